@@ -462,6 +462,27 @@ struct Cub {
         CK(cub::DeviceSelect::Unique(temp(b), b, in, out, num.p, (int)n, st));
         return read_num();
     }
+    // stable sort of (key, row) pairs ascending over bits [0, end_bit); the
+    // results end in k and v, k2 and v2 are scratch
+    void sort_pairs(dvec<uint64_t> &k, dvec<uint64_t> &k2, dvec<int32_t> &v, dvec<int32_t> &v2,
+                    int64_t n, int end_bit)
+    {
+        if (n <= 1) return;
+        cub::DoubleBuffer<uint64_t> dk(k.p, k2.p);
+        cub::DoubleBuffer<int32_t> dv(v.p, v2.p);
+        size_t b = 0;
+        CK(cub::DeviceRadixSort::SortPairs(nullptr, b, dk, dv, (int)n, 0, end_bit, st));
+        CK(cub::DeviceRadixSort::SortPairs(temp(b), b, dk, dv, (int)n, 0, end_bit, st));
+        if (dk.Current() != k.p) std::swap(k.p, k2.p);
+        if (dv.Current() != v.p) std::swap(v.p, v2.p);
+    }
+    template <class T>
+    void exclusive_sum(const T *in, T *out, int64_t n)
+    {
+        size_t b = 0;
+        CK(cub::DeviceScan::ExclusiveSum(nullptr, b, in, out, (int)n, st));
+        CK(cub::DeviceScan::ExclusiveSum(temp(b), b, in, out, (int)n, st));
+    }
     // runs of equal keys: unique values and lengths, copied to the host
     void rle(const uint64_t *in, int64_t n, std::vector<uint64_t> &uniq,
              std::vector<int32_t> &len)
@@ -482,6 +503,78 @@ struct Cub {
     }
 };
 
+// Sort key of every row for its sliced window: (window, longest first); rows of
+// more than kSellLong entries take the window after the last.
+constexpr int kSellKeyBits = 9;  // holds kSellLong - length, 0 .. kSellLong
+static_assert(kSellLong < (1 << kSellKeyBits), "row lengths of the sliced windows fit the key");
+__global__ void k_sell_keys(const int32_t *rp, int64_t n, Part part, int64_t nwin, uint64_t *key,
+                            int32_t *row)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t len = rp[i + 1] - rp[i];
+        const uint64_t w = len > kSellLong ? nwin : part.strided ? i / 1024 : part.owner(i);
+        key[i] = (w << kSellKeyBits) | (len > kSellLong ? 0 : kSellLong - len);
+        row[i] = (int32_t)i;
+    }
+}
+
+// A warp per window walks its sorted rows in steps of up to 32: lane l holds
+// the length of the l-th row from the chunk's first; the chunk ends before the
+// first row of less than half its length.  WRITE: the second pass, which
+// writes each chunk's entry and rows at the window's offsets; the first counts
+// chunks and slots (window nwin, the long rows, counts none and gives *first_long).
+template <bool WRITE>
+__global__ void k_sell_cut(const uint64_t *key, const int32_t *row, int64_t n, int64_t nwin,
+                           int64_t *nch, int64_t *nsl, const int64_t *och, const int64_t *osl,
+                           int2 *info, int32_t *perm, int64_t *first_long)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w <= nwin; w += warps) {
+        int64_t lim[2];  // the window's rows in the sorted order
+        for (int q = 0; q < 2; q++) {
+            int64_t lo = 0, hi = n;
+            const uint64_t x = (uint64_t)(w + q) << kSellKeyBits;
+            while (lo < hi) {
+                const int64_t mid = (lo + hi) >> 1;
+                if (key[mid] < x) lo = mid + 1;
+                else hi = mid;
+            }
+            lim[q] = lo;
+        }
+        if (w == nwin) {
+            if (!WRITE && lane == 0) {
+                nch[w] = nsl[w] = 0;
+                *first_long = lim[0];
+            }
+            continue;
+        }
+        int64_t c = WRITE ? och[w] : 0, slot = WRITE ? osl[w] : 0;
+        int64_t j = lim[0];
+        while (j < lim[1]) {
+            const bool in = j + lane < lim[1];
+            const int32_t len =
+                in ? kSellLong - (int32_t)(key[j + lane] & ((1u << kSellKeyBits) - 1)) : -1;
+            const int32_t width = __shfl_sync(0xffffffffu, len, 0);
+            const unsigned stop = __ballot_sync(0xffffffffu, !in || 2 * len < width);
+            const int nl = stop ? __ffs(stop) - 1 : 32;  // lane 0 never stops
+            if (WRITE) {
+                if (lane == 0) info[c] = make_int2((int)slot, (width << 6) | nl);
+                perm[32 * c + lane] = lane < nl ? row[j + lane] : -1;
+            }
+            // every chunk starts on a 4-slot (16-byte) boundary
+            slot += ((int64_t)width * nl + 3) & ~3ll;
+            c++;
+            j += nl;
+        }
+        if (!WRITE && lane == 0) {
+            nch[w] = c;
+            nsl[w] = slot;
+        }
+    }
+}
+
 // Sliced rows: one warp per chunk copies each lane's row into the chunk's
 // column-major slots (slot first + i * lanes + lane holds entry i of the
 // lane's row) and pads the slots past the row's end.
@@ -489,20 +582,21 @@ __global__ void k_sell_fill(const int32_t *rp, const uint32_t *col, const double
                             const float *val32, const int2 *info, const int32_t *perm,
                             int64_t nch, uint32_t *scol, double *sval, float *sval32)
 {
-    const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (c >= nch) return;
-    const int2 inf = info[c];
-    const int width = inf.y >> 6, nl = inf.y & 63;
-    if (lane >= nl) return;
-    const int row = perm[32 * c + lane];
-    const int k0 = rp[row], len = rp[row + 1] - k0;
-    for (int i = 0; i < width; i++) {
-        const int64_t q = (int64_t)inf.x + (int64_t)i * nl + lane;
-        const bool in = i < len;
-        scol[q] = in ? col[k0 + i] : kSellPad;
-        sval[q] = in ? val[k0 + i] : 0.0;
-        if (sval32) sval32[q] = in ? val32[k0 + i] : 0.0f;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < nch; c += warps) {
+        const int2 inf = info[c];
+        const int width = inf.y >> 6, nl = inf.y & 63;
+        if (lane >= nl) continue;
+        const int row = perm[32 * c + lane];
+        const int k0 = rp[row], len = rp[row + 1] - k0;
+        for (int i = 0; i < width; i++) {
+            const int64_t q = (int64_t)inf.x + (int64_t)i * nl + lane;
+            const bool in = i < len;
+            scol[q] = in ? col[k0 + i] : kSellPad;
+            sval[q] = in ? val[k0 + i] : 0.0;
+            if (sval32) sval32[q] = in ? val32[k0 + i] : 0.0f;
+        }
     }
 }
 
@@ -670,59 +764,60 @@ void host_stats(napspmv_plan_t *P)
 }
 
 // Sliced-row copy of one matrix part (which: 0 whole, 1 local, 2 remote) from
-// its CSR (host row pointer hrp, device arrays).  Windows: the rows of each
-// process (contiguous partition) or of each 1024-row block (strided).  Within
-// a window, rows of at most kSellLong entries are sorted by count, longest
-// first (ties by row), and cut into chunks of up to 32 whose counts are at
-// least half the first one's; longer rows are listed apart.  A part whose
-// padded slots would not fit 31-bit offsets is left without a sliced copy.
-void build_sell(napspmv_plan_t *P, int which, const std::vector<int32_t> &hrp,
-                const int32_t *d_rp, const uint32_t *d_col, const double *d_val,
-                const float *d_val32, const Part &part)
+// its CSR, built on the device.  Windows: the rows of each process (contiguous
+// partition) or of each 1024-row block (strided).  Within a window, rows of at
+// most kSellLong entries are sorted by count, longest first (ties by row), and
+// cut into chunks of up to 32 whose counts are at least half the first one's;
+// longer rows are listed apart.  A part whose padded slots would not fit 31-bit
+// offsets is left without a sliced copy.
+//
+// One radix sort of (window, length) keys orders every window at once; a warp
+// per window then cuts it, 32 rows to a step.  Sorting and cutting on the host
+// (a stable sort per window, three parts, and the upload of the row lists) took
+// most of a plan build: 41 of 56 ms of a 10^6-row 7-point plan on GB300, against 2.3 of
+// 17 ms this way (810 of 1,180 ms of the 2^23-row banded random plan, against 6 of 370).
+void build_sell(napspmv_plan_t *P, Cub &cb, int which, const int32_t *d_rp, const uint32_t *d_col,
+                const double *d_val, const float *d_val32, const Part &part)
 {
     SellPart &S = P->sell[which];
     const int64_t n = P->n;
-    std::vector<int2> info;
-    std::vector<int32_t> perm, lrows, ord;
-    int64_t slots = 0;
-    auto len = [&](int32_t r) { return hrp[r + 1] - hrp[r]; };
-    auto window = [&](int64_t r0, int64_t r1) {
-        ord.clear();
-        for (int64_t r = r0; r < r1; r++) {
-            if (len((int32_t)r) > kSellLong) lrows.push_back((int32_t)r);
-            else ord.push_back((int32_t)r);
-        }
-        std::stable_sort(ord.begin(), ord.end(),
-                         [&](int32_t a, int32_t b) { return len(a) > len(b); });
-        size_t j = 0;
-        while (j < ord.size()) {
-            const int32_t w = len(ord[j]);
-            size_t e = j + 1;
-            while (e < ord.size() && e - j < 32 && 2 * len(ord[e]) >= w) e++;
-            const int nl = (int)(e - j);
-            info.push_back(make_int2((int)std::min<int64_t>(slots, INT32_MAX), (w << 6) | nl));
-            for (int l = 0; l < 32; l++) perm.push_back(l < nl ? ord[j + l] : -1);
-            // every chunk starts on a 4-slot (16-byte) boundary: its column
-            // blocks are copied into shared memory with bulk copies
-            slots += ((int64_t)w * nl + 3) & ~3ll;
-            j = e;
-        }
-    };
-    if (part.strided) {
-        for (int64_t r0 = 0; r0 < n; r0 += 1024) window(r0, std::min<int64_t>(n, r0 + 1024));
-    } else {
-        for (int64_t r = 0; r < part.np; r++) window(part.start(r), part.start(r + 1));
-    }
+    const int64_t nwin = part.strided ? (n + 1023) / 1024 : part.np;
+    const int kb = kSellKeyBits + bits_for(nwin);
+    dvec<uint64_t> key(n), key2(n);
+    dvec<int32_t> row(n), row2(n);
+    k_sell_keys<<<blocks_for(n), 256>>>(d_rp, n, part, nwin, key.p, row.p);
+    CK(cudaGetLastError());
+    cb.sort_pairs(key, key2, row, row2, n, kb);
+    // per window: chunks and slots, then their exclusive sums (the last element
+    // is the total) and the first long row's position
+    dvec<int64_t> cnt(2 * (nwin + 1)), off(2 * (nwin + 1) + 1);
+    int64_t *nch = cnt.p, *nsl = cnt.p + nwin + 1, *och = off.p, *osl = off.p + nwin + 1;
+    const int wblocks = blocks_for(32 * (nwin + 1));
+    k_sell_cut<false><<<wblocks, 256>>>(key.p, row.p, n, nwin, nch, nsl, nullptr, nullptr, nullptr,
+                                        nullptr, off.p + 2 * (nwin + 1));
+    CK(cudaGetLastError());
+    cb.exclusive_sum(nch, och, nwin + 1);
+    cb.exclusive_sum(nsl, osl, nwin + 1);
+    int64_t tot[3];
+    CK(cudaMemcpy(&tot[0], och + nwin, sizeof(int64_t), cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(&tot[1], osl + nwin, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost));
+    const int64_t slots = tot[1];
     if (slots > (int64_t)INT32_MAX - 1024) {
         S.slots = -1;  // no sliced copy: NAPSPMV_PIPELINE_SELL is refused for this plan
         return;
     }
-    S.nch = (int64_t)info.size();
+    S.nch = tot[0];
     S.slots = slots;
-    S.n_long = (int32_t)lrows.size();
-    S.d_info = upload(info);
-    S.d_perm = upload(perm);
-    S.d_long = upload(lrows);
+    S.n_long = (int32_t)(n - tot[2]);
+    CK(cudaMalloc(&S.d_info, sizeof(int2) * std::max<int64_t>(S.nch, 1)));
+    CK(cudaMalloc(&S.d_perm, sizeof(int32_t) * 32 * std::max<int64_t>(S.nch, 1)));
+    CK(cudaMalloc(&S.d_long, sizeof(int32_t) * std::max<int64_t>(S.n_long, 1)));
+    if (S.n_long)
+        CK(cudaMemcpy(S.d_long, row.p + tot[2], sizeof(int32_t) * S.n_long,
+                      cudaMemcpyDeviceToDevice));
+    k_sell_cut<true><<<wblocks, 256>>>(key.p, row.p, n, nwin, nullptr, nullptr, och, osl, S.d_info,
+                                       S.d_perm, nullptr);
+    CK(cudaGetLastError());
     // padded past the last slot: a block's bulk copy is widened to 16 bytes
     auto al = [&](size_t sz) {
         void *q = nullptr;
@@ -1201,9 +1296,9 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
         for (int64_t i = 0; i <= n; i++) P->h_rowptr[i] = (int32_t)h[i];
     }
     // sliced-row copies of the whole matrix and of its two split parts
-    build_sell(P, 0, P->h_rowptr, P->d_rowptr, P->d_colenc, P->d_val, P->d_val32, part);
-    build_sell(P, 1, P->h_rowptrL, P->d_rowptrL, P->d_colL, P->d_valL, P->d_val32L, part);
-    build_sell(P, 2, P->h_rowptrR, P->d_rowptrR, P->d_colR, P->d_valR, P->d_val32R, part);
+    build_sell(P, cb, 0, P->d_rowptr, P->d_colenc, P->d_val, P->d_val32, part);
+    build_sell(P, cb, 1, P->d_rowptrL, P->d_colL, P->d_valL, P->d_val32L, part);
+    build_sell(P, cb, 2, P->d_rowptrR, P->d_colR, P->d_valR, P->d_val32R, part);
     CK(cudaDeviceSynchronize());
 
     host_stats(P);
