@@ -16,14 +16,15 @@
  *     (Sec. 2.1, Eqs. P, D) and the node-aware plan (Sec. 4.1, Eqs. N, E, T,
  *     U, G, I; Sec. 4.2, Eqs. L0/IL0, L1_send/IL1, L2/IL2), and the three-block
  *     CSR with each block's columns pointing into that block's receive buffer;
- *   - napspmv_apply runs, on the GPU, every message of the node-aware
- *     algorithm as a device gather or copy in HBM (on_node -> on_node and
+ *   - napspmv_apply runs, on the GPU, the messages of the node-aware
+ *     algorithm as device gathers and copies (on_node -> on_node and
  *     on_node -> off_node local exchanges, packing of g_send, the inter-node
  *     transfer g_send -> g_recv, the off_node -> on_node forwarding) and the
- *     three-block SpMV, for all simulated processes at once: by default as a
- *     CUDA graph of kernels in which the on_process part of the SpMV overlaps
- *     the message steps (NAPSPMV_ENGINE_OVERLAP), or in one persistent launch
- *     (NAPSPMV_ENGINE_FUSED).
+ *     three-block SpMV, for all simulated processes at once.  By default, for
+ *     matrices of short rows, in two passes: the inter-node messages go from
+ *     their owners to g_recv, and each block of a process's rows receives its
+ *     on-node and off-node values in the shared memory of the SM that sums
+ *     them.  The engines below run the steps one by one in HBM.
  *
  * Conventions for every call:
  *   - Return value: NAPSPMV_OK (0) or a negative NAPSPMV_ERR_* code; the
@@ -99,8 +100,8 @@ extern "C" {
 #define NAPSPMV_MAP_SPLIT (1u << 5)
 /* Composed gathers, an ablation with no counterpart in the paper: each
  * process's receive buffers are gathered straight from v (b_{l->l} as in the
- * on->on step, b_{nl->l} from the owners' values), skipping the on->off
- * gather, pack, transfer and off->on hops of Algorithm NAPSpMV.  The plan and
+ * on->on step, b_{nl->l} from the owners' values), skipping the hops of
+ * the inter-node exchange (on->off gather, pack, transfer, off->on).  The plan and
  * its statistics are unchanged; the result has the same bits as the literal
  * exchange.  Every engine, batches and the no-allocation entry run such
  * plans. */
@@ -110,6 +111,14 @@ extern "C" {
 #define NAPSPMV_PREC_F64 0 /* FP64 values, FP64 products and sums            */
 #define NAPSPMV_PREC_F32 1 /* FP32-stored values, FP32 products, FP64 sums   */
 
+/* With engine, pipeline, vec, tile_rows, tile_nnz, stages and halo all unset
+ * (engine PHASED alone counts as unset), a plan whose rows average at most 12
+ * entries runs on staged windows: every process's rows are cut into blocks, a
+ * CTA brings the values its block multiplies into shared memory, each once, and
+ * sums its sliced rows from there (the bits of vec = 1).  Such a plan needs at
+ * least 64 rows per process on average, no row of more than 256 entries and no
+ * composed gathers; others, and plans whose defaults napspmv_set_default_opts
+ * has set, run the engine and pipeline that napspmv_get_default_opts reports. */
 #define NAPSPMV_ENGINE_DEFAULT 0 /* the plan's default engine               */
 #define NAPSPMV_ENGINE_FUSED 1   /* one persistent, cooperative launch for all
                                     phases and all chained applies, in levels

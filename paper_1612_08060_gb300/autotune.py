@@ -104,6 +104,13 @@ def tune(plan, row_ptr, precision=nap.PREC_F64, reps=20, max_sweeps=2, cache_fil
             return float("inf")
 
     best_ms = measure(cur)
+    # sliced rows on the phased engine (with staged windows where the plan has
+    # them) are two options away from a tile pipeline: try the pair as a start
+    if nap.ENGINE_PHASED in CANDIDATES["engine"] and nap.PIPELINE_SELL in CANDIDATES.get("pipeline", ()):
+        trial = dict(cur, engine=nap.ENGINE_PHASED, pipeline=nap.PIPELINE_SELL)
+        ms = measure(trial)
+        if ms < best_ms:
+            best_ms, cur = ms, trial
     for _ in range(max_sweeps):
         improved = False
         for k, cands in CANDIDATES.items():

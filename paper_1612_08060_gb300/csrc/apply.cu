@@ -23,8 +23,12 @@
 // issue, not only HBM, bounds the SpMV on GB300).  Stages are sized to each
 // tile list's largest tile; tiles are handed to CTAs in contiguous runs.
 //
+// Staged windows (default for rows of at most 12 entries; k_send and k_window):
+// phases 1 to 3 of the inter-node messages in one pass, and the on_node and
+// off_node receives inside the SpMV's CTAs.
+//
 // Engines:
-//   overlapped (default for rows of at most 12 entries)  the matrix split into
+//   overlapped (for rows of at most 12 entries without windows)  the matrix split into
 //       its on_process part (local, needs no message) and its remote part; the
 //       local pass runs on a second stream while the message steps run, the
 //       remote pass continues each row's FMA chain from the local partial.
@@ -305,6 +309,20 @@ __device__ __forceinline__ double f32_product(float a, XT xv)
     if constexpr (sizeof(XT) == 4) xf = xv;
     else xf = d2f_rn(xv);
     return f2d_exact(__fmul_rn(a, xf));
+}
+// 0.0 + the widened product: the product itself, without an FP64 addition, unless
+// it is zero (0.0 + -0.0 is 0.0), subnormal, infinite or NaN.
+template <class XT>
+__device__ __forceinline__ double f32_first(float a, XT xv)
+{
+    float xf;
+    if constexpr (sizeof(XT) == 4) xf = xv;
+    else xf = d2f_rn(xv);
+    const float p = __fmul_rn(a, xf);
+    const uint32_t u = __float_as_uint(p), m = u & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(m << 29));
+    return __dadd_rn(0.0, f2d_exact(p));
 }
 template <bool F32, class XT>
 __device__ __forceinline__ double entry_add(double acc, const double *val, const float *val32,
@@ -1171,6 +1189,206 @@ __global__ void __launch_bounds__(32 * W, W == 8 ? (U >= 8 ? 4 : 6) : 1)
     griddep_done();
 }
 
+// --------------------------------------------------- staged-window SpMV
+// One CTA per block of a process's rows.  The CTA first brings the block's
+// window into shared memory: the vector entries its rows own, its on-node
+// receives (Eq. IL2) gathered from x and its off-node receives (Eq. IL1)
+// gathered from g_recv, each once; then it sums its sliced rows, one lane per
+// row in stored order, with every operand in shared memory.  b_{l->l} and
+// b_{nl->l} thus live in the SM that uses them.
+//
+// The block's runs, columns and values are constant plan data, each contiguous:
+// three bulk copies bring them into shared memory at the start, before the wait
+// for the previous kernel.  The window is gathered, and the rows are summed from
+// shared memory alone.  So a CTA passes through three memory latencies whatever
+// its size, and the CTAs that share an SM overlap one another's copies and sums.
+//
+// Bound by HBM with FP64 values (3D 7-point 128^3: 197 MB of DRAM in about 34 us,
+// 0.85 of the measured copy peak; 2-byte columns, 13 bytes of runs per 32 window
+// values, no row pointers) and by the FP64 pipe with FP32 values (Q1 2048^2: 74 us,
+// the pipe 72% busy with one DADD per entry but the first).  Per apply on GB300, against
+// the overlapped engine before it: 39.8 for 85.0 us, 75 for 130 us, and 60 for 154 us
+// on a strided 101^3.  Tried on 128^3: columns and values read from global memory by
+// each lane (512-row blocks), 85 us for this kernel alone, one latency after another;
+// 4- and 8-byte asynchronous copies in place of loads for the window, 66 for 61 us on
+// the strided plan; source lists in place of runs, 44.6 for 42.6 us per apply; 40
+// registers in place of 32, 42.6 us per apply; two threads per row, 60.7 us.
+struct WinView {
+    const WinBlock *blk;
+    const int2 *info;
+    const int32_t *perm;
+    const uint16_t *col;
+    const double *val;
+    const float *val32;
+    const uint32_t *runs;
+    int32_t cap_src, cap_slots, cap_words;  // largest block, multiples of 8, 8 and 4
+};
+
+// Shared memory of a CTA: two mbarriers, values, window, runs, columns.
+struct WinLayout {
+    int val, win, runs, col, bytes;
+};
+__host__ __device__ __forceinline__ WinLayout win_layout(int cap_src, int cap_slots, int cap_words,
+                                                         int vb)
+{
+    WinLayout L;
+    L.val = 32;
+    L.win = L.val + vb * cap_slots;
+    L.runs = L.win + vb * cap_src;
+    L.col = L.runs + 4 * cap_words;
+    L.bytes = L.col + 2 * cap_slots;
+    return L;
+}
+
+constexpr int kWinG = 4;  // window values in flight per thread
+constexpr int kWinThreads = 512;  // at most
+// STEP: on-node values come from b_{l->l} (napspmv_spmv_step).
+template <bool F32, bool STEP>
+__global__ void __launch_bounds__(kWinThreads, 4)
+    k_window(const __grid_constant__ WinView S, const void *xs, const void *gs, const void *ls,
+             double *y, float *y32, const Scale sc, int *err)
+{
+    using XT = typename std::conditional<F32, float, double>::type;
+    const XT *x = static_cast<const XT *>(xs), *g = static_cast<const XT *>(gs),
+             *l = static_cast<const XT *>(ls);
+    extern __shared__ __align__(16) unsigned char smem[];
+    const WinLayout L = win_layout(S.cap_src, S.cap_slots, S.cap_words, sizeof(XT));
+    TileStage lists{}, entries{};  // their mbarriers
+    lists.bar = reinterpret_cast<uint64_t *>(smem);
+    entries.bar = reinterpret_cast<uint64_t *>(smem + 16);
+    XT *val = reinterpret_cast<XT *>(smem + L.val), *win = reinterpret_cast<XT *>(smem + L.win);
+    uint32_t *runs = reinterpret_cast<uint32_t *>(smem + L.runs);
+    uint16_t *col = reinterpret_cast<uint16_t *>(smem + L.col);
+    const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, lane = tid & 31;
+    const WinBlock B = S.blk[blockIdx.x];
+    if (tid == 0) {
+        mbar_init(lists.bar, 1);
+        mbar_init(entries.bar, 1);
+        fence_barrier_init();
+        const uint32_t nrun = 4 * (uint32_t)B.words, nslot = (uint32_t)B.slots;
+        mbar_expect_tx(lists.bar, nrun);
+        if (nrun) bulk_g2s(runs, S.runs + 4 * (int64_t)B.word0, nrun, lists.bar);
+        mbar_expect_tx(entries.bar, nslot * (2 + (uint32_t)sizeof(XT)));
+        if (nslot) {
+            bulk_g2s(col, S.col + B.slot0, 2 * nslot, entries.bar);
+            if (F32) bulk_g2s(val, S.val32 + B.slot0, 4 * nslot, entries.bar);
+            else bulk_g2s(val, S.val + B.slot0, 8 * nslot, entries.bar);
+        }
+    }
+    // the warp's first chunk
+    int c = B.chunk0 + warp;
+    const int c1 = B.chunk0 + B.chunks;
+    int2 inf = c < c1 ? S.info[c] : make_int2(0, 0);
+    int row = c < c1 ? S.perm[32 * c + lane] : -1;
+    __syncthreads();  // the mbarriers are set up
+    bool ok = tile_wait(lists, 0, err);
+    griddep_wait();
+    // sticky error: no work until cleared (but the copies in flight land first)
+    ok = ok && !*(volatile const int *)err;
+    if (ok) {
+        const int tiles = (B.srcs + 31) >> 5, nw = nt >> 5;
+        const uint2 *head = reinterpret_cast<const uint2 *>(runs);
+        const uint32_t *first = runs + 2 * tiles;
+        for (int t0 = warp; t0 < tiles; t0 += kWinG * nw) {
+            XT v[kWinG];
+#pragma unroll
+            for (int u = 0; u < kWinG; u++) {
+                const int t = t0 + u * nw;
+                if (32 * t + lane >= B.srcs) continue;
+                const uint2 h = head[t];
+                const uint32_t m = h.x & (0xffffffffu >> (31 - lane));  // run starts up to this slot
+                const uint32_t s = first[h.y + __popc(m) - 1] + (lane - (31 - __clz(m)));
+                const XT *p = (s & kFromRecv) ? g + (s & ~kFromRecv) : x + s;
+                if (STEP && (s & (kFromRecv | kFromBll)) == kFromBll) p = l + (s & ~kFromBll);
+                v[u] = __ldg(p);
+            }
+#pragma unroll
+            for (int u = 0; u < kWinG; u++) {
+                const int k = 32 * (t0 + u * nw) + lane;
+                if (k < B.srcs) win[k] = v[u];
+            }
+        }
+    }
+    __syncthreads();
+    ok = tile_wait(entries, 0, err) && ok;
+    if (!ok) return;
+    while (c < c1) {
+        const int width = inf.y >> 6, nl = inf.y & 63;
+        if (lane < nl) {
+            double acc = 0.0;
+            int q = inf.x - B.slot0 + lane, i = 0;
+            if (F32 && width > 0 && col[q] != kWinPad) {
+                acc = f32_first(val[q], win[col[q]]);
+                i = 1;
+                q += nl;
+            }
+#pragma unroll 4
+            for (; i < width; i++, q += nl) {
+                const uint16_t cc = col[q];
+                if (cc == kWinPad) break;  // the padding ends the row
+                if constexpr (F32) acc = __dadd_rn(acc, f32_product(val[q], win[cc]));
+                else acc = fma(val[q], win[cc], acc);
+            }
+            const double r = apply_scale(acc, sc);
+            if (!F32 || y) y[row] = r;
+            if (F32 && y32) y32[row] = d2f_rn(r);
+        }
+        c += nt >> 5;
+        if (c < c1) {
+            inf = S.info[c];
+            row = S.perm[32 * c + lane];
+        }
+    }
+    griddep_done();
+}
+
+// Phases 1 (on_node -> off_node), 2 and 3 in one pass: element k of g_send, on
+// its way through the aggregator's buffer and g_send a register, goes from the
+// owner's x[j[k]] to its place in g_recv.  A warp moves groups of kSendGroup
+// elements, two at a time; within one message the places are consecutive, so a
+// group inside a message needs one number, its shift (kMixed: it crosses
+// messages, and every element's place is read).  Bound by the SM's sector loads: a gathered 8-byte value
+// costs up to a 32-byte sector.  Against the gather, pack and transfer kernels, 35.6 us
+// of 128^3, 9.3 us (GB300, cold, on their own).
+constexpr int kSendWarps = NT / 32;
+template <class T>
+__global__ void __launch_bounds__(NT)
+    k_send(const T *x, const int32_t *j, const int32_t *dst, const int32_t *shift, T *grecv, int n,
+           const int *err)
+{
+    constexpr int U = 2 * kSendGroup / 32;
+    if (*(volatile const int *)err) return;
+    const uint64_t pol = policy_evict_first();
+    const int lane = threadIdx.x & 31;
+    const int step = gridDim.x * kSendWarps * 2 * kSendGroup;
+    for (int b = (blockIdx.x * kSendWarps + (threadIdx.x >> 5)) * 2 * kSendGroup; b < n; b += step) {
+        int32_t ix[U], to[U];
+        T v[U];
+        const int32_t s0 = __ldg(shift + b / kSendGroup);
+        const int32_t s1 = b + kSendGroup < n ? __ldg(shift + b / kSendGroup + 1) : 0;
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int k = b + 32 * u + lane;
+            if (k < n) ix[u] = ld_stream_hint_s32(j + k, pol);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int k = b + 32 * u + lane;
+            const int32_t s = u < U / 2 ? s0 : s1;
+            to[u] = k + s;
+            if (s == kMixed && k < n) to[u] = ld_stream_hint_s32(dst + k, pol);
+        }
+        griddep_wait();
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (b + 32 * u + lane < n) v[u] = __ldg(x + ix[u]);
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (b + 32 * u + lane < n) grecv[to[u]] = v[u];
+    }
+    griddep_done();
+}
+
 // ---------------------------------------------------------- fused engine
 // One persistent, cooperative launch for every chained apply of one or more
 // independent jobs (a batch).  Each apply runs in five levels separated by
@@ -1422,22 +1640,33 @@ struct FusedKernelTable {
 
 static bool valid_vec(int v) { return v == 1 || v == 2 || v == 4 || v == 8 || v == 16 || v == 32; }
 
-napspmv_opts resolve_opts(const napspmv_plan_t *P, const napspmv_opts *o)
+bool leaves_path_open(const napspmv_opts &o)
 {
-    napspmv_opts r = P->defaults;
-    if (!o) return r;
-    r.precision = o->precision;  // 0 is FP64, a real choice
-    if (o->engine) r.engine = o->engine;
-    if (o->vec) r.vec = o->vec;
-    if (o->ctas_per_sm) r.ctas_per_sm = o->ctas_per_sm;
-    if (o->chunk) r.chunk = o->chunk;
-    if (o->tile_rows) r.tile_rows = o->tile_rows;
-    if (o->tile_nnz) r.tile_nnz = o->tile_nnz;
-    if (o->stages) r.stages = o->stages;
-    if (o->pipeline) r.pipeline = o->pipeline;
-    if (o->halo) r.halo = o->halo;
-    if (o->timeout_ms) r.timeout_ms = o->timeout_ms;
-    r.debug_stall = o->debug_stall;
+    return (!o.engine || o.engine == NAPSPMV_ENGINE_PHASED) && !o.pipeline && !o.vec &&
+           !o.tile_rows && !o.tile_nnz && !o.stages && !o.halo;
+}
+
+Opts resolve_opts(const napspmv_plan_t *P, const napspmv_opts *o)
+{
+    Opts r;
+    static_cast<napspmv_opts &>(r) = P->defaults;
+    if (o) {
+        r.precision = o->precision;  // 0 is FP64, a real choice
+        if (o->engine) r.engine = o->engine;
+        if (o->vec) r.vec = o->vec;
+        if (o->ctas_per_sm) r.ctas_per_sm = o->ctas_per_sm;
+        if (o->chunk) r.chunk = o->chunk;
+        if (o->tile_rows) r.tile_rows = o->tile_rows;
+        if (o->tile_nnz) r.tile_nnz = o->tile_nnz;
+        if (o->stages) r.stages = o->stages;
+        if (o->pipeline) r.pipeline = o->pipeline;
+        if (o->halo) r.halo = o->halo;
+        if (o->timeout_ms) r.timeout_ms = o->timeout_ms;
+        r.debug_stall = o->debug_stall;
+    }
+    r.window = P->win.blocks > 0 &&
+               ((P->auto_window && (!o || leaves_path_open(*o))) ||
+                (r.engine == NAPSPMV_ENGINE_PHASED && r.pipeline == NAPSPMV_PIPELINE_SELL));
     return r;
 }
 
@@ -1738,6 +1967,7 @@ static int launch_fused(int count, napspmv_plan_t *const *plans, napspmv_ws_t *c
             prm.off[l][i] = acc[l];
             acc[l] += prm.jobs[i].nunits[l];
         }
+        wi->bnl_stale = false;
         wi->buf_f32 = 0;  // this engine's receive buffers hold FP64 values in both modes
     }
     for (int l = 0; l < kLevels; l++) prm.off[l][count] = acc[l];
@@ -2116,9 +2346,115 @@ static int64_t enqueue_composed(const napspmv_plan_t *P, const void *x, napspmv_
     return 1;
 }
 
-static int enqueue_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, double *w, int reps,
-                          double scale, const napspmv_opts &o, cudaStream_t s, int64_t *kernels)
+using WinKernel = void (*)(const WinView, const void *, const void *, const void *, double *,
+                           float *, const Scale, int *);
+static WinKernel pick_window(bool f32, bool step)
 {
+    if (f32) return step ? k_window<true, true> : k_window<true, false>;
+    return step ? k_window<false, true> : k_window<false, false>;
+}
+int window_bytes(int64_t srcs, int64_t slots, int64_t words, int vb)
+{
+    return win_layout((int)((srcs + 7) & ~7ll), (int)((slots + 7) & ~7ll), (int)words, vb).bytes;
+}
+// What the launches of the staged windows need to know, taken once per plan.
+int window_prepare(napspmv_plan_t *P)
+{
+    if (!P->win.blocks) return NAPSPMV_OK;
+    for (int q = 0; q < 4; q++)
+        NAP_CUDA(cudaFuncSetAttribute((const void *)pick_window(q & 1, q & 2),
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, kWinSmem));
+    P->win.wave_gather[0] = one_wave(P, k_unpack<double>);
+    P->win.wave_gather[1] = one_wave(P, k_unpack<float>);
+    P->win.wave_send[0] = one_wave(P, k_send<double>);
+    P->win.wave_send[1] = one_wave(P, k_send<float>);
+    return NAPSPMV_OK;
+}
+// The SpMV over the staged windows; g, l: g_recv and b_{l->l} (step only).
+static int window_run(const napspmv_plan_t *P, const Opts &o, bool step, const void *x,
+                      const void *g, const void *l, double *y, float *y32, double scale,
+                      int *err, cudaStream_t s, bool pdl)
+{
+    const bool f32 = o.precision == NAPSPMV_PREC_F32;
+    const WinKernel fn = pick_window(f32, step);
+    const WinPart &W = P->win;
+    const SellPart &SP = P->sell[0];
+    const WinView V{W.d_blk[step], SP.d_info,        SP.d_perm,          W.d_col,
+                    SP.d_val,      SP.d_val32,       W.d_runs[step],     (W.max_src + 7) & ~7,
+                    (W.max_slots + 7) & ~7, W.max_words[step]};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)W.blocks);
+    cfg.blockDim = dim3((unsigned)W.threads);
+    cfg.dynamicSmemBytes = (size_t)window_bytes(W.max_src, W.max_slots, W.max_words[step], f32 ? 4 : 8);
+    if (o.ctas_per_sm > 0) {
+        // at most that many CTAs per SM: each takes its share of the 227 KB
+        const size_t share = 227 * 1024 / (size_t)o.ctas_per_sm;
+        if (share > 1024) cfg.dynamicSmemBytes = std::max(cfg.dynamicSmemBytes, share - 1024);
+    }
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    NAP_CUDA(cudaLaunchKernelEx(&cfg, fn, V, x, g, l, y, y32, make_scale(scale), err));
+    return NAPSPMV_OK;
+}
+
+// Applies on the staged windows: the inter-node messages from their owners to
+// g_recv in one pass, then the windowed SpMV, whose CTAs receive the on-node
+// and off-node values themselves.  The last apply of the chain also fills
+// b_{l->l}, which napspmv_spmv_step reads.
+template <class T>
+static int enqueue_window(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, double *w, int reps,
+                          double scale, const Opts &o, cudaStream_t s, int64_t *kernels)
+{
+    constexpr bool f32 = sizeof(T) == 4;
+    T *grecv = reinterpret_cast<T *>(ws->grecv), *bll = reinterpret_cast<T *>(ws->bll);
+    int64_t nk = 0;
+    if (f32) {
+        const int g = (int)std::max<int64_t>(1, std::min<int64_t>((P->n + NT * 8 - 1) / (NT * 8),
+                                                                  (int64_t)P->num_sms * 8));
+        launch_pdl(true, k_to_f32, g, 0, s, v, ws->x32[0], (int64_t)P->n, (const int *)ws->err);
+        nk++;
+    }
+    for (int k = 0; k < reps; k++) {
+        const bool last = k + 1 == reps;
+        const double *x = (k == 0) ? v : (((reps - k) & 1) == 0 ? w : ws->xtmp);
+        double *y = (((reps - 1 - k) & 1) == 0) ? w : ws->xtmp;
+        const T *xs = f32 ? reinterpret_cast<const T *>(ws->x32[k & 1])
+                          : reinterpret_cast<const T *>(x);
+        // FP32 mode: the next apply reads the FP32 copy only
+        float *y32 = f32 && !last ? ws->x32[(k + 1) & 1] : nullptr;
+        if (last && P->n_bll > 0) {
+            launch_pdl(true, k_unpack<T>, msg_grid(P, P->n_bll, P->win.wave_gather[f32]), 0, s, xs,
+                       (const int32_t *)P->lists[L_BLL].d_idx, bll, (int)P->n_bll,
+                       (const int *)ws->err);
+            nk++;
+        }
+        if (P->n_gs > 0) {
+            launch_pdl(true, k_send<T>, msg_grid(P, P->n_gs, P->win.wave_send[f32]), 0, s, xs,
+                       (const int32_t *)P->lists[L_INTER].d_idx, (const int32_t *)P->d_xfer_dst,
+                       (const int32_t *)P->d_xfer_shift, grecv, (int)P->n_gs, (const int *)ws->err);
+            nk++;
+        }
+        if (int rc = window_run(P, o, false, xs, grecv, nullptr, f32 && !last ? nullptr : y, y32,
+                                scale, ws->err, s, true))
+            return rc;
+        nk++;
+        NAP_CUDA(cudaGetLastError());
+    }
+    *kernels = nk;
+    return NAPSPMV_OK;
+}
+
+static int enqueue_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, double *w, int reps,
+                          double scale, const Opts &o, cudaStream_t s, int64_t *kernels)
+{
+    if (o.window)
+        return o.precision == NAPSPMV_PREC_F32
+                   ? enqueue_window<float>(P, ws, v, w, reps, scale, o, s, kernels)
+                   : enqueue_window<double>(P, ws, v, w, reps, scale, o, s, kernels);
     auto grid = [&](int64_t n) {
         return (int)std::max<int64_t>(1, std::min<int64_t>((n + NT * 8 - 1) / (NT * 8),
                                                             (int64_t)P->num_sms * 8));
@@ -2141,7 +2477,6 @@ static int enqueue_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, 
                    (const int *)ws->err);
         nk++;
     }
-    ws->buf_f32 = f32 ? 1 : 0;
     for (int k = 0; k < reps; k++) {
         const double *x = (k == 0) ? v : (((reps - k) & 1) == 0 ? w : ws->xtmp);
         double *y = (((reps - 1 - k) & 1) == 0) ? w : ws->xtmp;
@@ -2189,9 +2524,9 @@ static int enqueue_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, 
 // Chained applies on a capturable stream are recorded once into a CUDA graph
 // per (vectors, workspace, reps, scale, options) and replayed afterwards.
 static int launch_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, double *w, int reps,
-                         double scale, const napspmv_opts &o, cudaStream_t s)
+                         double scale, const Opts &o, cudaStream_t s)
 {
-    {
+    if (!o.window) {
         // attributes (dynamic shared memory) are set before any capture
         SpmvLaunch L;
         if (int rc = spmv_launch(P, o, kFull, L)) return rc;
@@ -2203,6 +2538,10 @@ static int launch_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, d
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     NAP_CUDA(cudaStreamIsCapturing(s, &cs));
     const bool use_graph = reps > 1 && s != nullptr && cs == cudaStreamCaptureStatusNone;
+    // what the workspace's receive buffers hold from now on
+    ws->buf_f32 = o.precision == NAPSPMV_PREC_F32 ? 1 : 0;
+    ws->bnl_stale = o.window;
+    if (o.window && cs != cudaStreamCaptureStatusNone) ws->bnl_captured = true;
     int64_t nk = 0;
     if (!use_graph) {
         int rc = enqueue_phased(P, ws, v, w, reps, scale, o, s, &nk);
@@ -2211,7 +2550,7 @@ static int launch_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, d
     }
     for (size_t i = 0; i < P->graphs.size(); i++) {
         auto &g = P->graphs[i];
-        if (g.v == v && g.w == w && g.ws == ws && g.reps == reps && g.scale == scale &&
+        if (g.v == v && g.w == w && g.ws == ws && g.window == o.window && g.reps == reps && g.scale == scale &&
             g.prec == o.precision && g.vec == o.vec && g.tile_rows == o.tile_rows &&
             g.tile_nnz == o.tile_nnz && g.engine == o.engine && g.stages == o.stages &&
             g.pipeline == o.pipeline && g.ctas_per_sm == o.ctas_per_sm && g.halo == o.halo) {
@@ -2237,7 +2576,7 @@ static int launch_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, d
         cudaGraphExecDestroy(P->graphs.front().exec);
         P->graphs.erase(P->graphs.begin());
     }
-    P->graphs.push_back({v, w, ws, reps, o.precision, o.vec, o.tile_rows, o.tile_nnz, o.engine,
+    P->graphs.push_back({v, w, ws, o.window, reps, o.precision, o.vec, o.tile_rows, o.tile_nnz, o.engine,
                          o.stages, o.pipeline, o.ctas_per_sm, o.halo, scale, exec, nk});
     NAP_CUDA(cudaGraphLaunch(exec, s));
     count_launch(nk);
@@ -2325,7 +2664,7 @@ int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const
     }
     // every entry resolves the unset fields against its own plan's defaults,
     // so that it runs with the row tiles its plan already holds
-    napspmv_opts oi[64];
+    Opts oi[64];
     int cur = 0;
     NAP_CUDA(cudaGetDevice(&cur));
     if (cur != P0->device) NAP_CUDA(cudaSetDevice(P0->device));
@@ -2345,7 +2684,10 @@ int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const
         oi[i] = resolve_opts(P, opts);
         // several entries share fused launches, whatever engine the options name:
         // validate them for that engine
-        if (count > 1) oi[i].engine = NAPSPMV_ENGINE_FUSED;
+        if (count > 1) {
+            oi[i].engine = NAPSPMV_ENGINE_FUSED;
+            oi[i].window = false;
+        }
         if ((rc = check_opts(P, oi[i]))) break;
         if ((rc = build_items(P, oi[i].tile_rows, oi[i].tile_nnz))) break;
         for (int q = 0; q < i; q++) {
@@ -2363,8 +2705,8 @@ int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const
         }
     }
     if (!rc && count == 1) {
-        const napspmv_opts &o = oi[0];
-        if (o.engine == NAPSPMV_ENGINE_PHASED || o.engine == NAPSPMV_ENGINE_OVERLAP)
+        const Opts &o = oi[0];
+        if (o.window || o.engine == NAPSPMV_ENGINE_PHASED || o.engine == NAPSPMV_ENGINE_OVERLAP)
             rc = launch_phased(P0, ws && ws[0] ? ws[0] : P0->ws, v[0], w[0], reps[0],
                                scale ? scale[0] : 1.0, o, s);
         else
@@ -2526,7 +2868,7 @@ extern "C" int napspmv_spmv_step(napspmv_plan_t *P, napspmv_ws_t *ws, const doub
         return NAPSPMV_ERR_ARG;
     }
     napspmv_ws_t *W = ws ? ws : P->ws;
-    napspmv_opts o = resolve_opts(P, opts);
+    const Opts o = resolve_opts(P, opts);
     int rc = check_opts(P, o);
     if (rc) return rc;
     int cur = 0;
@@ -2543,15 +2885,40 @@ extern "C" int napspmv_spmv_step(napspmv_plan_t *P, napspmv_ws_t *ws, const doub
         return NAPSPMV_ERR_STATE;
     }
     SpmvLaunch L;
-    if ((rc = spmv_launch(P, o, kFull, L))) return rc;
+    if (!o.window) {
+        if ((rc = spmv_launch(P, o, kFull, L))) return rc;
+        if ((W->bnl_stale || W->bnl_captured) && P->n_bnl > 0) {
+            // the last apply kept b_{nl->l} on chip: unpack it from g_recv
+            const cudaStream_t st = (cudaStream_t)stream;
+            if (f32)
+                launch_pdl(false, k_unpack<float>, msg_grid(P, P->n_bnl, one_wave(P, k_unpack<float>)),
+                           0, st, reinterpret_cast<const float *>(W->grecv),
+                           (const int32_t *)P->d_unp_src, reinterpret_cast<float *>(W->bnl),
+                           (int)P->n_bnl, (const int *)W->err);
+            else
+                launch_pdl(false, k_unpack<double>,
+                           msg_grid(P, P->n_bnl, one_wave(P, k_unpack<double>)), 0, st,
+                           (const double *)W->grecv, (const int32_t *)P->d_unp_src, W->bnl,
+                           (int)P->n_bnl, (const int *)W->err);
+            count_launch(1);
+            W->bnl_stale = false;
+        }
+    }
+    auto step = [&](const void *x) -> int {
+        if (o.window)
+            return window_run(P, o, true, x, W->grecv, W->bll, w, nullptr, scale, W->err,
+                              (cudaStream_t)stream, true);
+        spmv_run(L, x, W, w, nullptr, scale, o.stages, (cudaStream_t)stream, pdl);
+        return NAPSPMV_OK;
+    };
     if (f32) {
         const int g = (int)std::max<int64_t>(1, std::min<int64_t>((P->n + NT - 1) / NT,
                                                                   (int64_t)P->num_sms * 8));
         k_to_f32<<<g, NT, 0, (cudaStream_t)stream>>>(v, W->x32[0], P->n, W->err);
-        spmv_run(L, W->x32[0], W, w, nullptr, scale, o.stages, (cudaStream_t)stream, pdl);
+        if ((rc = step(W->x32[0]))) return rc;
         count_launch(2);
     } else {
-        spmv_run(L, v, W, w, nullptr, scale, o.stages, (cudaStream_t)stream, pdl);
+        if ((rc = step(v))) return rc;
         count_launch(1);
     }
     NAP_CUDA(cudaGetLastError());

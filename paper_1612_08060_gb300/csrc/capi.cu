@@ -208,7 +208,7 @@ int napspmv_get_default_opts(const napspmv_plan_t *P, napspmv_opts *out)
 int napspmv_set_default_opts(napspmv_plan_t *P, const napspmv_opts *opts)
 {
     if (!P || !opts) return arg_error("NULL plan or opts");
-    napspmv_opts o = resolve_opts(P, opts);
+    Opts o = resolve_opts(P, opts);
     o.debug_stall = 0;
     // every field is checked before it becomes a default (a bad timeout or
     // stage count would otherwise reach the kernels of later applies)
@@ -220,6 +220,7 @@ int napspmv_set_default_opts(napspmv_plan_t *P, const napspmv_opts *opts)
     if (cur != P->device) cudaSetDevice(cur);
     if (rc) return rc;
     P->defaults = o;
+    if (!leaves_path_open(*opts)) P->auto_window = false;
     return NAPSPMV_OK;
 }
 

@@ -36,6 +36,10 @@ constexpr uint32_t kIndexMask = (1u << 30) - 1;
 // A pack source with the top bit set reads the aggregator buffer b_{l->nl},
 // otherwise v.
 constexpr uint32_t kFromLbuf = 0x80000000u;
+// Groups of consecutive elements of g_send whose transfer destinations share one
+// shift from their positions; kMixed: they do not.
+constexpr int kSendGroup = 128;
+constexpr int32_t kMixed = INT32_MIN;
 
 // ------------------------------------------------- row tiles (CTA and warp)
 enum ItemKind : int32_t {
@@ -105,6 +109,42 @@ struct SellPart {
     int32_t *d_long = nullptr;  // rows of more than kSellLong entries
 };
 
+// ------------------------------------------------------ staged windows
+// Each process's rows are cut into blocks of `rows` rows, one CTA each.  A
+// block's window lists, once each, the values its rows multiply: own vector
+// entries, on-node receives (b_{l->l}) and off-node receives (b_{nl->l}), in
+// that order.  The CTA brings the window into shared memory (phase 4, and phase
+// 1's on-node part) and sums its sliced rows from there; the whole matrix's
+// sliced rows are sorted and cut per block, and stored entry s multiplies
+// window slot col[s].
+// Where the window's values come from is kept as runs.  For every 32 slots: a
+// mask of the slots that start a run (the first always does) and the index of
+// its first run, as two words; after them the source of every run's first slot.
+// Stencil windows are a few contiguous pieces, so this is about 13 bytes per 32
+// values instead of 128.
+constexpr uint16_t kWinPad = 0xffff;      // padding slots, as kSellPad
+constexpr uint32_t kFromRecv = 0x80000000u;  // source in g_recv, else in x
+constexpr uint32_t kFromBll = 0x40000000u;   // (step sources) source in b_{l->l}
+struct WinBlock {
+    int32_t chunk0, chunks;  // its chunks of the whole matrix's sliced rows
+    int32_t slot0, slots;    // its stored-entry slots
+    int32_t srcs;            // window slots
+    int32_t words, word0;    // its runs: words (a multiple of 4), and the first / 4
+    int32_t pad;
+};
+struct WinPart {
+    int32_t blocks = 0;   // 0: the plan has no windows
+    int32_t rows = 0;     // rows per block (a multiple of 32)
+    int32_t threads = 0;  // per CTA
+    // largest block: window slots, entry slots, run words (apply, step)
+    int32_t max_src = 0, max_slots = 0, max_words[2] = {};
+    int64_t wave_gather[2] = {}, wave_send[2] = {};  // CTAs the GPU holds at once (FP64, FP32)
+    uint16_t *d_col = nullptr;  // window slot of every sliced-row slot
+    // for an apply, and for a step with on-node values from b_{l->l}
+    WinBlock *d_blk[2] = {};
+    uint32_t *d_runs[2] = {};
+};
+
 }  // namespace nap
 
 struct napspmv_ws_s {
@@ -117,6 +157,9 @@ struct napspmv_ws_s {
     // read as float arrays)
     float *x32[2] = {nullptr, nullptr};
     int buf_f32 = 0;
+    // the staged windows leave b_{nl->l} in shared memory only: the buffer here is
+    // behind g_recv (stale), for good once such an apply was captured by the caller
+    bool bnl_stale = false, bnl_captured = false;
     double *hv = nullptr, *hw = nullptr;  // staging of napspmv_apply_host
     unsigned long long *ctr = nullptr;  // the fused engine's grid barrier: arrivals, generation
     int *err = nullptr;                 // sticky device status
@@ -159,6 +202,7 @@ struct napspmv_plan_s {
     int64_t n_bll = 0, n_lbuf = 0, n_gs = 0, n_bnl = 0;
     uint32_t *d_pack_src = nullptr;  // [n_gs]
     int32_t *d_xfer_dst = nullptr;   // [n_gs]
+    int32_t *d_xfer_shift = nullptr;  // [ceil(n_gs / kSendGroup)]
     int32_t *d_unp_src = nullptr;    // [n_bnl]
     // BLL / LBUF list idx arrays double as the J2 / J0 gather sources.
 
@@ -169,11 +213,16 @@ struct napspmv_plan_s {
     // sliced-row copies of the whole matrix, its local part and its remote
     // part (index 0, 1, 2), for NAPSPMV_PIPELINE_SELL; built with the plan
     nap::SellPart sell[3];
+    nap::WinPart win;  // staged windows over sell[0]
+    // an apply that leaves engine, pipeline and tile options unset runs on the
+    // staged windows (until napspmv_set_default_opts names an engine or pipeline)
+    bool auto_window = true;
 
     nap::ItemSet items;
     // instantiated CUDA graphs of chained phased applies, newest last
     struct GraphEntry {
         const void *v, *w, *ws;
+        bool window;
         int32_t reps, prec, vec, tile_rows, tile_nnz, engine, stages, pipeline, ctas_per_sm, halo;
         double scale;
         cudaGraphExec_t exec;
@@ -187,10 +236,19 @@ struct napspmv_plan_s {
 
 namespace nap {
 int build_items(napspmv_plan_t *P, int32_t tile_rows, int32_t tile_nnz);
+constexpr int kWinSmem = 226 * 1024;  // shared memory of a staged-window CTA, at most
+int window_bytes(int64_t srcs, int64_t slots, int64_t words, int vb);  // what one with this block needs
+int window_prepare(napspmv_plan_t *P);
 int ws_alloc(napspmv_plan_t *P, napspmv_ws_t *ws);
 void ws_free(napspmv_ws_t *ws);
 void plan_free(napspmv_plan_t *P);
-napspmv_opts resolve_opts(const napspmv_plan_t *P, const napspmv_opts *o);
+// Options with every unset field resolved; window: run on the staged windows.
+struct Opts : napspmv_opts {
+    bool window = false;
+};
+Opts resolve_opts(const napspmv_plan_t *P, const napspmv_opts *o);
+// the fields that name an engine, a pipeline or a tile shape are all unset
+bool leaves_path_open(const napspmv_opts &o);
 // ERR_ARG / ERR_STATE / ERR_UNSUPPORTED (with the message set) for resolved
 // options the plan cannot run, else NAPSPMV_OK
 int check_opts(const napspmv_plan_t *P, const napspmv_opts &o);

@@ -99,6 +99,17 @@ struct Part {
         if (strided) return j % np;
         return j < big ? j / (q + 1) : rem + (j - big) / q;
     }
+    // rows of rank r, and its k-th row
+    __host__ __device__ int64_t rows(int64_t r) const { return q + (r < rem ? 1 : 0); }
+    __host__ __device__ int64_t row(int64_t r, int64_t k) const
+    {
+        return strided ? r + k * np : start(r) + k;
+    }
+    // position of row i among its rank's rows
+    __host__ __device__ int64_t local(int64_t i) const
+    {
+        return strided ? i / np : i - start(owner(i));
+    }
     // first row of rank r (contiguous blocks only)
     __host__ __device__ int64_t start(int64_t r) const { return r * q + (r < rem ? r : rem); }
 };
@@ -262,6 +273,23 @@ __global__ void k_fill_gsend(int64_t n_gs, const int64_t *gs_off, int64_t n_msg,
         int64_t s = msg_src[lo], p = part.owner(j);
         j0key[e] = (p != s) ? (((uint64_t)p << (rb + jb)) | ((uint64_t)s << jb) | (uint64_t)j)
                             : SENT;
+    }
+}
+
+// Shift of every group of kSendGroup transfer destinations (a warp each).
+__global__ void k_xfer_shift(const int32_t *dst, int64_t n, int32_t *shift)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g * kSendGroup < n;
+         g += warps) {
+        const int64_t b = g * kSendGroup;
+        const int32_t s = dst[b] - (int32_t)b;
+        bool same = true;
+        for (int64_t k = b + lane; k < min(n, b + kSendGroup); k += 32)
+            same &= dst[k] - (int32_t)k == s;
+        same = __all_sync(0xffffffffu, same);
+        if (lane == 0) shift[g] = same ? s : kMixed;
     }
 }
 
@@ -476,6 +504,12 @@ struct Cub {
         if (dk.Current() != k.p) std::swap(k.p, k2.p);
         if (dv.Current() != v.p) std::swap(v.p, v2.p);
     }
+    void max_i32(const int32_t *in, int32_t *out, int64_t n)
+    {
+        size_t b = 0;
+        CK(cub::DeviceReduce::Max(nullptr, b, in, out, (int)n, st));
+        CK(cub::DeviceReduce::Max(temp(b), b, in, out, (int)n, st));
+    }
     template <class T>
     void exclusive_sum(const T *in, T *out, int64_t n)
     {
@@ -503,17 +537,33 @@ struct Cub {
     }
 };
 
+// The windows that sliced rows are sorted in: the blocks of the staged windows
+// (nsub blocks of `rows` rows per process), else whole processes, or 1024-row
+// blocks of a strided plan.
+struct SellCut {
+    int32_t nsub = 0, rows = 0;
+    __host__ __device__ int64_t count(const Part &part, int64_t n) const
+    {
+        return nsub ? part.np * nsub : part.strided ? (n + 1023) / 1024 : part.np;
+    }
+    __device__ int64_t window(const Part &part, int64_t i) const
+    {
+        if (nsub) return part.owner(i) * nsub + part.local(i) / rows;
+        return part.strided ? i / 1024 : part.owner(i);
+    }
+};
+
 // Sort key of every row for its sliced window: (window, longest first); rows of
 // more than kSellLong entries take the window after the last.
 constexpr int kSellKeyBits = 9;  // holds kSellLong - length, 0 .. kSellLong
 static_assert(kSellLong < (1 << kSellKeyBits), "row lengths of the sliced windows fit the key");
-__global__ void k_sell_keys(const int32_t *rp, int64_t n, Part part, int64_t nwin, uint64_t *key,
-                            int32_t *row)
+__global__ void k_sell_keys(const int32_t *rp, int64_t n, Part part, SellCut cut, int64_t nwin,
+                            uint64_t *key, int32_t *row)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int32_t len = rp[i + 1] - rp[i];
-        const uint64_t w = len > kSellLong ? nwin : part.strided ? i / 1024 : part.owner(i);
+        const uint64_t w = len > kSellLong ? nwin : cut.window(part, i);
         key[i] = (w << kSellKeyBits) | (len > kSellLong ? 0 : kSellLong - len);
         row[i] = (int32_t)i;
     }
@@ -563,8 +613,8 @@ __global__ void k_sell_cut(const uint64_t *key, const int32_t *row, int64_t n, i
                 if (lane == 0) info[c] = make_int2((int)slot, (width << 6) | nl);
                 perm[32 * c + lane] = lane < nl ? row[j + lane] : -1;
             }
-            // every chunk starts on a 4-slot (16-byte) boundary
-            slot += ((int64_t)width * nl + 3) & ~3ll;
+            // every chunk starts on an 8-slot boundary (16 bytes of 2-byte columns)
+            slot += ((int64_t)width * nl + 7) & ~7ll;
             c++;
             j += nl;
         }
@@ -777,15 +827,16 @@ void host_stats(napspmv_plan_t *P)
 // most of a plan build: 41 of 56 ms of a 10^6-row 7-point plan on GB300, against 2.3 of
 // 17 ms this way (810 of 1,180 ms of the 2^23-row banded random plan, against 6 of 370).
 void build_sell(napspmv_plan_t *P, Cub &cb, int which, const int32_t *d_rp, const uint32_t *d_col,
-                const double *d_val, const float *d_val32, const Part &part)
+                const double *d_val, const float *d_val32, const Part &part,
+                const SellCut &cut = SellCut(), dvec<int64_t> *win_off = nullptr)
 {
     SellPart &S = P->sell[which];
     const int64_t n = P->n;
-    const int64_t nwin = part.strided ? (n + 1023) / 1024 : part.np;
+    const int64_t nwin = cut.count(part, n);
     const int kb = kSellKeyBits + bits_for(nwin);
     dvec<uint64_t> key(n), key2(n);
     dvec<int32_t> row(n), row2(n);
-    k_sell_keys<<<blocks_for(n), 256>>>(d_rp, n, part, nwin, key.p, row.p);
+    k_sell_keys<<<blocks_for(n), 256>>>(d_rp, n, part, cut, nwin, key.p, row.p);
     CK(cudaGetLastError());
     cb.sort_pairs(key, key2, row, row2, n, kb);
     // per window: chunks and slots, then their exclusive sums (the last element
@@ -819,13 +870,13 @@ void build_sell(napspmv_plan_t *P, Cub &cb, int which, const int32_t *d_rp, cons
                                        S.d_perm, nullptr);
     CK(cudaGetLastError());
     // padded past the last slot: a block's bulk copy is widened to 16 bytes
-    auto al = [&](size_t sz) {
+    auto al = [&](size_t sz, int fill = 0) {
         void *q = nullptr;
         CK(cudaMalloc(&q, sz * (size_t)std::max<int64_t>(slots, 1) + 256));
-        CK(cudaMemset(q, 0, sz * (size_t)std::max<int64_t>(slots, 1) + 256));
+        CK(cudaMemset(q, fill, sz * (size_t)std::max<int64_t>(slots, 1) + 256));
         return q;
     };
-    S.d_col = (uint32_t *)al(4);
+    S.d_col = (uint32_t *)al(4, 0xff);  // kSellPad between chunks too
     S.d_val = (double *)al(8);
     if (d_val32) S.d_val32 = (float *)al(4);
     if (S.nch) {
@@ -834,6 +885,283 @@ void build_sell(napspmv_plan_t *P, Cub &cb, int which, const int32_t *d_rp, cons
                                                      S.d_val32);
         CK(cudaGetLastError());
     }
+    if (win_off) std::swap(win_off->p, off.p);
+}
+
+// A block takes at most this much shared memory in FP64: four CTAs to an SM.
+constexpr int kWinBytes = 56 * 1024;
+// Windows of more values per row than this (strided partitions, whose rows share
+// few operands) are mostly gathering: 128 rows to a block and two threads to a row
+// (strided 101^3 on GB300: 60.8 us per apply, 78 with 256 rows and a thread each).
+// Denser ones take 256 rows and a thread each (contiguous 128^3: 42.6 us, 46 with
+// 128 rows, 45 with 512, 59 with two threads).
+constexpr int kWinSparse = 5;
+
+// One CTA per block of the staged windows.  The positions of a process's full
+// window (own rows, b_{l->l}, b_{nl->l}) that the block's rows use are marked in
+// a shared-memory bitmap; a position's slot is its rank among the marked ones.
+// COUNT: the size of the block's window.  FILL: its sources and the slot of
+// every stored entry of its sliced rows.
+struct WinGeom {
+    Part part;
+    SellCut cut;
+    int32_t words;  // bitmap words of the largest process window
+    const int32_t *bll_ptr, *bnl_ptr;
+};
+template <bool FILL>
+__global__ void k_win_block(const int32_t *rp, const uint32_t *col, WinGeom G, int64_t nblk,
+                            int32_t *nsrc, int32_t *nent, int32_t *stat, const int64_t *osl,
+                            const int64_t *osrc,
+                            const int32_t *bll_j, const int32_t *unp_src, const uint32_t *scol,
+                            uint32_t *src, uint32_t *src_step, uint16_t *col16)
+{
+    extern __shared__ uint32_t bits[];  // [words], then (FILL) marked positions before each word
+    __shared__ int warp_sum[8];         // 256 threads
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int64_t b = blockIdx.x; b < nblk; b += gridDim.x) {
+        const int64_t t = b / G.cut.nsub, sub = b % G.cut.nsub;
+        const int32_t own = (int32_t)G.part.rows(t);
+        const int32_t l0 = G.bll_ptr[t], nl = G.bll_ptr[t + 1] - l0;
+        const int32_t r0 = G.bnl_ptr[t], nr = G.bnl_ptr[t + 1] - r0;
+        const int words = (own + nl + nr + 31) / 32;
+        auto position = [&](uint32_t c) {  // in the process's full window
+            const int32_t k = (int32_t)(c & kIndexMask);
+            const uint32_t blkno = c >> kBlockShift;
+            if (blkno == 0) return (int32_t)G.part.local(k);
+            return blkno == 1 ? own + k - l0 : own + nl + k - r0;
+        };
+        for (int w = tid; w < words; w += blockDim.x) bits[w] = 0;
+        __syncthreads();
+        const int32_t k1 = min(own, (int32_t)(sub + 1) * G.cut.rows);
+        int longest = 0, entries = 0;
+        for (int32_t k = (int32_t)sub * G.cut.rows + warp; k < k1; k += blockDim.x >> 5) {
+            const int64_t i = G.part.row(t, k);
+            const int32_t s = rp[i], e = rp[i + 1];
+            longest = max(longest, e - s);
+            entries += e - s;
+            for (int32_t q = s + lane; q < e; q += 32) {
+                const int32_t f = position(col[q]);
+                atomicOr(&bits[f >> 5], 1u << (f & 31));
+            }
+        }
+        __syncthreads();
+        // marked positions before this thread's run of words
+        const int per = (words + blockDim.x - 1) / blockDim.x;
+        const int w0 = min(words, tid * per), w1 = min(words, w0 + per);
+        int mine = 0;
+        for (int w = w0; w < w1; w++) mine += __popc(bits[w]);
+        int incl = mine;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += x;
+        }
+        if (lane == 31) warp_sum[warp] = incl;
+        __syncthreads();
+        int before = incl - mine;
+        for (int w = 0; w < warp; w++) before += warp_sum[w];
+        if (!FILL) {
+            if (tid == blockDim.x - 1) nsrc[b] = before + mine;
+            if (lane == 0 && longest) atomicMax(&stat[0], longest);
+            if (lane == 0 && entries) atomicAdd(&nent[b], entries);
+        } else {
+            uint32_t *pre = bits + G.words;
+            const int64_t s0 = osrc[b];
+            for (int w = w0; w < w1; w++) {
+                pre[w] = before;
+                for (uint32_t m = bits[w]; m; m &= m - 1) {
+                    const int32_t f = 32 * w + __ffs(m) - 1;
+                    uint32_t s, st;
+                    if (f < own) {
+                        s = st = (uint32_t)G.part.row(t, f);
+                    } else if (f < own + nl) {
+                        s = (uint32_t)bll_j[l0 + f - own];
+                        st = kFromBll | (uint32_t)(l0 + f - own);
+                    } else {
+                        s = st = kFromRecv | (uint32_t)unp_src[r0 + f - own - nl];
+                    }
+                    src[s0 + before] = s;
+                    src_step[s0 + before] = st;
+                    before++;
+                }
+            }
+            __syncthreads();
+            for (int64_t q = osl[b] + tid; q < osl[b + 1]; q += blockDim.x) {
+                const uint32_t c = scol[q];
+                if (c == kSellPad) {
+                    col16[q] = kWinPad;
+                } else {
+                    const int32_t f = position(c);
+                    col16[q] = (uint16_t)(pre[f >> 5] + __popc(bits[f >> 5] & ((1u << (f & 31)) - 1)));
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// Source runs of every block (a warp each) from its source list src[osrc ..].
+// COUNT: words needed, a multiple of 4.  WRITE: the runs.
+template <bool WRITE>
+__global__ void k_win_runs(int64_t nblk, const uint32_t *src, const int64_t *osrc,
+                           const int32_t *nsrc, int32_t *words, const int64_t *oword,
+                           uint32_t *runs)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < nblk; b += warps) {
+        const uint32_t *s = src + osrc[b];
+        const int n = nsrc[b], tiles = (n + 31) / 32;
+        uint32_t *out = WRITE ? runs + oword[b] : nullptr;
+        uint32_t r = 0;
+        for (int t = 0; t < tiles; t++) {
+            const int k = 32 * t + lane;
+            const bool start = k < n && (lane == 0 || s[k] != s[k - 1] + 1);
+            const uint32_t m = __ballot_sync(0xffffffffu, start);
+            if (WRITE) {
+                if (lane == 0) {
+                    out[2 * t] = m;
+                    out[2 * t + 1] = r;
+                }
+                if (start) out[2 * tiles + r + __popc(m & ((1u << lane) - 1))] = s[k];
+            }
+            r += __popc(m);
+        }
+        if (!WRITE && lane == 0) words[b] = (2 * tiles + (int)r + 3) & ~3;
+    }
+}
+
+__global__ void k_win_blocks(int64_t nblk, const int64_t *och, const int64_t *osl,
+                             const int32_t *nsrc, const int32_t *words, const int64_t *oword,
+                             WinBlock *blk)
+{
+    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (b >= nblk) return;
+    WinBlock B{};
+    B.chunk0 = (int32_t)och[b];
+    B.chunks = (int32_t)(och[b + 1] - och[b]);
+    B.slot0 = (int32_t)osl[b];
+    B.slots = (int32_t)(osl[b + 1] - osl[b]);
+    B.srcs = nsrc[b];
+    B.words = words[b];
+    B.word0 = (int32_t)(oword[b] / 4);
+    blk[b] = B;
+}
+__global__ void k_win_slots(int64_t nblk, const int64_t *osl, int32_t *slots)
+{
+    for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nblk;
+         b += (int64_t)gridDim.x * blockDim.x)
+        slots[b] = (int32_t)(osl[b + 1] - osl[b]);
+}
+__global__ void k_widen(const int32_t *in, int64_t n, int64_t *out)  // out[n] = 0
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        out[i] = i < n ? in[i] : 0;
+}
+
+// Chooses the block size of the staged windows and builds them with the whole
+// matrix's sliced rows.  No windows (the sliced rows then keep their own): rows
+// of more than 12 entries on average, a plan of composed gathers, a row of more
+// than kSellLong entries, fewer than 64 rows per process, or blocks that do not
+// fit the shared memory.
+void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *bll_ptr,
+                   const int32_t *bnl_ptr)
+{
+    WinPart &W = P->win;
+    const int64_t n = P->n;
+    auto plain = [&] {
+        build_sell(P, cb, 0, P->d_rowptr, P->d_colenc, P->d_val, P->d_val32, part);
+    };
+    int64_t wide = 0;  // largest process window
+    for (int64_t t = 0; t < part.np; t++)
+        wide = std::max<int64_t>(wide, part.rows(t) + P->h_bll_rank[t + 1] - P->h_bll_rank[t] +
+                                           P->h_bnl_rank[t + 1] - P->h_bnl_rank[t]);
+    const int64_t words = (wide + 31) / 32;
+    const int64_t max_rows = part.rows(0);
+    if (P->nnz > 12 * n || (P->flags & NAPSPMV_COMPOSED_GATHERS) || n / part.np < 64 ||
+        8 * words > 200 * 1024)
+        return plain();
+    WinGeom G{part, SellCut(), (int32_t)words, bll_ptr, bnl_ptr};
+    CK(cudaFuncSetAttribute((const void *)k_win_block<false>,
+                            cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    CK(cudaFuncSetAttribute((const void *)k_win_block<true>,
+                            cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    dvec<int32_t> nsrc, nent, stat(4);  // per block; longest row, largest window, most entries, words
+    int64_t nblk = 0;
+    int32_t st[4] = {};
+    bool fits = false;
+    int rows = 256;
+    for (; rows >= 32 && !fits; rows /= 2) {
+        G.cut.nsub = (int32_t)((max_rows + rows - 1) / rows);
+        G.cut.rows = (int32_t)((max_rows + G.cut.nsub - 1) / G.cut.nsub + 31) & ~31;
+        nblk = part.np * G.cut.nsub;
+        if (nblk >= (1ll << 31) - 1) break;
+        nsrc.alloc(nblk);
+        nent.alloc(nblk);
+        CK(cudaMemset(nent.p, 0, sizeof(int32_t) * nblk));
+        CK(cudaMemset(stat.p, 0, sizeof(st)));
+        const int grid = (int)std::min<int64_t>(nblk, 1 << 20);
+        k_win_block<false><<<grid, 256, 4 * words>>>(P->d_rowptr, P->d_colenc, G, nblk, nsrc.p,
+                                                     nent.p, stat.p, nullptr, nullptr, nullptr,
+                                                     nullptr, nullptr, nullptr, nullptr, nullptr);
+        CK(cudaGetLastError());
+        cb.max_i32(nsrc.p, stat.p + 1, nblk);
+        cb.max_i32(nent.p, stat.p + 2, nblk);
+        CK(cudaMemcpy(st, stat.p, sizeof(st), cudaMemcpyDeviceToHost));
+        if (st[0] > kSellLong) return plain();
+        const bool sparse = st[1] > kWinSparse * G.cut.rows;
+        W.threads = sparse ? 2 * G.cut.rows : G.cut.rows;
+        fits = window_bytes(st[1], st[2], st[1], 8) <= kWinBytes && !(sparse && rows > 128);
+    }
+    if (!fits) return plain();
+    dvec<int64_t> off, wide_n(nblk + 1), osrc(nblk + 1), oword(nblk + 1);
+    dvec<int32_t> nword(nblk);
+    build_sell(P, cb, 0, P->d_rowptr, P->d_colenc, P->d_val, P->d_val32, part, G.cut, &off);
+    if (P->sell[0].slots < 0) return;
+    // the most slots a block has, padding included
+    k_win_slots<<<blocks_for(nblk), 256>>>(nblk, off.p + nblk + 1, nent.p);
+    CK(cudaGetLastError());
+    cb.max_i32(nent.p, stat.p + 2, nblk);
+    auto offsets = [&](const int32_t *cnt, dvec<int64_t> &o) {  // and their total
+        k_widen<<<blocks_for(nblk + 1), 256>>>(cnt, nblk, wide_n.p);
+        CK(cudaGetLastError());
+        cb.exclusive_sum(wide_n.p, o.p, nblk + 1);
+        int64_t total = 0;
+        CK(cudaMemcpy(&total, o.p + nblk, sizeof(total), cudaMemcpyDeviceToHost));
+        return total;
+    };
+    const int64_t total = offsets(nsrc.p, osrc);
+    const size_t slots = (size_t)std::max<int64_t>(P->sell[0].slots, 1);
+    dvec<uint32_t> src(std::max<int64_t>(total, 1)), src_step(std::max<int64_t>(total, 1));
+    CK(cudaMalloc(&W.d_col, sizeof(uint16_t) * slots + 256));
+    const int grid = (int)std::min<int64_t>(nblk, 1 << 20);
+    k_win_block<true><<<grid, 256, 8 * words>>>(
+        P->d_rowptr, P->d_colenc, G, nblk, nullptr, nullptr, nullptr, off.p + nblk + 1, osrc.p,
+        P->lists[L_BLL].d_idx, P->d_unp_src, P->sell[0].d_col, src.p, src_step.p, W.d_col);
+    CK(cudaGetLastError());
+    for (int q = 0; q < 2; q++) {
+        const uint32_t *s = q ? src_step.p : src.p;
+        const int wgrid = blocks_for(32 * nblk);
+        k_win_runs<false><<<wgrid, 256>>>(nblk, s, osrc.p, nsrc.p, nword.p, nullptr, nullptr);
+        CK(cudaGetLastError());
+        cb.max_i32(nword.p, stat.p + 3, nblk);
+        const int64_t all = offsets(nword.p, oword);
+        if (all / 4 > (int64_t)INT32_MAX) return;
+        CK(cudaMalloc(&W.d_blk[q], sizeof(WinBlock) * nblk));
+        CK(cudaMalloc(&W.d_runs[q], sizeof(uint32_t) * std::max<int64_t>(all, 1)));
+        k_win_runs<true><<<wgrid, 256>>>(nblk, s, osrc.p, nsrc.p, nullptr, oword.p, W.d_runs[q]);
+        CK(cudaGetLastError());
+        k_win_blocks<<<(int)((nblk + 255) / 256), 256>>>(nblk, off.p, off.p + nblk + 1, nsrc.p,
+                                                         nword.p, oword.p, W.d_blk[q]);
+        CK(cudaGetLastError());
+        CK(cudaMemcpy(st, stat.p, sizeof(st), cudaMemcpyDeviceToHost));
+        if (window_bytes(st[1], st[2], st[3], 8) > kWinSmem || st[1] >= kWinPad) return;
+        W.max_words[q] = st[3];
+    }
+    W.rows = G.cut.rows;
+    W.max_src = st[1];
+    W.max_slots = st[2];
+    W.blocks = (int32_t)nblk;
 }
 
 void build(napspmv_plan_t *P, const napspmv_csr *A)
@@ -1150,6 +1478,13 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
         CK(cudaGetLastError());
     }
 
+    if (ngs) {
+        const int64_t groups = (ngs + kSendGroup - 1) / kSendGroup;
+        CK(cudaMalloc(&P->d_xfer_shift, sizeof(int32_t) * groups));
+        k_xfer_shift<<<blocks_for(32 * groups), 256>>>(P->d_xfer_dst, ngs, P->d_xfer_shift);
+        CK(cudaGetLastError());
+    }
+
     // ---- J0 (Eqs. L0, IL0) and the aggregator buffers b_{l->nl}
     int64_t nj0 = cb.select(j0key.p, ngs, j0alt.p, NotSent{});
     cb.sort(j0alt.p, j0key.p, nj0, 2 * rb + jb);
@@ -1296,7 +1631,7 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
         for (int64_t i = 0; i <= n; i++) P->h_rowptr[i] = (int32_t)h[i];
     }
     // sliced-row copies of the whole matrix and of its two split parts
-    build_sell(P, cb, 0, P->d_rowptr, P->d_colenc, P->d_val, P->d_val32, part);
+    build_windows(P, cb, part, d_bll_ptr.p, d_bnl_ptr.p);
     build_sell(P, cb, 1, P->d_rowptrL, P->d_colL, P->d_valL, P->d_val32L, part);
     build_sell(P, cb, 2, P->d_rowptrR, P->d_colR, P->d_valR, P->d_val32R, part);
     CK(cudaDeviceSynchronize());
@@ -1320,7 +1655,7 @@ void plan_free(napspmv_plan_t *P)
     for (auto &L : P->lists)
         if (L.d_idx) cudaFree(L.d_idx);
     void *ptrs[] = {P->d_split, P->d_rowptr, P->d_colenc, P->d_val, P->d_val32, P->d_pack_src,
-                    P->d_xfer_dst, P->d_unp_src,
+                    P->d_xfer_dst, P->d_xfer_shift, P->d_unp_src,
                     P->items.d_items, P->items.d_tilesL, P->items.d_tilesR,
                     P->items.d_wt, P->items.d_wtL, P->items.d_wtR, P->items.d_tilesRH,
                     P->d_rowptrL, P->d_rowptrR, P->d_colL, P->d_colR, P->d_valL, P->d_valR,
@@ -1335,6 +1670,9 @@ void plan_free(napspmv_plan_t *P)
         for (void *p : sp)
             if (p) cudaFree(p);
     }
+    void *wp[] = {P->win.d_col, P->win.d_blk[0], P->win.d_blk[1], P->win.d_runs[0], P->win.d_runs[1]};
+    for (void *p : wp)
+        if (p) cudaFree(p);
     delete P;
     cudaSetDevice(cur);
 }
@@ -1392,8 +1730,9 @@ int plan_create(const napspmv_csr *A, int32_t np, int32_t ppn, uint32_t flags,
         //    1.71 ms, against 2.18 ms overlapped with sliced rows and 2.00 ms
         //    overlapped with two-lane warp tiles (its SpMV step alone: 0.72 ms
         //    against 1.04 ms);
-        //  - shorter rows (the stencils): the overlapped engine with CTA tiles,
-        //    one lane per row, 512 rows / 1536 entries (3D 7-point 128^3: 76 us,
+        //  - shorter rows (the stencils): staged windows where the plan has them
+        //    (3D 7-point 128^3: 40 us); else, or when asked for, the overlapped
+        //    engine with CTA tiles, one lane per row, 512 rows / 1536 entries (76 us,
         //    against 79 us phased and 89 us overlapped with sliced rows).
         // The lane count and tile shape serve the CTA and warp pipelines when an
         // apply asks for them: one lane per row keeps exactly one FP64 FMA per
@@ -1425,6 +1764,7 @@ int plan_create(const napspmv_csr *A, int32_t np, int32_t ppn, uint32_t flags,
         P->defaults.debug_stall = 0;
         rc = build_items(P, P->defaults.tile_rows, P->defaults.tile_nnz);
         if (rc) throw NapError{rc, "row-tile construction failed"};
+        if ((rc = window_prepare(P))) throw NapError{rc, "staged windows"};
     } catch (const NapError &e) {
         plan_free(P);
         set_error(e.code, e.msg);

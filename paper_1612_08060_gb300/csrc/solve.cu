@@ -208,7 +208,7 @@ int cg_core(napspmv_plan_t *P, const double *b, double *x, double rtol, int max_
 int true_relres(napspmv_plan_t *P, const double *b, const double *x, CgBuffers &B, double *out)
 {
     cudaStream_t s = B.s;
-    napspmv_opts o = P->defaults;
+    napspmv_opts o{};  // unset fields: the plan's defaults
     o.precision = NAPSPMV_PREC_F64;
     int rc;
     if ((rc = napspmv_apply_ex(P, nullptr, x, B.q, 1, 1.0, &o, s))) return rc;
@@ -258,7 +258,7 @@ int napspmv_cg(napspmv_plan_t *P, const double *b, double *x, double rtol, int32
     CgBuffers B;
     int rc = cg_alloc(B, P->n, (cudaStream_t)stream);
     if (rc) return rc;
-    napspmv_opts o = P->defaults;
+    napspmv_opts o{};
     o.precision = NAPSPMV_PREC_F64;
     int it = 0;
     if ((rc = cg_core(P, b, x, rtol, max_it, o, B, &it))) return rc;
@@ -289,7 +289,7 @@ int napspmv_cg_ir(napspmv_plan_t *P, const double *b, double *x, double rtol, do
     int rc = cg_alloc(B, P->n, s);
     if (rc) return rc;
     if ((rc = cg_alloc(I, P->n, s))) return rc;
-    napspmv_opts o32 = P->defaults;
+    napspmv_opts o32{};
     o32.precision = NAPSPMV_PREC_F32;
     int outer = 0, inner_total = 0;
     double rr = 0;
@@ -500,7 +500,7 @@ int slot_apply(int32_t count, const napspmv_cg_slot *slots, bool from_x, int32_t
     int nb = 0;
     for (int i = 0; i < count; i++) {
         if (plans[i]->nnz >= NAPSPMV_SOLO_NNZ) {
-            napspmv_opts o = plans[i]->defaults;
+            napspmv_opts o{};  // unset fields: the plan's defaults
             o.precision = precision;
             o.engine = NAPSPMV_ENGINE_PHASED;
             if (int rc = apply_batch(1, &plans[i], &wss[i], &vs[i], &ws_[i], &reps[i], &sc[i], &o, st))
