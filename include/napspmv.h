@@ -20,11 +20,12 @@
  *     algorithm as device gathers and copies (on_node -> on_node and
  *     on_node -> off_node local exchanges, packing of g_send, the inter-node
  *     transfer g_send -> g_recv, the off_node -> on_node forwarding) and the
- *     three-block SpMV, for all simulated processes at once.  By default, for
- *     matrices of short rows, in two passes: the inter-node messages go from
- *     their owners to g_recv, and each block of a process's rows receives its
- *     on-node and off-node values in the shared memory of the SM that sums
- *     them.  The engines below run the steps one by one in HBM.
+ *     three-block SpMV, for all simulated processes at once.  By default in
+ *     two passes: the inter-node messages go from their owners to g_recv, and
+ *     each block of a process's rows receives its on-node and off-node values
+ *     in the shared memory of the SM that sums them.  The phased and overlapped
+ *     engines below keep every receive buffer in HBM, the fused engine every
+ *     message step.
  *
  * Conventions for every call:
  *   - Return value: NAPSPMV_OK (0) or a negative NAPSPMV_ERR_* code; the
@@ -112,13 +113,14 @@ extern "C" {
 #define NAPSPMV_PREC_F32 1 /* FP32-stored values, FP32 products, FP64 sums   */
 
 /* With engine, pipeline, vec, tile_rows, tile_nnz, stages and halo all unset
- * (engine PHASED alone counts as unset), a plan whose rows average at most 12
- * entries runs on staged windows: every process's rows are cut into blocks, a
- * CTA brings the values its block multiplies into shared memory, each once, and
- * sums its sliced rows from there (the bits of vec = 1).  Such a plan needs at
+ * (engine PHASED alone counts as unset, as do PHASED with PIPELINE_SELL), an
+ * apply runs on staged windows where it can: every process's rows are cut into
+ * blocks, a CTA brings the values its block multiplies into shared memory, each
+ * once, and sums its sliced rows from there (the bits of vec = 1).  That takes at
  * least 64 rows per process on average, no row of more than 256 entries and no
- * composed gathers; others, and plans whose defaults napspmv_set_default_opts
- * has set, run the engine and pipeline that napspmv_get_default_opts reports. */
+ * composed gathers, and with PREC_F32 rows of at most 12 entries on average or a
+ * small matrix; otherwise, and once napspmv_set_default_opts has set a plan's
+ * defaults, the engine and pipeline of napspmv_get_default_opts run. */
 #define NAPSPMV_ENGINE_DEFAULT 0 /* the plan's default engine               */
 #define NAPSPMV_ENGINE_FUSED 1   /* one persistent, cooperative launch for all
                                     phases and all chained applies, in levels

@@ -7,6 +7,8 @@
 //            on_node -> off_node  b_{l->nl}[k] = x[lbuf_j[k]]      (Eq. IL0)
 //   phase 2  pack g_send from x (own values) or b_{l->nl}          (Eq. I)
 //   phase 3  inter-node transfer g_send -> g_recv (the "network")
+//   (the fused engine runs 1 to 3 step by step; the others move each inter-node
+//   value from its owner to g_recv in one pass, see k_send)
 //   phase 4  off_node -> on_node  b_{nl->l}[k] = g_recv[unp_src[k]] (Eq. IL1)
 //   phase 5  three-block SpMV: on_process from x, on_node from b_{l->l},
 //            off_node from b_{nl->l} (the three local_spmv of the algorithm as
@@ -23,9 +25,8 @@
 // issue, not only HBM, bounds the SpMV on GB300).  Stages are sized to each
 // tile list's largest tile; tiles are handed to CTAs in contiguous runs.
 //
-// Staged windows (default for rows of at most 12 entries; k_send and k_window):
-// phases 1 to 3 of the inter-node messages in one pass, and the on_node and
-// off_node receives inside the SpMV's CTAs.
+// Staged windows (the default where a plan has them; k_send and k_window or
+// k_window_long): the on_node and off_node receives inside the SpMV's CTAs.
 //
 // Engines:
 //   overlapped (for rows of at most 12 entries without windows)  the matrix split into
@@ -626,29 +627,6 @@ __device__ __noinline__ void step_gather(T *dst, const T *src, const int32_t *id
         [&](int, uint32_t j) { return ldm<INKERNEL>(src + j); },
         [&](int k, uint32_t, T v) { dst[k] = v; });
 }
-template <bool INKERNEL, int U, class T = double, bool WAIT = false>
-__device__ __noinline__ void step_pack(T *gsend, const T *x, const T *lbuf, const uint32_t *src,
-                                       int b, int e, int tid)
-{
-    const uint64_t pol = policy_evict_first();
-    batched<U, T, WAIT>(
-        b, e, tid, [&](int k) { return ld_stream_hint_u32(src + k, pol); },
-        [&](int, uint32_t u) {
-            return (u & kFromLbuf) ? ldm<INKERNEL>(lbuf + (u & ~kFromLbuf)) : ldm<INKERNEL>(x + u);
-        },
-        [&](int k, uint32_t, T v) { gsend[k] = v; });
-}
-template <bool INKERNEL, int U, class T = double, bool WAIT = false>
-__device__ __noinline__ void step_transfer(T *grecv, const T *gsend, const int32_t *dst, int b,
-                                           int e, int tid)
-{
-    const uint64_t pol = policy_evict_first();
-    batched<U, T, WAIT>(
-        b, e, tid, [&](int k) { return (uint32_t)ld_stream_hint_s32(dst + k, pol); },
-        [&](int k, uint32_t) { return ldm<INKERNEL>(gsend + k); },
-        [&](int, uint32_t d, T v) { grecv[d] = v; });
-}
-
 __device__ __forceinline__ bool staged_tile(const Item &it, int cap)
 {
     return it.kind == kSpmv && it.k1 - it.k0 <= cap;
@@ -673,26 +651,6 @@ __global__ void __launch_bounds__(NT)
             step_gather<false, 8, T, true>(lbuf, x, lbuf_j, lb, le, threadIdx.x);
         }
     }
-    griddep_done();
-}
-template <class T>
-__global__ void __launch_bounds__(NT)
-    k_pack(const T *x, const T *lbuf, const uint32_t *src, T *gsend, int n, const int *err)
-{
-    if (*(volatile const int *)err) return;
-    const int per = NT * 8;
-    for (int b = blockIdx.x * per; b < n; b += gridDim.x * per)
-        step_pack<false, 8, T, true>(gsend, x, lbuf, src, b, min(b + per, n), threadIdx.x);
-    griddep_done();
-}
-template <class T>
-__global__ void __launch_bounds__(NT)
-    k_transfer(const T *gsend, const int32_t *dst, T *grecv, int n, const int *err)
-{
-    if (*(volatile const int *)err) return;
-    const int per = NT * 8;
-    for (int b = blockIdx.x * per; b < n; b += gridDim.x * per)
-        step_transfer<false, 8, T, true>(grecv, gsend, dst, b, min(b + per, n), threadIdx.x);
     griddep_done();
 }
 template <class T>
@@ -1342,6 +1300,210 @@ __global__ void __launch_bounds__(kWinThreads, 4)
     griddep_done();
 }
 
+__device__ __forceinline__ uint16_t ld_stream_hint_u16(const uint16_t *p, uint64_t pol)
+{
+    uint16_t v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.u16 %0, [%1], %2;" : "=h"(v) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+
+// Staged windows of long rows.  A block's entries outweigh its window, so only
+// windows are staged, two per CTA: the second half of the CTA's warps gather the
+// window of the CTA's next block while the first half sum the rows of the
+// current one, streaming columns and values from global memory two steps ahead
+// (one thread asks for the next block's in L2).  CTA b takes blocks b, b + grid,
+// ... so that all CTAs sweep the arrays together.
+//
+// Bound by the SM's load path, which takes a 32-byte sector per gathered value
+// where the sources are sparse (about 9.4 TB/s over the chip; the sums' shared
+// loads queue behind them) and then by the FP64 pipe (40% busy).  Per apply on
+// GB300, FP64 values, chains of 10: 1,002 us for the 2^23-row banded matrix, where
+// gathers into b_{l->l} and b_{nl->l} and the sliced-row pass take 1,193 (and
+// 1,436 with the message hops one by one), 484 against 545 at 4 * 10^6 rows, 109
+// against 129 at 10^6, 10.4 against 19.2 at 5 * 10^4.  Tried at 2^23 rows: 8
+// values in flight per thread 1,072, 2 1,028; 6 entries a step 1,109; no L2 request
+// 1,031; entries bulk-copied to shared memory as well (256-row blocks, 8 summing
+// warps) 1,784, since every shared load then waits behind the gathers.
+// Start bringing [p, p + bytes) into L2 (one thread; 16-byte multiples).
+__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+constexpr int kWinLongU = 4;  // entries per step of a row, two steps in flight
+constexpr int kWinLongG = 4;  // window values in flight per thread
+template <bool F32, bool STEP>
+__global__ void __launch_bounds__(1024, 1)
+    k_window_long(const __grid_constant__ WinView S, int nblk, const void *xs, const void *gs,
+                  const void *ls, double *y, float *y32, const Scale sc, int *err)
+{
+    using XT = typename std::conditional<F32, float, double>::type;
+    constexpr int U = kWinLongU, G = kWinLongG;
+    const XT *x = static_cast<const XT *>(xs), *g = static_cast<const XT *>(gs),
+             *l = static_cast<const XT *>(ls);
+    extern __shared__ __align__(16) unsigned char smem[];
+    // mbarriers: full 0, 1, empty 0, 1; then the two windows
+    auto bar = [&](int k) {
+        TileStage t{};
+        t.bar = reinterpret_cast<uint64_t *>(smem + 16 * k);
+        return t;
+    };
+    XT *win0 = reinterpret_cast<XT *>(smem + 64);
+    const int half = blockDim.x / 2, warps = half >> 5;  // of each kind
+    const int lane = threadIdx.x & 31;
+    const uint64_t pol = policy_evict_first();
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < 4; k++) mbar_init(bar(k).bar, warps);
+        fence_barrier_init();
+    }
+    __syncthreads();
+    int b = blockIdx.x;
+    if ((int)threadIdx.x >= half) {
+        // gather
+        const int tid = threadIdx.x - half;
+        uint32_t ix[G];
+        int n = S.blk[b].srcs, w0 = S.blk[b].word0;
+        auto load = [&](int k0) {
+#pragma unroll
+            for (int u = 0; u < G; u++) {
+                const int k = k0 + u * half;
+                if (k < n) ix[u] = ld_stream_hint_u32(S.runs + w0 + k, pol);
+            }
+        };
+        load(tid);
+        griddep_wait();
+        if (*(volatile const int *)err) return;  // sticky error: no work until cleared
+        for (int it = 0; b < nblk; it++) {
+            const int nb = b + gridDim.x;
+            int nn = 0, nw0 = 0;
+            if (nb < nblk) {
+                nn = S.blk[nb].srcs;
+                nw0 = S.blk[nb].word0;
+            }
+            XT *win = win0 + (it & 1) * S.cap_src;
+            if (it >= 2 && !tile_wait(bar(2 + (it & 1)), ((it >> 1) - 1) & 1, err)) return;
+            const int m = n;
+            for (int k0 = tid; k0 < m; k0 += G * half) {
+                XT v[G];
+#pragma unroll
+                for (int u = 0; u < G; u++) {
+                    if (k0 + u * half >= m) continue;
+                    const uint32_t s = ix[u];
+                    const XT *p = (s & kFromRecv) ? g + (s & ~kFromRecv) : x + s;
+                    if (STEP && (s & (kFromRecv | kFromBll)) == kFromBll) p = l + (s & ~kFromBll);
+                    v[u] = __ldg(p);
+                }
+                if (k0 + G * half < m) {
+                    load(k0 + G * half);
+                } else {
+                    n = nn;
+                    w0 = nw0;
+                    load(tid);  // the next block's first
+                }
+#pragma unroll
+                for (int u = 0; u < G; u++)
+                    if (k0 + u * half < m) win[k0 + u * half] = v[u];
+            }
+            if (tid >= m) {
+                n = nn;
+                w0 = nw0;
+                load(tid);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(it & 1).bar);
+            b = nb;
+        }
+    } else {
+        // sum
+        const int warp = threadIdx.x >> 5;
+        int c = S.blk[b].chunk0 + warp, c1 = S.blk[b].chunk0 + S.blk[b].chunks;
+        int2 inf = c < c1 ? S.info[c] : make_int2(0, 0);
+        int row = c < c1 ? S.perm[32 * c + lane] : -1;
+        uint16_t ca[U], cb[U];
+        XT aa[U], ab[U];
+        auto load = [&](int i, uint16_t (&cc)[U], XT (&a)[U]) {
+            const int nl = inf.y & 63, width = lane < nl ? inf.y >> 6 : 0;
+            const int64_t base = (int64_t)inf.x + lane;
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                cc[u] = kWinPad;
+                if (i + u < width) {
+                    const int64_t k = base + (int64_t)(i + u) * nl;
+                    cc[u] = ld_stream_hint_u16(S.col + k, pol);
+                    if constexpr (F32) a[u] = ld_stream_hint_f32(S.val32 + k, pol);
+                    else a[u] = ld_stream_hint_f64(S.val + k, pol);
+                }
+            }
+        };
+        load(0, ca, aa);
+        load(U, cb, ab);
+        griddep_wait();
+        if (*(volatile const int *)err) return;
+        for (int it = 0; b < nblk; it++) {
+            const int nb = b + gridDim.x;
+            int nc = 0, nc1 = 0;
+            if (nb < nblk) {
+                nc = S.blk[nb].chunk0 + warp;
+                nc1 = S.blk[nb].chunk0 + S.blk[nb].chunks;
+                if (threadIdx.x == 0 && S.blk[nb].slots) {
+                    const uint32_t m = (uint32_t)S.blk[nb].slots;
+                    prefetch_l2(S.col + S.blk[nb].slot0, 2 * m);
+                    if (F32) prefetch_l2(S.val32 + S.blk[nb].slot0, 4 * m);
+                    else prefetch_l2(S.val + S.blk[nb].slot0, 8 * m);
+                }
+            }
+            const XT *win = win0 + (it & 1) * S.cap_src;
+            if (!tile_wait(bar(it & 1), (it >> 1) & 1, err)) return;
+            int2 ninf = nc < nc1 ? S.info[nc] : make_int2(0, 0);
+            int nrow = nc < nc1 ? S.perm[32 * nc + lane] : -1;
+            while (c < c1) {
+                const int nl = inf.y & 63, width = inf.y >> 6;
+                double acc = 0.0;
+                auto add = [&](const uint16_t (&cc)[U], const XT (&a)[U]) {
+#pragma unroll
+                    for (int u = 0; u < U; u++) {
+                        if (cc[u] != kWinPad) {
+                            if constexpr (F32) acc = __dadd_rn(acc, f32_product(a[u], win[cc[u]]));
+                            else acc = fma(a[u], win[cc[u]], acc);
+                        }
+                    }
+                };
+                for (int i = 0; i < width; i += 2 * U) {
+                    add(ca, aa);
+                    load(i + 2 * U, ca, aa);
+                    add(cb, ab);
+                    load(i + 3 * U, cb, ab);
+                }
+                if (lane < nl) {
+                    const double r = apply_scale(acc, sc);
+                    if (!F32 || y) y[row] = r;
+                    if (F32 && y32) y32[row] = d2f_rn(r);
+                }
+                c += warps;
+                if (c < c1) {
+                    inf = S.info[c];
+                    row = S.perm[32 * c + lane];
+                    load(0, ca, aa);
+                    load(U, cb, ab);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(2 + (it & 1)).bar);
+            b = nb;
+            c = nc;
+            c1 = nc1;
+            inf = ninf;
+            row = nrow;
+            load(0, ca, aa);
+            load(U, cb, ab);
+        }
+    }
+    griddep_done();
+}
+
 // Phases 1 (on_node -> off_node), 2 and 3 in one pass: element k of g_send, on
 // its way through the aggregator's buffer and g_send a register, goes from the
 // owner's x[j[k]] to its place in g_recv.  A warp moves groups of kSendGroup
@@ -1349,7 +1511,8 @@ __global__ void __launch_bounds__(kWinThreads, 4)
 // group inside a message needs one number, its shift (kMixed: it crosses
 // messages, and every element's place is read).  Bound by the SM's sector loads: a gathered 8-byte value
 // costs up to a 32-byte sector.  Against the gather, pack and transfer kernels, 35.6 us
-// of 128^3, 9.3 us (GB300, cold, on their own).
+// of 128^3, 9.3 us (GB300, cold, on their own); 426 us of the 2^23-row banded
+// matrix, 162.
 constexpr int kSendWarps = NT / 32;
 template <class T>
 __global__ void __launch_bounds__(NT)
@@ -1640,6 +1803,12 @@ struct FusedKernelTable {
 
 static bool valid_vec(int v) { return v == 1 || v == 2 || v == 4 || v == 8 || v == 16 || v == 32; }
 
+// Long rows with FP32 values run on the windows up to this many entries: below
+// it launches count (5 * 10^4 rows: 12.5 us per apply against 20), above it the
+// sliced-row pass is as fast or faster (1.5 * 10^5 rows: 25.3 against 25.0 us,
+// 10^6: 110.5 against 106, 4 * 10^6: 444 against 425).
+constexpr int64_t kWinLongF32 = 2500000;
+
 bool leaves_path_open(const napspmv_opts &o)
 {
     return (!o.engine || o.engine == NAPSPMV_ENGINE_PHASED) && !o.pipeline && !o.vec &&
@@ -1664,7 +1833,7 @@ Opts resolve_opts(const napspmv_plan_t *P, const napspmv_opts *o)
         if (o->timeout_ms) r.timeout_ms = o->timeout_ms;
         r.debug_stall = o->debug_stall;
     }
-    r.window = P->win.blocks > 0 &&
+    r.window = P->win.blocks > 0 && (!P->win.long_rows || r.precision == NAPSPMV_PREC_F64 || P->nnz <= kWinLongF32) &&
                ((P->auto_window && (!o || leaves_path_open(*o))) ||
                 (r.engine == NAPSPMV_ENGINE_PHASED && r.pipeline == NAPSPMV_PIPELINE_SELL));
     return r;
@@ -2290,37 +2459,38 @@ static int msg_grid(const napspmv_plan_t *P, int64_t n, int64_t wave)
     return (int)std::max<int64_t>(1, std::min<int64_t>(chunks, g));
 }
 
-// The four message steps of one apply (phases 1-4) as kernels on stream s;
-// returns the number of launches.  The later steps are launched as
-// programmatic dependents of the earlier ones; pdl_first: the first step too.
+// The inter-node messages from their owners to g_recv.
 template <class T>
-static int64_t enqueue_messages(const napspmv_plan_t *P, const T *x, T *bll, T *lbuf, T *gsend,
-                                T *grecv, T *bnl, int *err, cudaStream_t s, bool pdl_first)
+static int64_t enqueue_send(const napspmv_plan_t *P, const T *x, T *grecv, int *err, cudaStream_t s,
+                            bool pdl)
 {
-    auto grid = [&](int64_t n, int64_t wave) { return msg_grid(P, n, wave); };
+    constexpr bool f32 = sizeof(T) == 4;
+    if (P->n_gs == 0) return 0;
+    launch_pdl(pdl, k_send<T>, msg_grid(P, P->n_gs, P->wave_send[f32]), 0, s, x,
+               (const int32_t *)P->lists[L_INTER].d_idx, (const int32_t *)P->d_xfer_dst,
+               (const int32_t *)P->d_xfer_shift, grecv, (int)P->n_gs, (const int *)err);
+    return 1;
+}
+
+// The messages of one apply (phases 1-4) as kernels on stream s: the on-node
+// receives, the inter-node messages from their owners to g_recv, the off-node
+// receives.  Returns the number of launches.  The later ones are launched as
+// programmatic dependents of the earlier; pdl_first: the first too.
+template <class T>
+static int64_t enqueue_messages(const napspmv_plan_t *P, const T *x, T *bll, T *grecv, T *bnl,
+                                int *err, cudaStream_t s, bool pdl_first)
+{
+    constexpr bool f32 = sizeof(T) == 4;
     int64_t nk = 0;
-    if (P->n_bll + P->n_lbuf > 0) {
-        launch_pdl(pdl_first, k_gather2<T>,
-                   grid(P->n_bll + P->n_lbuf, one_wave(P, k_gather2<T>)), 0, s, x,
-                   (const int32_t *)P->lists[L_BLL].d_idx, bll, (int)P->n_bll,
-                   (const int32_t *)P->lists[L_LBUF].d_idx, lbuf, (int)P->n_lbuf,
-                   (const int *)err);
+    auto gather = [&](T *dst, const T *src, const int32_t *idx, int64_t n) {
+        if (n == 0) return;
+        launch_pdl(nk > 0 || pdl_first, k_unpack<T>, msg_grid(P, n, P->wave_gather[f32]), 0, s, src,
+                   idx, dst, (int)n, (const int *)err);
         nk++;
-    }
-    if (P->n_gs > 0) {
-        launch_pdl(true, k_pack<T>, grid(P->n_gs, one_wave(P, k_pack<T>)), 0, s, x, (const T *)lbuf,
-                   (const uint32_t *)P->d_pack_src, gsend, (int)P->n_gs, (const int *)err);
-        launch_pdl(true, k_transfer<T>, grid(P->n_gs, one_wave(P, k_transfer<T>)), 0, s,
-                   (const T *)gsend,
-                   (const int32_t *)P->d_xfer_dst, grecv, (int)P->n_gs, (const int *)err);
-        nk += 2;
-    }
-    if (P->n_bnl > 0) {
-        launch_pdl(true, k_unpack<T>, grid(P->n_bnl, one_wave(P, k_unpack<T>)), 0, s,
-                   (const T *)grecv,
-                   (const int32_t *)P->d_unp_src, bnl, (int)P->n_bnl, (const int *)err);
-        nk++;
-    }
+    };
+    gather(bll, x, P->lists[L_BLL].d_idx, P->n_bll);
+    nk += enqueue_send<T>(P, x, grecv, err, s, nk > 0 || pdl_first);
+    gather(bnl, grecv, P->d_unp_src, P->n_bnl);
     return nk;
 }
 
@@ -2357,17 +2527,35 @@ int window_bytes(int64_t srcs, int64_t slots, int64_t words, int vb)
 {
     return win_layout((int)((srcs + 7) & ~7ll), (int)((slots + 7) & ~7ll), (int)words, vb).bytes;
 }
+using WinLongKernel = void (*)(const WinView, int, const void *, const void *, const void *,
+                               double *, float *, const Scale, int *);
+static WinLongKernel pick_window_long(bool f32, bool step)
+{
+    if (f32) return step ? k_window_long<true, true> : k_window_long<true, false>;
+    return step ? k_window_long<false, true> : k_window_long<false, false>;
+}
+int window_long_bytes(int64_t srcs, int vb) { return 64 + 2 * vb * (int)((srcs + 7) & ~7ll); }
 // What the launches of the staged windows need to know, taken once per plan.
 int window_prepare(napspmv_plan_t *P)
 {
+    P->wave_gather[0] = one_wave(P, k_unpack<double>);
+    P->wave_gather[1] = one_wave(P, k_unpack<float>);
+    P->wave_send[0] = one_wave(P, k_send<double>);
+    P->wave_send[1] = one_wave(P, k_send<float>);
     if (!P->win.blocks) return NAPSPMV_OK;
-    for (int q = 0; q < 4; q++)
+    for (int q = 0; q < 4; q++) {
         NAP_CUDA(cudaFuncSetAttribute((const void *)pick_window(q & 1, q & 2),
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kWinSmem));
-    P->win.wave_gather[0] = one_wave(P, k_unpack<double>);
-    P->win.wave_gather[1] = one_wave(P, k_unpack<float>);
-    P->win.wave_send[0] = one_wave(P, k_send<double>);
-    P->win.wave_send[1] = one_wave(P, k_send<float>);
+        NAP_CUDA(cudaFuncSetAttribute((const void *)pick_window_long(q & 1, q & 2),
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, kWinSmem));
+    }
+    for (int f32 = 0; P->win.long_rows && f32 < 2; f32++) {
+        int occ = 0;
+        NAP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &occ, (const void *)pick_window_long(f32, false), P->win.threads,
+            (size_t)window_long_bytes(P->win.max_src, f32 ? 4 : 8)));
+        P->win.long_ctas[f32] = std::max(occ, 1);
+    }
     return NAPSPMV_OK;
 }
 // The SpMV over the staged windows; g, l: g_recv and b_{l->l} (step only).
@@ -2385,8 +2573,15 @@ static int window_run(const napspmv_plan_t *P, const Opts &o, bool step, const v
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)W.blocks);
     cfg.blockDim = dim3((unsigned)W.threads);
-    cfg.dynamicSmemBytes = (size_t)window_bytes(W.max_src, W.max_slots, W.max_words[step], f32 ? 4 : 8);
-    if (o.ctas_per_sm > 0) {
+    if (W.long_rows) {
+        const int ctas = o.ctas_per_sm > 0 ? std::min(o.ctas_per_sm, W.long_ctas[f32]) : W.long_ctas[f32];
+        cfg.gridDim = dim3((unsigned)std::min(W.blocks, P->num_sms * ctas));
+        cfg.dynamicSmemBytes = (size_t)window_long_bytes(W.max_src, f32 ? 4 : 8);
+    } else {
+        cfg.dynamicSmemBytes =
+            (size_t)window_bytes(W.max_src, W.max_slots, W.max_words[step], f32 ? 4 : 8);
+    }
+    if (o.ctas_per_sm > 0 && !W.long_rows) {
         // at most that many CTAs per SM: each takes its share of the 227 KB
         const size_t share = 227 * 1024 / (size_t)o.ctas_per_sm;
         if (share > 1024) cfg.dynamicSmemBytes = std::max(cfg.dynamicSmemBytes, share - 1024);
@@ -2397,7 +2592,11 @@ static int window_run(const napspmv_plan_t *P, const Opts &o, bool step, const v
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = pdl ? 1 : 0;
-    NAP_CUDA(cudaLaunchKernelEx(&cfg, fn, V, x, g, l, y, y32, make_scale(scale), err));
+    if (W.long_rows)
+        NAP_CUDA(cudaLaunchKernelEx(&cfg, pick_window_long(f32, step), V, W.blocks, x, g, l, y, y32,
+                                    make_scale(scale), err));
+    else
+        NAP_CUDA(cudaLaunchKernelEx(&cfg, fn, V, x, g, l, y, y32, make_scale(scale), err));
     return NAPSPMV_OK;
 }
 
@@ -2427,17 +2626,12 @@ static int enqueue_window(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, 
         // FP32 mode: the next apply reads the FP32 copy only
         float *y32 = f32 && !last ? ws->x32[(k + 1) & 1] : nullptr;
         if (last && P->n_bll > 0) {
-            launch_pdl(true, k_unpack<T>, msg_grid(P, P->n_bll, P->win.wave_gather[f32]), 0, s, xs,
+            launch_pdl(true, k_unpack<T>, msg_grid(P, P->n_bll, P->wave_gather[f32]), 0, s, xs,
                        (const int32_t *)P->lists[L_BLL].d_idx, bll, (int)P->n_bll,
                        (const int *)ws->err);
             nk++;
         }
-        if (P->n_gs > 0) {
-            launch_pdl(true, k_send<T>, msg_grid(P, P->n_gs, P->win.wave_send[f32]), 0, s, xs,
-                       (const int32_t *)P->lists[L_INTER].d_idx, (const int32_t *)P->d_xfer_dst,
-                       (const int32_t *)P->d_xfer_shift, grecv, (int)P->n_gs, (const int *)ws->err);
-            nk++;
-        }
+        nk += enqueue_send<T>(P, xs, grecv, ws->err, s, true);
         if (int rc = window_run(P, o, false, xs, grecv, nullptr, f32 && !last ? nullptr : y, y32,
                                 scale, ws->err, s, true))
             return rc;
@@ -2501,13 +2695,10 @@ static int enqueue_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, 
             nk += enqueue_composed(P, f32 ? (const void *)x32 : (const void *)x, ws, f32, s, pdl);
         else if (f32)
             nk += enqueue_messages<float>(P, x32, reinterpret_cast<float *>(ws->bll),
-                                          reinterpret_cast<float *>(ws->lbuf),
-                                          reinterpret_cast<float *>(ws->gsend),
                                           reinterpret_cast<float *>(ws->grecv),
                                           reinterpret_cast<float *>(ws->bnl), ws->err, s, pdl);
         else
-            nk += enqueue_messages<double>(P, x, ws->bll, ws->lbuf, ws->gsend, ws->grecv, ws->bnl,
-                                           ws->err, s, pdl);
+            nk += enqueue_messages<double>(P, x, ws->bll, ws->grecv, ws->bnl, ws->err, s, pdl);
         if (overlap) {
             NAP_CUDA(cudaStreamWaitEvent(s, P->ev_join, 0));
             spmv_run(LR, xs, ws, y, y32, scale, o.stages, s, false);

@@ -121,7 +121,7 @@ struct SellPart {
 // mask of the slots that start a run (the first always does) and the index of
 // its first run, as two words; after them the source of every run's first slot.
 // Stencil windows are a few contiguous pieces, so this is about 13 bytes per 32
-// values instead of 128.
+// values instead of 128.  Plans of long rows keep a plain list: one source a slot.
 constexpr uint16_t kWinPad = 0xffff;      // padding slots, as kSellPad
 constexpr uint32_t kFromRecv = 0x80000000u;  // source in g_recv, else in x
 constexpr uint32_t kFromBll = 0x40000000u;   // (step sources) source in b_{l->l}
@@ -130,15 +130,17 @@ struct WinBlock {
     int32_t slot0, slots;    // its stored-entry slots
     int32_t srcs;            // window slots
     int32_t words, word0;    // its runs: words (a multiple of 4), and the first / 4
+                             // (long rows: sources, and the first)
     int32_t pad;
 };
 struct WinPart {
     int32_t blocks = 0;   // 0: the plan has no windows
     int32_t rows = 0;     // rows per block (a multiple of 32)
     int32_t threads = 0;  // per CTA
+    bool long_rows = false;     // rows of more than 12 entries: k_window_long
+    int32_t long_ctas[2] = {};  // its CTAs per SM (FP64, FP32)
     // largest block: window slots, entry slots, run words (apply, step)
     int32_t max_src = 0, max_slots = 0, max_words[2] = {};
-    int64_t wave_gather[2] = {}, wave_send[2] = {};  // CTAs the GPU holds at once (FP64, FP32)
     uint16_t *d_col = nullptr;  // window slot of every sliced-row slot
     // for an apply, and for a step with on-node values from b_{l->l}
     WinBlock *d_blk[2] = {};
@@ -214,6 +216,7 @@ struct napspmv_plan_s {
     // part (index 0, 1, 2), for NAPSPMV_PIPELINE_SELL; built with the plan
     nap::SellPart sell[3];
     nap::WinPart win;  // staged windows over sell[0]
+    int64_t wave_gather[2] = {}, wave_send[2] = {};  // CTAs the GPU holds at once (FP64, FP32)
     // an apply that leaves engine, pipeline and tile options unset runs on the
     // staged windows (until napspmv_set_default_opts names an engine or pipeline)
     bool auto_window = true;
@@ -238,6 +241,7 @@ namespace nap {
 int build_items(napspmv_plan_t *P, int32_t tile_rows, int32_t tile_nnz);
 constexpr int kWinSmem = 226 * 1024;  // shared memory of a staged-window CTA, at most
 int window_bytes(int64_t srcs, int64_t slots, int64_t words, int vb);  // what one with this block needs
+int window_long_bytes(int64_t srcs, int vb);
 int window_prepare(napspmv_plan_t *P);
 int ws_alloc(napspmv_plan_t *P, napspmv_ws_t *ws);
 void ws_free(napspmv_ws_t *ws);

@@ -896,6 +896,12 @@ constexpr int kWinBytes = 56 * 1024;
 // Denser ones take 256 rows and a thread each (contiguous 128^3: 42.6 us, 46 with
 // 128 rows, 45 with 512, 59 with two threads).
 constexpr int kWinSparse = 5;
+// Long rows: 512 rows to a block from this many entries on, 256 from that many,
+// else 128, and half of that until there are two blocks to an SM.  Larger blocks
+// gather denser windows, smaller ones overlap better (us per apply with 128 / 256 /
+// 512 rows on GB300: 10^6 rows of 20 entries 109 / 116 / 130, 4 * 10^6 510 / 484 /
+// 514, 2^23 1,241 / 1,237 / 1,002).
+constexpr int64_t kWinLong512 = 120000000, kWinLong256 = 50000000;
 
 // One CTA per block of the staged windows.  The positions of a process's full
 // window (own rows, b_{l->l}, b_{nl->l}) that the block's rows use are marked in
@@ -1032,7 +1038,7 @@ __global__ void k_win_runs(int64_t nblk, const uint32_t *src, const int64_t *osr
 
 __global__ void k_win_blocks(int64_t nblk, const int64_t *och, const int64_t *osl,
                              const int32_t *nsrc, const int32_t *words, const int64_t *oword,
-                             WinBlock *blk)
+                             int unit, WinBlock *blk)
 {
     const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (b >= nblk) return;
@@ -1043,7 +1049,7 @@ __global__ void k_win_blocks(int64_t nblk, const int64_t *och, const int64_t *os
     B.slots = (int32_t)(osl[b + 1] - osl[b]);
     B.srcs = nsrc[b];
     B.words = words[b];
-    B.word0 = (int32_t)(oword[b] / 4);
+    B.word0 = (int32_t)(oword[b] / unit);
     blk[b] = B;
 }
 __global__ void k_win_slots(int64_t nblk, const int64_t *osl, int32_t *slots)
@@ -1060,10 +1066,9 @@ __global__ void k_widen(const int32_t *in, int64_t n, int64_t *out)  // out[n] =
 }
 
 // Chooses the block size of the staged windows and builds them with the whole
-// matrix's sliced rows.  No windows (the sliced rows then keep their own): rows
-// of more than 12 entries on average, a plan of composed gathers, a row of more
-// than kSellLong entries, fewer than 64 rows per process, or blocks that do not
-// fit the shared memory.
+// matrix's sliced rows.  No windows (the sliced rows then keep their own): a
+// plan of composed gathers, a row of more than kSellLong entries, fewer than 64
+// rows per process, or blocks that do not fit the shared memory.
 void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *bll_ptr,
                    const int32_t *bnl_ptr)
 {
@@ -1078,7 +1083,7 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
                                            P->h_bnl_rank[t + 1] - P->h_bnl_rank[t]);
     const int64_t words = (wide + 31) / 32;
     const int64_t max_rows = part.rows(0);
-    if (P->nnz > 12 * n || (P->flags & NAPSPMV_COMPOSED_GATHERS) || n / part.np < 64 ||
+    if ((P->flags & NAPSPMV_COMPOSED_GATHERS) || n / part.np < 64 ||
         8 * words > 200 * 1024)
         return plain();
     WinGeom G{part, SellCut(), (int32_t)words, bll_ptr, bnl_ptr};
@@ -1090,7 +1095,8 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
     int64_t nblk = 0;
     int32_t st[4] = {};
     bool fits = false;
-    int rows = 256;
+    W.long_rows = P->nnz > 12 * n;
+    int rows = !W.long_rows ? 256 : P->nnz >= kWinLong512 ? 512 : P->nnz >= kWinLong256 ? 256 : 128;
     for (; rows >= 32 && !fits; rows /= 2) {
         G.cut.nsub = (int32_t)((max_rows + rows - 1) / rows);
         G.cut.rows = (int32_t)((max_rows + G.cut.nsub - 1) / G.cut.nsub + 31) & ~31;
@@ -1109,6 +1115,12 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
         cb.max_i32(nent.p, stat.p + 2, nblk);
         CK(cudaMemcpy(st, stat.p, sizeof(st), cudaMemcpyDeviceToHost));
         if (st[0] > kSellLong) return plain();
+        if (W.long_rows) {
+            W.threads = 2 * std::max(64, G.cut.rows);
+            fits = window_long_bytes(st[1], 8) <= kWinSmem &&
+                   (rows <= 64 || nblk >= 2 * (int64_t)P->num_sms);
+            continue;
+        }
         const bool sparse = st[1] > kWinSparse * G.cut.rows;
         W.threads = sparse ? 2 * G.cut.rows : G.cut.rows;
         fits = window_bytes(st[1], st[2], st[1], 8) <= kWinBytes && !(sparse && rows > 128);
@@ -1139,7 +1151,15 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
         P->d_rowptr, P->d_colenc, G, nblk, nullptr, nullptr, nullptr, off.p + nblk + 1, osrc.p,
         P->lists[L_BLL].d_idx, P->d_unp_src, P->sell[0].d_col, src.p, src_step.p, W.d_col);
     CK(cudaGetLastError());
-    for (int q = 0; q < 2; q++) {
+    for (int q = 0; q < 2 && W.long_rows; q++) {  // plain lists
+        if (total > INT32_MAX || st[1] >= kWinPad) return;
+        CK(cudaMalloc(&W.d_blk[q], sizeof(WinBlock) * nblk));
+        k_win_blocks<<<(int)((nblk + 255) / 256), 256>>>(nblk, off.p, off.p + nblk + 1, nsrc.p,
+                                                         nsrc.p, osrc.p, 1, W.d_blk[q]);
+        CK(cudaGetLastError());
+        W.d_runs[q] = q ? src_step.release() : src.release();
+    }
+    for (int q = 0; q < 2 && !W.long_rows; q++) {
         const uint32_t *s = q ? src_step.p : src.p;
         const int wgrid = blocks_for(32 * nblk);
         k_win_runs<false><<<wgrid, 256>>>(nblk, s, osrc.p, nsrc.p, nword.p, nullptr, nullptr);
@@ -1152,7 +1172,7 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
         k_win_runs<true><<<wgrid, 256>>>(nblk, s, osrc.p, nsrc.p, nullptr, oword.p, W.d_runs[q]);
         CK(cudaGetLastError());
         k_win_blocks<<<(int)((nblk + 255) / 256), 256>>>(nblk, off.p, off.p + nblk + 1, nsrc.p,
-                                                         nword.p, oword.p, W.d_blk[q]);
+                                                         nword.p, oword.p, 4, W.d_blk[q]);
         CK(cudaGetLastError());
         CK(cudaMemcpy(st, stat.p, sizeof(st), cudaMemcpyDeviceToHost));
         if (window_bytes(st[1], st[2], st[3], 8) > kWinSmem || st[1] >= kWinPad) return;
@@ -1724,16 +1744,18 @@ int plan_create(const napspmv_csr *A, int32_t np, int32_t ppn, uint32_t flags,
         if (rc) throw NapError{rc, "workspace allocation failed"};
         P->ws->owned_by_plan = true;
         // defaults, measured on GB300 (FP64, per apply):
+        //  - staged windows where the plan has them (k_window, k_window_long);
+        //    else, or when asked for, by row length:
         //  - rows of more than 12 stored entries on average: the phased engine
         //    with the sliced rows (one lane per row, no shared-memory stage,
         //    chunk groups dealt round robin).  2^23-row banded random workload:
         //    1.71 ms, against 2.18 ms overlapped with sliced rows and 2.00 ms
         //    overlapped with two-lane warp tiles (its SpMV step alone: 0.72 ms
         //    against 1.04 ms);
-        //  - shorter rows (the stencils): staged windows where the plan has them
-        //    (3D 7-point 128^3: 40 us); else, or when asked for, the overlapped
-        //    engine with CTA tiles, one lane per row, 512 rows / 1536 entries (76 us,
-        //    against 79 us phased and 89 us overlapped with sliced rows).
+        //  - shorter rows (the stencils): the overlapped engine with CTA tiles,
+        //    one lane per row, 512 rows / 1536 entries (3D 7-point 128^3: 76 us,
+        //    against 79 us phased and 89 us overlapped with sliced rows; staged
+        //    windows: 40 us).
         // The lane count and tile shape serve the CTA and warp pipelines when an
         // apply asks for them: one lane per row keeps exactly one FP64 FMA per
         // stored entry (GB300's FP64 pipe is the scarce unit); longer rows take

@@ -1,4 +1,4 @@
-"""Staged windows (the default of short-row plans) against the one-lane tile pass, bit for
+"""Staged windows (the default) against the one-lane tile pass, bit for
 bit: both sum each row in its stored order with one FMA per entry, and messages are
 copies, so nothing may differ.  Sizes at the edges: rows per process around 32, the
 blocks' 128 and 256 rows and several blocks; send groups of 128 elements that cross
@@ -61,6 +61,21 @@ def test_bits(rows, n_p, ppn, flags, near):
                 assert np.array_equal(a, b), (prec, reps)
 
 
+@pytest.mark.parametrize("flags", [0, nap.PARTITION_STRIDED])
+@pytest.mark.parametrize("rows,n_p,ppn,near", [(64, 3, 2, 0), (65, 9, 2, 0), (130, 7, 3, 200), (513, 5, 4, 0),
+                                               (1000, 41, 8, 300)])
+def test_long_rows_bits(rows, n_p, ppn, near, flags):
+    """Rows of about 20 entries (the last case fills 128-row blocks)."""
+    A = sparse(rows * n_p + 1, 20, rows, near)
+    plan = gpu_plan(A, n_p, ppn, nap.F32_VALUES | flags)
+    buf = torch.from_numpy(I.vector(A.n + 1, rows)).cuda()
+    for vd in (buf[:A.n], buf[1:]):
+        for prec in (nap.PREC_F64, nap.PREC_F32):
+            for reps in (1, 2, 3):
+                a, b = both(plan, vd, reps, 0.5, prec)
+                assert np.array_equal(a, b), (prec, reps)
+
+
 @pytest.mark.parametrize("make,n_p,ppn", [(lambda: I.poisson2d(47), 7, 3), (lambda: I.poisson3d(17), 5, 2),
                                           (lambda: I.aniso_q1(40), 9, 4)])
 @pytest.mark.parametrize("flags", [0, nap.PARTITION_STRIDED])
@@ -79,11 +94,12 @@ def test_stencils_and_special_values(make, n_p, ppn, flags):
 
 @pytest.mark.parametrize("flags", [0, nap.PARTITION_STRIDED])
 @pytest.mark.parametrize("prec", [nap.PREC_F64, nap.PREC_F32])
-def test_step_keeps_the_receives_of_the_last_apply(flags, prec):
+@pytest.mark.parametrize("mat", ["short", "long"])
+def test_step_keeps_the_receives_of_the_last_apply(flags, prec, mat):
     """napspmv_spmv_step multiplies a new v with the receive buffers of the last apply:
     the same on the windows, and on the tiles after an apply that kept b_{nl->l} on chip
     (also when that apply was captured and replayed)."""
-    A = I.poisson3d(18)
+    A = I.poisson3d(18) if mat == "short" else sparse(1500, 20, 5)
     plan = gpu_plan(A, 7, 3, nap.F32_VALUES | flags)
     v1, v2 = (torch.from_numpy(I.vector(A.n, s)).cuda() for s in (1, 2))
     tiles = nap.make_opts(precision=prec, **TILES)
