@@ -275,11 +275,13 @@ int napspmv_spmv_step(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, doub
 int napspmv_apply_host(napspmv_plan_t *P, const double *v_host, double *w_host, int32_t reps,
                        double scale, void *stream);
 
-/* Persistent launches over `count` independent applies (each with its own
+/* Shared launches over `count` independent applies (each with its own
  * plan, workspace, vectors, reps and scale): the batched form used by the
  * request server.  ws[i] may be NULL only if no other entry uses the same
  * plan's own workspace.  count <= 64; all plans on one device.  count = 1
- * runs as napspmv_apply_ex with the given options; count > 1 runs on the
+ * runs as napspmv_apply_ex with the given options.  With count > 1, entries of
+ * short-row plans with staged windows (see NAPSPMV_ENGINE_DEFAULT) share those
+ * launches where `opts` leaves the path open; every other entry runs on the
  * fused engine, whatever engine `opts` names.  Options: each entry resolves
  * the fields of `opts` left 0 (or opts NULL) against its own plan's
  * defaults.  Entries whose resolved launch options agree share one fused

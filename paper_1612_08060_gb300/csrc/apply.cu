@@ -1165,7 +1165,7 @@ __global__ void __launch_bounds__(32 * W, W == 8 ? (U >= 8 ? 4 : 6) : 1)
 // 0.85 of the measured copy peak; 2-byte columns, 13 bytes of runs per 32 window
 // values, no row pointers) and by the FP64 pipe with FP32 values (Q1 2048^2: 74 us,
 // the pipe 72% busy with one DADD per entry but the first).  Per apply on GB300, against
-// the overlapped engine before it: 39.8 for 85.0 us, 75 for 130 us, and 60 for 154 us
+// the overlapped engine before it: 39.0 for 85.9 us, 74 for 130 us, and 52.5 for 155 us
 // on a strided 101^3.  Tried on 128^3: columns and values read from global memory by
 // each lane (512-row blocks), 85 us for this kernel alone, one latency after another;
 // 4- and 8-byte asynchronous copies in place of loads for the window, 66 for 61 us on
@@ -1198,17 +1198,67 @@ __host__ __device__ __forceinline__ WinLayout win_layout(int cap_src, int cap_sl
     return L;
 }
 
+// One windowed SpMV of a launch: its matrix, x, g_recv, for a step the vector that
+// the on-node receives come from (l), the results, and its first CTA.
+struct WinJob {
+    WinView S;
+    const void *x, *g, *l;
+    double *y;
+    float *y32;
+    Scale sc;
+    int *err;
+    int32_t block0;
+};
+template <int MAXJ>
+struct WinJobs {
+    int32_t n;
+    WinJob job[MAXJ];
+};
+static_assert(sizeof(WinJobs<64>) <= 32764, "kernel parameters are limited to 32,764 bytes");
+
+__device__ __forceinline__ double to_xt(double, double v) { return v; }
+__device__ __forceinline__ float to_xt(float, double v) { return d2f_rn(v); }
+__device__ __forceinline__ float to_xt(float, float v) { return v; }
+// A window value: from g_recv, from x (XS: its type; FP32 mode rounds FP64 sources), or
+// for a step's on-node receives from l.
+template <class XT, class XS, bool STEP>
+__device__ __forceinline__ XT window_value(uint32_t s, const XS *x, const XT *g, const XS *l)
+{
+    const uint32_t k = s & kIndexMask;
+    if constexpr (sizeof(XT) == sizeof(XS)) {
+        const XT *p = (s & kFromRecv) ? g + k : x + k;
+        if (STEP && (s & kFromNode)) p = l + k;
+        return __ldg(p);
+    } else {
+        if (s & kFromRecv) return __ldg(g + k);
+        return to_xt(XT(0), __ldg((STEP && (s & kFromNode)) ? l + k : x + k));
+    }
+}
+
 constexpr int kWinG = 4;  // window values in flight per thread
 constexpr int kWinThreads = 512;  // at most
-// STEP: on-node values come from b_{l->l} (napspmv_spmv_step).
-template <bool F32, bool STEP>
+template <bool F32, class XS, bool STEP, int MAXJ>
 __global__ void __launch_bounds__(kWinThreads, 4)
-    k_window(const __grid_constant__ WinView S, const void *xs, const void *gs, const void *ls,
-             double *y, float *y32, const Scale sc, int *err)
+    k_window(const __grid_constant__ WinJobs<MAXJ> jobs)
 {
     using XT = typename std::conditional<F32, float, double>::type;
-    const XT *x = static_cast<const XT *>(xs), *g = static_cast<const XT *>(gs),
-             *l = static_cast<const XT *>(ls);
+    int jn = 0;
+    if (MAXJ > 1) {  // the last job that starts at or before this CTA
+        int hi = jobs.n - 1;
+        while (jn < hi) {
+            const int mid = (jn + hi + 1) >> 1;
+            if (jobs.job[mid].block0 <= (int)blockIdx.x) jn = mid;
+            else hi = mid - 1;
+        }
+    }
+    const WinJob &J = jobs.job[jn];
+    const WinView &S = J.S;
+    const XS *x = static_cast<const XS *>(J.x), *l = static_cast<const XS *>(J.l);
+    const XT *g = static_cast<const XT *>(J.g);
+    double *y = J.y;
+    float *y32 = J.y32;
+    const Scale sc = J.sc;
+    int *err = J.err;
     extern __shared__ __align__(16) unsigned char smem[];
     const WinLayout L = win_layout(S.cap_src, S.cap_slots, S.cap_words, sizeof(XT));
     TileStage lists{}, entries{};  // their mbarriers
@@ -1218,7 +1268,7 @@ __global__ void __launch_bounds__(kWinThreads, 4)
     uint32_t *runs = reinterpret_cast<uint32_t *>(smem + L.runs);
     uint16_t *col = reinterpret_cast<uint16_t *>(smem + L.col);
     const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, lane = tid & 31;
-    const WinBlock B = S.blk[blockIdx.x];
+    const WinBlock B = S.blk[(int)blockIdx.x - J.block0];
     if (tid == 0) {
         mbar_init(lists.bar, 1);
         mbar_init(entries.bar, 1);
@@ -1256,9 +1306,7 @@ __global__ void __launch_bounds__(kWinThreads, 4)
                 const uint2 h = head[t];
                 const uint32_t m = h.x & (0xffffffffu >> (31 - lane));  // run starts up to this slot
                 const uint32_t s = first[h.y + __popc(m) - 1] + (lane - (31 - __clz(m)));
-                const XT *p = (s & kFromRecv) ? g + (s & ~kFromRecv) : x + s;
-                if (STEP && (s & (kFromRecv | kFromBll)) == kFromBll) p = l + (s & ~kFromBll);
-                v[u] = __ldg(p);
+                v[u] = window_value<XT, XS, STEP>(s, x, g, l);
             }
 #pragma unroll
             for (int u = 0; u < kWinG; u++) {
@@ -1335,15 +1383,19 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
 }
 constexpr int kWinLongU = 4;  // entries per step of a row, two steps in flight
 constexpr int kWinLongG = 4;  // window values in flight per thread
-template <bool F32, bool STEP>
+template <bool F32, class XS, bool STEP>
 __global__ void __launch_bounds__(1024, 1)
-    k_window_long(const __grid_constant__ WinView S, int nblk, const void *xs, const void *gs,
-                  const void *ls, double *y, float *y32, const Scale sc, int *err)
+    k_window_long(const __grid_constant__ WinJob J, int nblk)
 {
     using XT = typename std::conditional<F32, float, double>::type;
     constexpr int U = kWinLongU, G = kWinLongG;
-    const XT *x = static_cast<const XT *>(xs), *g = static_cast<const XT *>(gs),
-             *l = static_cast<const XT *>(ls);
+    const WinView &S = J.S;
+    const XS *x = static_cast<const XS *>(J.x), *l = static_cast<const XS *>(J.l);
+    const XT *g = static_cast<const XT *>(J.g);
+    double *y = J.y;
+    float *y32 = J.y32;
+    const Scale sc = J.sc;
+    int *err = J.err;
     extern __shared__ __align__(16) unsigned char smem[];
     // mbarriers: full 0, 1, empty 0, 1; then the two windows
     auto bar = [&](int k) {
@@ -1391,10 +1443,7 @@ __global__ void __launch_bounds__(1024, 1)
 #pragma unroll
                 for (int u = 0; u < G; u++) {
                     if (k0 + u * half >= m) continue;
-                    const uint32_t s = ix[u];
-                    const XT *p = (s & kFromRecv) ? g + (s & ~kFromRecv) : x + s;
-                    if (STEP && (s & (kFromRecv | kFromBll)) == kFromBll) p = l + (s & ~kFromBll);
-                    v[u] = __ldg(p);
+                    v[u] = window_value<XT, XS, STEP>(ix[u], x, g, l);
                 }
                 if (k0 + G * half < m) {
                     load(k0 + G * half);
@@ -1513,41 +1562,97 @@ __global__ void __launch_bounds__(1024, 1)
 // costs up to a 32-byte sector.  Against the gather, pack and transfer kernels, 35.6 us
 // of 128^3, 9.3 us (GB300, cold, on their own); 426 us of the 2^23-row banded
 // matrix, 162.
+// The copy of x that a later napspmv_spmv_step takes the on-node receives from
+// (SendJob::keep) is made by further CTAs of the same launch.
 constexpr int kSendWarps = NT / 32;
-template <class T>
-__global__ void __launch_bounds__(NT)
-    k_send(const T *x, const int32_t *j, const int32_t *dst, const int32_t *shift, T *grecv, int n,
-           const int *err)
+struct SendJob {
+    const void *x;
+    const int32_t *j, *dst, *shift;
+    void *grecv;
+    double *keep;  // null: no copy
+    int *state;    // not null: set to 1
+    const int *err;
+    int64_t n;  // of x
+    int32_t n_gs;
+    int32_t block0, send_blocks, blocks;
+};
+template <int MAXJ>
+struct SendJobs {
+    int32_t n;
+    SendJob job[MAXJ];
+};
+static_assert(sizeof(SendJobs<64>) <= 32764, "kernel parameters are limited to 32,764 bytes");
+template <class T, class XS, int MAXJ>
+__global__ void __launch_bounds__(NT) k_send(const __grid_constant__ SendJobs<MAXJ> jobs)
 {
+    int jn = 0;
+    if (MAXJ > 1) {  // the last job that starts at or before this CTA
+        int hi = jobs.n - 1;
+        while (jn < hi) {
+            const int mid = (jn + hi + 1) >> 1;
+            if (jobs.job[mid].block0 <= (int)blockIdx.x) jn = mid;
+            else hi = mid - 1;
+        }
+    }
+    const SendJob &J = jobs.job[jn];
+    if (*(volatile const int *)J.err) return;
     constexpr int U = 2 * kSendGroup / 32;
-    if (*(volatile const int *)err) return;
+    const XS *x = static_cast<const XS *>(J.x);
+    T *grecv = static_cast<T *>(J.grecv);
+    const int block = (int)blockIdx.x - J.block0, n = J.n_gs;
+    if (block >= J.send_blocks) {
+        griddep_wait();
+        if (J.state && block == J.send_blocks && threadIdx.x == 0) *J.state = 1;
+        if (J.keep)
+            for (int64_t i = (int64_t)(block - J.send_blocks) * NT + threadIdx.x; i < J.n;
+                 i += (int64_t)(J.blocks - J.send_blocks) * NT)
+                J.keep[i] = (double)x[i];
+        griddep_done();
+        return;
+    }
     const uint64_t pol = policy_evict_first();
     const int lane = threadIdx.x & 31;
-    const int step = gridDim.x * kSendWarps * 2 * kSendGroup;
-    for (int b = (blockIdx.x * kSendWarps + (threadIdx.x >> 5)) * 2 * kSendGroup; b < n; b += step) {
+    const int step = J.send_blocks * kSendWarps * 2 * kSendGroup;
+    for (int b = (block * kSendWarps + (threadIdx.x >> 5)) * 2 * kSendGroup; b < n; b += step) {
         int32_t ix[U], to[U];
         T v[U];
-        const int32_t s0 = __ldg(shift + b / kSendGroup);
-        const int32_t s1 = b + kSendGroup < n ? __ldg(shift + b / kSendGroup + 1) : 0;
+        const int32_t s0 = __ldg(J.shift + b / kSendGroup);
+        const int32_t s1 = b + kSendGroup < n ? __ldg(J.shift + b / kSendGroup + 1) : 0;
 #pragma unroll
         for (int u = 0; u < U; u++) {
             const int k = b + 32 * u + lane;
-            if (k < n) ix[u] = ld_stream_hint_s32(j + k, pol);
+            if (k < n) ix[u] = ld_stream_hint_s32(J.j + k, pol);
         }
 #pragma unroll
         for (int u = 0; u < U; u++) {
             const int k = b + 32 * u + lane;
             const int32_t s = u < U / 2 ? s0 : s1;
             to[u] = k + s;
-            if (s == kMixed && k < n) to[u] = ld_stream_hint_s32(dst + k, pol);
+            if (s == kMixed && k < n) to[u] = ld_stream_hint_s32(J.dst + k, pol);
         }
         griddep_wait();
 #pragma unroll
         for (int u = 0; u < U; u++)
-            if (b + 32 * u + lane < n) v[u] = __ldg(x + ix[u]);
+            if (b + 32 * u + lane < n) v[u] = to_xt(T(0), __ldg(x + ix[u]));
 #pragma unroll
         for (int u = 0; u < U; u++)
             if (b + 32 * u + lane < n) grecv[to[u]] = v[u];
+    }
+    griddep_done();
+}
+
+// Both receive buffers from a kept vector (no more work where *state is 0).
+template <class T>
+__global__ void __launch_bounds__(NT)
+    k_receives(const double *x, const int32_t *bll_j, T *bll, int n_bll, const int32_t *bnl_j,
+               T *bnl, int n_bnl, const int *state, const int *err)
+{
+    griddep_wait();
+    if (*(volatile const int *)err || (state && !*state)) return;
+    for (int64_t k = blockIdx.x * (int64_t)NT + threadIdx.x; k < (int64_t)n_bll + n_bnl;
+         k += (int64_t)gridDim.x * NT) {
+        if (k < n_bll) bll[k] = to_xt(T(0), __ldg(x + bll_j[k]));
+        else bnl[k - n_bll] = to_xt(T(0), __ldg(x + bnl_j[k - n_bll]));
     }
     griddep_done();
 }
@@ -2015,11 +2120,12 @@ int ws_alloc(napspmv_plan_t *P, napspmv_ws_t *ws)
         al(&ws->grecv, P->n_gs) || al(&ws->bnl, P->n_bnl + 4) || al(&ws->xtmp, P->n) ||
         alf(&ws->x32[0], P->n) || alf(&ws->x32[1], P->n) ||
         cudaMalloc(&ws->ctr, sizeof(unsigned long long) * ctr_count(P)) ||
-        cudaMalloc(&ws->err, sizeof(int))) {
+        cudaMalloc(&ws->err, 2 * sizeof(int))) {
         ws_free(ws);
         return cuda_error(cudaErrorMemoryAllocation, "workspace");
     }
-    if (cudaMemset(ws->err, 0, sizeof(int)) != cudaSuccess) {
+    ws->state = ws->err + 1;
+    if (cudaMemset(ws->err, 0, 2 * sizeof(int)) != cudaSuccess) {
         ws_free(ws);
         return cuda_error(cudaGetLastError(), "workspace");
     }
@@ -2035,7 +2141,7 @@ void ws_free(napspmv_ws_t *ws)
     ws->bll = ws->lbuf = ws->gsend = ws->grecv = ws->bnl = ws->xtmp = ws->hv = ws->hw = nullptr;
     ws->x32[0] = ws->x32[1] = nullptr;
     ws->ctr = nullptr;
-    ws->err = nullptr;
+    ws->err = ws->state = nullptr;
 }
 
 static Scale make_scale(double s)
@@ -2070,6 +2176,18 @@ static SellView sell_view(const napspmv_plan_t *P, int part, bool f32)
 }
 
 static int32_t cdiv(int64_t a, int64_t b) { return (int32_t)((a + b - 1) / b); }
+
+// What a workspace's receive buffers hold after the applies about to be queued;
+// every engine calls this.  A workspace that the caller once captured has its
+// device word cleared with every apply: the buffers are valid in HBM.
+static int note_receives(napspmv_ws_t *ws, bool f32, bool vector, bool capturing, cudaStream_t s)
+{
+    ws->buf_f32 = f32 ? 1 : 0;
+    ws->recv_vector = vector;
+    if (capturing) ws->captured = true;
+    if (ws->captured && ws->state) NAP_CUDA(cudaMemsetAsync(ws->state, 0, sizeof(int), s));
+    return NAPSPMV_OK;
+}
 
 static FJob make_job(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, double *w, int reps,
                      double scale, bool f32, int32_t chunk)
@@ -2136,8 +2254,11 @@ static int launch_fused(int count, napspmv_plan_t *const *plans, napspmv_ws_t *c
             prm.off[l][i] = acc[l];
             acc[l] += prm.jobs[i].nunits[l];
         }
-        wi->bnl_stale = false;
-        wi->buf_f32 = 0;  // this engine's receive buffers hold FP64 values in both modes
+        // this engine's receive buffers hold FP64 values in both modes
+        wi->recv_f32 = false;
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        NAP_CUDA(cudaStreamIsCapturing(s, &cs));
+        if (int rc = note_receives(wi, false, false, cs != cudaStreamCaptureStatusNone, s)) return rc;
     }
     for (int l = 0; l < kLevels; l++) prm.off[l][count] = acc[l];
     // barrier words and the test hook's counter: the first job's workspace words
@@ -2460,15 +2581,29 @@ static int msg_grid(const napspmv_plan_t *P, int64_t n, int64_t wave)
 }
 
 // The inter-node messages from their owners to g_recv.
+static SendJob send_job(const napspmv_plan_t *P, bool f32, const void *x, void *grecv, const int *err)
+{
+    SendJob J{};
+    J.x = x;
+    J.j = P->lists[L_INTER].d_idx;
+    J.dst = P->d_xfer_dst;
+    J.shift = P->d_xfer_shift;
+    J.grecv = grecv;
+    J.err = err;
+    J.n = P->n;
+    J.n_gs = (int32_t)P->n_gs;
+    J.send_blocks = J.blocks = P->n_gs > 0 ? msg_grid(P, P->n_gs, P->wave_send[f32]) : 0;
+    return J;
+}
 template <class T>
 static int64_t enqueue_send(const napspmv_plan_t *P, const T *x, T *grecv, int *err, cudaStream_t s,
                             bool pdl)
 {
-    constexpr bool f32 = sizeof(T) == 4;
     if (P->n_gs == 0) return 0;
-    launch_pdl(pdl, k_send<T>, msg_grid(P, P->n_gs, P->wave_send[f32]), 0, s, x,
-               (const int32_t *)P->lists[L_INTER].d_idx, (const int32_t *)P->d_xfer_dst,
-               (const int32_t *)P->d_xfer_shift, grecv, (int)P->n_gs, (const int *)err);
+    SendJobs<1> S{};
+    S.n = 1;
+    S.job[0] = send_job(P, sizeof(T) == 4, x, grecv, err);
+    launch_pdl(pdl, k_send<T, T, 1>, S.job[0].blocks, 0, s, S);
     return 1;
 }
 
@@ -2516,39 +2651,49 @@ static int64_t enqueue_composed(const napspmv_plan_t *P, const void *x, napspmv_
     return 1;
 }
 
-using WinKernel = void (*)(const WinView, const void *, const void *, const void *, double *,
-                           float *, const Scale, int *);
-static WinKernel pick_window(bool f32, bool step)
+// The windowed kernels by source (0 FP64 values; FP32 values from 1 an FP32, 2 an
+// FP64 vector), and for a step.
+template <int MAXJ>
+using WinKernel = void (*)(const WinJobs<MAXJ>);
+template <int MAXJ>
+static WinKernel<MAXJ> pick_window(int source, bool step)
 {
-    if (f32) return step ? k_window<true, true> : k_window<true, false>;
-    return step ? k_window<false, true> : k_window<false, false>;
+    if (step) return source ? k_window<true, double, true, MAXJ> : k_window<false, double, true, MAXJ>;
+    return source == 0   ? k_window<false, double, false, MAXJ>
+           : source == 1 ? k_window<true, float, false, MAXJ>
+                         : k_window<true, double, false, MAXJ>;
+}
+using WinLongKernel = void (*)(const WinJob, int);
+static WinLongKernel pick_window_long(int source, bool step)
+{
+    if (step) return source ? k_window_long<true, double, true> : k_window_long<false, double, true>;
+    return source == 0   ? k_window_long<false, double, false>
+           : source == 1 ? k_window_long<true, float, false>
+                         : k_window_long<true, double, false>;
 }
 int window_bytes(int64_t srcs, int64_t slots, int64_t words, int vb)
 {
     return win_layout((int)((srcs + 7) & ~7ll), (int)((slots + 7) & ~7ll), (int)words, vb).bytes;
 }
-using WinLongKernel = void (*)(const WinView, int, const void *, const void *, const void *,
-                               double *, float *, const Scale, int *);
-static WinLongKernel pick_window_long(bool f32, bool step)
-{
-    if (f32) return step ? k_window_long<true, true> : k_window_long<true, false>;
-    return step ? k_window_long<false, true> : k_window_long<false, false>;
-}
 int window_long_bytes(int64_t srcs, int vb) { return 64 + 2 * vb * (int)((srcs + 7) & ~7ll); }
-// What the launches of the staged windows need to know, taken once per plan.
+// What the launches of the message kernels and the staged windows need to know,
+// taken once per plan.
 int window_prepare(napspmv_plan_t *P)
 {
     P->wave_gather[0] = one_wave(P, k_unpack<double>);
     P->wave_gather[1] = one_wave(P, k_unpack<float>);
-    P->wave_send[0] = one_wave(P, k_send<double>);
-    P->wave_send[1] = one_wave(P, k_send<float>);
+    P->wave_send[0] = one_wave(P, k_send<double, double, 1>);
+    P->wave_send[1] = one_wave(P, k_send<float, float, 1>);
     if (!P->win.blocks) return NAPSPMV_OK;
-    for (int q = 0; q < 4; q++) {
-        NAP_CUDA(cudaFuncSetAttribute((const void *)pick_window(q & 1, q & 2),
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, kWinSmem));
-        NAP_CUDA(cudaFuncSetAttribute((const void *)pick_window_long(q & 1, q & 2),
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, kWinSmem));
-    }
+    auto allow = [](const void *fn) {
+        return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kWinSmem);
+    };
+    for (int q = 0; q < 3; q++)
+        for (int step = 0; step < 2; step++) {
+            NAP_CUDA(allow((const void *)pick_window<1>(q, step)));
+            NAP_CUDA(allow((const void *)pick_window_long(q, step)));
+            NAP_CUDA(allow((const void *)pick_window<64>(q, step)));
+        }
     for (int f32 = 0; P->win.long_rows && f32 < 2; f32++) {
         int occ = 0;
         NAP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
@@ -2558,83 +2703,155 @@ int window_prepare(napspmv_plan_t *P)
     }
     return NAPSPMV_OK;
 }
-// The SpMV over the staged windows; g, l: g_recv and b_{l->l} (step only).
-static int window_run(const napspmv_plan_t *P, const Opts &o, bool step, const void *x,
-                      const void *g, const void *l, double *y, float *y32, double scale,
-                      int *err, cudaStream_t s, bool pdl)
+static WinJob window_job(const napspmv_plan_t *P, const napspmv_ws_t *ws, const void *x,
+                         const void *l, double *y, float *y32, double scale)
 {
-    const bool f32 = o.precision == NAPSPMV_PREC_F32;
-    const WinKernel fn = pick_window(f32, step);
     const WinPart &W = P->win;
     const SellPart &SP = P->sell[0];
-    const WinView V{W.d_blk[step], SP.d_info,        SP.d_perm,          W.d_col,
-                    SP.d_val,      SP.d_val32,       W.d_runs[step],     (W.max_src + 7) & ~7,
-                    (W.max_slots + 7) & ~7, W.max_words[step]};
+    WinJob J{};
+    J.S = WinView{W.d_blk,  SP.d_info,  SP.d_perm, W.d_col, SP.d_val,
+                  SP.d_val32, W.d_runs, (W.max_src + 7) & ~7, (W.max_slots + 7) & ~7, W.max_words};
+    J.x = x;
+    J.g = ws->grecv;
+    J.l = l;
+    J.y = y;
+    J.y32 = y32;
+    J.sc = make_scale(scale);
+    J.err = ws->err;
+    return J;
+}
+// One launch of windowed SpMVs: several jobs of short rows, or one job.
+template <int MAXJ>
+static int window_launch(int count, const napspmv_plan_t *const *plans, WinJobs<MAXJ> &jobs,
+                         int source, bool step, const Opts &o, cudaStream_t s)
+{
+    const int vb = source ? 4 : 8;
+    const napspmv_plan_t *P = plans[0];
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)W.blocks);
-    cfg.blockDim = dim3((unsigned)W.threads);
-    if (W.long_rows) {
-        const int ctas = o.ctas_per_sm > 0 ? std::min(o.ctas_per_sm, W.long_ctas[f32]) : W.long_ctas[f32];
-        cfg.gridDim = dim3((unsigned)std::min(W.blocks, P->num_sms * ctas));
-        cfg.dynamicSmemBytes = (size_t)window_long_bytes(W.max_src, f32 ? 4 : 8);
-    } else {
-        cfg.dynamicSmemBytes =
-            (size_t)window_bytes(W.max_src, W.max_slots, W.max_words[step], f32 ? 4 : 8);
+    int blocks = 0, threads = 0;
+    size_t smem = 0;
+    jobs.n = count;
+    for (int i = 0; i < count; i++) {
+        const WinPart &W = plans[i]->win;
+        jobs.job[i].block0 = blocks;
+        blocks += W.blocks;
+        threads = std::max(threads, W.threads);
+        smem = std::max(smem, (size_t)(W.long_rows
+                                           ? window_long_bytes(W.max_src, vb)
+                                           : window_bytes(W.max_src, W.max_slots, W.max_words, vb)));
     }
-    if (o.ctas_per_sm > 0 && !W.long_rows) {
+    if (P->win.long_rows) {
+        const int ctas = P->win.long_ctas[source != 0];
+        blocks = std::min(blocks, P->num_sms * (o.ctas_per_sm > 0 ? std::min(o.ctas_per_sm, ctas) : ctas));
+    } else if (o.ctas_per_sm > 0) {
         // at most that many CTAs per SM: each takes its share of the 227 KB
         const size_t share = 227 * 1024 / (size_t)o.ctas_per_sm;
-        if (share > 1024) cfg.dynamicSmemBytes = std::max(cfg.dynamicSmemBytes, share - 1024);
+        if (share > 1024) smem = std::max(smem, share - 1024);
     }
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = pdl ? 1 : 0;
-    if (W.long_rows)
-        NAP_CUDA(cudaLaunchKernelEx(&cfg, pick_window_long(f32, step), V, W.blocks, x, g, l, y, y32,
-                                    make_scale(scale), err));
+    cfg.numAttrs = 1;
+    if (P->win.long_rows)
+        NAP_CUDA(cudaLaunchKernelEx(&cfg, pick_window_long(source, step), jobs.job[0], P->win.blocks));
     else
-        NAP_CUDA(cudaLaunchKernelEx(&cfg, fn, V, x, g, l, y, y32, make_scale(scale), err));
+        NAP_CUDA(cudaLaunchKernelEx(&cfg, pick_window<MAXJ>(source, step), jobs));
     return NAPSPMV_OK;
 }
 
-// Applies on the staged windows: the inter-node messages from their owners to
-// g_recv in one pass, then the windowed SpMV, whose CTAs receive the on-node
-// and off-node values themselves.  The last apply of the chain also fills
-// b_{l->l}, which napspmv_spmv_step reads.
 template <class T>
-static int enqueue_window(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, double *w, int reps,
-                          double scale, const Opts &o, cudaStream_t s, int64_t *kernels)
+static void receives_launch(const napspmv_plan_t *P, const napspmv_ws_t *ws, const double *x,
+                            const int *state, cudaStream_t s)
+{
+    const int64_t n = P->n_bll + P->n_bnl;
+    if (n == 0) return;
+    const int g = (int)std::min<int64_t>((n + NT - 1) / NT, (int64_t)P->num_sms * 32);
+    launch_pdl(true, k_receives<T>, g, 0, s, x, (const int32_t *)P->lists[L_BLL].d_idx,
+               reinterpret_cast<T *>(ws->bll), (int)P->n_bll,
+               (const int32_t *)P->lists[L_BNL].d_idx, reinterpret_cast<T *>(ws->bnl),
+               (int)P->n_bnl, state, (const int *)ws->err);
+}
+
+// Chained applies on the staged windows, of one plan or of several short-row
+// plans at once (one precision): per apply the inter-node messages go from their
+// owners to g_recv in one launch, then the windowed SpMV, whose CTAs receive the
+// on-node and off-node values themselves.
+// keep: napspmv_spmv_step may follow.  It needs the receives of the last apply,
+// so that apply's vector stays in xtmp (a copy if it was v; in FP32 mode the
+// chain's FP64 rows before the last) and g_recv with it; where the caller
+// captures, both receive buffers are filled instead (in FP64 after a batch, as
+// the fused engine does).  Filling b_{l->l} after every call in place of the copy
+// cost a launch and a gather: 118 against 105 us for one apply of a 10^6-row
+// banded matrix, 60 against 52.5 us for the strided 101^3 (GB300).
+// Several plans: 32 Poisson matrices of 10^3 to 10^5 rows take two launches, 52
+// against 82 us per call on the fused engine's four grid barriers, and 8 CG
+// iterations over 16 of them 352 against 749 us.
+template <class T, int MAXJ>
+static int enqueue_windows(int count, napspmv_plan_t *const *plans, napspmv_ws_t *const *ws,
+                           const double *const *v, double *const *w, const int32_t *reps,
+                           const double *scale, const Opts &o, bool keep, bool fill,
+                           cudaStream_t s, int64_t *kernels)
 {
     constexpr bool f32 = sizeof(T) == 4;
-    T *grecv = reinterpret_cast<T *>(ws->grecv), *bll = reinterpret_cast<T *>(ws->bll);
+    const bool fill32 = f32 && count == 1 && !o.batch;
+    int kmax = 0;
+    for (int i = 0; i < count; i++) kmax = std::max(kmax, reps[i]);
     int64_t nk = 0;
-    if (f32) {
-        const int g = (int)std::max<int64_t>(1, std::min<int64_t>((P->n + NT * 8 - 1) / (NT * 8),
-                                                                  (int64_t)P->num_sms * 8));
-        launch_pdl(true, k_to_f32, g, 0, s, v, ws->x32[0], (int64_t)P->n, (const int *)ws->err);
-        nk++;
-    }
-    for (int k = 0; k < reps; k++) {
-        const bool last = k + 1 == reps;
-        const double *x = (k == 0) ? v : (((reps - k) & 1) == 0 ? w : ws->xtmp);
-        double *y = (((reps - 1 - k) & 1) == 0) ? w : ws->xtmp;
-        const T *xs = f32 ? reinterpret_cast<const T *>(ws->x32[k & 1])
-                          : reinterpret_cast<const T *>(x);
-        // FP32 mode: the next apply reads the FP32 copy only
-        float *y32 = f32 && !last ? ws->x32[(k + 1) & 1] : nullptr;
-        if (last && P->n_bll > 0) {
-            launch_pdl(true, k_unpack<T>, msg_grid(P, P->n_bll, P->wave_gather[f32]), 0, s, xs,
-                       (const int32_t *)P->lists[L_BLL].d_idx, bll, (int)P->n_bll,
-                       (const int *)ws->err);
+    SendJobs<MAXJ> sends;
+    WinJobs<MAXJ> wins;
+    const napspmv_plan_t *wp[MAXJ];
+    for (int k = 0; k < kmax; k++) {
+        int ns = 0, nw = 0, blocks = 0;
+        for (int i = 0; i < count; i++) {
+            if (k >= reps[i]) continue;
+            napspmv_plan_t *P = plans[i];
+            napspmv_ws_t *W = ws[i];
+            const int left = reps[i] - 1 - k;  // applies after this one
+            const double *x = (k == 0) ? v[i] : ((left & 1) ? w[i] : W->xtmp);
+            double *y = (left & 1) ? W->xtmp : w[i];
+            const void *xs = f32 && k > 0 ? (const void *)W->x32[left & 1] : (const void *)x;
+            // FP32 mode: the next apply reads the FP32 copy only
+            float *y32 = f32 && left > 0 ? W->x32[(left - 1) & 1] : nullptr;
+            if (f32 && left > 0 && !(keep && left == 1)) y = nullptr;
+            SendJob S = send_job(P, f32, xs, W->grecv, W->err);
+            const bool hold = keep && left == 0 && !fill;
+            if (hold) {
+                S.state = W->state;
+                S.keep = k == 0 ? W->xtmp : nullptr;
+                S.blocks += S.keep ? (int)std::min<int64_t>((P->n + 8 * NT - 1) / (8 * NT),
+                                                            4 * (int64_t)P->num_sms)
+                                   : 1;
+            }
+            if (S.blocks) {
+                S.block0 = blocks;
+                blocks += S.blocks;
+                sends.job[ns++] = S;
+            }
+            if (keep && fill && left == 0) {
+                const double *src = k == 0 ? v[i] : W->xtmp;
+                if (fill32) receives_launch<float>(P, W, src, nullptr, s);
+                else receives_launch<double>(P, W, src, nullptr, s);
+                nk += P->n_bll + P->n_bnl > 0;
+            }
+            wp[nw] = P;
+            wins.job[nw++] = window_job(P, W, xs, nullptr, y, y32, scale ? scale[i] : 1.0);
+        }
+        sends.n = ns;
+        if (ns) {
+            if constexpr (f32) {
+                if (k > 0) launch_pdl(true, k_send<T, float, MAXJ>, blocks, 0, s, sends);
+                else launch_pdl(true, k_send<T, double, MAXJ>, blocks, 0, s, sends);
+            } else {
+                launch_pdl(true, k_send<T, double, MAXJ>, blocks, 0, s, sends);
+            }
             nk++;
         }
-        nk += enqueue_send<T>(P, xs, grecv, ws->err, s, true);
-        if (int rc = window_run(P, o, false, xs, grecv, nullptr, f32 && !last ? nullptr : y, y32,
-                                scale, ws->err, s, true))
-            return rc;
+        if (int rc = window_launch<MAXJ>(nw, wp, wins, !f32 ? 0 : k > 0 ? 1 : 2, false, o, s)) return rc;
         nk++;
         NAP_CUDA(cudaGetLastError());
     }
@@ -2643,12 +2860,15 @@ static int enqueue_window(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, 
 }
 
 static int enqueue_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, double *w, int reps,
-                          double scale, const Opts &o, cudaStream_t s, int64_t *kernels)
+                          double scale, const Opts &o, bool keep, cudaStream_t s,
+                          int64_t *kernels)
 {
     if (o.window)
         return o.precision == NAPSPMV_PREC_F32
-                   ? enqueue_window<float>(P, ws, v, w, reps, scale, o, s, kernels)
-                   : enqueue_window<double>(P, ws, v, w, reps, scale, o, s, kernels);
+                   ? enqueue_windows<float, 1>(1, &P, &ws, &v, &w, &reps, &scale, o, keep,
+                                               ws->captured, s, kernels)
+                   : enqueue_windows<double, 1>(1, &P, &ws, &v, &w, &reps, &scale, o, keep,
+                                                ws->captured, s, kernels);
     auto grid = [&](int64_t n) {
         return (int)std::max<int64_t>(1, std::min<int64_t>((n + NT * 8 - 1) / (NT * 8),
                                                             (int64_t)P->num_sms * 8));
@@ -2715,7 +2935,7 @@ static int enqueue_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, 
 // Chained applies on a capturable stream are recorded once into a CUDA graph
 // per (vectors, workspace, reps, scale, options) and replayed afterwards.
 static int launch_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, double *w, int reps,
-                         double scale, const Opts &o, cudaStream_t s)
+                         double scale, const Opts &o, bool keep, cudaStream_t s)
 {
     if (!o.window) {
         // attributes (dynamic shared memory) are set before any capture
@@ -2729,19 +2949,22 @@ static int launch_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, d
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     NAP_CUDA(cudaStreamIsCapturing(s, &cs));
     const bool use_graph = reps > 1 && s != nullptr && cs == cudaStreamCaptureStatusNone;
-    // what the workspace's receive buffers hold from now on
-    ws->buf_f32 = o.precision == NAPSPMV_PREC_F32 ? 1 : 0;
-    ws->bnl_stale = o.window;
-    if (o.window && cs != cudaStreamCaptureStatusNone) ws->bnl_captured = true;
+    const bool capturing = cs != cudaStreamCaptureStatusNone;
+    const bool f32 = o.precision == NAPSPMV_PREC_F32;
+    ws->recv_f32 = f32;
+    if (keep || !o.window)
+        if (int rc = note_receives(ws, f32 && !o.batch, o.window && !ws->captured && !capturing,
+                                   capturing, s))
+            return rc;
     int64_t nk = 0;
     if (!use_graph) {
-        int rc = enqueue_phased(P, ws, v, w, reps, scale, o, s, &nk);
+        int rc = enqueue_phased(P, ws, v, w, reps, scale, o, keep, s, &nk);
         if (!rc) count_launch(nk);
         return rc;
     }
     for (size_t i = 0; i < P->graphs.size(); i++) {
         auto &g = P->graphs[i];
-        if (g.v == v && g.w == w && g.ws == ws && g.window == o.window && g.reps == reps && g.scale == scale &&
+        if (g.v == v && g.w == w && g.ws == ws && g.window == o.window && g.fill == (ws->captured || !keep) && g.reps == reps && g.scale == scale &&
             g.prec == o.precision && g.vec == o.vec && g.tile_rows == o.tile_rows &&
             g.tile_nnz == o.tile_nnz && g.engine == o.engine && g.stages == o.stages &&
             g.pipeline == o.pipeline && g.ctas_per_sm == o.ctas_per_sm && g.halo == o.halo) {
@@ -2752,7 +2975,7 @@ static int launch_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, d
     }
     cudaGraph_t graph = nullptr;
     NAP_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-    int rc = enqueue_phased(P, ws, v, w, reps, scale, o, s, &nk);
+    int rc = enqueue_phased(P, ws, v, w, reps, scale, o, keep, s, &nk);
     cudaError_t e = cudaStreamEndCapture(s, &graph);
     if (rc) {
         if (graph) cudaGraphDestroy(graph);
@@ -2767,7 +2990,7 @@ static int launch_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, d
         cudaGraphExecDestroy(P->graphs.front().exec);
         P->graphs.erase(P->graphs.begin());
     }
-    P->graphs.push_back({v, w, ws, o.window, reps, o.precision, o.vec, o.tile_rows, o.tile_nnz, o.engine,
+    P->graphs.push_back({v, w, ws, o.window, ws->captured || !keep, reps, o.precision, o.vec, o.tile_rows, o.tile_nnz, o.engine,
                          o.stages, o.pipeline, o.ctas_per_sm, o.halo, scale, exec, nk});
     NAP_CUDA(cudaGraphLaunch(exec, s));
     count_launch(nk);
@@ -2842,7 +3065,7 @@ static bool same_launch(const napspmv_opts &a, const napspmv_opts &b)
 
 int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const *ws,
                 const double *const *v, double *const *w, const int32_t *reps, const double *scale,
-                const napspmv_opts *opts, cudaStream_t s)
+                const napspmv_opts *opts, cudaStream_t s, bool keep, bool as_batch)
 {
     if (count < 1 || count > 64 || !plans || !v || !w || !reps) {
         set_error(NAPSPMV_ERR_ARG, "batch needs 1..64 entries and non-NULL arrays");
@@ -2856,6 +3079,7 @@ int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const
     // every entry resolves the unset fields against its own plan's defaults,
     // so that it runs with the row tiles its plan already holds
     Opts oi[64];
+    const bool opens = !opts || leaves_path_open(*opts);
     int cur = 0;
     NAP_CUDA(cudaGetDevice(&cur));
     if (cur != P0->device) NAP_CUDA(cudaSetDevice(P0->device));
@@ -2875,9 +3099,12 @@ int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const
         oi[i] = resolve_opts(P, opts);
         // several entries share fused launches, whatever engine the options name:
         // validate them for that engine
-        if (count > 1) {
-            oi[i].engine = NAPSPMV_ENGINE_FUSED;
-            oi[i].window = false;
+        oi[i].batch = count > 1 || as_batch;
+        if (oi[i].batch) {
+            // several entries run together: on staged windows where the options
+            // leave the path open and the plan has them, else on the fused engine
+            oi[i].window = oi[i].window && opens && !P->win.long_rows && !oi[i].debug_stall;
+            if (!oi[i].window) oi[i].engine = NAPSPMV_ENGINE_FUSED;
         }
         if ((rc = check_opts(P, oi[i]))) break;
         if ((rc = build_items(P, oi[i].tile_rows, oi[i].tile_nnz))) break;
@@ -2899,7 +3126,7 @@ int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const
         const Opts &o = oi[0];
         if (o.window || o.engine == NAPSPMV_ENGINE_PHASED || o.engine == NAPSPMV_ENGINE_OVERLAP)
             rc = launch_phased(P0, ws && ws[0] ? ws[0] : P0->ws, v[0], w[0], reps[0],
-                               scale ? scale[0] : 1.0, o, s);
+                               scale ? scale[0] : 1.0, o, keep, s);
         else
             rc = launch_fused<1>(1, plans, ws, v, w, reps, scale, o, s);
     } else if (!rc) {
@@ -2907,6 +3134,46 @@ int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const
         // appearance; an entry's bits are those of its plan applied alone on the
         // fused engine with its resolved options, whatever else is in the batch
         bool done[64] = {};
+        {
+            napspmv_plan_t *gp[64];
+            napspmv_ws_t *gw[64];
+            const double *gv[64];
+            double *gx[64];
+            int32_t gr[64];
+            double gs[64];
+            int m = 0, first = -1;
+            bool fill = false;
+            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+            cudaStreamIsCapturing(s, &cs);
+            const bool capturing = cs != cudaStreamCaptureStatusNone;
+            for (int j = 0; j < count; j++) {
+                if (!oi[j].window) continue;
+                napspmv_ws_t *W = ws && ws[j] ? ws[j] : plans[j]->ws;
+                fill = fill || W->captured || capturing;
+            }
+            for (int j = 0; j < count && !rc; j++) {
+                if (!oi[j].window) continue;
+                done[j] = true;
+                if (first < 0) first = j;
+                gp[m] = plans[j];
+                gw[m] = ws && ws[j] ? ws[j] : plans[j]->ws;
+                gv[m] = v[j];
+                gx[m] = w[j];
+                gr[m] = reps[j];
+                gs[m] = scale ? scale[j] : 1.0;
+                gw[m]->recv_f32 = oi[j].precision == NAPSPMV_PREC_F32;
+                if (keep) rc = note_receives(gw[m], false, !fill, capturing, s);
+                m++;
+            }
+            int64_t nk = 0;
+            if (m && !rc)
+                rc = oi[first].precision == NAPSPMV_PREC_F32
+                         ? enqueue_windows<float, 64>(m, gp, gw, gv, gx, gr, gs, oi[first], keep,
+                                                      fill, s, &nk)
+                         : enqueue_windows<double, 64>(m, gp, gw, gv, gx, gr, gs, oi[first], keep,
+                                                       fill, s, &nk);
+            if (m && !rc) count_launch(nk);
+        }
         for (int i = 0; i < count && !rc; i++) {
             if (done[i]) continue;
             napspmv_plan_t *gp[64];
@@ -3075,42 +3342,36 @@ extern "C" int napspmv_spmv_step(napspmv_plan_t *P, napspmv_ws_t *ws, const doub
                                      "for FP32) before the step");
         return NAPSPMV_ERR_STATE;
     }
-    SpmvLaunch L;
-    if (!o.window) {
-        if ((rc = spmv_launch(P, o, kFull, L))) return rc;
-        if ((W->bnl_stale || W->bnl_captured) && P->n_bnl > 0) {
-            // the last apply kept b_{nl->l} on chip: unpack it from g_recv
-            const cudaStream_t st = (cudaStream_t)stream;
-            if (f32)
-                launch_pdl(false, k_unpack<float>, msg_grid(P, P->n_bnl, one_wave(P, k_unpack<float>)),
-                           0, st, reinterpret_cast<const float *>(W->grecv),
-                           (const int32_t *)P->d_unp_src, reinterpret_cast<float *>(W->bnl),
-                           (int)P->n_bnl, (const int *)W->err);
-            else
-                launch_pdl(false, k_unpack<double>,
-                           msg_grid(P, P->n_bnl, one_wave(P, k_unpack<double>)), 0, st,
-                           (const double *)W->grecv, (const int32_t *)P->d_unp_src, W->bnl,
-                           (int)P->n_bnl, (const int *)W->err);
-            count_launch(1);
-            W->bnl_stale = false;
-        }
-    }
-    auto step = [&](const void *x) -> int {
-        if (o.window)
-            return window_run(P, o, true, x, W->grecv, W->bll, w, nullptr, scale, W->err,
-                              (cudaStream_t)stream, true);
-        spmv_run(L, x, W, w, nullptr, scale, o.stages, (cudaStream_t)stream, pdl);
-        return NAPSPMV_OK;
-    };
-    if (f32) {
-        const int g = (int)std::max<int64_t>(1, std::min<int64_t>((P->n + NT - 1) / NT,
-                                                                  (int64_t)P->num_sms * 8));
-        k_to_f32<<<g, NT, 0, (cudaStream_t)stream>>>(v, W->x32[0], P->n, W->err);
-        if ((rc = step(W->x32[0]))) return rc;
-        count_launch(2);
-    } else {
-        if ((rc = step(v))) return rc;
+    const cudaStream_t st = (cudaStream_t)stream;
+    if (o.window && W->recv_vector && !W->captured && W->recv_f32 == f32) {
+        // on the windows: on-node receives from the kept vector, off-node from g_recv
+        WinJobs<1> jobs{};
+        jobs.job[0] = window_job(P, W, v, W->xtmp, w, nullptr, scale);
+        const napspmv_plan_t *pl[1] = {P};
+        if ((rc = window_launch<1>(1, pl, jobs, f32 ? 2 : 0, true, o, st))) return rc;
         count_launch(1);
+    } else {
+        if (W->recv_vector || W->captured) {
+            // the receive buffers from the kept vector (after a capture, if the
+            // device word says that the last apply kept one)
+            const int *state = W->captured ? W->state : nullptr;
+            if (f32) receives_launch<float>(P, W, W->xtmp, state, st);
+            else receives_launch<double>(P, W, W->xtmp, state, st);
+            count_launch(1);
+            if (!W->captured) W->recv_vector = false;
+        }
+        SpmvLaunch L;
+        if ((rc = spmv_launch(P, o, kFull, L))) return rc;
+        if (f32) {
+            const int g = (int)std::max<int64_t>(1, std::min<int64_t>((P->n + NT - 1) / NT,
+                                                                      (int64_t)P->num_sms * 8));
+            k_to_f32<<<g, NT, 0, st>>>(v, W->x32[0], P->n, W->err);
+            spmv_run(L, W->x32[0], W, w, nullptr, scale, o.stages, st, pdl);
+            count_launch(2);
+        } else {
+            spmv_run(L, v, W, w, nullptr, scale, o.stages, st, pdl);
+            count_launch(1);
+        }
     }
     NAP_CUDA(cudaGetLastError());
     if (cur != P->device) cudaSetDevice(cur);

@@ -124,7 +124,7 @@ struct SellPart {
 // values instead of 128.  Plans of long rows keep a plain list: one source a slot.
 constexpr uint16_t kWinPad = 0xffff;      // padding slots, as kSellPad
 constexpr uint32_t kFromRecv = 0x80000000u;  // source in g_recv, else in x
-constexpr uint32_t kFromBll = 0x40000000u;   // (step sources) source in b_{l->l}
+constexpr uint32_t kFromNode = 0x40000000u;  // an on-node receive, source in x
 struct WinBlock {
     int32_t chunk0, chunks;  // its chunks of the whole matrix's sliced rows
     int32_t slot0, slots;    // its stored-entry slots
@@ -139,12 +139,10 @@ struct WinPart {
     int32_t threads = 0;  // per CTA
     bool long_rows = false;     // rows of more than 12 entries: k_window_long
     int32_t long_ctas[2] = {};  // its CTAs per SM (FP64, FP32)
-    // largest block: window slots, entry slots, run words (apply, step)
-    int32_t max_src = 0, max_slots = 0, max_words[2] = {};
+    int32_t max_src = 0, max_slots = 0, max_words = 0;  // largest block: slots, entry slots, run words
     uint16_t *d_col = nullptr;  // window slot of every sliced-row slot
-    // for an apply, and for a step with on-node values from b_{l->l}
-    WinBlock *d_blk[2] = {};
-    uint32_t *d_runs[2] = {};
+    WinBlock *d_blk = nullptr;
+    uint32_t *d_runs = nullptr;
 };
 
 }  // namespace nap
@@ -159,9 +157,13 @@ struct napspmv_ws_s {
     // read as float arrays)
     float *x32[2] = {nullptr, nullptr};
     int buf_f32 = 0;
-    // the staged windows leave b_{nl->l} in shared memory only: the buffer here is
-    // behind g_recv (stale), for good once such an apply was captured by the caller
-    bool bnl_stale = false, bnl_captured = false;
+    // the staged windows keep the receives in shared memory: what a later
+    // napspmv_spmv_step takes them from is the last apply's vector, in xtmp, and
+    // g_recv (recv_f32: of FP32 copies).  captured: the caller captured an apply,
+    // whose replays the host does not see; *state (device) is then 1 only while
+    // the last apply that ran kept its vector, and later applies fill the buffers.
+    bool recv_vector = false, recv_f32 = false, captured = false;
+    int *state = nullptr;
     double *hv = nullptr, *hw = nullptr;  // staging of napspmv_apply_host
     unsigned long long *ctr = nullptr;  // the fused engine's grid barrier: arrivals, generation
     int *err = nullptr;                 // sticky device status
@@ -225,7 +227,7 @@ struct napspmv_plan_s {
     // instantiated CUDA graphs of chained phased applies, newest last
     struct GraphEntry {
         const void *v, *w, *ws;
-        bool window;
+        bool window, fill;
         int32_t reps, prec, vec, tile_rows, tile_nnz, engine, stages, pipeline, ctas_per_sm, halo;
         double scale;
         cudaGraphExec_t exec;
@@ -249,6 +251,7 @@ void plan_free(napspmv_plan_t *P);
 // Options with every unset field resolved; window: run on the staged windows.
 struct Opts : napspmv_opts {
     bool window = false;
+    bool batch = false;  // FP64 receive buffers in both precisions, as on the fused engine
 };
 Opts resolve_opts(const napspmv_plan_t *P, const napspmv_opts *o);
 // the fields that name an engine, a pipeline or a tile shape are all unset
@@ -258,5 +261,6 @@ bool leaves_path_open(const napspmv_opts &o);
 int check_opts(const napspmv_plan_t *P, const napspmv_opts &o);
 int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const *ws,
                 const double *const *v, double *const *w, const int32_t *reps,
-                const double *scale, const napspmv_opts *opts, cudaStream_t s);
+                const double *scale, const napspmv_opts *opts, cudaStream_t s, bool keep = true,
+                bool as_batch = false);
 }  // namespace nap

@@ -919,7 +919,7 @@ __global__ void k_win_block(const int32_t *rp, const uint32_t *col, WinGeom G, i
                             int32_t *nsrc, int32_t *nent, int32_t *stat, const int64_t *osl,
                             const int64_t *osrc,
                             const int32_t *bll_j, const int32_t *unp_src, const uint32_t *scol,
-                            uint32_t *src, uint32_t *src_step, uint16_t *col16)
+                            uint32_t *src, uint16_t *col16)
 {
     extern __shared__ uint32_t bits[];  // [words], then (FILL) marked positions before each word
     __shared__ int warp_sum[8];         // 256 threads
@@ -976,17 +976,9 @@ __global__ void k_win_block(const int32_t *rp, const uint32_t *col, WinGeom G, i
                 pre[w] = before;
                 for (uint32_t m = bits[w]; m; m &= m - 1) {
                     const int32_t f = 32 * w + __ffs(m) - 1;
-                    uint32_t s, st;
-                    if (f < own) {
-                        s = st = (uint32_t)G.part.row(t, f);
-                    } else if (f < own + nl) {
-                        s = (uint32_t)bll_j[l0 + f - own];
-                        st = kFromBll | (uint32_t)(l0 + f - own);
-                    } else {
-                        s = st = kFromRecv | (uint32_t)unp_src[r0 + f - own - nl];
-                    }
-                    src[s0 + before] = s;
-                    src_step[s0 + before] = st;
+                    src[s0 + before] = f < own        ? (uint32_t)G.part.row(t, f)
+                                       : f < own + nl ? kFromNode | (uint32_t)bll_j[l0 + f - own]
+                                                      : kFromRecv | (uint32_t)unp_src[r0 + f - own - nl];
                     before++;
                 }
             }
@@ -1109,7 +1101,7 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
         const int grid = (int)std::min<int64_t>(nblk, 1 << 20);
         k_win_block<false><<<grid, 256, 4 * words>>>(P->d_rowptr, P->d_colenc, G, nblk, nsrc.p,
                                                      nent.p, stat.p, nullptr, nullptr, nullptr,
-                                                     nullptr, nullptr, nullptr, nullptr, nullptr);
+                                                     nullptr, nullptr, nullptr, nullptr);
         CK(cudaGetLastError());
         cb.max_i32(nsrc.p, stat.p + 1, nblk);
         cb.max_i32(nent.p, stat.p + 2, nblk);
@@ -1144,39 +1136,38 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
     };
     const int64_t total = offsets(nsrc.p, osrc);
     const size_t slots = (size_t)std::max<int64_t>(P->sell[0].slots, 1);
-    dvec<uint32_t> src(std::max<int64_t>(total, 1)), src_step(std::max<int64_t>(total, 1));
+    dvec<uint32_t> src(std::max<int64_t>(total, 1));
     CK(cudaMalloc(&W.d_col, sizeof(uint16_t) * slots + 256));
     const int grid = (int)std::min<int64_t>(nblk, 1 << 20);
     k_win_block<true><<<grid, 256, 8 * words>>>(
         P->d_rowptr, P->d_colenc, G, nblk, nullptr, nullptr, nullptr, off.p + nblk + 1, osrc.p,
-        P->lists[L_BLL].d_idx, P->d_unp_src, P->sell[0].d_col, src.p, src_step.p, W.d_col);
+        P->lists[L_BLL].d_idx, P->d_unp_src, P->sell[0].d_col, src.p, W.d_col);
     CK(cudaGetLastError());
-    for (int q = 0; q < 2 && W.long_rows; q++) {  // plain lists
-        if (total > INT32_MAX || st[1] >= kWinPad) return;
-        CK(cudaMalloc(&W.d_blk[q], sizeof(WinBlock) * nblk));
-        k_win_blocks<<<(int)((nblk + 255) / 256), 256>>>(nblk, off.p, off.p + nblk + 1, nsrc.p,
-                                                         nsrc.p, osrc.p, 1, W.d_blk[q]);
+    if (st[1] >= kWinPad) return;
+    CK(cudaMalloc(&W.d_blk, sizeof(WinBlock) * nblk));
+    const int bgrid = (int)((nblk + 255) / 256);
+    if (W.long_rows) {  // plain lists
+        if (total > INT32_MAX) return;
+        k_win_blocks<<<bgrid, 256>>>(nblk, off.p, off.p + nblk + 1, nsrc.p, nsrc.p, osrc.p, 1,
+                                     W.d_blk);
         CK(cudaGetLastError());
-        W.d_runs[q] = q ? src_step.release() : src.release();
-    }
-    for (int q = 0; q < 2 && !W.long_rows; q++) {
-        const uint32_t *s = q ? src_step.p : src.p;
+        W.d_runs = src.release();
+    } else {
         const int wgrid = blocks_for(32 * nblk);
-        k_win_runs<false><<<wgrid, 256>>>(nblk, s, osrc.p, nsrc.p, nword.p, nullptr, nullptr);
+        k_win_runs<false><<<wgrid, 256>>>(nblk, src.p, osrc.p, nsrc.p, nword.p, nullptr, nullptr);
         CK(cudaGetLastError());
         cb.max_i32(nword.p, stat.p + 3, nblk);
         const int64_t all = offsets(nword.p, oword);
         if (all / 4 > (int64_t)INT32_MAX) return;
-        CK(cudaMalloc(&W.d_blk[q], sizeof(WinBlock) * nblk));
-        CK(cudaMalloc(&W.d_runs[q], sizeof(uint32_t) * std::max<int64_t>(all, 1)));
-        k_win_runs<true><<<wgrid, 256>>>(nblk, s, osrc.p, nsrc.p, nullptr, oword.p, W.d_runs[q]);
+        CK(cudaMalloc(&W.d_runs, sizeof(uint32_t) * std::max<int64_t>(all, 1)));
+        k_win_runs<true><<<wgrid, 256>>>(nblk, src.p, osrc.p, nsrc.p, nullptr, oword.p, W.d_runs);
         CK(cudaGetLastError());
-        k_win_blocks<<<(int)((nblk + 255) / 256), 256>>>(nblk, off.p, off.p + nblk + 1, nsrc.p,
-                                                         nword.p, oword.p, 4, W.d_blk[q]);
+        k_win_blocks<<<bgrid, 256>>>(nblk, off.p, off.p + nblk + 1, nsrc.p, nword.p, oword.p, 4,
+                                     W.d_blk);
         CK(cudaGetLastError());
         CK(cudaMemcpy(st, stat.p, sizeof(st), cudaMemcpyDeviceToHost));
-        if (window_bytes(st[1], st[2], st[3], 8) > kWinSmem || st[1] >= kWinPad) return;
-        W.max_words[q] = st[3];
+        if (window_bytes(st[1], st[2], st[3], 8) > kWinSmem) return;
+        W.max_words = st[3];
     }
     W.rows = G.cut.rows;
     W.max_src = st[1];
@@ -1690,7 +1681,7 @@ void plan_free(napspmv_plan_t *P)
         for (void *p : sp)
             if (p) cudaFree(p);
     }
-    void *wp[] = {P->win.d_col, P->win.d_blk[0], P->win.d_blk[1], P->win.d_runs[0], P->win.d_runs[1]};
+    void *wp[] = {P->win.d_col, P->win.d_blk, P->win.d_runs};
     for (void *p : wp)
         if (p) cudaFree(p);
     delete P;

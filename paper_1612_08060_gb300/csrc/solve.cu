@@ -154,22 +154,34 @@ int cg_alloc(CgBuffers &B, int64_t n, cudaStream_t s)
     return NAPSPMV_OK;
 }
 
+// q <- A p with the plan's default options.  keep: the caller's last apply, whose
+// receives napspmv_spmv_step may ask for.
+int apply_one(napspmv_plan_t *P, const double *p, double *q, int32_t precision, bool keep,
+              cudaStream_t s)
+{
+    napspmv_opts o{};
+    o.precision = precision;
+    const int32_t reps = 1;
+    const double scale = 1.0;
+    return apply_batch(1, &P, nullptr, &p, &q, &reps, &scale, &o, s, keep);
+}
+
 int grid_for(const napspmv_plan_t *P, int64_t n)
 {
     return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)P->num_sms * 8));
 }
 
-// CG on A x = b from the x given, with the apply options `o`.  Stops when the
+// CG on A x = b from the x given, products at `precision`.  Stops when the
 // recursive residual satisfies ||r|| <= rtol * ||b|| or after max_it
 // iterations (checked on the host every `poll` iterations).  x, b: device.
 int cg_core(napspmv_plan_t *P, const double *b, double *x, double rtol, int max_it,
-            const napspmv_opts &o, CgBuffers &B, int *iters)
+            int32_t precision, CgBuffers &B, int *iters)
 {
     cudaStream_t s = B.s;
     const int64_t n = P->n;
     const int g = grid_for(P, n);
     int rc;
-    if ((rc = napspmv_apply_ex(P, nullptr, x, B.q, 1, 1.0, &o, s))) return rc;
+    if ((rc = apply_one(P, x, B.q, precision, false, s))) return rc;
     k_resid<<<g, 256, 0, s>>>(B.r, B.p, b, B.q, n);
     count_launch(1);
     if ((rc = dot_launch(b, b, n, &B.sc->bb, B.ds, s))) return rc;
@@ -183,7 +195,7 @@ int cg_core(napspmv_plan_t *P, const double *b, double *x, double rtol, int max_
     bool done = std::sqrt(h.rr) <= rtol * bn;
     while (!done && it < max_it) {
         for (int q = 0; q < poll && it < max_it; q++, it++) {
-            if ((rc = napspmv_apply_ex(P, nullptr, B.p, B.q, 1, 1.0, &o, s))) return rc;
+            if ((rc = apply_one(P, B.p, B.q, precision, false, s))) return rc;
             if ((rc = dot_launch(B.p, B.q, n, &B.sc->pq, B.ds, s))) return rc;
             k_alpha<<<1, 1, 0, s>>>(B.sc);
             k_update_xr<<<g, 256, 0, s>>>(x, B.r, B.p, B.q, n, B.sc);
@@ -208,10 +220,8 @@ int cg_core(napspmv_plan_t *P, const double *b, double *x, double rtol, int max_
 int true_relres(napspmv_plan_t *P, const double *b, const double *x, CgBuffers &B, double *out)
 {
     cudaStream_t s = B.s;
-    napspmv_opts o{};  // unset fields: the plan's defaults
-    o.precision = NAPSPMV_PREC_F64;
     int rc;
-    if ((rc = napspmv_apply_ex(P, nullptr, x, B.q, 1, 1.0, &o, s))) return rc;
+    if ((rc = apply_one(P, x, B.q, NAPSPMV_PREC_F64, true, s))) return rc;
     k_resid<<<grid_for(P, P->n), 256, 0, s>>>(B.r, nullptr, b, B.q, P->n);
     count_launch(1);
     if ((rc = dot_launch(B.r, B.r, P->n, &B.sc->rnorm0, B.ds, s))) return rc;
@@ -258,10 +268,8 @@ int napspmv_cg(napspmv_plan_t *P, const double *b, double *x, double rtol, int32
     CgBuffers B;
     int rc = cg_alloc(B, P->n, (cudaStream_t)stream);
     if (rc) return rc;
-    napspmv_opts o{};
-    o.precision = NAPSPMV_PREC_F64;
     int it = 0;
-    if ((rc = cg_core(P, b, x, rtol, max_it, o, B, &it))) return rc;
+    if ((rc = cg_core(P, b, x, rtol, max_it, NAPSPMV_PREC_F64, B, &it))) return rc;
     double rr = 0;
     if ((rc = true_relres(P, b, x, B, &rr))) return rc;
     if (info) {
@@ -289,8 +297,6 @@ int napspmv_cg_ir(napspmv_plan_t *P, const double *b, double *x, double rtol, do
     int rc = cg_alloc(B, P->n, s);
     if (rc) return rc;
     if ((rc = cg_alloc(I, P->n, s))) return rc;
-    napspmv_opts o32{};
-    o32.precision = NAPSPMV_PREC_F32;
     int outer = 0, inner_total = 0;
     double rr = 0;
     for (;;) {
@@ -299,7 +305,7 @@ int napspmv_cg_ir(napspmv_plan_t *P, const double *b, double *x, double rtol, do
         // inner solve A d = r with FP32-stored values, d_0 = 0
         NAP_CUDA(cudaMemsetAsync(I.d, 0, sizeof(double) * P->n, s));
         int it = 0;
-        if ((rc = cg_core(P, B.r, I.d, inner_rtol, inner_max, o32, I, &it))) return rc;
+        if ((rc = cg_core(P, B.r, I.d, inner_rtol, inner_max, NAPSPMV_PREC_F32, I, &it))) return rc;
         k_add<<<grid_for(P, P->n), 256, 0, s>>>(x, I.d, P->n);
         count_launch(1);
         NAP_CUDA(cudaGetLastError());
@@ -472,7 +478,7 @@ int slot_setup(int32_t count, const napspmv_cg_slot *slots, SlotVecs &S)
 }
 
 int slot_apply(int32_t count, const napspmv_cg_slot *slots, bool from_x, int32_t precision,
-               cudaStream_t st)
+               bool keep, cudaStream_t st)
 {
     napspmv_plan_t *plans[kMaxSlots];
     napspmv_ws_t *wss[kMaxSlots];
@@ -489,8 +495,9 @@ int slot_apply(int32_t count, const napspmv_cg_slot *slots, bool from_x, int32_t
         sc[i] = 1.0;
     }
     // A slot whose matrix holds NAPSPMV_SOLO_NNZ or more stored entries gets an
-    // apply of its own on the phased engine; the others share one persistent
-    // launch.  Measured on GB300 (FP32 mode, one apply): a 2.0M-row 7-point
+    // apply of its own (staged windows or the phased engine); the others share
+    // launches: the windows' two per apply, or the persistent one of the plans
+    // without windows.  Measured on GB300 (FP32 mode, one apply): a 2.0M-row 7-point
     // plan takes 77 us phased against 191 us in the persistent launch, a
     // 0.4M-row one 33 against 70 us; below about half a million entries the
     // shared launch costs less than a call per slot.  The choice depends on the
@@ -503,7 +510,7 @@ int slot_apply(int32_t count, const napspmv_cg_slot *slots, bool from_x, int32_t
             napspmv_opts o{};  // unset fields: the plan's defaults
             o.precision = precision;
             o.engine = NAPSPMV_ENGINE_PHASED;
-            if (int rc = apply_batch(1, &plans[i], &wss[i], &vs[i], &ws_[i], &reps[i], &sc[i], &o, st))
+            if (int rc = apply_batch(1, &plans[i], &wss[i], &vs[i], &ws_[i], &reps[i], &sc[i], &o, st, keep))
                 return rc;
         } else {
             plans[nb] = plans[i];
@@ -516,8 +523,7 @@ int slot_apply(int32_t count, const napspmv_cg_slot *slots, bool from_x, int32_t
     if (nb == 0) return NAPSPMV_OK;
     napspmv_opts o{};  // unset fields: each slot's own plan defaults
     o.precision = precision;
-    o.engine = NAPSPMV_ENGINE_FUSED;
-    return apply_batch(nb, plans, wss, vs, ws_, reps, sc, &o, st);
+    return apply_batch(nb, plans, wss, vs, ws_, reps, sc, &o, st, keep, true);
 }
 
 struct Partials {
@@ -545,7 +551,7 @@ int napspmv_cg_batch_init(int32_t count, const napspmv_cg_slot *slots, int32_t p
     P.s = st;
     NAP_CUDA(cudaMallocAsync(&P.p, sizeof(double) * 2 * kSlotBlocksMax * count, st));
     if (x_is_zero) return slot_vec(S, 4, P.p, st);
-    if ((rc = slot_apply(count, slots, true, precision, st))) return rc;
+    if ((rc = slot_apply(count, slots, true, precision, true, st))) return rc;
     return slot_vec(S, 0, P.p, st);
 }
 
@@ -564,7 +570,7 @@ int napspmv_cg_batch_iterate(int32_t count, const napspmv_cg_slot *slots, int32_
     P.s = st;
     NAP_CUDA(cudaMallocAsync(&P.p, sizeof(double) * 2 * kSlotBlocksMax * count, st));
     for (int it = 0; it < iters; it++) {
-        if ((rc = slot_apply(count, slots, false, precision, st))) return rc;
+        if ((rc = slot_apply(count, slots, false, precision, it + 1 == iters, st))) return rc;
         if ((rc = slot_vec(S, 1, P.p, st))) return rc;
         if ((rc = slot_vec(S, 2, P.p, st))) return rc;
         if ((rc = slot_vec(S, 3, P.p, st))) return rc;

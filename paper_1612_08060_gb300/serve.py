@@ -16,7 +16,7 @@ cache ``key``) and right-hand side (``rhs``).  The server:
   the host reads the other group's scalars (one device-to-host copy per step,
   awaited on its own event), retires what finished and queues that group's next
   step, so the device never idles on a host decision;
-* a step of those groups launches one batched fused apply for the group's SpMV
+* a step of those groups launches one batched apply for the group's SpMV
   requests, one batched CG-residual step (FP64 values) for the solves entering
   an outer iteration and ``iters_per_step`` batched CG iterations (FP32 values)
   for the solves in their inner loop;
@@ -27,9 +27,9 @@ cache ``key``) and right-hand side (``rhs``).  The server:
   needs thousands of CG iterations, and with 8 per step its host round trips,
   not its arithmetic, set the slowest latencies.
 
-Each request's arithmetic is independent of what else is in flight: a fixed
-engine per request (the fused engine with its own plan's options, or the phased
-engine on a large matrix), a fixed number of CG iterations per step (by its
+Each request's arithmetic is independent of what else is in flight: engines of
+equal bits per request (staged windows or the fused engine, or the phased engine
+on a large matrix), a fixed number of CG iterations per step (by its
 matrix's size), fixed per-row and per-slot reduction orders and the same
 sequence of steps whatever its group holds, so a request served alone and in a
 mix gives the same bits.  ``max_active=1`` is the plain per-request loop
@@ -101,7 +101,10 @@ class Server:
         self.stream = torch.cuda.Stream(self.dev)       # fused launches and CG kernels
         self.solo_stream = torch.cuda.Stream(self.dev)  # products on large matrices
         self.solo_opts = nap.make_opts(engine=nap.ENGINE_PHASED)
-        # unset fields: each plan's own defaults (one launch per option set)
+        # unset fields: each plan's own defaults.  Several entries left open share the
+        # staged windows' launches, or the fused engine's where a plan has none; one
+        # entry takes the fused engine, which gives the same bits as either
+        self.batch_opts = nap.make_opts()
         self.fused_opts = nap.make_opts(engine=nap.ENGINE_FUSED)
         self.tune_cache = tune_cache
         self.hbuf = [torch.zeros(max_active, 2, 8, dtype=torch.float64).pin_memory()
@@ -236,7 +239,8 @@ class Server:
                 for grp in self._chunks(spmv):
                     nap.napspmv_apply_batch([r.m.plan for r in grp], [r.v for r in grp],
                                             [r.w for r in grp], [1] * len(grp),
-                                            opts=self.fused_opts, ws=[r.ws for r in grp], stream=s)
+                                            opts=self.batch_opts if len(grp) > 1 else self.fused_opts,
+                                            ws=[r.ws for r in grp], stream=s)
             for grp in self._chunks(outer):
                 nap.napspmv_cg_batch_init([r.outer_slot for r in grp], nap.PREC_F64, stream=s)
             for grp in self._chunks(inner):
