@@ -132,22 +132,6 @@ __device__ __forceinline__ uint32_t ld_stream_hint_u32(const uint32_t *p, uint64
     return v;
 }
 
-// Programmatic dependent launch (sm_90 and later).  A kernel launched with the
-// programmatic-serialization attribute may become resident while its
-// predecessor in the stream drains: griddep_wait() waits, in hardware, until
-// the predecessor grid has completed and its writes are visible, and
-// griddep_done(), called when a CTA has issued its last work, lets the
-// dependent grid start as this grid's CTAs finish (a CTA that exits early
-// counts as done).  Without a programmatic predecessor both are no-ops.
-__device__ __forceinline__ void griddep_wait()
-{
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-__device__ __forceinline__ void griddep_done()
-{
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 __device__ __forceinline__ long long globaltimer()
 {
     long long t;

@@ -27,6 +27,24 @@ void count_launch(int64_t n = 1);
         if (e_ != cudaSuccess) return ::nap::cuda_error(e_, #call); \
     } while (0)
 
+#ifdef __CUDACC__
+// Programmatic dependent launch (sm_90 and later).  A kernel launched with the
+// programmatic-serialization attribute may become resident while its
+// predecessor in the stream drains: griddep_wait() waits, in hardware, until
+// the predecessor grid has completed and its writes are visible, and
+// griddep_done(), called when a CTA has issued its last work, lets the
+// dependent grid start as this grid's CTAs finish (a CTA that exits early
+// counts as done).  Without a programmatic predecessor both are no-ops.
+__device__ __forceinline__ void griddep_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void griddep_done()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 // ----------------------------------------------------------- column coding
 // A column of the three-block CSR stores its block in the top two bits:
 // 0 = on-process (index into v), 1 = on-node (index into b_{l->l}),

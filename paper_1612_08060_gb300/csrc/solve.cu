@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <utility>
 
 #include "internal.h"
 
@@ -34,65 +35,128 @@ __device__ __forceinline__ double block_sum(double v, double *sh)
     return v;  // valid in thread 0
 }
 
-// Partial sums per block over indices i = b*256 + t + q*1024*256; the last
-// block to finish adds the 1024 partials in index order and resets the ticket.
-__global__ void __launch_bounds__(kThreads)
-    k_dot(const double *__restrict__ x, const double *__restrict__ y, int64_t n,
-          double *partial, unsigned *ticket, double *result)
-{
-    __shared__ double sh[kThreads / 32];
-    __shared__ bool last;
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n;
-         i += (int64_t)kDotBlocks * kThreads)
-        s = fma(x[i], y[i], s);
-    s = block_sum(s, sh);
-    if (threadIdx.x == 0) {
-        partial[blockIdx.x] = s;
-        __threadfence();
-        last = atomicAdd(ticket, 1u) == kDotBlocks - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    double a = 0.0;
-    for (int b = threadIdx.x; b < kDotBlocks; b += kThreads) a += __ldcg(partial + b);
-    a = block_sum(a, sh);
-    if (threadIdx.x == 0) {
-        *result = a;
-        *ticket = 0;
-    }
-}
-
 struct Scal {
     double rr, rr_new, pq, alpha, beta, bb, rnorm0;
+    int err, pad;  // the workspace's error flag, as the last CG iteration saw it
 };
 
-__global__ void k_alpha(Scal *s) { s->alpha = s->rr / s->pq; }
-__global__ void k_beta(Scal *s)
+// Sum of 256 values (a group of 8 warps, numbered g in its block) in a fixed tree;
+// valid in the group's thread 0.
+__device__ __forceinline__ double group_sum(double v, double *sh, int g)
 {
-    s->beta = s->rr_new / s->rr;
-    s->rr = s->rr_new;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    if (l == 0) sh[w] = v;
+    __syncthreads();
+    if ((w & 7) == 0) {
+        v = l < 8 ? sh[8 * g + l] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    }
+    __syncthreads();
+    return v;
 }
 
-// x += alpha p ; r -= alpha q
-__global__ void k_update_xr(double *x, double *r, const double *p, const double *q, int64_t n,
-                            const Scal *s)
+// FP64 dot products over a fixed partition: partial b, of 1,024, sums the indices
+// i = b*256 + t + q*1024*256 over the 256 threads t of a group, and the last CTA
+// to finish adds the partials in index order and resets the ticket.  A CTA is
+// four groups, so that a quarter of the tickets are drawn; partials past the
+// vector's end are 0 and not launched.
+// WHAT: kDot    *result = x.y
+//       kAlpha  pq = x.y (x = p, y = q), alpha = rr / pq
+//       kUpdate x += alpha p, r -= alpha q, rr_new = r.r, beta = rr_new / rr, rr = rr_new
+// The scalar recurrences ride on the last CTA: on their own they were two more
+// launches per CG iteration, and the update and its dot product two passes.  With
+// the windows an iteration is five launches in place of ten: 39 us of a CG-IR
+// solve on 63^3 with FP32 values, where it was 55 (GB300); latency-bound.
+enum CgOp { kDot, kAlpha, kUpdate };
+constexpr int kDotGroups = 4;
+struct CgVecs {
+    const double *x, *y;  // kUpdate: p, q
+    double *sol, *res;    // kUpdate: x, r
+    int64_t n;
+    double *partial;
+    unsigned *ticket;
+    double *result;
+    Scal *sc;
+    const int *err;
+};
+template <int WHAT>
+__global__ void __launch_bounds__(kThreads *kDotGroups) k_cg(const CgVecs V)
 {
-    const double a = s->alpha;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        x[i] = fma(a, p[i], x[i]);
-        r[i] = fma(-a, q[i], r[i]);
+    __shared__ double sh[8 * kDotGroups];
+    __shared__ bool last;
+    griddep_wait();
+    const int g = threadIdx.x / kThreads, t = threadIdx.x % kThreads;
+    const int b = blockIdx.x * kDotGroups + g;
+    const double a = WHAT == kUpdate ? V.sc->alpha : 0.0;
+    double s = 0.0;
+    for (int64_t i = (int64_t)b * kThreads + t; i < V.n; i += (int64_t)kDotBlocks * kThreads) {
+        if (WHAT == kUpdate) {
+            V.sol[i] = fma(a, V.x[i], V.sol[i]);
+            const double r = fma(-a, V.y[i], V.res[i]);
+            V.res[i] = r;
+            s = fma(r, r, s);
+        } else {
+            s = fma(V.x[i], V.y[i], s);
+        }
+    }
+    s = group_sum(s, sh, g);
+    if (t == 0) V.partial[b] = s;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(V.ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    griddep_done();
+    if (!last) return;
+    __threadfence();
+    const int nb = gridDim.x * kDotGroups;
+    double v = 0.0;
+    if (g == 0)
+        for (int q = t; q < kDotBlocks; q += kThreads) v += q < nb ? __ldcg(V.partial + q) : 0.0;
+    v = group_sum(v, sh, g);
+    if (threadIdx.x == 0) {
+        *V.ticket = 0;
+        if (WHAT == kDot) *V.result = v;
+        if (WHAT == kAlpha) {
+            V.sc->pq = v;
+            V.sc->alpha = V.sc->rr / v;
+        }
+        if (WHAT == kUpdate) {
+            V.sc->rr_new = v;
+            V.sc->beta = v / V.sc->rr;
+            V.sc->rr = v;
+            V.sc->err = *(volatile const int *)V.err;
+        }
     }
 }
 // p = r + beta p
-__global__ void k_update_p(double *p, const double *r, int64_t n, const Scal *s)
+__global__ void __launch_bounds__(kThreads) k_update_p(double *p, const double *r, int64_t n, const Scal *s)
 {
+    griddep_wait();
     const double b = s->beta;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
         p[i] = fma(b, p[i], r[i]);
+    griddep_done();
+}
+// Launch as a programmatic dependent of the stream's last kernel.
+template <typename... KArgs, typename... Args>
+int launch_dependent(void (*kern)(KArgs...), dim3 grid, int threads, cudaStream_t s, Args &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    NAP_CUDA(cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...));
+    count_launch(1);
+    return NAPSPMV_OK;
 }
 // r = b - q ; p = r
 __global__ void k_resid(double *r, double *p, const double *b, const double *q, int64_t n)
@@ -117,13 +181,17 @@ struct DotScratch {
     unsigned *ticket = nullptr;
 };
 
+dim3 dot_grid(int64_t n)
+{
+    const int64_t per = kThreads * kDotGroups;
+    return dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>((n + per - 1) / per,
+                                                                 kDotBlocks / kDotGroups)));
+}
 int dot_launch(const double *x, const double *y, int64_t n, double *result, DotScratch &ds,
                cudaStream_t s)
 {
-    k_dot<<<kDotBlocks, kThreads, 0, s>>>(x, y, n, ds.partial, ds.ticket, result);
-    count_launch(1);
-    NAP_CUDA(cudaGetLastError());
-    return NAPSPMV_OK;
+    const CgVecs V{x, y, nullptr, nullptr, n, ds.partial, ds.ticket, result, nullptr, nullptr};
+    return launch_dependent(k_cg<kDot>, dot_grid(n), kThreads * kDotGroups, s, V);
 }
 
 struct CgBuffers {
@@ -196,19 +264,20 @@ int cg_core(napspmv_plan_t *P, const double *b, double *x, double rtol, int max_
     while (!done && it < max_it) {
         for (int q = 0; q < poll && it < max_it; q++, it++) {
             if ((rc = apply_one(P, B.p, B.q, precision, false, s))) return rc;
-            if ((rc = dot_launch(B.p, B.q, n, &B.sc->pq, B.ds, s))) return rc;
-            k_alpha<<<1, 1, 0, s>>>(B.sc);
-            k_update_xr<<<g, 256, 0, s>>>(x, B.r, B.p, B.q, n, B.sc);
-            count_launch(2);
-            if ((rc = dot_launch(B.r, B.r, n, &B.sc->rr_new, B.ds, s))) return rc;
-            k_beta<<<1, 1, 0, s>>>(B.sc);
-            k_update_p<<<g, 256, 0, s>>>(B.p, B.r, n, B.sc);
-            count_launch(2);
+            const CgVecs V{B.p, B.q, x,       B.r,         n,
+                           B.ds.partial, B.ds.ticket, nullptr, B.sc, P->ws->err};
+            const dim3 dg = dot_grid(n);
+            if ((rc = launch_dependent(k_cg<kAlpha>, dg, kThreads * kDotGroups, s, V))) return rc;
+            if ((rc = launch_dependent(k_cg<kUpdate>, dg, kThreads * kDotGroups, s, V))) return rc;
+            if ((rc = launch_dependent(k_update_p, dim3((unsigned)g), kThreads, s, B.p,
+                                       (const double *)B.r, n, (const Scal *)B.sc)))
+                return rc;
         }
-        NAP_CUDA(cudaGetLastError());
         NAP_CUDA(cudaMemcpyAsync(&h, B.sc, sizeof(Scal), cudaMemcpyDeviceToHost, s));
         NAP_CUDA(cudaStreamSynchronize(s));
-        if ((rc = napspmv_ws_status(P->ws, s))) return rc;
+        // (a flag set by the last product itself is read here too: it was set
+        // before the update kernel read it)
+        if (h.err && (rc = napspmv_ws_status(P->ws, s))) return rc;
         if (!std::isfinite(h.rr)) break;
         done = std::sqrt(h.rr) <= rtol * bn;
     }
@@ -356,41 +425,48 @@ struct SlotVecs {
     double *x[kMaxSlots], *r[kMaxSlots], *p[kMaxSlots], *q[kMaxSlots], *scal[kMaxSlots];
 };
 
-__device__ __forceinline__ double block_sum_any(double v, double *sh)
-{
-    return block_sum(v, sh);
-}
-
 // mode 0: r = b - q, p = r, partial(r.r) and partial(b.b)
 // mode 1: partial(p.q)
 // mode 2: x += alpha p, r -= alpha q, partial(r.r)
 // mode 3: p = r + beta p
 // mode 4: r = b, p = b, partial(r.r), partial(b.b)   (x = 0)
-__global__ void __launch_bounds__(kThreads) k_slot_vec(const __grid_constant__ SlotVecs S, int mode,
-                                                       double *partial)
+// The slot's last block to finish adds its partials in a fixed order (lane l of a
+// warp adds partials l, l + 32, ... in order, then a fixed shuffle tree), applies
+// the scalar recurrences of CG and resets the slot's ticket.  It brings the
+// partials into shared memory first: a warp that read them from L2 one by one, in
+// a launch of its own, took 15 us per sum of a 1.7M-element slot (GB300; its CG
+// iteration falls from 96 to 73 us, bound by the FP64 pipe and HBM in turn).
+constexpr int kSumRound = 2048;  // partials in shared memory at a time
+template <int MODE>
+__global__ void __launch_bounds__(kThreads)
+    k_slot_vec(const __grid_constant__ SlotVecs S, double *partial, unsigned *ticket)
 {
+    constexpr bool both = MODE == 0 || MODE == 4;
     __shared__ double sh[kThreads / 32];
+    __shared__ double part[MODE == 3 ? 1 : kSumRound];
+    __shared__ bool last;
+    griddep_wait();
     const int i = blockIdx.y;
     const int64_t n = S.n[i];
     const int nb = slot_blocks(n);
     if ((int)blockIdx.x >= nb) return;  // the whole block: this slot needs fewer
     const double *b = S.b[i];
     double *x = S.x[i], *r = S.r[i], *p = S.p[i], *q = S.q[i];
-    const double alpha = mode == 2 ? S.scal[i][S_ALPHA] : 0.0;
-    const double beta = mode == 3 ? S.scal[i][S_BETA] : 0.0;
+    const double alpha = MODE == 2 ? S.scal[i][S_ALPHA] : 0.0;
+    const double beta = MODE == 3 ? S.scal[i][S_BETA] : 0.0;
     double s1 = 0.0, s2 = 0.0;
     for (int64_t k = (int64_t)blockIdx.x * kThreads + threadIdx.x; k < n;
          k += (int64_t)nb * kThreads) {
-        if (mode == 0 || mode == 4) {
-            const double v = mode == 0 ? b[k] - q[k] : b[k];
+        if (both) {
+            const double v = MODE == 0 ? b[k] - q[k] : b[k];
             r[k] = v;
             p[k] = v;
-            if (mode == 4) x[k] = 0.0;
+            if (MODE == 4) x[k] = 0.0;
             s1 = fma(v, v, s1);
             s2 = fma(b[k], b[k], s2);
-        } else if (mode == 1) {
+        } else if (MODE == 1) {
             s1 = fma(p[k], q[k], s1);
-        } else if (mode == 2) {
+        } else if (MODE == 2) {
             x[k] = fma(alpha, p[k], x[k]);
             const double v = fma(-alpha, q[k], r[k]);
             r[k] = v;
@@ -399,57 +475,80 @@ __global__ void __launch_bounds__(kThreads) k_slot_vec(const __grid_constant__ S
             p[k] = fma(beta, p[k], r[k]);
         }
     }
-    if (mode == 3) return;
-    s1 = block_sum_any(s1, sh);
-    if (mode == 0 || mode == 4) s2 = block_sum_any(s2, sh);
+    if (MODE == 3) {
+        griddep_done();
+        return;
+    }
+    double *mine = partial + (int64_t)i * 2 * kSlotBlocksMax;  // r.r or p.q, then b.b
+    s1 = block_sum(s1, sh);
+    if (both) s2 = block_sum(s2, sh);
     if (threadIdx.x == 0) {
-        partial[((int64_t)i * kSlotBlocksMax + blockIdx.x) * 2 + 0] = s1;
-        partial[((int64_t)i * kSlotBlocksMax + blockIdx.x) * 2 + 1] = s2;
+        mine[blockIdx.x] = s1;
+        if (both) mine[kSlotBlocksMax + blockIdx.x] = s2;
+        __threadfence();
+        last = atomicAdd(ticket + i, 1u) == (unsigned)nb - 1;
     }
-}
-
-// Fixed-order sums of the partials (lane l adds partials l, l + 32, ... in
-// order, then a fixed shuffle tree) and the scalar recurrences of CG.
-__global__ void k_slot_final(const __grid_constant__ SlotVecs S, int mode, const double *partial)
-{
-    const int i = blockIdx.x, lane = threadIdx.x;
-    double a = 0.0, c = 0.0;
-    const int nb = slot_blocks(S.n[i]);
-    for (int q = lane; q < nb; q += 32) {
-        a += partial[((int64_t)i * kSlotBlocksMax + q) * 2 + 0];
-        c += partial[((int64_t)i * kSlotBlocksMax + q) * 2 + 1];
+    __syncthreads();
+    griddep_done();
+    if (!last) return;
+    __threadfence();
+    double sum[2] = {0.0, 0.0};
+    for (int w = 0; w < (both ? 2 : 1); w++) {
+        double a = 0.0;
+        for (int q0 = 0; q0 < nb; q0 += kSumRound) {
+            const int m = min(kSumRound, nb - q0);
+            __syncthreads();
+            for (int k = threadIdx.x; k < m; k += kThreads)
+                part[k] = __ldcg(mine + w * kSlotBlocksMax + q0 + k);
+            __syncthreads();
+            if (threadIdx.x < 32)
+                for (int k = threadIdx.x; k < m; k += 32) a += part[k];
+        }
+        if (threadIdx.x < 32)
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        sum[w] = a;
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        c += __shfl_xor_sync(0xffffffffu, c, o);
-    }
-    if (lane != 0) return;
+    if (threadIdx.x != 0) return;
+    ticket[i] = 0;
     double *s = S.scal[i];
-    if (mode == 0 || mode == 4) {
-        s[S_RR] = a;
-        s[S_BB] = c;
-    } else if (mode == 1) {
-        s[S_PQ] = a;
-        s[S_ALPHA] = s[S_RR] / a;
-    } else if (mode == 2) {
-        s[S_RRNEW] = a;
-        s[S_BETA] = a / s[S_RR];
-        s[S_RR] = a;
+    if (both) {
+        s[S_RR] = sum[0];
+        s[S_BB] = sum[1];
+    } else if (MODE == 1) {
+        s[S_PQ] = sum[0];
+        s[S_ALPHA] = s[S_RR] / sum[0];
+    } else {
+        s[S_RRNEW] = sum[0];
+        s[S_BETA] = sum[0] / s[S_RR];
+        s[S_RR] = sum[0];
     }
 }
 
-int slot_vec(const SlotVecs &S, int mode, double *partial, cudaStream_t st)
+struct Partials {
+    double *p = nullptr;
+    unsigned *ticket = nullptr;
+    cudaStream_t s = 0;
+    ~Partials()
+    {
+        if (p) cudaFreeAsync(p, s);
+    }
+    int alloc(int count, cudaStream_t st)
+    {
+        s = st;
+        const size_t sums = sizeof(double) * 2 * kSlotBlocksMax * count;
+        NAP_CUDA(cudaMallocAsync(&p, sums + sizeof(unsigned) * count, st));
+        ticket = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(p) + sums);
+        NAP_CUDA(cudaMemsetAsync(ticket, 0, sizeof(unsigned) * count, st));
+        return NAPSPMV_OK;
+    }
+};
+
+template <int MODE>
+int slot_vec(const SlotVecs &S, const Partials &P)
 {
     int gx = 1;
     for (int i = 0; i < S.count; i++) gx = std::max(gx, slot_blocks(S.n[i]));
-    k_slot_vec<<<dim3(gx, S.count), kThreads, 0, st>>>(S, mode, partial);
-    count_launch(1);
-    if (mode != 3) {
-        k_slot_final<<<S.count, 32, 0, st>>>(S, mode, partial);
-        count_launch(1);
-    }
-    NAP_CUDA(cudaGetLastError());
-    return NAPSPMV_OK;
+    return launch_dependent(k_slot_vec<MODE>, dim3(gx, S.count), kThreads, P.s, S, P.p, P.ticket);
 }
 
 int slot_setup(int32_t count, const napspmv_cg_slot *slots, SlotVecs &S)
@@ -526,15 +625,6 @@ int slot_apply(int32_t count, const napspmv_cg_slot *slots, bool from_x, int32_t
     return apply_batch(nb, plans, wss, vs, ws_, reps, sc, &o, st, keep, true);
 }
 
-struct Partials {
-    double *p = nullptr;
-    cudaStream_t s = 0;
-    ~Partials()
-    {
-        if (p) cudaFreeAsync(p, s);
-    }
-};
-
 }  // namespace
 }  // namespace nap
 
@@ -548,11 +638,10 @@ int napspmv_cg_batch_init(int32_t count, const napspmv_cg_slot *slots, int32_t p
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     Partials P;
-    P.s = st;
-    NAP_CUDA(cudaMallocAsync(&P.p, sizeof(double) * 2 * kSlotBlocksMax * count, st));
-    if (x_is_zero) return slot_vec(S, 4, P.p, st);
+    if ((rc = P.alloc(count, st))) return rc;
+    if (x_is_zero) return slot_vec<4>(S, P);
     if ((rc = slot_apply(count, slots, true, precision, true, st))) return rc;
-    return slot_vec(S, 0, P.p, st);
+    return slot_vec<0>(S, P);
 }
 
 int napspmv_cg_batch_iterate(int32_t count, const napspmv_cg_slot *slots, int32_t precision,
@@ -567,13 +656,12 @@ int napspmv_cg_batch_iterate(int32_t count, const napspmv_cg_slot *slots, int32_
     }
     cudaStream_t st = (cudaStream_t)stream;
     Partials P;
-    P.s = st;
-    NAP_CUDA(cudaMallocAsync(&P.p, sizeof(double) * 2 * kSlotBlocksMax * count, st));
+    if ((rc = P.alloc(count, st))) return rc;
     for (int it = 0; it < iters; it++) {
         if ((rc = slot_apply(count, slots, false, precision, it + 1 == iters, st))) return rc;
-        if ((rc = slot_vec(S, 1, P.p, st))) return rc;
-        if ((rc = slot_vec(S, 2, P.p, st))) return rc;
-        if ((rc = slot_vec(S, 3, P.p, st))) return rc;
+        if ((rc = slot_vec<1>(S, P))) return rc;
+        if ((rc = slot_vec<2>(S, P))) return rc;
+        if ((rc = slot_vec<3>(S, P))) return rc;
     }
     return NAPSPMV_OK;
 }

@@ -1,0 +1,51 @@
+"""The dot products' partition at its edges: napspmv_dot and the batched CG scalars on
+inputs whose products and sums are exact in FP64 (small integers times powers of two), so
+that a lost, doubled or stale partial shows whatever the order.  Lengths around a group
+(256), a CTA of four groups, the whole partition (1,024 groups), a batched block (1,024
+values) and a shared-memory round of partials (2,048 blocks)."""
+from fractions import Fraction
+
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import gpu_plan
+from paper_1612_08060_gb300 import inputs as I
+from paper_1612_08060_gb300 import napspmv as nap
+
+pytestmark = pytest.mark.gpu
+
+
+def vectors(n, seed):
+    rng = np.random.default_rng(seed)
+    return (rng.integers(-3, 4, n) * 0.5 ** rng.integers(0, 3, n) for _ in range(2))
+
+
+@pytest.mark.parametrize("n", [1, 255, 256, 257, 1024, 1025, 4096, 262143, 262144, 262145, 600001])
+def test_dot(n):
+    x, y = vectors(n, n)
+    out = torch.empty(1, dtype=torch.float64, device="cuda")
+    xd, yd = torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda()
+    for _ in range(2):  # the ticket is back at 0
+        nap.napspmv_dot(xd, yd, n, out)
+    assert Fraction(out.item()) == sum(map(Fraction, (x * y).tolist()))
+
+
+@pytest.mark.parametrize("n", [64, 1023, 1025, 40000, 2048 * 1024 + 5])
+def test_batched_scalars(n):
+    """Two slots of one call, A = I."""
+    A = I.CSR(np.arange(n + 1, dtype=np.int64), np.arange(n, dtype=np.int32), np.ones(n))
+    plan = gpu_plan(A, 1, 1)
+    slots, want = [], []
+    for k in range(2):
+        b, _ = vectors(n, n + k)
+        z = lambda: torch.zeros(n, dtype=torch.float64, device="cuda")  # noqa: E731
+        slots.append(dict(plan=plan, ws=nap.Workspace(plan), b=torch.from_numpy(b).cuda(), x=z(), r=z(), p=z(), q=z(),
+                          scal=torch.zeros(8, dtype=torch.float64, device="cuda")))
+        want.append(float(np.sum(b * b)))
+    nap.napspmv_cg_batch_init(slots, nap.PREC_F64, x_is_zero=True)
+    nap.napspmv_cg_batch_iterate(slots, nap.PREC_F64, 1)  # A = I: alpha = 1, x = b, r = 0
+    for s, bb in zip(slots, want):
+        scal = s["scal"].cpu().numpy()
+        assert scal[5] == bb and scal[1] == bb and scal[2] == 1.0 and scal[0] == 0.0
+        assert torch.equal(s["x"], s["b"]) and not s["r"].any()
