@@ -2843,6 +2843,42 @@ static int enqueue_windows(int count, napspmv_plan_t *const *plans, napspmv_ws_t
     return NAPSPMV_OK;
 }
 
+bool runs_on_windows(const napspmv_plan_t *P, int32_t precision)
+{
+    napspmv_opts o{};
+    o.precision = precision;
+    return resolve_opts(P, &o).window;
+}
+SendList send_list(const napspmv_plan_t *P)
+{
+    return SendList{P->lists[L_INTER].d_idx, P->d_xfer_dst, P->d_xfer_shift, P->ws->grecv, P->ws->err,
+                    (int32_t)P->n_gs};
+}
+int send_alone(napspmv_plan_t *P, int32_t precision, const double *x, cudaStream_t s)
+{
+    if (P->n_gs == 0) return NAPSPMV_OK;
+    const bool f32 = precision == NAPSPMV_PREC_F32;
+    SendJobs<1> S{};
+    S.n = 1;
+    S.job[0] = send_job(P, f32, x, P->ws->grecv, P->ws->err);
+    launch_pdl(true, f32 ? k_send<float, double, 1> : k_send<double, double, 1>, S.job[0].blocks, 0, s, S);
+    count_launch(1);
+    NAP_CUDA(cudaGetLastError());
+    return NAPSPMV_OK;
+}
+int window_alone(napspmv_plan_t *P, int32_t precision, const double *x, double *y, cudaStream_t s)
+{
+    napspmv_opts o{};
+    o.precision = precision;
+    const bool f32 = precision == NAPSPMV_PREC_F32;
+    WinJobs<1> W;
+    W.job[0] = window_job(P, P->ws, x, nullptr, y, nullptr, 1.0);
+    const napspmv_plan_t *pl[1] = {P};
+    P->ws->recv_f32 = f32;
+    count_launch(1);
+    return window_launch<1>(1, pl, W, f32 ? 2 : 0, false, resolve_opts(P, &o), s);
+}
+
 static int enqueue_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, double *w, int reps,
                           double scale, const Opts &o, bool keep, cudaStream_t s,
                           int64_t *kernels)

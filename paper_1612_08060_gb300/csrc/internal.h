@@ -281,4 +281,17 @@ int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const
                 const double *const *v, double *const *w, const int32_t *reps,
                 const double *scale, const napspmv_opts *opts, cudaStream_t s, bool keep = true,
                 bool as_batch = false);
+// Pieces of an apply for a caller that makes its vector itself (CG): whether
+// applies at this precision run on staged windows by default; the inter-node
+// messages of x alone; the windowed SpMV alone; and where the messages go.
+bool runs_on_windows(const napspmv_plan_t *P, int32_t precision);
+int send_alone(napspmv_plan_t *P, int32_t precision, const double *x, cudaStream_t s);
+int window_alone(napspmv_plan_t *P, int32_t precision, const double *x, double *y, cudaStream_t s);
+struct SendList {
+    const int32_t *j, *dst, *shift;  // see k_send
+    void *grecv;
+    const int *err;
+    int32_t n;
+};
+SendList send_list(const napspmv_plan_t *P);
 }  // namespace nap

@@ -19,126 +19,180 @@ namespace {
 constexpr int kDotBlocks = 1024;  // fixed grid: the partition of every dot product
 constexpr int kThreads = 256;
 
-__device__ __forceinline__ double block_sum(double v, double *sh)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) sh[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        v = l < (kThreads / 32) ? sh[l] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    }
-    __syncthreads();
-    return v;  // valid in thread 0
-}
-
 struct Scal {
-    double rr, rr_new, pq, alpha, beta, bb, rnorm0;
+    double rr[2];  // r.r before the next iteration, by the parity of its number
+    double bb, rnorm0;
     int err, pad;  // the workspace's error flag, as the last CG iteration saw it
 };
 
-// Sum of 256 values (a group of 8 warps, numbered g in its block) in a fixed tree;
-// valid in the group's thread 0.
+// Sum of 256 values, one per thread of a group of 8 warps (group g of its CTA), in
+// a fixed tree: lanes 16, 8, 4, 2, 1 apart within each warp, then the 8 warps' sums
+// 4, 2, 1 apart; valid in the group's first warp.  GB300 issues an FP64 addition per
+// warp every 84 cycles or so on a quarter of an SM, whatever its lanes hold, so the
+// 248 additions of the tree are packed into full warps through shared memory: 13
+// instructions, where a shuffle tree in every warp takes 45.  A CG iteration on 63^3
+// fell from 36.7 to 31.8 us, a served one of 1.7M elements from 73 to 70.
+constexpr int kSumDoubles = 256 + 128 + 64;  // shared memory of a group
 __device__ __forceinline__ double group_sum(double v, double *sh, int g)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) sh[w] = v;
+    double *a = sh + kSumDoubles * g, *b = a + 256, *c = b + 128;
+    const int t = threadIdx.x % kThreads;
+    a[t] = v;
     __syncthreads();
-    if ((w & 7) == 0) {
-        v = l < 8 ? sh[8 * g + l] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (t < 128) b[t] = a[32 * (t >> 4) + (t & 15)] + a[32 * (t >> 4) + (t & 15) + 16];
+    __syncthreads();
+    if (t < 64) c[t] = b[16 * (t >> 3) + (t & 7)] + b[16 * (t >> 3) + (t & 7) + 8];
+    __syncthreads();
+    if (t < 32) {
+        v = c[8 * (t >> 2) + (t & 3)] + c[8 * (t >> 2) + (t & 3) + 4];
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        v += 0.0;  // a sum of -0.0 counts as 0.0
+        v += __shfl_xor_sync(0xffffffffu, v, 16);  // warps 4, 2, 1 apart
+        v += __shfl_xor_sync(0xffffffffu, v, 8);
+        v += __shfl_xor_sync(0xffffffffu, v, 4);
     }
     __syncthreads();
     return v;
 }
 
 // FP64 dot products over a fixed partition: partial b, of 1,024, sums the indices
-// i = b*256 + t + q*1024*256 over the 256 threads t of a group, and the last CTA
-// to finish adds the partials in index order and resets the ticket.  A CTA is
-// four groups, so that a quarter of the tickets are drawn; partials past the
-// vector's end are 0 and not launched.
-// WHAT: kDot    *result = x.y
-//       kAlpha  pq = x.y (x = p, y = q), alpha = rr / pq
-//       kUpdate x += alpha p, r -= alpha q, rr_new = r.r, beta = rr_new / rr, rr = rr_new
-// The scalar recurrences ride on the last CTA: on their own they were two more
-// launches per CG iteration, and the update and its dot product two passes.  With
-// the windows an iteration is five launches in place of ten: 39 us of a CG-IR
-// solve on 63^3 with FP32 values, where it was 55 (GB300); latency-bound.
-enum CgOp { kDot, kAlpha, kUpdate };
+// i = b*256 + t + q*1024*256 over the 256 threads t of a group, and the partials
+// are added in a fixed order.  A CTA is four groups; partials past the vector's
+// end are 0 and not launched.
 constexpr int kDotGroups = 4;
-struct CgVecs {
-    const double *x, *y;  // kUpdate: p, q
-    double *sol, *res;    // kUpdate: x, r
-    int64_t n;
-    double *partial;
-    unsigned *ticket;
-    double *result;
-    Scal *sc;
-    const int *err;
-};
-template <int WHAT>
-__global__ void __launch_bounds__(kThreads *kDotGroups) k_cg(const CgVecs V)
+// All threads of a CTA: f of the sum of the first nb partials (the others are 0),
+// f taken by one thread: an FP64 division by every warp costs more than the sum.
+template <class F>
+__device__ __forceinline__ double sum_partials(const double *partial, int nb, double *sh, F f)
 {
-    __shared__ double sh[8 * kDotGroups];
+    __shared__ double total;
+    const int g = threadIdx.x / kThreads, t = threadIdx.x % kThreads;
+    double v = 0.0;
+    if (g == 0)
+        for (int q = t; q < kDotBlocks; q += kThreads) v += q < nb ? __ldcg(partial + q) : 0.0;
+    v = group_sum(v, sh, g);
+    if (threadIdx.x == 0) total = f(v);
+    __syncthreads();
+    return total;
+}
+
+// *result = x.y: the last CTA to finish adds the partials and resets the ticket.
+__global__ void __launch_bounds__(kThreads *kDotGroups)
+    k_dot(const double *x, const double *y, int64_t n, double *partial, unsigned *ticket,
+          double *result)
+{
+    __shared__ double sh[kSumDoubles * kDotGroups];
     __shared__ bool last;
     griddep_wait();
     const int g = threadIdx.x / kThreads, t = threadIdx.x % kThreads;
     const int b = blockIdx.x * kDotGroups + g;
-    const double a = WHAT == kUpdate ? V.sc->alpha : 0.0;
     double s = 0.0;
-    for (int64_t i = (int64_t)b * kThreads + t; i < V.n; i += (int64_t)kDotBlocks * kThreads) {
-        if (WHAT == kUpdate) {
-            V.sol[i] = fma(a, V.x[i], V.sol[i]);
-            const double r = fma(-a, V.y[i], V.res[i]);
-            V.res[i] = r;
-            s = fma(r, r, s);
-        } else {
-            s = fma(V.x[i], V.y[i], s);
-        }
-    }
+    for (int64_t i = (int64_t)b * kThreads + t; i < n; i += (int64_t)kDotBlocks * kThreads)
+        s = fma(x[i], y[i], s);
     s = group_sum(s, sh, g);
-    if (t == 0) V.partial[b] = s;
+    if (t == 0) partial[b] = s;
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(V.ticket, 1u) == gridDim.x - 1;
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     __syncthreads();
     griddep_done();
     if (!last) return;
     __threadfence();
-    const int nb = gridDim.x * kDotGroups;
-    double v = 0.0;
-    if (g == 0)
-        for (int q = t; q < kDotBlocks; q += kThreads) v += q < nb ? __ldcg(V.partial + q) : 0.0;
-    v = group_sum(v, sh, g);
+    const double v = sum_partials(partial, gridDim.x * kDotGroups, sh, [](double a) { return a; });
     if (threadIdx.x == 0) {
-        *V.ticket = 0;
-        if (WHAT == kDot) *V.result = v;
-        if (WHAT == kAlpha) {
-            V.sc->pq = v;
-            V.sc->alpha = V.sc->rr / v;
-        }
-        if (WHAT == kUpdate) {
-            V.sc->rr_new = v;
-            V.sc->beta = v / V.sc->rr;
-            V.sc->rr = v;
-            V.sc->err = *(volatile const int *)V.err;
-        }
+        *ticket = 0;
+        *result = v;
     }
 }
-// p = r + beta p
-__global__ void __launch_bounds__(kThreads) k_update_p(double *p, const double *r, int64_t n, const Scal *s)
+
+// A CG iteration after q = A p is three kernels, each CTA of the second and third
+// adding the partials of the one before for itself (8 KB from L2), so that no sum
+// and no scalar has a launch, a ticket or a last CTA of its own:
+//   k_pq        partials of p.q
+//   k_update    alpha = rr / p.q; x += alpha p, r -= alpha q, partials of r.r
+//   k_next_p    beta = r.r / rr; p' = r + beta p into the other vector, and the
+//               inter-node messages of p' (each sender's element is formed again
+//               from p and r, the same operation), so that q = A p' is the windowed
+//               SpMV alone
+// Latency-bound at the sizes of a served solve.  Per iteration on 63^3 with FP32
+// values (GB300): 31.8 us in four launches; 39 in five, the last CTA of a dot
+// product summing and the messages in their own launch (with shuffle trees, 36.7
+// against 39); 55 in ten.
+struct CgIter {
+    double *x, *r, *p, *p2, *q;
+    int64_t n;
+    double *pq, *rr;  // partials
+    int nb;           // of them
+    Scal *sc;
+    int parity;
+};
+__global__ void __launch_bounds__(kThreads *kDotGroups) k_pq(const CgIter I)
 {
+    __shared__ double sh[kSumDoubles * kDotGroups];
     griddep_wait();
-    const double b = s->beta;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = fma(b, p[i], r[i]);
+    const int g = threadIdx.x / kThreads, b = blockIdx.x * kDotGroups + g;
+    double s = 0.0;
+    for (int64_t i = (int64_t)b * kThreads + threadIdx.x % kThreads; i < I.n;
+         i += (int64_t)kDotBlocks * kThreads)
+        s = fma(I.p[i], I.q[i], s);
+    s = group_sum(s, sh, g);
+    if (threadIdx.x % kThreads == 0) I.pq[b] = s;
+    griddep_done();
+}
+__global__ void __launch_bounds__(kThreads *kDotGroups) k_update(const CgIter I)
+{
+    __shared__ double sh[kSumDoubles * kDotGroups];
+    griddep_wait();
+    const double a = sum_partials(I.pq, I.nb, sh, [&](double pq) { return I.sc->rr[I.parity] / pq; });
+    const int g = threadIdx.x / kThreads, b = blockIdx.x * kDotGroups + g;
+    double s = 0.0;
+    for (int64_t i = (int64_t)b * kThreads + threadIdx.x % kThreads; i < I.n;
+         i += (int64_t)kDotBlocks * kThreads) {
+        I.x[i] = fma(a, I.p[i], I.x[i]);
+        const double r = fma(-a, I.q[i], I.r[i]);
+        I.r[i] = r;
+        s = fma(r, r, s);
+    }
+    s = group_sum(s, sh, g);
+    if (threadIdx.x % kThreads == 0) I.rr[b] = s;
+    griddep_done();
+}
+// The first vec_blocks CTAs form p', the others send it (none where the product
+// brings its own messages).
+template <class T>
+__global__ void __launch_bounds__(kThreads *kDotGroups)
+    k_next_p(const CgIter I, const SendList L, int vec_blocks)
+{
+    __shared__ double sh[kSumDoubles * kDotGroups];
+    griddep_wait();
+    const double beta = sum_partials(I.rr, I.nb, sh, [&](double rr) {
+        if (blockIdx.x == 0) {
+            I.sc->rr[I.parity ^ 1] = rr;
+            I.sc->err = *(volatile const int *)L.err;
+        }
+        return rr / I.sc->rr[I.parity];
+    });
+    if ((int)blockIdx.x < vec_blocks) {
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < I.n;
+             i += (int64_t)vec_blocks * blockDim.x)
+            I.p2[i] = fma(beta, I.p[i], I.r[i]);
+    } else if (!*(volatile const int *)L.err) {
+        const int lane = threadIdx.x & 31, warps = blockDim.x / 32;
+        const int block = (int)blockIdx.x - vec_blocks, step = ((int)gridDim.x - vec_blocks) * warps;
+        for (int g = block * warps + (threadIdx.x >> 5); g * kSendGroup < L.n; g += step) {
+            const int32_t shift = __ldg(L.shift + g);
+#pragma unroll
+            for (int u = 0; u < kSendGroup / 32; u++) {
+                const int k = g * kSendGroup + 32 * u + lane;
+                if (k >= L.n) continue;
+                const int32_t j = __ldg(L.j + k), to = shift == kMixed ? __ldg(L.dst + k) : k + shift;
+                const double v = fma(beta, I.p[j], I.r[j]);
+                if constexpr (sizeof(T) == 4) static_cast<T *>(L.grecv)[to] = __double2float_rn(v);
+                else static_cast<T *>(L.grecv)[to] = v;
+            }
+        }
+    }
     griddep_done();
 }
 // Launch as a programmatic dependent of the stream's last kernel.
@@ -190,18 +244,18 @@ dim3 dot_grid(int64_t n)
 int dot_launch(const double *x, const double *y, int64_t n, double *result, DotScratch &ds,
                cudaStream_t s)
 {
-    const CgVecs V{x, y, nullptr, nullptr, n, ds.partial, ds.ticket, result, nullptr, nullptr};
-    return launch_dependent(k_cg<kDot>, dot_grid(n), kThreads * kDotGroups, s, V);
+    return launch_dependent(k_dot, dot_grid(n), kThreads * kDotGroups, s, x, y, n, ds.partial, ds.ticket,
+                            result);
 }
 
 struct CgBuffers {
-    double *r = nullptr, *p = nullptr, *q = nullptr, *d = nullptr;
+    double *r = nullptr, *p = nullptr, *p2 = nullptr, *q = nullptr, *d = nullptr;
     Scal *sc = nullptr;
     DotScratch ds;
     cudaStream_t s = 0;
     ~CgBuffers()
     {
-        void *ptrs[] = {r, p, q, d, sc, ds.partial, ds.ticket};
+        void *ptrs[] = {r, p, p2, q, d, sc, ds.partial, ds.ticket};
         for (void *x : ptrs)
             if (x) cudaFreeAsync(x, s);
     }
@@ -212,10 +266,11 @@ int cg_alloc(CgBuffers &B, int64_t n, cudaStream_t s)
     B.s = s;
     NAP_CUDA(cudaMallocAsync(&B.r, sizeof(double) * n, s));
     NAP_CUDA(cudaMallocAsync(&B.p, sizeof(double) * n, s));
+    NAP_CUDA(cudaMallocAsync(&B.p2, sizeof(double) * n, s));
     NAP_CUDA(cudaMallocAsync(&B.q, sizeof(double) * n, s));
     NAP_CUDA(cudaMallocAsync(&B.d, sizeof(double) * n, s));
     NAP_CUDA(cudaMallocAsync(&B.sc, sizeof(Scal), s));
-    NAP_CUDA(cudaMallocAsync(&B.ds.partial, sizeof(double) * kDotBlocks, s));
+    NAP_CUDA(cudaMallocAsync(&B.ds.partial, sizeof(double) * 2 * kDotBlocks, s));
     NAP_CUDA(cudaMallocAsync(&B.ds.ticket, sizeof(unsigned), s));
     NAP_CUDA(cudaMemsetAsync(B.ds.ticket, 0, sizeof(unsigned), s));
     NAP_CUDA(cudaMemsetAsync(B.sc, 0, sizeof(Scal), s));
@@ -253,33 +308,46 @@ int cg_core(napspmv_plan_t *P, const double *b, double *x, double rtol, int max_
     k_resid<<<g, 256, 0, s>>>(B.r, B.p, b, B.q, n);
     count_launch(1);
     if ((rc = dot_launch(b, b, n, &B.sc->bb, B.ds, s))) return rc;
-    if ((rc = dot_launch(B.r, B.r, n, &B.sc->rr, B.ds, s))) return rc;
+    if ((rc = dot_launch(B.r, B.r, n, &B.sc->rr[0], B.ds, s))) return rc;
     Scal h{};
     NAP_CUDA(cudaMemcpyAsync(&h, B.sc, sizeof(Scal), cudaMemcpyDeviceToHost, s));
     NAP_CUDA(cudaStreamSynchronize(s));
     const double bn = h.bb > 0 ? std::sqrt(h.bb) : 1.0;
     int it = 0;
     const int poll = 8;
-    bool done = std::sqrt(h.rr) <= rtol * bn;
+    // on staged windows the iteration sends p itself, the first time from here
+    const bool windows = runs_on_windows(P, precision), f32 = precision == NAPSPMV_PREC_F32;
+    const SendList sends = send_list(P);
+    const int64_t groups = (sends.n + kSendGroup - 1) / kSendGroup;
+    const int send_blocks =
+        windows ? (int)std::min<int64_t>((groups + kThreads * kDotGroups / 32 - 1) / (kThreads * kDotGroups / 32),
+                                     (int64_t)P->num_sms)
+                : 0;
+    const dim3 dg = dot_grid(n);
+    if (windows && (rc = send_alone(P, precision, B.p, s))) return rc;
+    bool done = std::sqrt(h.rr[0]) <= rtol * bn;
     while (!done && it < max_it) {
         for (int q = 0; q < poll && it < max_it; q++, it++) {
-            if ((rc = apply_one(P, B.p, B.q, precision, false, s))) return rc;
-            const CgVecs V{B.p, B.q, x,       B.r,         n,
-                           B.ds.partial, B.ds.ticket, nullptr, B.sc, P->ws->err};
-            const dim3 dg = dot_grid(n);
-            if ((rc = launch_dependent(k_cg<kAlpha>, dg, kThreads * kDotGroups, s, V))) return rc;
-            if ((rc = launch_dependent(k_cg<kUpdate>, dg, kThreads * kDotGroups, s, V))) return rc;
-            if ((rc = launch_dependent(k_update_p, dim3((unsigned)g), kThreads, s, B.p,
-                                       (const double *)B.r, n, (const Scal *)B.sc)))
+            if (windows) rc = window_alone(P, precision, B.p, B.q, s);
+            else rc = apply_one(P, B.p, B.q, precision, false, s);
+            if (rc) return rc;
+            const CgIter I{x, B.r, B.p, B.p2, B.q, n, B.ds.partial, B.ds.partial + kDotBlocks,
+                           (int)dg.x * kDotGroups, B.sc, it & 1};
+            if ((rc = launch_dependent(k_pq, dg, kThreads * kDotGroups, s, I))) return rc;
+            if ((rc = launch_dependent(k_update, dg, kThreads * kDotGroups, s, I))) return rc;
+            if ((rc = launch_dependent(f32 ? k_next_p<float> : k_next_p<double>,
+                                       dim3(dg.x + (unsigned)send_blocks), kThreads * kDotGroups, s, I, sends,
+                                       (int)dg.x)))
                 return rc;
+            std::swap(B.p, B.p2);
         }
         NAP_CUDA(cudaMemcpyAsync(&h, B.sc, sizeof(Scal), cudaMemcpyDeviceToHost, s));
         NAP_CUDA(cudaStreamSynchronize(s));
         // (a flag set by the last product itself is read here too: it was set
         // before the update kernel read it)
         if (h.err && (rc = napspmv_ws_status(P->ws, s))) return rc;
-        if (!std::isfinite(h.rr)) break;
-        done = std::sqrt(h.rr) <= rtol * bn;
+        if (!std::isfinite(h.rr[it & 1])) break;
+        done = std::sqrt(h.rr[it & 1]) <= rtol * bn;
     }
     *iters = it;
     return NAPSPMV_OK;
@@ -442,7 +510,7 @@ __global__ void __launch_bounds__(kThreads)
     k_slot_vec(const __grid_constant__ SlotVecs S, double *partial, unsigned *ticket)
 {
     constexpr bool both = MODE == 0 || MODE == 4;
-    __shared__ double sh[kThreads / 32];
+    __shared__ double sh[kSumDoubles];
     __shared__ double part[MODE == 3 ? 1 : kSumRound];
     __shared__ bool last;
     griddep_wait();
@@ -480,8 +548,8 @@ __global__ void __launch_bounds__(kThreads)
         return;
     }
     double *mine = partial + (int64_t)i * 2 * kSlotBlocksMax;  // r.r or p.q, then b.b
-    s1 = block_sum(s1, sh);
-    if (both) s2 = block_sum(s2, sh);
+    s1 = group_sum(s1, sh, 0);
+    if (both) s2 = group_sum(s2, sh, 0);
     if (threadIdx.x == 0) {
         mine[blockIdx.x] = s1;
         if (both) mine[kSlotBlocksMax + blockIdx.x] = s2;
