@@ -1941,146 +1941,10 @@ int build_items(napspmv_plan_t *P, int32_t tile_rows, int32_t tile_nnz)
         return NAPSPMV_ERR_ARG;
     }
     ItemSet &S = P->items;
-    if (S.d_items && S.tile_rows == tile_rows && S.tile_nnz == tile_nnz) return NAPSPMV_OK;
-    const int nn = P->nn;
-    // CTA tiles of the whole matrix, cut within each node's rows
-    std::vector<Item> items;
-    const std::vector<int32_t> &rp = P->h_rowptr;
-    for (int x = 0; x < nn; x++) {
-        int64_t r = P->node_rows[x];
-        const int64_t end = P->node_rows[x + 1];
-        while (r < end) {
-            int64_t e = r;
-            while (e < end && e - r < tile_rows && rp[e + 1] - rp[r] <= tile_nnz) e++;
-            if (e == r) e = r + 1;  // one row longer than the capacity
-            Item it{};
-            it.kind = kSpmv;
-            it.node = x;
-            it.b = (int32_t)r;
-            it.e = (int32_t)e;
-            it.k0 = rp[r];
-            it.k1 = rp[e];
-            items.push_back(it);
-            r = e;
-        }
-    }
-
-    // tiles of the local / remote parts (overlapped engine), same size limits
-    auto cut = [&](const std::vector<int32_t> &rp2, std::vector<Item> &out) {
-        const int64_t n = (int64_t)rp2.size() - 1;
-        int64_t r = 0;
-        while (r < n) {
-            int64_t e = r;
-            while (e < n && e - r < tile_rows && rp2[e + 1] - rp2[r] <= tile_nnz) e++;
-            if (e == r) e = r + 1;
-            Item it{};
-            it.kind = kSpmv;
-            it.b = (int32_t)r;
-            it.e = (int32_t)e;
-            it.k0 = rp2[r];
-            it.k1 = rp2[e];
-            out.push_back(it);
-            r = e;
-        }
-    };
-    std::vector<Item> tl, tr, trh;
-    if (!P->h_rowptrL.empty()) {
-        cut(P->h_rowptrL, tl);
-        cut(P->h_rowptrR, tr);
-        if (!(P->flags & NAPSPMV_PARTITION_STRIDED)) {
-            // remote tiles never straddle two processes: Item::msg is the
-            // process, whose receive buffers the remote pass may stage
-            const int64_t n = P->n, q = n / P->np, rem = n % P->np;
-            std::vector<int32_t> sub;
-            for (int32_t r = 0; r < P->np; r++) {
-                const int64_t r0 = r * q + std::min<int64_t>(r, rem);
-                const int64_t r1 = r0 + q + (r < rem ? 1 : 0);
-                sub.assign(P->h_rowptrR.begin() + r0, P->h_rowptrR.begin() + r1 + 1);
-                const size_t first = trh.size();
-                cut(sub, trh);
-                for (size_t k = first; k < trh.size(); k++) {
-                    trh[k].b += (int32_t)r0;
-                    trh[k].e += (int32_t)r0;
-                    trh[k].msg = r;
-                }
-            }
-        }
-    }
-    // warp tiles: the same cutting with a warp's share of a CTA tile
-    std::vector<Item> wt, wtl, wtr;
-    {
-        const int32_t trows = tile_rows, tnnz = tile_nnz;
-        tile_rows = std::max(1, trows / 8);
-        tile_nnz = std::max(32, tnnz / 8);
-        cut(P->h_rowptr, wt);
-        if (!P->h_rowptrL.empty()) {
-            cut(P->h_rowptrL, wtl);
-            cut(P->h_rowptrR, wtr);
-        }
-        tile_rows = trows;
-        tile_nnz = tnnz;
-    }
-    // the stage each list needs: its largest tile that is staged at all
-    auto fit = [](const std::vector<Item> &v, int32_t tnnz, int32_t &cap, int32_t &rows) {
-        cap = 32;
-        rows = 1;
-        for (const Item &it : v)
-            if (it.kind == kSpmv && it.k1 - it.k0 <= tnnz) {
-                cap = std::max(cap, it.k1 - it.k0);
-                rows = std::max(rows, it.e - it.b);
-            }
-        cap = std::min(tnnz, (cap + 15) & ~15);
-    };
-    {
-        const int32_t wn = std::max(32, tile_nnz / 8);
-        fit(items, tile_nnz, S.fit_nnz[0], S.fit_rows[0]);
-        fit(tl, tile_nnz, S.fit_nnz[1], S.fit_rows[1]);
-        fit(tr, tile_nnz, S.fit_nnz[2], S.fit_rows[2]);
-        fit(trh, tile_nnz, S.fit_nnz[6], S.fit_rows[6]);
-        fit(wt, wn, S.fit_nnz[3], S.fit_rows[3]);
-        fit(wtl, wn, S.fit_nnz[4], S.fit_rows[4]);
-        fit(wtr, wn, S.fit_nnz[5], S.fit_rows[5]);
-    }
-    auto upload_items = [&](const std::vector<Item> &v, Item **d, int32_t *n) -> int {
-        if (*d) cudaFree(*d);
-        *d = nullptr;
-        *n = (int32_t)v.size();
-        if (v.empty()) return NAPSPMV_OK;
-        NAP_CUDA(cudaMalloc(d, sizeof(Item) * v.size()));
-        NAP_CUDA(cudaMemcpy(*d, v.data(), sizeof(Item) * v.size(), cudaMemcpyHostToDevice));
-        return NAPSPMV_OK;
-    };
-    if (int rc = upload_items(wt, &S.d_wt, &S.n_wt)) return rc;
-    if (int rc = upload_items(trh, &S.d_tilesRH, &S.n_tilesRH)) return rc;
-    if (int rc = upload_items(wtl, &S.d_wtL, &S.n_wtL)) return rc;
-    if (int rc = upload_items(wtr, &S.d_wtR, &S.n_wtR)) return rc;
-    Item *d_tl = nullptr, *d_tr = nullptr;
-    if (!tl.empty()) {
-        NAP_CUDA(cudaMalloc(&d_tl, sizeof(Item) * tl.size()));
-        NAP_CUDA(cudaMalloc(&d_tr, sizeof(Item) * tr.size()));
-        NAP_CUDA(cudaMemcpy(d_tl, tl.data(), sizeof(Item) * tl.size(), cudaMemcpyHostToDevice));
-        NAP_CUDA(cudaMemcpy(d_tr, tr.data(), sizeof(Item) * tr.size(), cudaMemcpyHostToDevice));
-    }
-    if (S.d_tilesL) cudaFree(S.d_tilesL);
-    if (S.d_tilesR) cudaFree(S.d_tilesR);
-    S.d_tilesL = d_tl;
-    S.d_tilesR = d_tr;
-    S.n_tilesL = (int32_t)tl.size();
-    S.n_tilesR = (int32_t)tr.size();
-
-    Item *d_items = nullptr;
-    if (!items.empty()) {
-        NAP_CUDA(cudaMalloc(&d_items, sizeof(Item) * items.size()));
-        NAP_CUDA(cudaMemcpy(d_items, items.data(), sizeof(Item) * items.size(),
-                            cudaMemcpyHostToDevice));
-    }
-    if (S.d_items) cudaFree(S.d_items);
+    if (S.built && S.tile_rows == tile_rows && S.tile_nnz == tile_nnz) return NAPSPMV_OK;
+    if (int rc = cut_tiles(P, tile_rows, tile_nnz)) return rc;
     for (auto &g : P->graphs) cudaGraphExecDestroy(g.exec);  // they captured the old tiles
     P->graphs.clear();
-    S.d_items = d_items;
-    S.n_items = (int32_t)items.size();
-    S.tile_rows = tile_rows;
-    S.tile_nnz = tile_nnz;
     return NAPSPMV_OK;
 }
 
@@ -2362,7 +2226,7 @@ static size_t halo_smem(const napspmv_plan_t *P, const napspmv_opts &o)
 {
     if (o.halo != NAPSPMV_HALO_ON || o.pipeline == NAPSPMV_PIPELINE_SELL ||
         (P->flags & NAPSPMV_PARTITION_STRIDED) ||
-        P->h_bll_rank.size() != (size_t)P->np + 1 || P->items.n_tilesRH == 0 ||
+        P->h_bll_rank.size() != (size_t)P->np + 1 || P->items.list[kTilesRH].n == 0 ||
         P->nnzR < 8 * P->n)
         return 0;
     const bool f32 = o.precision == NAPSPMV_PREC_F32;
@@ -2375,7 +2239,7 @@ static size_t halo_smem(const napspmv_plan_t *P, const napspmv_opts &o)
         const int64_t n1 = (P->h_bnl_rank[r + 1] + al - 1) & ~(al - 1);
         wcap = std::max(wcap, (b1 - b0) + (n1 - n0));
     }
-    const size_t sm = (size_t)tile_smem_bytes(P->items.fit_nnz[6], P->items.fit_rows[6], o.stages,
+    const size_t sm = (size_t)tile_smem_bytes(P->items.list[kTilesRH].fit_nnz, P->items.list[kTilesRH].fit_rows, o.stages,
                                               es) + 16 + (size_t)wcap * es;
     int smem_sm = 0, reserved = 0;
     if (cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, P->device) ||
@@ -2423,39 +2287,39 @@ static int spmv_launch(const napspmv_plan_t *P, const napspmv_opts &o, int mode,
     const bool warp = o.pipeline == NAPSPMV_PIPELINE_WARP;
     const ItemSet &S = P->items;
     const int list = (warp ? 3 : 0) + (mode == kLocal ? 1 : mode == kRemote ? 2 : 0);
-    L.cap = S.fit_nnz[list];
-    L.rows = S.fit_rows[list];
+    L.cap = S.list[list].fit_nnz;
+    L.rows = S.list[list].fit_rows;
     const int vb = f32 ? 4 : 8;  // bytes per staged value
     L.sm = warp ? (size_t)warp_smem_bytes(L.cap, L.rows, o.stages, vb)
                 : smem_bytes(L.cap, L.rows, o.stages, vb);
     if (mode == kLocal) {
         L.A = Csr3{P->d_rowptrL, P->d_colL, P->d_valL, f32 ? P->d_val32L : nullptr};
         L.fn = f32 ? pick_spmv<true, kLocal>(o.vec, warp) : pick_spmv<false, kLocal>(o.vec, warp);
-        L.tiles = warp ? S.d_wtL : S.d_tilesL;
-        L.n = warp ? S.n_wtL : S.n_tilesL;
+        L.tiles = S.list[list].d;
+        L.n = S.list[list].n;
     } else if (mode == kRemote) {
         L.A = Csr3{P->d_rowptrR, P->d_colR, P->d_valR, f32 ? P->d_val32R : nullptr};
         if (const size_t hs = halo_smem(P, o)) {
             // CTA tiles cut at process boundaries, receive buffers staged
             L.hfn = f32 ? pick_halo<true>(o.vec) : pick_halo<false>(o.vec);
-            L.cap = S.fit_nnz[6];
-            L.rows = S.fit_rows[6];
+            L.cap = S.list[kTilesRH].fit_nnz;
+            L.rows = S.list[kTilesRH].fit_rows;
             L.sm = hs;
-            L.tiles = S.d_tilesRH;
-            L.n = S.n_tilesRH;
+            L.tiles = S.list[kTilesRH].d;
+            L.n = S.list[kTilesRH].n;
             L.bll_rank = P->d_bll_rank;
             L.bnl_rank = P->d_bnl_rank;
         } else {
             L.fn = f32 ? pick_spmv<true, kRemote>(o.vec, warp)
                        : pick_spmv<false, kRemote>(o.vec, warp);
-            L.tiles = warp ? S.d_wtR : S.d_tilesR;
-            L.n = warp ? S.n_wtR : S.n_tilesR;
+            L.tiles = S.list[list].d;
+            L.n = S.list[list].n;
         }
     } else {
         L.A = Csr3{P->d_rowptr, P->d_colenc, P->d_val, f32 ? P->d_val32 : nullptr};
         L.fn = f32 ? pick_spmv<true, kFull>(o.vec, warp) : pick_spmv<false, kFull>(o.vec, warp);
-        L.tiles = warp ? S.d_wt : S.d_items;
-        L.n = warp ? S.n_wt : S.n_items;
+        L.tiles = S.list[list].d;
+        L.n = S.list[list].n;
     }
     const void *kf = L.hfn ? (const void *)L.hfn : (const void *)L.fn;
     if (L.sm > 48 * 1024)
@@ -2894,7 +2758,7 @@ static int enqueue_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, 
                                                             (int64_t)P->num_sms * 8));
     };
     const ItemSet &S = P->items;
-    const bool overlap = o.engine == NAPSPMV_ENGINE_OVERLAP && S.n_tilesL > 0;
+    const bool overlap = o.engine == NAPSPMV_ENGINE_OVERLAP && S.list[kTilesL].n > 0;
     SpmvLaunch LF, LL, LR;
     if (int rc = spmv_launch(P, o, kFull, LF)) return rc;
     if (overlap) {
@@ -2961,7 +2825,7 @@ static int launch_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, d
         // attributes (dynamic shared memory) are set before any capture
         SpmvLaunch L;
         if (int rc = spmv_launch(P, o, kFull, L)) return rc;
-        if (o.engine == NAPSPMV_ENGINE_OVERLAP && P->items.n_tilesL > 0) {
+        if (o.engine == NAPSPMV_ENGINE_OVERLAP && P->items.list[kTilesL].n > 0) {
             if (int rc = spmv_launch(P, o, kLocal, L)) return rc;
             if (int rc = spmv_launch(P, o, kRemote, L)) return rc;
         }

@@ -66,31 +66,28 @@ enum ItemKind : int32_t {
 
 struct Item {
     int32_t kind;
-    int32_t node;    // node of the rows
     int32_t b, e;    // row range
     int32_t msg;     // remote tiles cut at process bounds: the process
     int32_t k0, k1;  // stored-entry range [row_ptr[b], row_ptr[e])
-    int32_t pad;
+    int32_t pad[2];
 };
 
+// The tile lists: CTA tiles of the whole matrix (cut within each node's rows), of
+// its local and remote parts; warp tiles (at most tile_rows / 8 rows, tile_nnz / 8
+// entries) of the three; remote CTA tiles cut at process bounds (Item::msg =
+// process), for the remote pass with staged receive buffers.
+enum TileList { kTiles = 0, kTilesL, kTilesR, kWarpTiles, kWarpTilesL, kWarpTilesR, kTilesRH, kTileLists };
 struct ItemSet {
+    bool built = false;
     int32_t tile_rows = 0, tile_nnz = 0;
-    int32_t n_items = 0;  // CTA tiles of the whole matrix (d_items)
-    Item *d_tilesL = nullptr, *d_tilesR = nullptr;  // tiles of the split parts
-    int32_t n_tilesL = 0, n_tilesR = 0;
-    // remote tiles cut at process boundaries (Item::msg = process), for the
-    // remote pass with staged receive buffers
-    Item *d_tilesRH = nullptr;
-    int32_t n_tilesRH = 0;
-    // warp tiles (at most tile_rows / 8 rows, tile_nnz / 8 entries) of the whole
-    // matrix and of its two split parts
-    Item *d_wt = nullptr, *d_wtL = nullptr, *d_wtR = nullptr;
-    int32_t n_wt = 0, n_wtL = 0, n_wtR = 0;
-    // largest staged tile (entries, rows) of each list, in the order whole /
-    // local / remote CTA tiles, whole / local / remote warp tiles, remote tiles
-    // cut per process: a stage is sized to what its list needs, not to tile_nnz
-    int32_t fit_nnz[7] = {}, fit_rows[7] = {};
-    Item *d_items = nullptr;
+    Item *d_all = nullptr;  // the lists, one after another
+    struct {
+        Item *d = nullptr;
+        int32_t n = 0;
+        // largest staged tile (entries, rows): a stage is sized to what its list
+        // needs, not to tile_nnz
+        int32_t fit_nnz = 0, fit_rows = 0;
+    } list[kTileLists];
 };
 
 // --------------------------------------------------------------- plan lists
@@ -213,7 +210,6 @@ struct napspmv_plan_s {
     uint32_t *d_colL = nullptr, *d_colR = nullptr;
     double *d_valL = nullptr, *d_valR = nullptr;
     float *d_val32L = nullptr, *d_val32R = nullptr;
-    std::vector<int32_t> h_rowptrL, h_rowptrR;
     // per-process offsets of b_{l->l} and b_{nl->l} (np + 1 each), host and device
     std::vector<int32_t> h_bll_rank, h_bnl_rank;
     int32_t *d_bll_rank = nullptr, *d_bnl_rank = nullptr;
@@ -227,10 +223,6 @@ struct napspmv_plan_s {
     int32_t *d_xfer_shift = nullptr;  // [ceil(n_gs / kSendGroup)]
     int32_t *d_unp_src = nullptr;    // [n_bnl]
     // BLL / LBUF list idx arrays double as the J2 / J0 gather sources.
-
-    // first row of every node (host), where the CTA row tiles are cut
-    std::vector<int64_t> node_rows;  // [nn+1]
-    std::vector<int32_t> h_rowptr;         // host copy of the row pointer, for tiling
 
     // sliced-row copies of the whole matrix, its local part and its remote
     // part (index 0, 1, 2), for NAPSPMV_PIPELINE_SELL; built with the plan
@@ -258,6 +250,7 @@ struct napspmv_plan_s {
 };
 
 namespace nap {
+int cut_tiles(napspmv_plan_t *P, int32_t tile_rows, int32_t tile_nnz);  // of every list
 int build_items(napspmv_plan_t *P, int32_t tile_rows, int32_t tile_nnz);
 constexpr int kWinSmem = 226 * 1024;  // shared memory of a staged-window CTA, at most
 int window_bytes(int64_t srcs, int64_t slots, int64_t words, int vb);  // what one with this block needs

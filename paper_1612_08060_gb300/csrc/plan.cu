@@ -21,6 +21,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cstring>
+#include <map>
 #include <numeric>
 
 #include "internal.h"
@@ -43,28 +44,99 @@ inline void ck(cudaError_t e, const char *what)
 }
 #define CK(x) ck((x), #x)
 
+// Temporaries of one plan build, on one stream: a block given back serves the next
+// request that fits it, and all are freed with the build.  About a hundred arrays
+// come and go, and each allocation and release of one synchronised the device:
+// about 3.4 of 12.4 ms of a 10^6-row 7-point plan (GB300).
+struct Scratch {
+    std::multimap<size_t, void *> idle;
+    Scratch *outer = current;
+    static thread_local Scratch *current;
+    Scratch() { current = this; }
+    ~Scratch()
+    {
+        trim();
+        current = outer;
+    }
+    void trim()
+    {
+        for (auto &b : idle) cudaFree(b.second);
+        idle.clear();
+    }
+    void *take(size_t &bytes)
+    {
+        auto it = idle.lower_bound(bytes);
+        if (it != idle.end() && it->first <= 2 * bytes + 4096) {
+            void *p = it->second;
+            bytes = it->first;
+            idle.erase(it);
+            return p;
+        }
+        void *p = nullptr;
+        cudaError_t e = cudaMalloc(&p, bytes);
+        if (e == cudaErrorMemoryAllocation && !idle.empty()) {
+            cudaGetLastError();
+            trim();
+            e = cudaMalloc(&p, bytes);
+        }
+        CK(e);
+        return p;
+    }
+};
+thread_local Scratch *Scratch::current = nullptr;
+// Memory that stays with the plan; idle temporaries make room for it.
+template <class T>
+cudaError_t device_alloc(T **p, size_t bytes)
+{
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && Scratch::current && !Scratch::current->idle.empty()) {
+        cudaGetLastError();
+        Scratch::current->trim();
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
 template <class T>
 struct dvec {
     T *p = nullptr;
     int64_t n = 0;
+    size_t bytes = 0;  // of a block that came from the scratch
     dvec() = default;
     explicit dvec(int64_t count) { alloc(count); }
     void alloc(int64_t count)
     {
-        if (p) cudaFree(p);
-        p = nullptr;
+        drop();
         n = count;
-        if (count > 0) CK(cudaMalloc(&p, sizeof(T) * (size_t)count));
+        if (count <= 0) return;
+        size_t b = (sizeof(T) * (size_t)count + 511) & ~(size_t)511;
+        if (Scratch::current) {
+            p = static_cast<T *>(Scratch::current->take(b));
+            bytes = b;
+        } else {
+            CK(device_alloc(&p, b));
+        }
     }
-    ~dvec()
+    void drop()
     {
-        if (p) cudaFree(p);
+        if (p && bytes && Scratch::current) Scratch::current->idle.emplace(bytes, p);
+        else if (p) cudaFree(p);
+        p = nullptr;
+        bytes = 0;
     }
+    ~dvec() { drop(); }
     T *release()
     {
         T *q = p;
         p = nullptr;
+        bytes = 0;
         return q;
+    }
+    void swap(dvec &o)
+    {
+        std::swap(p, o.p);
+        std::swap(n, o.n);
+        std::swap(bytes, o.bytes);
     }
     dvec(const dvec &) = delete;
     dvec &operator=(const dvec &) = delete;
@@ -75,7 +147,7 @@ T *upload(const std::vector<T> &h)
 {
     T *d = nullptr;
     size_t bytes = sizeof(T) * std::max<size_t>(h.size(), 1);
-    CK(cudaMalloc(&d, bytes));
+    CK(device_alloc(&d, bytes));
     if (!h.empty()) CK(cudaMemcpy(d, h.data(), sizeof(T) * h.size(), cudaMemcpyHostToDevice));
     return d;
 }
@@ -501,8 +573,8 @@ struct Cub {
         size_t b = 0;
         CK(cub::DeviceRadixSort::SortPairs(nullptr, b, dk, dv, (int)n, 0, end_bit, st));
         CK(cub::DeviceRadixSort::SortPairs(temp(b), b, dk, dv, (int)n, 0, end_bit, st));
-        if (dk.Current() != k.p) std::swap(k.p, k2.p);
-        if (dv.Current() != v.p) std::swap(v.p, v2.p);
+        if (dk.Current() != k.p) k.swap(k2);
+        if (dv.Current() != v.p) v.swap(v2);
     }
     void max_i32(const int32_t *in, int32_t *out, int64_t n)
     {
@@ -722,7 +794,7 @@ void make_list(Cub &cb, const uint64_t *keys, int64_t cnt, int fb, int jb, HostL
         }
         L.ptr[k + 1] = L.ptr[k] + len[k];
     }
-    CK(cudaMalloc(&L.d_idx, sizeof(int32_t) * cnt));
+    CK(device_alloc(&L.d_idx, sizeof(int32_t) * cnt));
     k_low<<<blocks_for(cnt), 256, 0, cb.st>>>(keys, cnt, (1ull << jb) - 1, L.d_idx);
     CK(cudaGetLastError());
 }
@@ -860,9 +932,9 @@ void build_sell(napspmv_plan_t *P, Cub &cb, int which, const int32_t *d_rp, cons
     S.nch = tot[0];
     S.slots = slots;
     S.n_long = (int32_t)(n - tot[2]);
-    CK(cudaMalloc(&S.d_info, sizeof(int2) * std::max<int64_t>(S.nch, 1)));
-    CK(cudaMalloc(&S.d_perm, sizeof(int32_t) * 32 * std::max<int64_t>(S.nch, 1)));
-    CK(cudaMalloc(&S.d_long, sizeof(int32_t) * std::max<int64_t>(S.n_long, 1)));
+    CK(device_alloc(&S.d_info, sizeof(int2) * std::max<int64_t>(S.nch, 1)));
+    CK(device_alloc(&S.d_perm, sizeof(int32_t) * 32 * std::max<int64_t>(S.nch, 1)));
+    CK(device_alloc(&S.d_long, sizeof(int32_t) * std::max<int64_t>(S.n_long, 1)));
     if (S.n_long)
         CK(cudaMemcpy(S.d_long, row.p + tot[2], sizeof(int32_t) * S.n_long,
                       cudaMemcpyDeviceToDevice));
@@ -872,7 +944,7 @@ void build_sell(napspmv_plan_t *P, Cub &cb, int which, const int32_t *d_rp, cons
     // padded past the last slot: a block's bulk copy is widened to 16 bytes
     auto al = [&](size_t sz, int fill = 0) {
         void *q = nullptr;
-        CK(cudaMalloc(&q, sz * (size_t)std::max<int64_t>(slots, 1) + 256));
+        CK(device_alloc(&q, sz * (size_t)std::max<int64_t>(slots, 1) + 256));
         CK(cudaMemset(q, fill, sz * (size_t)std::max<int64_t>(slots, 1) + 256));
         return q;
     };
@@ -885,7 +957,7 @@ void build_sell(napspmv_plan_t *P, Cub &cb, int which, const int32_t *d_rp, cons
                                                      S.d_val32);
         CK(cudaGetLastError());
     }
-    if (win_off) std::swap(win_off->p, off.p);
+    if (win_off) win_off->swap(off);
 }
 
 // A block takes at most this much shared memory in FP64: four CTAs to an SM.
@@ -1137,14 +1209,14 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
     const int64_t total = offsets(nsrc.p, osrc);
     const size_t slots = (size_t)std::max<int64_t>(P->sell[0].slots, 1);
     dvec<uint32_t> src(std::max<int64_t>(total, 1));
-    CK(cudaMalloc(&W.d_col, sizeof(uint16_t) * slots + 256));
+    CK(device_alloc(&W.d_col, sizeof(uint16_t) * slots + 256));
     const int grid = (int)std::min<int64_t>(nblk, 1 << 20);
     k_win_block<true><<<grid, 256, 8 * words>>>(
         P->d_rowptr, P->d_colenc, G, nblk, nullptr, nullptr, nullptr, off.p + nblk + 1, osrc.p,
         P->lists[L_BLL].d_idx, P->d_unp_src, P->sell[0].d_col, src.p, W.d_col);
     CK(cudaGetLastError());
     if (st[1] >= kWinPad) return;
-    CK(cudaMalloc(&W.d_blk, sizeof(WinBlock) * nblk));
+    CK(device_alloc(&W.d_blk, sizeof(WinBlock) * nblk));
     const int bgrid = (int)((nblk + 255) / 256);
     if (W.long_rows) {  // plain lists
         if (total > INT32_MAX) return;
@@ -1159,7 +1231,7 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
         cb.max_i32(nword.p, stat.p + 3, nblk);
         const int64_t all = offsets(nword.p, oword);
         if (all / 4 > (int64_t)INT32_MAX) return;
-        CK(cudaMalloc(&W.d_runs, sizeof(uint32_t) * std::max<int64_t>(all, 1)));
+        CK(device_alloc(&W.d_runs, sizeof(uint32_t) * std::max<int64_t>(all, 1)));
         k_win_runs<true><<<wgrid, 256>>>(nblk, src.p, osrc.p, nsrc.p, nullptr, oword.p, W.d_runs);
         CK(cudaGetLastError());
         k_win_blocks<<<bgrid, 256>>>(nblk, off.p, off.p + nblk + 1, nsrc.p, nword.p, oword.p, 4,
@@ -1179,6 +1251,7 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
 {
     const int64_t n = A->n, nnz = A->nnz;
     const int32_t np = P->np, ppn = P->ppn, nn = P->nn;
+    Scratch scratch;  // outlives every temporary below
     Cub cb;
     Part part{n / np, n % np, (n % np) * (n / np + 1), np,
               (P->flags & NAPSPMV_PARTITION_STRIDED) != 0};
@@ -1480,8 +1553,8 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
     dvec<int32_t> msg_of(ngs);
     dvec<uint64_t> j0key(ngs), j0alt(ngs);
     if (ngs) {
-        CK(cudaMalloc(&P->lists[L_INTER].d_idx, sizeof(int32_t) * ngs));
-        CK(cudaMalloc(&P->d_xfer_dst, sizeof(int32_t) * ngs));
+        CK(device_alloc(&P->lists[L_INTER].d_idx, sizeof(int32_t) * ngs));
+        CK(device_alloc(&P->d_xfer_dst, sizeof(int32_t) * ngs));
         k_fill_gsend<<<blocks_for(ngs), 256>>>(ngs, d_gs_off.p, NM, d_msg_pair.p, d_msg_src.p,
                                               d_msg_gr.p, d_msg_lo.p, d_node_ptr.p, ND.d_idx,
                                               part, rb, jb, P->lists[L_INTER].d_idx,
@@ -1491,7 +1564,7 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
 
     if (ngs) {
         const int64_t groups = (ngs + kSendGroup - 1) / kSendGroup;
-        CK(cudaMalloc(&P->d_xfer_shift, sizeof(int32_t) * groups));
+        CK(device_alloc(&P->d_xfer_shift, sizeof(int32_t) * groups));
         k_xfer_shift<<<blocks_for(32 * groups), 256>>>(P->d_xfer_dst, ngs, P->d_xfer_shift);
         CK(cudaGetLastError());
     }
@@ -1525,7 +1598,7 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
     d_bll_ptr.p = upload(bll_ptr);
     d_bnl_ptr.p = upload(bnl_ptr);
     if (ngs) {
-        CK(cudaMalloc(&P->d_pack_src, sizeof(uint32_t) * ngs));
+        CK(device_alloc(&P->d_pack_src, sizeof(uint32_t) * ngs));
         k_pack_src<<<blocks_for(ngs), 256>>>(ngs, P->lists[L_INTER].d_idx, msg_of.p, d_msg_src.p,
                                             d_lbuf_ptr.p, P->lists[L_LBUF].d_idx, part,
                                             P->d_pack_src, bad.p);
@@ -1548,7 +1621,7 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
     d_piece_dst.p = upload(piece_dst);
     dvec<uint64_t> j1key(nbnl), j1alt(nbnl);
     if (nbnl) {
-        CK(cudaMalloc(&P->d_unp_src, sizeof(int32_t) * nbnl));
+        CK(device_alloc(&P->d_unp_src, sizeof(int32_t) * nbnl));
         k_unpack_src<<<blocks_for(nbnl), 256>>>(nbnl, bnl_keys.p, jb, part, ppn, nb, M,
                                                d_pair_key.p, d_pair_piece.p, d_piece_lo.p,
                                                d_piece_dst.p, d_piece_gr.p, d_node_ptr.p,
@@ -1565,13 +1638,13 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
 
     // ---- three-block CSR
     // padded so that 16-byte bulk copies of a row range may read past the end
-    CK(cudaMalloc(&P->d_rowptr, sizeof(int32_t) * (n + 16)));
+    CK(device_alloc(&P->d_rowptr, sizeof(int32_t) * (n + 16)));
     CK(cudaMemset(P->d_rowptr, 0, sizeof(int32_t) * (n + 16)));
-    CK(cudaMalloc(&P->d_colenc, sizeof(uint32_t) * std::max<int64_t>(nnz, 1) + 64));
-    CK(cudaMalloc(&P->d_val, sizeof(double) * std::max<int64_t>(nnz, 1) + 64));
-    CK(cudaMalloc(&P->d_split, sizeof(int32_t) * 3 * n));
+    CK(device_alloc(&P->d_colenc, sizeof(uint32_t) * std::max<int64_t>(nnz, 1) + 64));
+    CK(device_alloc(&P->d_val, sizeof(double) * std::max<int64_t>(nnz, 1) + 64));
+    CK(device_alloc(&P->d_split, sizeof(int32_t) * 3 * n));
     if (P->flags & NAPSPMV_F32_VALUES)
-        CK(cudaMalloc(&P->d_val32, sizeof(float) * std::max<int64_t>(nnz, 1) + 64));
+        CK(device_alloc(&P->d_val32, sizeof(float) * std::max<int64_t>(nnz, 1) + 64));
     k_three_block<<<blocks_for(n), 256>>>(rp.p, n, col.p, val.p, tag.p, part, d_bll_ptr.p,
                                          P->lists[L_BLL].d_idx, d_bnl_ptr.p,
                                          P->lists[L_BNL].d_idx, P->d_colenc, P->d_val,
@@ -1582,8 +1655,8 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
     // ---- local / remote split
     {
         dvec<int32_t> lenL(n + 1), lenR(n + 1);
-        CK(cudaMalloc(&P->d_rowptrL, sizeof(int32_t) * (n + 16)));
-        CK(cudaMalloc(&P->d_rowptrR, sizeof(int32_t) * (n + 16)));
+        CK(device_alloc(&P->d_rowptrL, sizeof(int32_t) * (n + 16)));
+        CK(device_alloc(&P->d_rowptrR, sizeof(int32_t) * (n + 16)));
         CK(cudaMemset(P->d_rowptrL, 0, sizeof(int32_t) * (n + 16)));
         CK(cudaMemset(P->d_rowptrR, 0, sizeof(int32_t) * (n + 16)));
         k_split_lens<<<blocks_for(n + 1), 256>>>(P->d_split, n, lenL.p, lenR.p);
@@ -1593,18 +1666,12 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
         void *tmp = cb.temp(b);
         CK(cub::DeviceScan::ExclusiveSum(tmp, b, lenL.p, P->d_rowptrL, (int)(n + 1)));
         CK(cub::DeviceScan::ExclusiveSum(tmp, b, lenR.p, P->d_rowptrR, (int)(n + 1)));
-        P->h_rowptrL.resize(n + 1);
-        P->h_rowptrR.resize(n + 1);
-        CK(cudaMemcpy(P->h_rowptrL.data(), P->d_rowptrL, sizeof(int32_t) * (n + 1),
-                      cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(P->h_rowptrR.data(), P->d_rowptrR, sizeof(int32_t) * (n + 1),
-                      cudaMemcpyDeviceToHost));
-        P->nnzL = P->h_rowptrL[n];
-        P->nnzR = P->h_rowptrR[n];
+        P->nnzL = P->stats.nnz_on_process;
+        P->nnzR = nnz - P->nnzL;
         const bool f32 = P->d_val32 != nullptr;
         auto al = [&](int64_t m, size_t sz) {
             void *q = nullptr;
-            CK(cudaMalloc(&q, sz * (size_t)std::max<int64_t>(m, 1) + 64));
+            CK(device_alloc(&q, sz * (size_t)std::max<int64_t>(m, 1) + 64));
             return q;
         };
         P->d_colL = (uint32_t *)al(P->nnzL, 4);
@@ -1627,20 +1694,6 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
     }
     CK(cudaDeviceSynchronize());
 
-    // ---- first row of every node, where the CTA row tiles are cut
-    P->node_rows.assign(nn + 1, 0);
-    for (int32_t x = 0; x <= nn; x++) {
-        int32_t r = std::min<int64_t>((int64_t)x * ppn, np);
-        // strided: every node's rows interleave; the row tiles are cut over
-        // all rows as one range
-        P->node_rows[x] = part.strided ? (x == 0 ? 0 : n) : part.start(r);
-    }
-    {
-        std::vector<int64_t> h(n + 1);
-        CK(cudaMemcpy(h.data(), rp.p, sizeof(int64_t) * (n + 1), cudaMemcpyDeviceToHost));
-        P->h_rowptr.resize(n + 1);
-        for (int64_t i = 0; i <= n; i++) P->h_rowptr[i] = (int32_t)h[i];
-    }
     // sliced-row copies of the whole matrix and of its two split parts
     build_windows(P, cb, part, d_bll_ptr.p, d_bnl_ptr.p);
     build_sell(P, cb, 1, P->d_rowptrL, P->d_colL, P->d_valL, P->d_val32L, part);
@@ -1651,6 +1704,160 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
 }
 
 }  // namespace
+
+// Row tiles.  A list's rows are cut into segments (at most kSegment rows, within a
+// node's or a process's rows where the list wants that); a warp per segment lays
+// tiles one after another, each as many rows as fit tile_rows rows and tile_nnz
+// entries (a longer single row alone).  Cutting the seven lists on the host, row by
+// row, took 5.1 of 17.6 ms of a 10^6-row 7-point plan, and their three row pointers
+// 0.8 ms to bring there; this way 0.65 ms (GB300).
+namespace {
+constexpr int kSegment = 16384;
+struct TileCut {
+    const int32_t *rp[kTileLists];
+    int32_t rows[kTileLists], cap[kTileLists];
+    int64_t segs[kTileLists];   // of every list
+    int32_t group[kTileLists];  // processes per unit that tiles stay within; 0: none
+    int32_t sub[kTileLists];    // segments per unit
+    Part part;
+    int64_t n;
+};
+template <bool WRITE>
+__global__ void k_cut_tiles(TileCut C, int32_t *count, const int64_t *off, int32_t *fit, Item *items)
+{
+    const int list = blockIdx.y, lane = threadIdx.x & 31;
+    const int32_t *rp = C.rp[list];
+    const int32_t rows = C.rows[list], cap = C.cap[list];
+    int64_t base = 0;  // of this list among all segments
+    for (int q = 0; q < list; q++) base += C.segs[q];
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < C.segs[list]; s += warps) {
+        int64_t r, e;
+        int32_t unit = 0;
+        if (C.group[list]) {
+            unit = (int32_t)(s / C.sub[list]);
+            const int64_t u0 = C.part.start(min((int64_t)unit * C.group[list], C.part.np));
+            const int64_t u1 = C.part.start(min((int64_t)(unit + 1) * C.group[list], C.part.np));
+            r = min(u1, u0 + s % C.sub[list] * kSegment);
+            e = min(u1, r + kSegment);
+        } else {
+            r = s * kSegment;
+            e = min(C.n, r + kSegment);
+        }
+        int64_t at = WRITE ? off[base + s] : 0;
+        int32_t most = 0, tall = 0;
+        while (r < e) {
+            const int32_t k0 = rp[r];
+            const int32_t limit = (int32_t)min((int64_t)rows, e - r);
+            int32_t m = 0;  // rows of the tile
+            for (;;) {
+                const int32_t i = m + lane + 1;
+                const unsigned ok = __ballot_sync(0xffffffffu, i <= limit && rp[r + min(i, limit)] - k0 <= cap);
+                if (ok == 0xffffffffu) {
+                    m += 32;
+                    continue;
+                }
+                m += __ffs(~ok) - 1;  // (the row pointer ascends: a prefix fits)
+                break;
+            }
+            m = max(m, 1);
+            const int32_t k1 = rp[r + m];
+            if (WRITE && lane == 0) {
+                Item it{};
+                it.kind = kSpmv;
+                it.b = (int32_t)r;
+                it.e = (int32_t)(r + m);
+                it.msg = list == kTilesRH ? unit : 0;
+                it.k0 = k0;
+                it.k1 = k1;
+                items[at] = it;
+            }
+            if (k1 - k0 <= cap) {
+                most = max(most, k1 - k0);
+                tall = max(tall, m);
+            }
+            at++;
+            r += m;
+        }
+        if (!WRITE && lane == 0) {
+            count[base + s] = (int32_t)at;
+            atomicMax(&fit[2 * list], most);
+            atomicMax(&fit[2 * list + 1], tall);
+        }
+    }
+}
+}  // namespace
+
+int cut_tiles(napspmv_plan_t *P, int32_t tile_rows, int32_t tile_nnz)
+{
+    try {
+        const int64_t n = P->n;
+        const bool strided = (P->flags & NAPSPMV_PARTITION_STRIDED) != 0;
+        TileCut C{};
+        C.part = Part{n / P->np, n % P->np, (n % P->np) * (n / P->np + 1), P->np, strided};
+        C.n = n;
+        int64_t all = 0;
+        for (int q = 0; q < kTileLists; q++) {
+            const bool warp = q == kWarpTiles || q == kWarpTilesL || q == kWarpTilesR;
+            C.rp[q] = q == kTilesL || q == kWarpTilesL   ? P->d_rowptrL
+                      : q == kTiles || q == kWarpTiles ? P->d_rowptr
+                                                       : P->d_rowptrR;
+            C.rows[q] = warp ? std::max(1, tile_rows / 8) : tile_rows;
+            C.cap[q] = warp ? std::max(32, tile_nnz / 8) : tile_nnz;
+            C.segs[q] = (n + kSegment - 1) / kSegment;
+            if (q == kTilesRH && strided) C.segs[q] = 0;
+            if (!strided && (q == kTiles || q == kTilesRH)) {
+                C.group[q] = q == kTiles ? P->ppn : 1;
+                const int64_t units = q == kTiles ? P->nn : P->np;
+                const int64_t most = std::min<int64_t>(C.group[q], P->np) * C.part.rows(0);
+                C.sub[q] = (int32_t)((most + kSegment - 1) / kSegment);
+                C.segs[q] = units * C.sub[q];
+            }
+            all += C.segs[q];
+        }
+        Cub cb;
+        dvec<int32_t> count(all + 1), fit(2 * kTileLists);
+        dvec<int64_t> wide(all + 1), off(all + 1);
+        CK(cudaMemset(fit.p, 0, sizeof(int32_t) * 2 * kTileLists));
+        const int64_t most = *std::max_element(C.segs, C.segs + kTileLists);
+        const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>((most + 7) / 8, 1 << 16)), kTileLists);
+        k_cut_tiles<false><<<grid, 256>>>(C, count.p, nullptr, fit.p, nullptr);
+        k_widen<<<blocks_for(all + 1), 256>>>(count.p, all, wide.p);
+        CK(cudaGetLastError());
+        cb.exclusive_sum(wide.p, off.p, all + 1);
+        int64_t first[kTileLists + 1], base = 0;
+        int32_t hf[2 * kTileLists];
+        for (int q = 0; q <= kTileLists; q++) {
+            CK(cudaMemcpyAsync(&first[q], off.p + base, sizeof(int64_t), cudaMemcpyDeviceToHost));
+            if (q < kTileLists) base += C.segs[q];
+        }
+        CK(cudaMemcpy(hf, fit.p, sizeof(hf), cudaMemcpyDeviceToHost));
+        Item *d = nullptr;
+        CK(device_alloc(&d, sizeof(Item) * std::max<int64_t>(first[kTileLists], 1)));
+        k_cut_tiles<true><<<grid, 256>>>(C, nullptr, off.p, nullptr, d);
+        const cudaError_t e = cudaStreamSynchronize(0);
+        if (e != cudaSuccess) cudaFree(d);
+        CK(e);
+        ItemSet &S = P->items;
+        if (S.d_all) cudaFree(S.d_all);
+        S.d_all = d;
+        for (int q = 0; q < kTileLists; q++) {
+            auto &L = S.list[q];
+            L.d = d + first[q];
+            L.n = (int32_t)(first[q + 1] - first[q]);
+            // the stage the list needs: its largest tile that is staged at all
+            L.fit_nnz = std::min(C.cap[q], (std::max(32, hf[2 * q]) + 15) & ~15);
+            L.fit_rows = std::max(1, hf[2 * q + 1]);
+        }
+        S.tile_rows = tile_rows;
+        S.tile_nnz = tile_nnz;
+        S.built = true;
+    } catch (const NapError &e) {
+        set_error(e.code, e.msg);
+        return e.code;
+    }
+    return NAPSPMV_OK;
+}
 
 void plan_free(napspmv_plan_t *P)
 {
@@ -1667,8 +1874,7 @@ void plan_free(napspmv_plan_t *P)
         if (L.d_idx) cudaFree(L.d_idx);
     void *ptrs[] = {P->d_split, P->d_rowptr, P->d_colenc, P->d_val, P->d_val32, P->d_pack_src,
                     P->d_xfer_dst, P->d_xfer_shift, P->d_unp_src,
-                    P->items.d_items, P->items.d_tilesL, P->items.d_tilesR,
-                    P->items.d_wt, P->items.d_wtL, P->items.d_wtR, P->items.d_tilesRH,
+                    P->items.d_all,
                     P->d_rowptrL, P->d_rowptrR, P->d_colL, P->d_colR, P->d_valL, P->d_valR,
                     P->d_val32L, P->d_val32R, P->d_bll_rank, P->d_bnl_rank};
     if (P->aux) cudaStreamDestroy(P->aux);

@@ -56,3 +56,34 @@ def test_bits_of_the_tile_pass(kind, rows, n_p, flags):
         if prec == nap.PREC_F64:
             for w in out:
                 assert_close_fp64(w, O.spmv(A.row_ptr, A.col, A.val, v), abs_row_bound(A, v))
+
+
+@pytest.mark.parametrize("n,n_p,ppn,flags", [(16383, 1, 1, 0), (16384, 3, 2, 0), (16385, 1, 1, 0), (32769, 2, 1, 0),
+                                             (32768 + 31, 700, 3, 0), (16385, 5, 2, nap.PARTITION_STRIDED)])
+@pytest.mark.parametrize("rows,nnz", [(1, 32), (33, 64), (512, 1536), (4000, 6000)])
+def test_tiles_around_a_segment(n, n_p, ppn, flags, rows, nnz):
+    """Row tiles are cut in segments of 16,384 rows: every row in one tile of each list,
+    whatever the tile shape, so the tile passes give the sliced pass's bits."""
+    rng = np.random.default_rng(n + rows)
+    length = rng.integers(0, 9, n)
+    length[rng.integers(0, n, 5)] = 150  # past the smaller tiles
+    off = np.arange(150) * 7
+    cols = [np.sort((i + off[:k]) % n) for i, k in enumerate(length)]
+    row_ptr = np.zeros(n + 1, np.int64)
+    np.cumsum(length, out=row_ptr[1:])
+    A = I.CSR(row_ptr, np.concatenate(cols).astype(np.int32), rng.uniform(-1, 1, int(row_ptr[-1])))
+    plan = gpu_plan(A, n_p, ppn, flags)
+    vd = torch.from_numpy(I.vector(n, 2)).cuda()
+    out = {}
+    for engine in (nap.ENGINE_PHASED, nap.ENGINE_OVERLAP):
+        for pipe in (nap.PIPELINE_SELL, nap.PIPELINE_CTA, nap.PIPELINE_WARP):
+            w = torch.full_like(vd, float("nan"))
+            o = nap.make_opts(engine=engine, pipeline=pipe, vec=1, tile_rows=rows, tile_nnz=nnz)
+            nap.napspmv_apply_ex(plan, vd, w, 1, 1.0, o)
+            assert nap.napspmv_status(plan) == 0
+            out[engine, pipe] = w.cpu().numpy()
+    short = length < 150  # a row past a tile is a tree sum
+    want = out[nap.ENGINE_PHASED, nap.PIPELINE_SELL]
+    for w in out.values():
+        assert np.array_equal(w[short].view(np.int64), want[short].view(np.int64))
+        assert_close_fp64(w, want, abs_row_bound(A, vd.cpu().numpy()))
