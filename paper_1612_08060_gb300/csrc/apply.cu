@@ -2711,36 +2711,59 @@ bool runs_on_windows(const napspmv_plan_t *P, int32_t precision)
 {
     napspmv_opts o{};
     o.precision = precision;
-    return resolve_opts(P, &o).window;
+    return !P->win.long_rows && resolve_opts(P, &o).window;
 }
-SendList send_list(const napspmv_plan_t *P)
+SendList send_list(const napspmv_plan_t *P, const napspmv_ws_t *ws)
 {
-    return SendList{P->lists[L_INTER].d_idx, P->d_xfer_dst, P->d_xfer_shift, P->ws->grecv, P->ws->err,
+    return SendList{P->lists[L_INTER].d_idx, P->d_xfer_dst, P->d_xfer_shift, ws->grecv, ws->err,
                     (int32_t)P->n_gs};
 }
-int send_alone(napspmv_plan_t *P, int32_t precision, const double *x, cudaStream_t s)
+template <int MAXJ>
+static int send_jobs(int count, napspmv_plan_t *const *plans, napspmv_ws_t *const *ws, bool f32,
+                     const double *const *x, cudaStream_t s)
 {
-    if (P->n_gs == 0) return NAPSPMV_OK;
-    const bool f32 = precision == NAPSPMV_PREC_F32;
-    SendJobs<1> S{};
-    S.n = 1;
-    S.job[0] = send_job(P, f32, x, P->ws->grecv, P->ws->err);
-    launch_pdl(true, f32 ? k_send<float, double, 1> : k_send<double, double, 1>, S.job[0].blocks, 0, s, S);
+    SendJobs<MAXJ> S;
+    S.n = 0;
+    int blocks = 0;
+    for (int i = 0; i < count; i++) {
+        if (plans[i]->n_gs == 0) continue;
+        SendJob J = send_job(plans[i], f32, x[i], ws[i]->grecv, ws[i]->err);
+        J.block0 = blocks;
+        blocks += J.blocks;
+        S.job[S.n++] = J;
+    }
+    if (S.n == 0) return NAPSPMV_OK;
+    launch_pdl(true, f32 ? k_send<float, double, MAXJ> : k_send<double, double, MAXJ>, blocks, 0, s, S);
     count_launch(1);
     NAP_CUDA(cudaGetLastError());
     return NAPSPMV_OK;
 }
-int window_alone(napspmv_plan_t *P, int32_t precision, const double *x, double *y, cudaStream_t s)
+template <int MAXJ>
+static int window_jobs(int count, napspmv_plan_t *const *plans, napspmv_ws_t *const *ws,
+                       int32_t precision, const double *const *x, double *const *y, cudaStream_t s)
 {
     napspmv_opts o{};
     o.precision = precision;
     const bool f32 = precision == NAPSPMV_PREC_F32;
-    WinJobs<1> W;
-    W.job[0] = window_job(P, P->ws, x, nullptr, y, nullptr, 1.0);
-    const napspmv_plan_t *pl[1] = {P};
-    P->ws->recv_f32 = f32;
+    WinJobs<MAXJ> W;
+    for (int i = 0; i < count; i++) {
+        W.job[i] = window_job(plans[i], ws[i], x[i], nullptr, y[i], nullptr, 1.0);
+        ws[i]->recv_f32 = f32;
+    }
     count_launch(1);
-    return window_launch<1>(1, pl, W, f32 ? 2 : 0, false, resolve_opts(P, &o), s);
+    return window_launch<MAXJ>(count, plans, W, f32 ? 2 : 0, false, resolve_opts(plans[0], &o), s);
+}
+int send_alone(int count, napspmv_plan_t *const *plans, napspmv_ws_t *const *ws, int32_t precision,
+               const double *const *x, cudaStream_t s)
+{
+    const bool f32 = precision == NAPSPMV_PREC_F32;
+    return count == 1 ? send_jobs<1>(1, plans, ws, f32, x, s) : send_jobs<64>(count, plans, ws, f32, x, s);
+}
+int window_alone(int count, napspmv_plan_t *const *plans, napspmv_ws_t *const *ws, int32_t precision,
+                 const double *const *x, double *const *y, cudaStream_t s)
+{
+    return count == 1 ? window_jobs<1>(1, plans, ws, precision, x, y, s)
+                      : window_jobs<64>(count, plans, ws, precision, x, y, s);
 }
 
 static int enqueue_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, double *w, int reps,

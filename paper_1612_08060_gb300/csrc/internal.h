@@ -275,16 +275,19 @@ int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const
                 const double *scale, const napspmv_opts *opts, cudaStream_t s, bool keep = true,
                 bool as_batch = false);
 // Pieces of an apply for a caller that makes its vector itself (CG): whether
-// applies at this precision run on staged windows by default; the inter-node
-// messages of x alone; the windowed SpMV alone; and where the messages go.
+// applies at this precision run on short-row staged windows by default; the
+// inter-node messages of several vectors alone (one each for distinct plans or
+// workspaces); the windowed SpMVs alone; and where the messages go.
 bool runs_on_windows(const napspmv_plan_t *P, int32_t precision);
-int send_alone(napspmv_plan_t *P, int32_t precision, const double *x, cudaStream_t s);
-int window_alone(napspmv_plan_t *P, int32_t precision, const double *x, double *y, cudaStream_t s);
+int send_alone(int count, napspmv_plan_t *const *plans, napspmv_ws_t *const *ws, int32_t precision,
+               const double *const *x, cudaStream_t s);
+int window_alone(int count, napspmv_plan_t *const *plans, napspmv_ws_t *const *ws, int32_t precision,
+                 const double *const *x, double *const *y, cudaStream_t s);
 struct SendList {
     const int32_t *j, *dst, *shift;  // see k_send
     void *grecv;
     const int *err;
     int32_t n;
 };
-SendList send_list(const napspmv_plan_t *P);
+SendList send_list(const napspmv_plan_t *P, const napspmv_ws_t *ws);
 }  // namespace nap

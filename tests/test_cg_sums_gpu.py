@@ -49,3 +49,34 @@ def test_batched_scalars(n):
         scal = s["scal"].cpu().numpy()
         assert scal[5] == bb and scal[1] == bb and scal[2] == 1.0 and scal[0] == 0.0
         assert torch.equal(s["x"], s["b"]) and not s["r"].any()
+
+
+@pytest.mark.parametrize("prec", [nap.PREC_F64, nap.PREC_F32])
+@pytest.mark.parametrize("iters", [2, 5, 8])
+def test_iterations_in_one_call(prec, iters):
+    """Several iterations in one call (the direction alternating with the workspace's vector
+    and sent as it is formed) against one iteration a call: the same operations, the same
+    bits, and the same receives for a step afterwards."""
+    mats = [(I.poisson2d(70), 5, 16, 0), (I.poisson3d(12), 4, 2, 0), (I.poisson2d(40), 20, 4, nap.PARTITION_STRIDED),
+            (I.poisson2d(330), 53, 16, 0)]  # the last one past NAPSPMV_SOLO_NNZ
+    runs = []
+    for calls in ([iters], [1] * iters):
+        slots = []
+        for k, (A, n_p, ppn, fl) in enumerate(mats):
+            plan = gpu_plan(A, n_p, ppn, nap.F32_VALUES | fl)
+            z = lambda: torch.zeros(A.n, dtype=torch.float64, device="cuda")  # noqa: E731, B023
+            slots.append(dict(plan=plan, ws=nap.Workspace(plan), b=torch.from_numpy(I.vector(A.n, k)).cuda(), x=z(), r=z(),
+                              p=z(), q=z(), scal=torch.zeros(8, dtype=torch.float64, device="cuda")))
+        nap.napspmv_cg_batch_init(slots, prec, x_is_zero=True)
+        for c in calls:
+            nap.napspmv_cg_batch_iterate(slots, prec, c)
+        out = [s[f].clone() for s in slots for f in ("x", "r", "p", "q", "scal")]
+        for k, s in enumerate(slots):
+            assert nap.napspmv_ws_status(s["ws"]) == 0
+            big = mats[k][0].nnz >= nap.SOLO_NNZ
+            step = torch.empty_like(s["x"])
+            nap.napspmv_spmv_step(s["plan"], s["b"], step, 1.0, nap.make_opts(precision=prec if big else nap.PREC_F64), ws=s["ws"])
+            out.append(step)
+        runs.append([o.cpu().numpy().view(np.int64) for o in out])
+    for k, (a, b) in enumerate(zip(*runs)):
+        assert np.array_equal(a, b), k
