@@ -118,8 +118,7 @@ extern "C" {
  * blocks, a CTA brings the values its block multiplies into shared memory, each
  * once, and sums its sliced rows from there (the bits of vec = 1).  That takes at
  * least 64 rows per process on average, no row of more than 256 entries and no
- * composed gathers, and with PREC_F32 rows of at most 12 entries on average or a
- * small matrix; otherwise, and once napspmv_set_default_opts has set a plan's
+ * composed gathers; otherwise, and once napspmv_set_default_opts has set a plan's
  * defaults, the engine and pipeline of napspmv_get_default_opts run. */
 #define NAPSPMV_ENGINE_DEFAULT 0 /* the plan's default engine               */
 #define NAPSPMV_ENGINE_FUSED 1   /* one persistent, cooperative launch for all

@@ -1122,9 +1122,12 @@ __global__ void __launch_bounds__(32 * W, W == 8 ? (U >= 8 ? 4 : 6) : 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint64_t pol = policy_evict_first();  // the matrix streams once per apply
     const int ngroups = (S.nch + G - 1) / G;
-    for (int g = blockIdx.x; g < ngroups; g += gridDim.x)
-        for (int c = g * G + warp; c < min(S.nch, (g + 1) * G); c += WPB)
-            sell_chunk<F32, false, MODE, U>(S, c, x, bll, bnl, y, y32, sc, lane, pol);
+    // chunks of a group are sorted by length: every other group is dealt backwards,
+    // so that no warp takes the longest of each
+    for (int g = blockIdx.x, back = 0; g < ngroups; g += gridDim.x, back ^= 1) {
+        const int c = g * G + (back ? G - 1 - warp : warp);
+        if (c < S.nch) sell_chunk<F32, false, MODE, U>(S, c, x, bll, bnl, y, y32, sc, lane, pol);
+    }
     // rows longer than kSellLong: a warp each
     const int gw = blockIdx.x * WPB + warp, nw = gridDim.x * WPB;
     for (int q = gw; q < S.n_long; q += nw) row_warp<F32, MODE>(S.A, x, bll, bnl, y, y32, sc, S.lrows[q], lane);
@@ -1353,13 +1356,16 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 // Bound by the SM's load path, which takes a 32-byte sector per gathered value
 // where the sources are sparse (about 9.4 TB/s over the chip; the sums' shared
 // loads queue behind them) and then by the FP64 pipe (40% busy).  Per apply on
-// GB300, FP64 values, chains of 10: 1,002 us for the 2^23-row banded matrix, where
+// GB300, FP64 values, chains of 10: 940 us for the 2^23-row banded matrix, where
 // gathers into b_{l->l} and b_{nl->l} and the sliced-row pass take 1,193 (and
-// 1,436 with the message hops one by one), 484 against 545 at 4 * 10^6 rows, 109
-// against 129 at 10^6, 10.4 against 19.2 at 5 * 10^4.  Tried at 2^23 rows: 8
+// 1,436 with the message hops one by one), 449 against 545 at 4 * 10^6 rows, 102
+// against 129 at 10^6, 10.4 against 19.2 at 5 * 10^4; FP32 values 827 against 879,
+// 405 against 427, 99 against 111 and 12.3 against 20.  Chunks dealt by length
+// alone, longest to the first warp, took 1,002 us at 2^23 rows (FP64), and then 8
 // values in flight per thread 1,072, 2 1,028; 6 entries a step 1,109; no L2 request
 // 1,031; entries bulk-copied to shared memory as well (256-row blocks, 8 summing
-// warps) 1,784, since every shared load then waits behind the gathers.
+// warps) 1,784, since every shared load then waits behind the gathers.  Four FP32
+// products tested and widened at once: no gain.
 // Start bringing [p, p + bytes) into L2 (one thread; 16-byte multiples).
 __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
 {
@@ -1451,7 +1457,10 @@ __global__ void __launch_bounds__(1024, 1)
         }
     } else {
         // sum
-        const int warp = threadIdx.x >> 5;
+        // chunks of a block are sorted by length: every other block is dealt backwards,
+        // so that no warp takes the longest of each (the second window gives a block
+        // of slack)
+        const int warp = threadIdx.x >> 5, drawn = warps - 1 - warp;
         int c = S.blk[b].chunk0 + warp, c1 = S.blk[b].chunk0 + S.blk[b].chunks;
         int2 inf = c < c1 ? S.info[c] : make_int2(0, 0);
         int row = c < c1 ? S.perm[32 * c + lane] : -1;
@@ -1479,7 +1488,7 @@ __global__ void __launch_bounds__(1024, 1)
             const int nb = b + gridDim.x;
             int nc = 0, nc1 = 0;
             if (nb < nblk) {
-                nc = S.blk[nb].chunk0 + warp;
+                nc = S.blk[nb].chunk0 + (it & 1 ? warp : drawn);
                 nc1 = S.blk[nb].chunk0 + S.blk[nb].chunks;
                 if (threadIdx.x == 0 && S.blk[nb].slots) {
                     const uint32_t m = (uint32_t)S.blk[nb].slots;
@@ -1892,12 +1901,6 @@ struct FusedKernelTable {
 
 static bool valid_vec(int v) { return v == 1 || v == 2 || v == 4 || v == 8 || v == 16 || v == 32; }
 
-// Long rows with FP32 values run on the windows up to this many entries: below
-// it launches count (5 * 10^4 rows: 12.5 us per apply against 20), above it the
-// sliced-row pass is as fast or faster (1.5 * 10^5 rows: 25.3 against 25.0 us,
-// 10^6: 110.5 against 106, 4 * 10^6: 444 against 425).
-constexpr int64_t kWinLongF32 = 2500000;
-
 bool leaves_path_open(const napspmv_opts &o)
 {
     return (!o.engine || o.engine == NAPSPMV_ENGINE_PHASED) && !o.pipeline && !o.vec &&
@@ -1922,7 +1925,7 @@ Opts resolve_opts(const napspmv_plan_t *P, const napspmv_opts *o)
         if (o->timeout_ms) r.timeout_ms = o->timeout_ms;
         r.debug_stall = o->debug_stall;
     }
-    r.window = P->win.blocks > 0 && (!P->win.long_rows || r.precision == NAPSPMV_PREC_F64 || P->nnz <= kWinLongF32) &&
+    r.window = P->win.blocks > 0 &&
                ((P->auto_window && (!o || leaves_path_open(*o))) ||
                 (r.engine == NAPSPMV_ENGINE_PHASED && r.pipeline == NAPSPMV_PIPELINE_SELL));
     return r;

@@ -968,11 +968,12 @@ constexpr int kWinBytes = 56 * 1024;
 // Denser ones take 256 rows and a thread each (contiguous 128^3: 42.6 us, 46 with
 // 128 rows, 45 with 512, 59 with two threads).
 constexpr int kWinSparse = 5;
-// Long rows: 512 rows to a block from this many entries on, 256 from that many,
-// else 128, and half of that until there are two blocks to an SM.  Larger blocks
-// gather denser windows, smaller ones overlap better (us per apply with 128 / 256 /
-// 512 rows on GB300: 10^6 rows of 20 entries 109 / 116 / 130, 4 * 10^6 510 / 484 /
-// 514, 2^23 1,241 / 1,237 / 1,002).
+// Long rows: 512 rows to a block from this many entries on, 256 from that many in a
+// plan without FP32 values, else 128, and half of that until there are two blocks to
+// an SM.  Larger blocks gather denser windows, smaller ones overlap better (us per
+// apply with 128 / 256 / 512 rows on GB300: 10^6 rows of 20 entries 103 / 107 / 120
+// (FP32 values 101 / 104 / 117), 4 * 10^6 480 / 449 / 491 (405 / 424 / 482), 2^23
+// 1,135 / 1,060 / 948 (839 / 834 / 835)).
 constexpr int64_t kWinLong512 = 120000000, kWinLong256 = 50000000;
 
 // One CTA per block of the staged windows.  The positions of a process's full
@@ -1160,7 +1161,10 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
     int32_t st[4] = {};
     bool fits = false;
     W.long_rows = P->nnz > 12 * n;
-    int rows = !W.long_rows ? 256 : P->nnz >= kWinLong512 ? 512 : P->nnz >= kWinLong256 ? 256 : 128;
+    int rows = !W.long_rows                                ? 256
+               : P->nnz >= kWinLong512                     ? 512
+               : P->nnz >= kWinLong256 && !P->d_val32 ? 256
+                                                           : 128;
     for (; rows >= 32 && !fits; rows /= 2) {
         G.cut.nsub = (int32_t)((max_rows + rows - 1) / rows);
         G.cut.rows = (int32_t)((max_rows + G.cut.nsub - 1) / G.cut.nsub + 31) & ~31;
