@@ -2431,12 +2431,18 @@ static int msg_grid(const napspmv_plan_t *P, int64_t n, int64_t wave)
     return (int)std::max<int64_t>(1, std::min<int64_t>(chunks, g));
 }
 
-// The inter-node messages from their owners to g_recv.
-static SendJob send_job(const napspmv_plan_t *P, bool f32, const void *x, void *grecv, const int *err)
+// The inter-node messages from their owners to g_recv; windows: in the order of
+// the staged windows' receives.
+static const int32_t *send_order(const napspmv_plan_t *P, bool windows)
+{
+    return windows && P->win.d_send ? P->win.d_send : P->lists[L_INTER].d_idx;
+}
+static SendJob send_job(const napspmv_plan_t *P, bool f32, bool windows, const void *x, void *grecv,
+                        const int *err)
 {
     SendJob J{};
     J.x = x;
-    J.j = P->lists[L_INTER].d_idx;
+    J.j = send_order(P, windows);
     J.dst = P->d_xfer_dst;
     J.shift = P->d_xfer_shift;
     J.grecv = grecv;
@@ -2453,7 +2459,7 @@ static int64_t enqueue_send(const napspmv_plan_t *P, const T *x, T *grecv, int *
     if (P->n_gs == 0) return 0;
     SendJobs<1> S{};
     S.n = 1;
-    S.job[0] = send_job(P, sizeof(T) == 4, x, grecv, err);
+    S.job[0] = send_job(P, sizeof(T) == 4, false, x, grecv, err);
     launch_pdl(pdl, k_send<T, T, 1>, S.job[0].blocks, 0, s, S);
     return 1;
 }
@@ -2669,7 +2675,7 @@ static int enqueue_windows(int count, napspmv_plan_t *const *plans, napspmv_ws_t
             // FP32 mode: the next apply reads the FP32 copy only
             float *y32 = f32 && left > 0 ? W->x32[(left - 1) & 1] : nullptr;
             if (f32 && left > 0 && !(keep && left == 1)) y = nullptr;
-            SendJob S = send_job(P, f32, xs, W->grecv, W->err);
+            SendJob S = send_job(P, f32, true, xs, W->grecv, W->err);
             const bool hold = keep && left == 0 && !fill;
             if (hold) {
                 S.state = W->state;
@@ -2718,7 +2724,7 @@ bool runs_on_windows(const napspmv_plan_t *P, int32_t precision)
 }
 SendList send_list(const napspmv_plan_t *P, const napspmv_ws_t *ws)
 {
-    return SendList{P->lists[L_INTER].d_idx, P->d_xfer_dst, P->d_xfer_shift, ws->grecv, ws->err,
+    return SendList{send_order(P, true), P->d_xfer_dst, P->d_xfer_shift, ws->grecv, ws->err,
                     (int32_t)P->n_gs};
 }
 template <int MAXJ>
@@ -2730,7 +2736,7 @@ static int send_jobs(int count, napspmv_plan_t *const *plans, napspmv_ws_t *cons
     int blocks = 0;
     for (int i = 0; i < count; i++) {
         if (plans[i]->n_gs == 0) continue;
-        SendJob J = send_job(plans[i], f32, x[i], ws[i]->grecv, ws[i]->err);
+        SendJob J = send_job(plans[i], f32, true, x[i], ws[i]->grecv, ws[i]->err);
         J.block0 = blocks;
         blocks += J.blocks;
         S.job[S.n++] = J;

@@ -158,6 +158,7 @@ struct WinPart {
     uint16_t *d_col = nullptr;  // window slot of every sliced-row slot
     WinBlock *d_blk = nullptr;
     uint32_t *d_runs = nullptr;
+    int32_t *d_send = nullptr;  // not null: the order of g_send the windows' receives want (order_receives)
 };
 
 }  // namespace nap

@@ -974,7 +974,7 @@ constexpr int kWinSparse = 5;
 // apply with 128 / 256 / 512 rows on GB300: 10^6 rows of 20 entries 103 / 107 / 120
 // (FP32 values 101 / 104 / 117), 4 * 10^6 480 / 449 / 491 (405 / 424 / 482), 2^23
 // 1,135 / 1,060 / 948 (839 / 834 / 835)).
-constexpr int64_t kWinLong512 = 120000000, kWinLong256 = 50000000;
+constexpr int64_t kWinLong512 = 140000000, kWinLong256 = 36000000;
 
 // One CTA per block of the staged windows.  The positions of a process's full
 // window (own rows, b_{l->l}, b_{nl->l}) that the block's rows use are marked in
@@ -1130,12 +1130,114 @@ __global__ void k_widen(const int32_t *in, int64_t n, int64_t *out)  // out[n] =
         out[i] = i < n ? in[i] : 0;
 }
 
+// Far columns: a message's elements are used by one block of rows each and lie far
+// apart in x, sorted by index, and what a block takes of them costs a sector per
+// value in g_recv.  Sent in the order of the blocks instead, a block's share is
+// contiguous.  Messages of which an element has 1.5 users or more on average (near
+// columns) keep their order, for the neighbours in index are what the next rows use;
+// and so do messages with an element in fewer than 16 of x, whose owners' values then
+// share sectors with the index order only.  Us per apply on GB300, FP64, nodes of 2^15
+// rows of 20 entries, a fifth of them far, without / with the order, and an element
+// in how many: 10^6 rows 102.8 / 105.7 (8), 2 * 10^6 215 / 213 (15), 4 * 10^6
+// 449 / 431 (30), 2^23 948 / 900 (64); FP32 values 100.8 / 103.7, 200 / 201, 405 / 399,
+// 839 / 810.
+constexpr int kFarSpan = 16;
+
+// first[p], uses[p] of g_recv position p: the first block that uses it, how many do
+__global__ void k_recv_uses(int64_t nblk, const uint32_t *src, const int64_t *osrc,
+                            const int32_t *nsrc, int32_t *first, int32_t *uses)
+{
+    for (int64_t b = blockIdx.x; b < nblk; b += gridDim.x)
+        for (int k = threadIdx.x; k < nsrc[b]; k += blockDim.x) {
+            const uint32_t s = src[osrc[b] + k];
+            if (!(s & kFromRecv)) continue;
+            atomicMin(&first[s & kIndexMask], (int32_t)b);
+            atomicAdd(&uses[s & kIndexMask], 1);
+        }
+}
+// Sort keys (message, first user) of the elements of g_send, a CTA per message;
+// any: some message is reordered.
+__global__ void k_recv_keys(int64_t n_msg, const int64_t *gs_off, const int32_t *gs_j,
+                            const int32_t *dst,
+                            const int32_t *first, const int32_t *uses, int bits, uint64_t *key,
+                            int32_t *val, int *any)
+{
+    __shared__ unsigned long long all;
+    for (int64_t m = blockIdx.x; m < n_msg; m += gridDim.x) {
+        const int64_t b = gs_off[m], e = gs_off[m + 1];
+        if (threadIdx.x == 0) all = 0;
+        __syncthreads();
+        unsigned long long sum = 0;
+        for (int64_t k = b + threadIdx.x; k < e; k += blockDim.x) sum += uses[dst[k]];
+        atomicAdd(&all, sum);
+        __syncthreads();
+        const bool far = e > b && 2 * all < 3 * (unsigned long long)(e - b) &&
+                         gs_j[e - 1] - gs_j[b] >= kFarSpan * (e - b);
+        if (far && threadIdx.x == 0) *any = 1;
+        for (int64_t k = b + threadIdx.x; k < e; k += blockDim.x) {
+            key[k] = ((uint64_t)m << bits) | (uint64_t)(far ? min(first[dst[k]], (1 << bits) - 1) : 0);
+            val[k] = (int32_t)k;
+        }
+        __syncthreads();
+    }
+}
+// Element k of g_send becomes the former element from[k]; its place in g_recv moves along.
+__global__ void k_recv_order(int64_t n_gs, const int32_t *from, const int32_t *gs_j,
+                             const int32_t *dst, int32_t *send, int32_t *place)
+{
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n_gs;
+         k += (int64_t)gridDim.x * blockDim.x) {
+        send[k] = gs_j[from[k]];
+        place[dst[from[k]]] = dst[k];
+    }
+}
+__global__ void k_recv_move(int64_t n, const int32_t *place, uint32_t *src)
+{
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
+         k += (int64_t)gridDim.x * blockDim.x)
+        if (src[k] & kFromRecv) src[k] = kFromRecv | (uint32_t)place[src[k] & kIndexMask];
+}
+// The order in which g_send suits the windows, and their sources moved to it;
+// null: the messages stay as they are.
+int32_t *order_receives(napspmv_plan_t *P, Cub &cb, int64_t nblk, const int32_t *nsrc,
+                        const int64_t *osrc, uint32_t *src, int64_t total, const int64_t *gs_off,
+                        int64_t n_msg)
+{
+    const int64_t n = P->n_gs;
+    if (n == 0) return nullptr;
+    dvec<int32_t> first(n), uses(n), val(n), val2(n);
+    dvec<uint64_t> key(n), key2(n);
+    dvec<int> any(1);
+    const int bits = bits_for(nblk);
+    CK(cudaMemset(first.p, 0x7f, sizeof(int32_t) * n));
+    CK(cudaMemset(uses.p, 0, sizeof(int32_t) * n));
+    CK(cudaMemset(any.p, 0, sizeof(int)));
+    k_recv_uses<<<(int)std::min<int64_t>(nblk, 1 << 20), 256>>>(nblk, src, osrc, nsrc, first.p,
+                                                                uses.p);
+    CK(cudaGetLastError());
+    k_recv_keys<<<(int)std::min<int64_t>(n_msg, 1 << 20), 256>>>(
+        n_msg, gs_off, P->lists[L_INTER].d_idx, P->d_xfer_dst, first.p, uses.p, bits, key.p, val.p, any.p);
+    CK(cudaGetLastError());
+    int some = 0;
+    CK(cudaMemcpy(&some, any.p, sizeof(int), cudaMemcpyDeviceToHost));
+    if (!some) return nullptr;
+    cb.sort_pairs(key, key2, val, val2, n, bits + bits_for(n_msg));
+    int32_t *send = nullptr;
+    CK(device_alloc(&send, sizeof(int32_t) * n));
+    k_recv_order<<<blocks_for(n), 256>>>(n, val.p, P->lists[L_INTER].d_idx, P->d_xfer_dst, send,
+                                         first.p);
+    CK(cudaGetLastError());
+    k_recv_move<<<blocks_for(total), 256>>>(total, first.p, src);
+    CK(cudaGetLastError());
+    return send;
+}
+
 // Chooses the block size of the staged windows and builds them with the whole
 // matrix's sliced rows.  No windows (the sliced rows then keep their own): a
 // plan of composed gathers, a row of more than kSellLong entries, fewer than 64
 // rows per process, or blocks that do not fit the shared memory.
 void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *bll_ptr,
-                   const int32_t *bnl_ptr)
+                   const int32_t *bnl_ptr, const int64_t *gs_off, int64_t n_msg)
 {
     WinPart &W = P->win;
     const int64_t n = P->n;
@@ -1161,10 +1263,10 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
     int32_t st[4] = {};
     bool fits = false;
     W.long_rows = P->nnz > 12 * n;
-    int rows = !W.long_rows                                ? 256
-               : P->nnz >= kWinLong512                     ? 512
+    int rows = !W.long_rows                           ? 256
+               : P->nnz >= kWinLong512                ? 512
                : P->nnz >= kWinLong256 && !P->d_val32 ? 256
-                                                           : 128;
+                                                      : 128;
     for (; rows >= 32 && !fits; rows /= 2) {
         G.cut.nsub = (int32_t)((max_rows + rows - 1) / rows);
         G.cut.rows = (int32_t)((max_rows + G.cut.nsub - 1) / G.cut.nsub + 31) & ~31;
@@ -1227,6 +1329,7 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
         k_win_blocks<<<bgrid, 256>>>(nblk, off.p, off.p + nblk + 1, nsrc.p, nsrc.p, osrc.p, 1,
                                      W.d_blk);
         CK(cudaGetLastError());
+        W.d_send = order_receives(P, cb, nblk, nsrc.p, osrc.p, src.p, total, gs_off, n_msg);
         W.d_runs = src.release();
     } else {
         const int wgrid = blocks_for(32 * nblk);
@@ -1699,7 +1802,7 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
     CK(cudaDeviceSynchronize());
 
     // sliced-row copies of the whole matrix and of its two split parts
-    build_windows(P, cb, part, d_bll_ptr.p, d_bnl_ptr.p);
+    build_windows(P, cb, part, d_bll_ptr.p, d_bnl_ptr.p, d_gs_off.p, NM);
     build_sell(P, cb, 1, P->d_rowptrL, P->d_colL, P->d_valL, P->d_val32L, part);
     build_sell(P, cb, 2, P->d_rowptrR, P->d_colR, P->d_valR, P->d_val32R, part);
     CK(cudaDeviceSynchronize());
@@ -1891,7 +1994,7 @@ void plan_free(napspmv_plan_t *P)
         for (void *p : sp)
             if (p) cudaFree(p);
     }
-    void *wp[] = {P->win.d_col, P->win.d_blk, P->win.d_runs};
+    void *wp[] = {P->win.d_col, P->win.d_blk, P->win.d_runs, P->win.d_send};
     for (void *p : wp)
         if (p) cudaFree(p);
     delete P;

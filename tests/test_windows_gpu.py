@@ -76,6 +76,41 @@ def test_long_rows_bits(rows, n_p, ppn, near, flags):
                 assert np.array_equal(a, b), (prec, reps)
 
 
+def near_and_far(n, near, far, seed):
+    """16 columns a row within `near` of the diagonal and `far` anywhere."""
+    rng = np.random.default_rng(seed)
+    i = np.arange(n)[:, None]
+    cols = np.concatenate([(i + rng.integers(-near, near + 1, (n, 16))) % n, rng.integers(0, n, (n, far))], 1)
+    key = np.unique(i * n + cols)
+    row_ptr = np.searchsorted(key, np.arange(n + 1) * n)
+    return I.CSR(row_ptr.astype(np.int64), (key % n).astype(np.int32), rng.uniform(-1, 1, len(key)))
+
+
+@pytest.mark.parametrize("flags", [0, nap.MAP_SPLIT])
+@pytest.mark.parametrize("rows,n_p,ppn,near,far", [(1000, 30, 4, 300, 3), (257, 64, 2, 5, 1), (300, 80, 1, 700, 1)])
+def test_far_columns_in_block_order(rows, n_p, ppn, near, far, flags):
+    """Messages whose elements have one user each and lie 16 apart or more are sent in
+    another order (no message of the first case, the far ones of the others); the other
+    engines, which read the same buffer, and the step that follows either kind of apply
+    do not notice."""
+    A = near_and_far(rows * n_p + 1, near, far, rows)
+    plan = gpu_plan(A, n_p, ppn, nap.F32_VALUES | flags)
+    vd = torch.from_numpy(I.vector(A.n, rows)).cuda()
+    for prec in (nap.PREC_F64, nap.PREC_F32):
+        for reps in (1, 2, 3):
+            a, b = both(plan, vd, reps, 0.5, prec)
+            assert np.array_equal(a, b), (prec, reps)
+        steps = []
+        for first in ({}, TILES):
+            for then in ({}, TILES):
+                w, z = torch.empty_like(vd), torch.full_like(vd, float("nan"))
+                nap.napspmv_apply_ex(plan, vd, w, 1, 1.0, nap.make_opts(precision=prec, **first))
+                nap.napspmv_spmv_step(plan, vd, z, 1.0, nap.make_opts(precision=prec, **then))
+                assert nap.napspmv_status(plan) == 0
+                steps.append(z.cpu().numpy().view(np.int64))
+        assert all(np.array_equal(steps[0], z) for z in steps), prec
+
+
 @pytest.mark.parametrize("make,n_p,ppn", [(lambda: I.poisson2d(47), 7, 3), (lambda: I.poisson3d(17), 5, 2),
                                           (lambda: I.aniso_q1(40), 9, 4)])
 @pytest.mark.parametrize("flags", [0, nap.PARTITION_STRIDED])
