@@ -647,13 +647,18 @@ __global__ void __launch_bounds__(NT)
         step_gather<false, 8, T, true>(bnl, grecv, src, b, min(b + per, n), threadIdx.x);
     griddep_done();
 }
-// FP32 copy of an input vector (first apply of a chain in FP32 mode)
-__global__ void __launch_bounds__(NT) k_to_f32(const double *v, float *v32, int64_t n, const int *err)
+// FP32 copy of an input vector (first apply of a chain in FP32 mode); keep, if not
+// null, gets the vector itself
+__global__ void __launch_bounds__(NT)
+    k_to_f32(const double *v, float *v32, double *keep, int64_t n, const int *err)
 {
     griddep_wait();
     if (*(volatile const int *)err) return;
-    for (int64_t i = blockIdx.x * (int64_t)NT + threadIdx.x; i < n; i += (int64_t)gridDim.x * NT)
-        v32[i] = d2f_rn(ld_stream_f64(v + i));
+    for (int64_t i = blockIdx.x * (int64_t)NT + threadIdx.x; i < n; i += (int64_t)gridDim.x * NT) {
+        const double d = ld_stream_f64(v + i);
+        v32[i] = d2f_rn(d);
+        if (keep) keep[i] = d;
+    }
     griddep_done();
 }
 template <int V, bool F32, int MODE = kFull>
@@ -1373,15 +1378,15 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
 }
 constexpr int kWinLongU = 4;  // entries per step of a row, two steps in flight
 constexpr int kWinLongG = 4;  // window values in flight per thread
-template <bool F32, class XS, bool STEP>
+template <bool F32, bool STEP>
 __global__ void __launch_bounds__(1024, 1)
     k_window_long(const __grid_constant__ WinJob J, int nblk)
 {
     using XT = typename std::conditional<F32, float, double>::type;
     constexpr int U = kWinLongU, G = kWinLongG;
     const WinView &S = J.S;
-    const XS *x = static_cast<const XS *>(J.x), *l = static_cast<const XS *>(J.l);
-    const XT *g = static_cast<const XT *>(J.g);
+    const XT *x = static_cast<const XT *>(J.x), *g = static_cast<const XT *>(J.g),
+             *l = static_cast<const XT *>(J.l);
     double *y = J.y;
     float *y32 = J.y32;
     const Scale sc = J.sc;
@@ -1433,7 +1438,7 @@ __global__ void __launch_bounds__(1024, 1)
 #pragma unroll
                 for (int u = 0; u < G; u++) {
                     if (k0 + u * half >= m) continue;
-                    v[u] = window_value<XT, XS, STEP>(ix[u], x, g, l);
+                    v[u] = window_value<XT, XT, STEP>(ix[u], x, g, l);
                 }
                 if (k0 + G * half < m) {
                     load(k0 + G * half);
@@ -2521,12 +2526,10 @@ static WinKernel<MAXJ> pick_window(int source, bool step)
                          : k_window<true, double, false, MAXJ>;
 }
 using WinLongKernel = void (*)(const WinJob, int);
-static WinLongKernel pick_window_long(int source, bool step)
+static WinLongKernel pick_window_long(bool f32, bool step)
 {
-    if (step) return source ? k_window_long<true, double, true> : k_window_long<false, double, true>;
-    return source == 0   ? k_window_long<false, double, false>
-           : source == 1 ? k_window_long<true, float, false>
-                         : k_window_long<true, double, false>;
+    if (step) return f32 ? k_window_long<true, true> : k_window_long<false, true>;
+    return f32 ? k_window_long<true, false> : k_window_long<false, false>;
 }
 int window_bytes(int64_t srcs, int64_t slots, int64_t words, int vb)
 {
@@ -2656,6 +2659,11 @@ static int enqueue_windows(int count, napspmv_plan_t *const *plans, napspmv_ws_t
 {
     constexpr bool f32 = sizeof(T) == 4;
     const bool fill32 = f32 && count == 1 && !o.batch;
+    // Long rows take a value about ten times from all over x: FP32 copies of x are made
+    // first, where the windows of short rows, which take it about once, round FP64
+    // sources (one FP32 apply of 20-entry rows, us on GB300: 3 * 10^5 rows 40.1 against
+    // 43.1 with FP64 sources, 10^6 102 against 126, 3 * 10^6 303 against 376).
+    const bool convert = f32 && plans[0]->win.long_rows;
     int kmax = 0;
     for (int i = 0; i < count; i++) kmax = std::max(kmax, reps[i]);
     int64_t nk = 0;
@@ -2671,15 +2679,22 @@ static int enqueue_windows(int count, napspmv_plan_t *const *plans, napspmv_ws_t
             const int left = reps[i] - 1 - k;  // applies after this one
             const double *x = (k == 0) ? v[i] : ((left & 1) ? w[i] : W->xtmp);
             double *y = (left & 1) ? W->xtmp : w[i];
-            const void *xs = f32 && k > 0 ? (const void *)W->x32[left & 1] : (const void *)x;
+            const void *xs = f32 && (k > 0 || convert) ? (const void *)W->x32[left & 1] : (const void *)x;
             // FP32 mode: the next apply reads the FP32 copy only
             float *y32 = f32 && left > 0 ? W->x32[(left - 1) & 1] : nullptr;
             if (f32 && left > 0 && !(keep && left == 1)) y = nullptr;
             SendJob S = send_job(P, f32, true, xs, W->grecv, W->err);
             const bool hold = keep && left == 0 && !fill;
+            if (convert && k == 0) {
+                const int g = (int)std::max<int64_t>(1, std::min<int64_t>((P->n + NT * 8 - 1) / (NT * 8),
+                                                                          (int64_t)P->num_sms * 8));
+                launch_pdl(true, k_to_f32, g, 0, s, x, W->x32[left & 1],
+                           hold ? W->xtmp : (double *)nullptr, (int64_t)P->n, (const int *)W->err);
+                nk++;
+            }
             if (hold) {
                 S.state = W->state;
-                S.keep = k == 0 ? W->xtmp : nullptr;
+                S.keep = k == 0 && !convert ? W->xtmp : nullptr;
                 S.blocks += S.keep ? (int)std::min<int64_t>((P->n + 8 * NT - 1) / (8 * NT),
                                                             4 * (int64_t)P->num_sms)
                                    : 1;
@@ -2701,14 +2716,14 @@ static int enqueue_windows(int count, napspmv_plan_t *const *plans, napspmv_ws_t
         sends.n = ns;
         if (ns) {
             if constexpr (f32) {
-                if (k > 0) launch_pdl(true, k_send<T, float, MAXJ>, blocks, 0, s, sends);
+                if (k > 0 || convert) launch_pdl(true, k_send<T, float, MAXJ>, blocks, 0, s, sends);
                 else launch_pdl(true, k_send<T, double, MAXJ>, blocks, 0, s, sends);
             } else {
                 launch_pdl(true, k_send<T, double, MAXJ>, blocks, 0, s, sends);
             }
             nk++;
         }
-        if (int rc = window_launch<MAXJ>(nw, wp, wins, !f32 ? 0 : k > 0 ? 1 : 2, false, o, s)) return rc;
+        if (int rc = window_launch<MAXJ>(nw, wp, wins, !f32 ? 0 : k > 0 || convert ? 1 : 2, false, o, s)) return rc;
         nk++;
         NAP_CUDA(cudaGetLastError());
     }
@@ -2803,8 +2818,8 @@ static int enqueue_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, 
     const bool f32 = o.precision == NAPSPMV_PREC_F32;
     int64_t nk = 0;
     if (f32) {
-        launch_pdl(!overlap, k_to_f32, grid(P->n), 0, s, v, ws->x32[0], (int64_t)P->n,
-                   (const int *)ws->err);
+        launch_pdl(!overlap, k_to_f32, grid(P->n), 0, s, v, ws->x32[0], (double *)nullptr,
+                   (int64_t)P->n, (const int *)ws->err);
         nk++;
     }
     for (int k = 0; k < reps; k++) {
@@ -3259,12 +3274,29 @@ extern "C" int napspmv_spmv_step(napspmv_plan_t *P, napspmv_ws_t *ws, const doub
         return NAPSPMV_ERR_STATE;
     }
     const cudaStream_t st = (cudaStream_t)stream;
+    auto to_f32 = [&](const double *src, float *dst) {
+        const int g = (int)std::max<int64_t>(1, std::min<int64_t>((P->n + NT - 1) / NT,
+                                                                  (int64_t)P->num_sms * 8));
+        k_to_f32<<<g, NT, 0, st>>>(src, dst, nullptr, P->n, W->err);
+        count_launch(1);
+    };
     if (o.window && W->recv_vector && !W->captured && W->recv_f32 == f32) {
-        // on the windows: on-node receives from the kept vector, off-node from g_recv
+        // on the windows: on-node receives from the kept vector, off-node from g_recv.
+        // It receives again what an apply that filled the buffers had received: a step
+        // alone on 10^6 rows of 20 entries takes 88 us (73 from filled buffers), an
+        // apply and a step 188 (222).
+        const void *x = v, *l = W->xtmp;
+        const bool convert = f32 && P->win.long_rows;  // as enqueue_windows
+        if (convert) {
+            to_f32(v, W->x32[0]);
+            to_f32(W->xtmp, W->x32[1]);
+            x = W->x32[0];
+            l = W->x32[1];
+        }
         WinJobs<1> jobs{};
-        jobs.job[0] = window_job(P, W, v, W->xtmp, w, nullptr, scale);
+        jobs.job[0] = window_job(P, W, x, l, w, nullptr, scale);
         const napspmv_plan_t *pl[1] = {P};
-        if ((rc = window_launch<1>(1, pl, jobs, f32 ? 2 : 0, true, o, st))) return rc;
+        if ((rc = window_launch<1>(1, pl, jobs, convert ? 1 : f32 ? 2 : 0, true, o, st))) return rc;
         count_launch(1);
     } else {
         if (W->recv_vector || W->captured) {
@@ -3279,15 +3311,12 @@ extern "C" int napspmv_spmv_step(napspmv_plan_t *P, napspmv_ws_t *ws, const doub
         SpmvLaunch L;
         if ((rc = spmv_launch(P, o, kFull, L))) return rc;
         if (f32) {
-            const int g = (int)std::max<int64_t>(1, std::min<int64_t>((P->n + NT - 1) / NT,
-                                                                      (int64_t)P->num_sms * 8));
-            k_to_f32<<<g, NT, 0, st>>>(v, W->x32[0], P->n, W->err);
+            to_f32(v, W->x32[0]);
             spmv_run(L, W->x32[0], W, w, nullptr, scale, o.stages, st, pdl);
-            count_launch(2);
         } else {
             spmv_run(L, v, W, w, nullptr, scale, o.stages, st, pdl);
-            count_launch(1);
         }
+        count_launch(1);
     }
     NAP_CUDA(cudaGetLastError());
     if (cur != P->device) cudaSetDevice(cur);
