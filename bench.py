@@ -149,7 +149,8 @@ def ncu_record(workload, what):
 
 
 # kernels of an apply and of the SpMV step, as ncu names them
-_APPLY_KERNELS = re.compile(r"k_gather2|k_pack|k_transfer|k_unpack|k_spmv|k_to_f32|k_fused")
+_APPLY_KERNELS = re.compile(r"k_gather2|k_pack|k_transfer|k_unpack|k_spmv|k_to_f32|k_fused|"
+                            r"k_send|k_window|k_receives")
 
 
 def ncu_launches(csv_path):
@@ -172,11 +173,14 @@ def ncu_launches(csv_path):
 def ncu_summary(csv_path, nsteps=2, per_step=1):
     """DRAM record of one `--profile-spmv nsteps` run: the kernels after the
     last plan-build kernel are one apply, then nsteps SpMV steps of per_step
-    launches each (FP32 values: the FP32 copy of x, then the SpMV)."""
+    launches each (FP32 values: the FP32 copy of x, then the SpMV; one launch on the
+    staged windows)."""
     items = []
     for name, m in ncu_launches(csv_path):
         short = name.split("(")[0].replace("void ", "").replace("nap::", "")
         items.append((short.replace("<unnamed>::", ""), m))
+    if "k_window" in items[-1][0]:
+        per_step = 1
     first = max(j for j, (n, _) in enumerate(items) if not _APPLY_KERNELS.search(n))
     rest = items[first + 1:]
     steps, apply_ = rest[len(rest) - nsteps * per_step:], rest[:len(rest) - nsteps * per_step]
@@ -311,14 +315,14 @@ def run_reference(args):
     ot.close()
     val = B * args.steps / el / 1e9
     line = {
-        "impl": "reference", "metric": METRIC, "value": round(val, 3), "unit": "GB/s",
+        "impl": "reference", "metric": METRIC, "value": round(val, 6), "unit": "GB/s",
         "n_gpus": ws, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": round(el / args.steps * 1e3, 3), "ms_per_apply": round(el / args.steps * 1e3, 3),
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",
         "data": "synthetic",
         "config": {"workload": w.name, "n": A.n, "nnz": A.nnz, "n_p": w.n_p, "ppn": w.ppn,
                    "partition": "contiguous", "gathers": "literal", "applies_per_step": 1},
-        "cpu_baseline": {"value": round(val, 3), "unit": "GB/s", "cores": T, "kind": "oracle",
+        "cpu_baseline": {"value": round(val, 6), "unit": "GB/s", "cores": T, "kind": "oracle",
                          "sample": f"{args.steps} plain FP64 CSR SpMVs of the full matrix on {T} "
                                    "threads (row blocks of equal stored entries); bytes counted as "
                                    "for the GPU apply, so the ratio of the two values is the "
@@ -326,7 +330,7 @@ def run_reference(args):
                          "ms_per_apply": round(el / args.steps * 1e3, 3),
                          "plan_stats": src,
                          "plan_build_s": None if plan_s is None else round(plan_s, 3)},
-        "e2e": {"value": round(val, 3), "unit": "GB/s", "h2d_bytes_per_step": 0,
+        "e2e": {"value": round(val, 6), "unit": "GB/s", "h2d_bytes_per_step": 0,
                 "d2h_bytes_per_step": 0},
     }
     print(json.dumps(line), flush=True)
@@ -529,6 +533,9 @@ def measure(nap, torch, dev, args, cfg, precision, reps, steps, warmup, ws=1, wi
             "l2": "inputs larger than L2 (129 MB): each apply streams the matrix "
                   f"({(12 if not f32 else 8) * A.nnz / 1e6:.0f} MB of columns and values); "
                   "not flushed between steps"}
+    # messages and windows: two launches per apply (FP32 copies of x: one per step more)
+    cfgd["staged_windows"] = args.gathers == "literal" and launches in (
+        2 * reps * steps, (2 * reps + 1) * steps)
     what = f"{precision}|{cfgd['engine']}|{cfgd['pipeline']}"
     rec = ncu_record(w.name, what)
     spmv_traffic = None if rec is None else rec.get("spmv_step_bytes")
@@ -549,7 +556,7 @@ def measure(nap, torch, dev, args, cfg, precision, reps, steps, warmup, ws=1, wi
                                "on the benchmark stream after the timed region" + (
                                    "; inside it the overlapped engine runs the same rows as a "
                                    "local and a remote launch" if engine == nap.ENGINE_OVERLAP
-                                   else "; inside it the phased engine runs the same launch"
+                                   else "; inside it the apply runs the same launch"
                                    if engine == nap.ENGINE_PHASED
                                    else "; inside it the fused kernel's last level sums the "
                                    "same rows"),
@@ -557,7 +564,9 @@ def measure(nap, torch, dev, args, cfg, precision, reps, steps, warmup, ws=1, wi
         "step_roofline": {"bound": "hbm", "achieved": round(achieved, 3), "peak": peak,
                           "frac": round(achieved / peak, 4),
                           "frac_of_nominal_8tbs": round(achieved / NOMINAL_GBS, 4),
-                          "what": "whole apply (message steps + SpMV), algorithmic bytes"},
+                          "what": "whole apply (message steps + SpMV), algorithmic bytes of the "
+                                  "step-by-step exchange; the staged windows move each "
+                                  "message once, so its DRAM bytes (apply_dram) are fewer"},
         "gpu_launches": int(launches),
         "clocks": clocks,
         "plan": {"gpu_plan_ms": round(plan_ms, 2), "std_msgs": st["std_msgs"],

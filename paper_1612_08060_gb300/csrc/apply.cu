@@ -15,8 +15,9 @@
 //            one pass over each row, blocks in that order)
 //
 // SpMV pipelines: sliced rows (rows sorted by length, 32 to a chunk,
-// column-major, one lane per row, no shared-memory stage; the default for rows
-// of more than 12 entries and the fused engine's), and CTA or warp row tiles.
+// column-major, one lane per row, no shared-memory stage; the rows of the fused
+// engine and of plans without windows whose rows have more than 12 entries), and
+// CTA or warp row tiles.
 // A row tile: one thread copies the tile's row-pointer, column and value slices
 // into a shared-memory stage with bulk asynchronous copies counted on an
 // mbarrier; the next tile's copy overlaps the current tile.  Each row is then
@@ -35,7 +36,7 @@
 //       remote pass continues each row's FMA chain from the local partial.
 //       Where remote rows are gather-heavy, the remote pass stages each
 //       process's receive buffers in shared memory.
-//   phased (default for longer rows)  one kernel per phase per apply with the
+//   phased (for longer rows without windows)  one kernel per phase per apply with the
 //       single-pass SpMV.
 //   fused    one persistent, cooperative launch for all phases and applies of
 //       one or more jobs, in levels separated by bounded grid barriers (see
@@ -1361,14 +1362,14 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 // Bound by the SM's load path, which takes a 32-byte sector per gathered value
 // where the sources are sparse (about 9.4 TB/s over the chip; the sums' shared
 // loads queue behind them) and then by the FP64 pipe (40% busy).  Per apply on
-// GB300, FP64 values, chains of 10: 940 us for the 2^23-row banded matrix, where
+// GB300, FP64 values, chains of 10: 896 us for the 2^23-row banded matrix, where
 // gathers into b_{l->l} and b_{nl->l} and the sliced-row pass take 1,193 (and
-// 1,436 with the message hops one by one), 449 against 545 at 4 * 10^6 rows, 102
-// against 129 at 10^6, 10.4 against 19.2 at 5 * 10^4; FP32 values 827 against 879,
-// 405 against 427, 99 against 111 and 12.3 against 20.  Chunks dealt by length
-// alone, longest to the first warp, took 1,002 us at 2^23 rows (FP64), and then 8
-// values in flight per thread 1,072, 2 1,028; 6 entries a step 1,109; no L2 request
-// 1,031; entries bulk-copied to shared memory as well (256-row blocks, 8 summing
+// 1,436 with the message hops one by one), 429 against 545 at 4 * 10^6 rows, 102
+// against 129 at 10^6, 10.4 against 19.2 at 5 * 10^4; FP32 values 806 against 879,
+// 396 against 427, 99 against 111 and 12.3 against 20.  With far messages in index
+// order 2^23 rows took 940 us, and with chunks dealt by length alone, longest to the
+// first warp, 1,002; of that form 8 values in flight per thread 1,072, 2 1,028; 6
+// entries a step 1,109; no L2 request 1,031; entries bulk-copied to shared memory as well (256-row blocks, 8 summing
 // warps) 1,784, since every shared load then waits behind the gathers.  Four FP32
 // products tested and widened at once: no gain.
 // Start bringing [p, p + bytes) into L2 (one thread; 16-byte multiples).
