@@ -173,16 +173,17 @@ def ncu_launches(csv_path):
 def ncu_summary(csv_path, nsteps=2, per_step=1):
     """DRAM record of one `--profile-spmv nsteps` run: the kernels after the
     last plan-build kernel are one apply, then nsteps SpMV steps of per_step
-    launches each (FP32 values: the FP32 copy of x, then the SpMV; one launch on the
-    staged windows)."""
+    launches each (FP32 values: the FP32 copy of x, then the SpMV; on the staged
+    windows, whose first launch ends the apply, as many as there are)."""
     items = []
     for name, m in ncu_launches(csv_path):
         short = name.split("(")[0].replace("void ", "").replace("nap::", "")
         items.append((short.replace("<unnamed>::", ""), m))
-    if "k_window" in items[-1][0]:
-        per_step = 1
     first = max(j for j, (n, _) in enumerate(items) if not _APPLY_KERNELS.search(n))
     rest = items[first + 1:]
+    if "k_window" in rest[-1][0]:
+        done = next(j for j, (n, _) in enumerate(rest) if "k_window" in n)
+        per_step = (len(rest) - done - 1) // nsteps
     steps, apply_ = rest[len(rest) - nsteps * per_step:], rest[:len(rest) - nsteps * per_step]
     b = lambda m: m.get("dram__bytes_read.sum", 0) + m.get("dram__bytes_write.sum", 0)  # noqa: E731
     t = lambda m: m.get("gpu__time_duration.sum", 0) / 1e3  # noqa: E731

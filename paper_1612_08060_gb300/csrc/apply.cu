@@ -1557,10 +1557,11 @@ __global__ void __launch_bounds__(1024, 1)
 // owner's x[j[k]] to its place in g_recv.  A warp moves groups of kSendGroup
 // elements, two at a time; within one message the places are consecutive, so a
 // group inside a message needs one number, its shift (kMixed: it crosses
-// messages, and every element's place is read).  Bound by the SM's sector loads: a gathered 8-byte value
-// costs up to a 32-byte sector.  Against the gather, pack and transfer kernels, 35.6 us
-// of 128^3, 9.3 us (GB300, cold, on their own); 426 us of the 2^23-row banded
-// matrix, 162.
+// messages, and every element's place is read).  Bound by the SM's sector loads: a
+// gathered 8-byte value costs up to a 32-byte sector.  Against the gather, pack and
+// transfer kernels, 35.6 us of 128^3, 9.3 us (GB300, cold, on their own); 426 us of the
+// 2^23-row banded matrix, 162 in index order and 205 with the far messages in the order
+// that the windows gain from.
 // The copy of x that a later napspmv_spmv_step takes the on-node receives from
 // (SendJob::keep) is made by further CTAs of the same launch.
 constexpr int kSendWarps = NT / 32;
