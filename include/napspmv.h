@@ -283,9 +283,9 @@ int napspmv_apply_host(napspmv_plan_t *P, const double *v_host, double *w_host, 
  * launches where `opts` leaves the path open; every other entry runs on the
  * fused engine, whatever engine `opts` names.  Options: each entry resolves
  * the fields of `opts` left 0 (or opts NULL) against its own plan's
- * defaults.  Entries whose resolved launch options agree share one fused
- * launch; the launches are issued on `stream` in order of each option set's
- * first entry.  Each entry's result is bit-identical to napspmv_apply_ex of
+ * defaults.  Entries whose resolved launch options agree (on the windows:
+ * precision and ctas_per_sm) share their launches; these are issued on `stream`
+ * in order of each option set's first entry.  Each entry's result is bit-identical to napspmv_apply_ex of
  * its plan on the fused engine with its resolved options, whatever else is
  * in the batch.  Errors stay per entry: an entry whose wait times out sets
  * its workspace's error flag (napspmv_ws_status) and its remaining work is

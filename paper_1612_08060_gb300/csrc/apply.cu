@@ -2996,6 +2996,37 @@ static bool same_launch(const napspmv_opts &a, const napspmv_opts &b)
            a.debug_stall == b.debug_stall;
 }
 
+// The same for the staged windows' shared launches.
+static bool same_windows(const napspmv_opts &a, const napspmv_opts &b)
+{
+    return a.precision == b.precision && a.ctas_per_sm == b.ctas_per_sm;
+}
+
+// Entries of a batch that share the staged windows' launches.
+static int launch_windows(int count, napspmv_plan_t *const *plans, napspmv_ws_t *const *ws,
+                          const double *const *v, double *const *w, const int32_t *reps,
+                          const double *scale, const Opts &o, bool keep, cudaStream_t s)
+{
+    const bool f32 = o.precision == NAPSPMV_PREC_F32;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    NAP_CUDA(cudaStreamIsCapturing(s, &cs));
+    const bool capturing = cs != cudaStreamCaptureStatusNone;
+    bool fill = capturing;
+    for (int i = 0; i < count; i++) fill = fill || ws[i]->captured;
+    for (int i = 0; i < count; i++) {
+        ws[i]->recv_f32 = f32;
+        if (!keep) continue;
+        if (int rc = note_receives(ws[i], false, !fill, capturing, s)) return rc;
+    }
+    int64_t nk = 0;
+    const int rc = f32 ? enqueue_windows<float, 64>(count, plans, ws, v, w, reps, scale, o, keep,
+                                                    fill, s, &nk)
+                       : enqueue_windows<double, 64>(count, plans, ws, v, w, reps, scale, o, keep,
+                                                     fill, s, &nk);
+    if (!rc) count_launch(nk);
+    return rc;
+}
+
 int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const *ws,
                 const double *const *v, double *const *w, const int32_t *reps, const double *scale,
                 const napspmv_opts *opts, cudaStream_t s, bool keep, bool as_batch)
@@ -3063,50 +3094,11 @@ int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const
         else
             rc = launch_fused<1>(1, plans, ws, v, w, reps, scale, o, s);
     } else if (!rc) {
-        // one fused launch per distinct launch option set, in order of first
-        // appearance; an entry's bits are those of its plan applied alone on the
-        // fused engine with its resolved options, whatever else is in the batch
+        // one set of launches per path (windows or fused) and distinct launch option
+        // set, in order of first appearance; an entry's bits are those of its plan
+        // applied alone on the fused engine with its resolved options, whatever else
+        // is in the batch
         bool done[64] = {};
-        {
-            napspmv_plan_t *gp[64];
-            napspmv_ws_t *gw[64];
-            const double *gv[64];
-            double *gx[64];
-            int32_t gr[64];
-            double gs[64];
-            int m = 0, first = -1;
-            bool fill = false;
-            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-            cudaStreamIsCapturing(s, &cs);
-            const bool capturing = cs != cudaStreamCaptureStatusNone;
-            for (int j = 0; j < count; j++) {
-                if (!oi[j].window) continue;
-                napspmv_ws_t *W = ws && ws[j] ? ws[j] : plans[j]->ws;
-                fill = fill || W->captured || capturing;
-            }
-            for (int j = 0; j < count && !rc; j++) {
-                if (!oi[j].window) continue;
-                done[j] = true;
-                if (first < 0) first = j;
-                gp[m] = plans[j];
-                gw[m] = ws && ws[j] ? ws[j] : plans[j]->ws;
-                gv[m] = v[j];
-                gx[m] = w[j];
-                gr[m] = reps[j];
-                gs[m] = scale ? scale[j] : 1.0;
-                gw[m]->recv_f32 = oi[j].precision == NAPSPMV_PREC_F32;
-                if (keep) rc = note_receives(gw[m], false, !fill, capturing, s);
-                m++;
-            }
-            int64_t nk = 0;
-            if (m && !rc)
-                rc = oi[first].precision == NAPSPMV_PREC_F32
-                         ? enqueue_windows<float, 64>(m, gp, gw, gv, gx, gr, gs, oi[first], keep,
-                                                      fill, s, &nk)
-                         : enqueue_windows<double, 64>(m, gp, gw, gv, gx, gr, gs, oi[first], keep,
-                                                       fill, s, &nk);
-            if (m && !rc) count_launch(nk);
-        }
         for (int i = 0; i < count && !rc; i++) {
             if (done[i]) continue;
             napspmv_plan_t *gp[64];
@@ -3116,8 +3108,11 @@ int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const
             int32_t gr[64];
             double gs[64];
             int m = 0;
+            const bool window = oi[i].window;
             for (int j = i; j < count; j++) {
-                if (done[j] || !same_launch(oi[i], oi[j])) continue;
+                if (done[j] || oi[j].window != window ||
+                    !(window ? same_windows(oi[i], oi[j]) : same_launch(oi[i], oi[j])))
+                    continue;
                 done[j] = true;
                 gp[m] = plans[j];
                 gw[m] = ws && ws[j] ? ws[j] : plans[j]->ws;
@@ -3127,8 +3122,9 @@ int apply_batch(int32_t count, napspmv_plan_t *const *plans, napspmv_ws_t *const
                 gs[m] = scale ? scale[j] : 1.0;
                 m++;
             }
-            rc = m == 1 ? launch_fused<1>(1, gp, gw, gv, gx, gr, gs, oi[i], s)
-                        : launch_fused<64>(m, gp, gw, gv, gx, gr, gs, oi[i], s);
+            rc = window   ? launch_windows(m, gp, gw, gv, gx, gr, gs, oi[i], keep, s)
+                 : m == 1 ? launch_fused<1>(1, gp, gw, gv, gx, gr, gs, oi[i], s)
+                          : launch_fused<64>(m, gp, gw, gv, gx, gr, gs, oi[i], s);
         }
     }
     if (cur != P0->device) cudaSetDevice(cur);
