@@ -1,5 +1,6 @@
 """Which path a call takes around the staged windows, and that it answers the same on every
 path: batches of plans with different default options."""
+import numpy as np
 import pytest
 import torch
 
