@@ -617,15 +617,24 @@ __device__ __forceinline__ bool staged_tile(const Item &it, int cap)
     return it.kind == kSpmv && it.k1 - it.k0 <= cap;
 }
 
+// Sticky error of the kernels that load their indices before the wait: no work until
+// cleared (a flag set by the programmatic predecessor itself is seen by the next
+// launch).  The wait is made all the same: a launch of which no CTA waits could end
+// before the kernel in front of it, and the kernel behind waits for that launch alone.
+__device__ __forceinline__ bool sticky_error(const int *err)
+{
+    if (!*(volatile const int *)err) return false;
+    griddep_wait();
+    return true;
+}
+
 // --------------------------------------------------------- phased engine
 template <class T>
 __global__ void __launch_bounds__(NT)
     k_gather2(const T *x, const int32_t *bll_j, T *bll, int n_bll, const int32_t *lbuf_j, T *lbuf,
               int n_lbuf, const int *err)
 {
-    // sticky error: no work until cleared (a flag set by the programmatic
-    // predecessor itself is seen by the next launch)
-    if (*(volatile const int *)err) return;
+    if (sticky_error(err)) return;
     const int per = NT * 8;
     for (int b = blockIdx.x * per; b < n_bll + n_lbuf; b += gridDim.x * per) {
         const int e = min(b + per, n_bll + n_lbuf);
@@ -642,7 +651,7 @@ template <class T>
 __global__ void __launch_bounds__(NT)
     k_unpack(const T *grecv, const int32_t *src, T *bnl, int n, const int *err)
 {
-    if (*(volatile const int *)err) return;
+    if (sticky_error(err)) return;
     const int per = NT * 8;
     for (int b = blockIdx.x * per; b < n; b += gridDim.x * per)
         step_gather<false, 8, T, true>(bnl, grecv, src, b, min(b + per, n), threadIdx.x);
@@ -1595,7 +1604,7 @@ __global__ void __launch_bounds__(NT) k_send(const __grid_constant__ SendJobs<MA
         }
     }
     const SendJob &J = jobs.job[jn];
-    if (*(volatile const int *)J.err) return;
+    if (sticky_error(J.err)) return;
     constexpr int U = 2 * kSendGroup / 32;
     const XS *x = static_cast<const XS *>(J.x);
     T *grecv = static_cast<T *>(J.grecv);

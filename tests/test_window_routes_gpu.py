@@ -1,5 +1,5 @@
 """Which path a call takes around the staged windows, and that it answers the same on every
-path: batches of plans with different default options."""
+path: batches of plans with different default options, workspaces in error."""
 import numpy as np
 import pytest
 import torch
@@ -45,3 +45,27 @@ def test_batch_keeps_each_plans_default_precision(first):
         (want if fused else got).extend(bits(w) for w in outs)
     for k, (a, b) in enumerate(zip(got, want)):
         assert np.array_equal(a, b), k
+
+
+@pytest.mark.parametrize("message_less", [False, True])
+def test_workspace_in_error_leaves_the_rest_of_a_windowed_batch_alone(message_less):
+    """A workspace whose flag is set skips its part of the shared launches; a healthy entry,
+    with messages or without, reads the vector that the launch before them wrote."""
+    A, B = gpu_plan(I.poisson3d(16), 16, 4), gpu_plan(I.poisson2d(60), 1 if message_less else 20, 4)
+    va, vb = vec(A.n, 1), vec(B.n, 2)
+    wa, wb, vb2 = torch.full_like(va, 7.0), torch.empty_like(vb), torch.empty_like(vb)
+    nap.napspmv_apply_ex(A, va, wa, 1, 1.0, nap.make_opts(engine=nap.ENGINE_FUSED, debug_stall=1, timeout_ms=50))
+    torch.cuda.synchronize()
+    wa.fill_(7.0)
+    want = torch.empty_like(vb)
+    nap.napspmv_apply_ex(B, vb, vb2, 1, 1.0, nap.make_opts(engine=nap.ENGINE_FUSED))
+    nap.napspmv_apply_ex(B, vb2, want, 1, 1.0, nap.make_opts(engine=nap.ENGINE_FUSED))
+    for _ in range(20):
+        vb2.fill_(float("nan"))
+        nap.napspmv_apply(B, vb, vb2)  # its windows end in the launch that the batch depends on
+        nap.napspmv_apply_batch([A, B], [va, vb2], [wa, wb], [1, 1])
+        assert torch.equal(wb, want)
+    assert nap.napspmv_status(B) == nap.OK
+    assert torch.all(wa == 7.0) and nap.napspmv_status(A) == nap.ERR_TIMEOUT
+    nap.napspmv_apply_batch([A, B], [va, vb2], [wa, wb], [1, 1])
+    assert nap.napspmv_status(A) == nap.OK and not torch.any(wa == 7.0)
