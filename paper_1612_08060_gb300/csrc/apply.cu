@@ -1579,10 +1579,10 @@ struct SendJob {
     const int32_t *j, *dst, *shift;
     void *grecv;
     double *keep;  // null: no copy
-    int *state;    // not null: set to 1
+    int *state;    // not null: set to value
     const int *err;
     int64_t n;  // of x
-    int32_t n_gs;
+    int32_t n_gs, value;
     int32_t block0, send_blocks, blocks;
 };
 template <int MAXJ>
@@ -1609,9 +1609,10 @@ __global__ void __launch_bounds__(NT) k_send(const __grid_constant__ SendJobs<MA
     const XS *x = static_cast<const XS *>(J.x);
     T *grecv = static_cast<T *>(J.grecv);
     const int block = (int)blockIdx.x - J.block0, n = J.n_gs;
+    const bool tells = J.state && block == J.blocks - 1 && threadIdx.x == 0;
     if (block >= J.send_blocks) {
         griddep_wait();
-        if (J.state && block == J.send_blocks && threadIdx.x == 0) *J.state = 1;
+        if (tells) *J.state = J.value;
         if (J.keep)
             for (int64_t i = (int64_t)(block - J.send_blocks) * NT + threadIdx.x; i < J.n;
                  i += (int64_t)(J.blocks - J.send_blocks) * NT)
@@ -1647,21 +1648,39 @@ __global__ void __launch_bounds__(NT) k_send(const __grid_constant__ SendJobs<MA
         for (int u = 0; u < U; u++)
             if (b + 32 * u + lane < n) grecv[to[u]] = v[u];
     }
+    if (tells) {
+        griddep_wait();
+        *J.state = J.value;
+    }
     griddep_done();
 }
 
-// Both receive buffers from a kept vector (no more work where *state is 0).
+// Both receive buffers from a kept vector, where *state is 1; the last CTA to finish
+// clears it (state[1]: their count), for the buffers are what a later step reads.
 template <class T>
 __global__ void __launch_bounds__(NT)
     k_receives(const double *x, const int32_t *bll_j, T *bll, int n_bll, const int32_t *bnl_j,
-               T *bnl, int n_bnl, const int *state, const int *err)
+               T *bnl, int n_bnl, int *state, const int *err)
 {
     griddep_wait();
-    if (*(volatile const int *)err || (state && !*state)) return;
-    for (int64_t k = blockIdx.x * (int64_t)NT + threadIdx.x; k < (int64_t)n_bll + n_bnl;
-         k += (int64_t)gridDim.x * NT) {
-        if (k < n_bll) bll[k] = to_xt(T(0), __ldg(x + bll_j[k]));
-        else bnl[k - n_bll] = to_xt(T(0), __ldg(x + bnl_j[k - n_bll]));
+    if (*(volatile const int *)err || !*(volatile int *)state) return;
+    const uint64_t pol = policy_evict_first();
+    auto gather = [&](T *dst, const int32_t *idx, int b, int e) {
+        batched<8, T>(
+            b, e, threadIdx.x, [&](int k) { return (uint32_t)ld_stream_hint_s32(idx + k, pol); },
+            [&](int, uint32_t j) { return to_xt(T(0), __ldg(x + j)); },
+            [&](int k, uint32_t, T v) { dst[k] = v; });
+    };
+    const int64_t n = (int64_t)n_bll + n_bnl, per = NT * 8;
+    for (int64_t b = blockIdx.x * per; b < n; b += gridDim.x * per) {
+        const int64_t e = min(b + per, n);
+        if (b < n_bll) gather(bll, bll_j, (int)b, (int)min(e, (int64_t)n_bll));
+        if (e > n_bll) gather(bnl, bnl_j, (int)(max(b, (int64_t)n_bll) - n_bll), (int)(e - n_bll));
+    }
+    __syncthreads();  // every thread of the CTA has read the word
+    if (threadIdx.x == 0 && atomicAdd(state + 1, 1) == (int)gridDim.x - 1) {
+        state[0] = 0;
+        state[1] = 0;
     }
     griddep_done();
 }
@@ -1717,6 +1736,7 @@ struct FJob {
     int32_t nmsg[kLevels];      // message units per level
     int32_t ch;                 // elements per message unit (option chunk)
     int32_t nunits[kLevels];    // all units per level
+    int *state;                 // cleared (may be null)
 };
 
 template <int MAXJ>
@@ -1890,6 +1910,8 @@ __global__ void __launch_bounds__(NT, 4) k_fused(const __grid_constant__ FusedPa
                     !wait_ge(prm.stallctr, 1, prm.jobs[0].err, prm.timeout_ns))
                     skip = 1;
                 s_skip[tid] = skip;
+                // the receive buffers hold the receives (see note_receives)
+                if (blockIdx.x == 0 && lvl == 0 && prm.jobs[tid].state) *prm.jobs[tid].state = 0;
             }
             __syncthreads();
             for (int j = 0; j < prm.njobs; j++) {
@@ -1987,12 +2009,12 @@ int ws_alloc(napspmv_plan_t *P, napspmv_ws_t *ws)
         al(&ws->grecv, P->n_gs) || al(&ws->bnl, P->n_bnl + 4) || al(&ws->xtmp, P->n) ||
         alf(&ws->x32[0], P->n) || alf(&ws->x32[1], P->n) ||
         cudaMalloc(&ws->ctr, sizeof(unsigned long long) * ctr_count(P)) ||
-        cudaMalloc(&ws->err, 2 * sizeof(int))) {
+        cudaMalloc(&ws->err, 3 * sizeof(int))) {
         ws_free(ws);
         return cuda_error(cudaErrorMemoryAllocation, "workspace");
     }
     ws->state = ws->err + 1;
-    if (cudaMemset(ws->err, 0, 2 * sizeof(int)) != cudaSuccess) {
+    if (cudaMemset(ws->err, 0, 3 * sizeof(int)) != cudaSuccess) {
         ws_free(ws);
         return cuda_error(cudaGetLastError(), "workspace");
     }
@@ -2044,16 +2066,15 @@ static SellView sell_view(const napspmv_plan_t *P, int part, bool f32)
 
 static int32_t cdiv(int64_t a, int64_t b) { return (int32_t)((a + b - 1) / b); }
 
-// What a workspace's receive buffers hold after the applies about to be queued;
-// every engine calls this.  A workspace that the caller once captured has its
-// device word cleared with every apply: the buffers are valid in HBM.
-static int note_receives(napspmv_ws_t *ws, bool f32, bool vector, bool capturing, cudaStream_t s)
+// What a workspace's receives are after the applies about to be queued; every engine
+// calls this.  vector: the last apply keeps its vector, in replays too, and sets the
+// device word (k_send); otherwise the receive buffers are filled in HBM and a kernel of
+// the apply clears the word (k_send, k_fused; a plan without windows never sets it).
+static void note_receives(napspmv_ws_t *ws, bool f32, bool vector, bool capturing)
 {
+    ws->captured = ws->captured || capturing;
     ws->buf_f32 = f32 ? 1 : 0;
     ws->recv_vector = vector;
-    if (capturing) ws->captured = true;
-    if (ws->captured && ws->state) NAP_CUDA(cudaMemsetAsync(ws->state, 0, sizeof(int), s));
-    return NAPSPMV_OK;
 }
 
 static FJob make_job(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, double *w, int reps,
@@ -2085,6 +2106,7 @@ static FJob make_job(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, doubl
     J.bnl = ws->bnl;
     J.xtmp = ws->xtmp;
     J.err = ws->err;
+    J.state = ws->state;
     J.v = v;
     J.w = w;
     // units of every level: message chunks (levels 0-2), the sliced rows'
@@ -2125,7 +2147,7 @@ static int launch_fused(int count, napspmv_plan_t *const *plans, napspmv_ws_t *c
         wi->recv_f32 = false;
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         NAP_CUDA(cudaStreamIsCapturing(s, &cs));
-        if (int rc = note_receives(wi, false, false, cs != cudaStreamCaptureStatusNone, s)) return rc;
+        note_receives(wi, false, false, cs != cudaStreamCaptureStatusNone);
     }
     for (int l = 0; l < kLevels; l++) prm.off[l][count] = acc[l];
     // barrier words and the test hook's counter: the first job's workspace words
@@ -2468,14 +2490,16 @@ static SendJob send_job(const napspmv_plan_t *P, bool f32, bool windows, const v
     J.send_blocks = J.blocks = P->n_gs > 0 ? msg_grid(P, P->n_gs, P->wave_send[f32]) : 0;
     return J;
 }
+// For the engines that fill the receive buffers (state: cleared, see note_receives).
 template <class T>
-static int64_t enqueue_send(const napspmv_plan_t *P, const T *x, T *grecv, int *err, cudaStream_t s,
-                            bool pdl)
+static int64_t enqueue_send(const napspmv_plan_t *P, const T *x, T *grecv, int *err, int *state,
+                            cudaStream_t s, bool pdl)
 {
     if (P->n_gs == 0) return 0;
     SendJobs<1> S{};
     S.n = 1;
     S.job[0] = send_job(P, sizeof(T) == 4, false, x, grecv, err);
+    S.job[0].state = state;
     launch_pdl(pdl, k_send<T, T, 1>, S.job[0].blocks, 0, s, S);
     return 1;
 }
@@ -2486,7 +2510,7 @@ static int64_t enqueue_send(const napspmv_plan_t *P, const T *x, T *grecv, int *
 // programmatic dependents of the earlier; pdl_first: the first too.
 template <class T>
 static int64_t enqueue_messages(const napspmv_plan_t *P, const T *x, T *bll, T *grecv, T *bnl,
-                                int *err, cudaStream_t s, bool pdl_first)
+                                int *err, int *state, cudaStream_t s, bool pdl_first)
 {
     constexpr bool f32 = sizeof(T) == 4;
     int64_t nk = 0;
@@ -2497,7 +2521,7 @@ static int64_t enqueue_messages(const napspmv_plan_t *P, const T *x, T *bll, T *
         nk++;
     };
     gather(bll, x, P->lists[L_BLL].d_idx, P->n_bll);
-    nk += enqueue_send<T>(P, x, grecv, err, s, nk > 0 || pdl_first);
+    nk += enqueue_send<T>(P, x, grecv, err, state, s, nk > 0 || pdl_first);
     gather(bnl, grecv, P->d_unp_src, P->n_bnl);
     return nk;
 }
@@ -2637,15 +2661,16 @@ static int window_launch(int count, const napspmv_plan_t *const *plans, WinJobs<
 
 template <class T>
 static void receives_launch(const napspmv_plan_t *P, const napspmv_ws_t *ws, const double *x,
-                            const int *state, cudaStream_t s)
+                            cudaStream_t s)
 {
+    // one resident wave: after a capture most launches find the buffers filled
     const int64_t n = P->n_bll + P->n_bnl;
-    if (n == 0) return;
-    const int g = (int)std::min<int64_t>((n + NT - 1) / NT, (int64_t)P->num_sms * 32);
+    const int g = (int)std::max<int64_t>(1, std::min<int64_t>((n + NT * 8 - 1) / (NT * 8),
+                                                              P->wave_gather[sizeof(T) == 4]));
     launch_pdl(true, k_receives<T>, g, 0, s, x, (const int32_t *)P->lists[L_BLL].d_idx,
                reinterpret_cast<T *>(ws->bll), (int)P->n_bll,
                (const int32_t *)P->lists[L_BNL].d_idx, reinterpret_cast<T *>(ws->bnl),
-               (int)P->n_bnl, state, (const int *)ws->err);
+               (int)P->n_bnl, ws->state, (const int *)ws->err);
 }
 
 // Chained applies on the staged windows, of one plan or of several short-row
@@ -2654,22 +2679,20 @@ static void receives_launch(const napspmv_plan_t *P, const napspmv_ws_t *ws, con
 // on-node and off-node values themselves.
 // keep: napspmv_spmv_step may follow.  It needs the receives of the last apply,
 // so that apply's vector stays in xtmp (a copy if it was v; in FP32 mode the
-// chain's FP64 rows before the last) and g_recv with it; where the caller
-// captures, both receive buffers are filled instead (in FP64 after a batch, as
-// the fused engine does).  Filling b_{l->l} after every call in place of the copy
-// cost a launch and a gather: 118 against 105 us for one apply of a 10^6-row
-// banded matrix, 60 against 52.5 us for the strided 101^3 (GB300).
+// chain's FP64 rows before the last), which the send says in the workspace's device
+// word, for a step after a replay that the host does not see.  Filling b_{l->l} after
+// every call in place of the copy cost a launch and a gather: 118 against 105 us for
+// one apply of a 10^6-row banded matrix, 60 against 52.5 us for the strided 101^3 (GB300).
 // Several plans: 32 Poisson matrices of 10^3 to 10^5 rows take two launches, 52
 // against 82 us per call on the fused engine's four grid barriers, and 8 CG
 // iterations over 16 of them 352 against 749 us.
 template <class T, int MAXJ>
 static int enqueue_windows(int count, napspmv_plan_t *const *plans, napspmv_ws_t *const *ws,
                            const double *const *v, double *const *w, const int32_t *reps,
-                           const double *scale, const Opts &o, bool keep, bool fill,
-                           cudaStream_t s, int64_t *kernels)
+                           const double *scale, const Opts &o, bool keep, cudaStream_t s,
+                           int64_t *kernels)
 {
     constexpr bool f32 = sizeof(T) == 4;
-    const bool fill32 = f32 && count == 1 && !o.batch;
     // Long rows take a value about ten times from all over x: FP32 copies of x are made
     // first, where the windows of short rows, which take it about once, round FP64
     // sources (one FP32 apply of 20-entry rows, us on GB300: 3 * 10^5 rows 40.1 against
@@ -2695,7 +2718,7 @@ static int enqueue_windows(int count, napspmv_plan_t *const *plans, napspmv_ws_t
             float *y32 = f32 && left > 0 ? W->x32[(left - 1) & 1] : nullptr;
             if (f32 && left > 0 && !(keep && left == 1)) y = nullptr;
             SendJob S = send_job(P, f32, true, xs, W->grecv, W->err);
-            const bool hold = keep && left == 0 && !fill;
+            const bool hold = keep && left == 0;
             if (convert && k == 0) {
                 const int g = (int)std::max<int64_t>(1, std::min<int64_t>((P->n + NT * 8 - 1) / (NT * 8),
                                                                           (int64_t)P->num_sms * 8));
@@ -2705,6 +2728,7 @@ static int enqueue_windows(int count, napspmv_plan_t *const *plans, napspmv_ws_t
             }
             if (hold) {
                 S.state = W->state;
+                S.value = 1;
                 S.keep = k == 0 && !convert ? W->xtmp : nullptr;
                 S.blocks += S.keep ? (int)std::min<int64_t>((P->n + 8 * NT - 1) / (8 * NT),
                                                             4 * (int64_t)P->num_sms)
@@ -2714,12 +2738,6 @@ static int enqueue_windows(int count, napspmv_plan_t *const *plans, napspmv_ws_t
                 S.block0 = blocks;
                 blocks += S.blocks;
                 sends.job[ns++] = S;
-            }
-            if (keep && fill && left == 0) {
-                const double *src = k == 0 ? v[i] : W->xtmp;
-                if (fill32) receives_launch<float>(P, W, src, nullptr, s);
-                else receives_launch<double>(P, W, src, nullptr, s);
-                nk += P->n_bll + P->n_bnl > 0;
             }
             wp[nw] = P;
             wins.job[nw++] = window_job(P, W, xs, nullptr, y, y32, scale ? scale[i] : 1.0);
@@ -2807,10 +2825,8 @@ static int enqueue_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, 
 {
     if (o.window)
         return o.precision == NAPSPMV_PREC_F32
-                   ? enqueue_windows<float, 1>(1, &P, &ws, &v, &w, &reps, &scale, o, keep,
-                                               ws->captured, s, kernels)
-                   : enqueue_windows<double, 1>(1, &P, &ws, &v, &w, &reps, &scale, o, keep,
-                                                ws->captured, s, kernels);
+                   ? enqueue_windows<float, 1>(1, &P, &ws, &v, &w, &reps, &scale, o, keep, s, kernels)
+                   : enqueue_windows<double, 1>(1, &P, &ws, &v, &w, &reps, &scale, o, keep, s, kernels);
     auto grid = [&](int64_t n) {
         return (int)std::max<int64_t>(1, std::min<int64_t>((n + NT * 8 - 1) / (NT * 8),
                                                             (int64_t)P->num_sms * 8));
@@ -2858,9 +2874,9 @@ static int enqueue_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, 
         else if (f32)
             nk += enqueue_messages<float>(P, x32, reinterpret_cast<float *>(ws->bll),
                                           reinterpret_cast<float *>(ws->grecv),
-                                          reinterpret_cast<float *>(ws->bnl), ws->err, s, pdl);
+                                          reinterpret_cast<float *>(ws->bnl), ws->err, ws->state, s, pdl);
         else
-            nk += enqueue_messages<double>(P, x, ws->bll, ws->grecv, ws->bnl, ws->err, s, pdl);
+            nk += enqueue_messages<double>(P, x, ws->bll, ws->grecv, ws->bnl, ws->err, ws->state, s, pdl);
         if (overlap) {
             NAP_CUDA(cudaStreamWaitEvent(s, P->ev_join, 0));
             spmv_run(LR, xs, ws, y, y32, scale, o.stages, s, false);
@@ -2894,10 +2910,10 @@ static int launch_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, d
     const bool capturing = cs != cudaStreamCaptureStatusNone;
     const bool f32 = o.precision == NAPSPMV_PREC_F32;
     ws->recv_f32 = f32;
-    if (keep || !o.window)
-        if (int rc = note_receives(ws, f32 && !o.batch, o.window && !ws->captured && !capturing,
-                                   capturing, s))
-            return rc;
+    if (keep || !o.window) note_receives(ws, f32 && !o.batch, o.window, capturing);
+    // (no message kernel to clear the word: see enqueue_messages)
+    if (!o.window && P->win.blocks && P->n_gs == 0)
+        NAP_CUDA(cudaMemsetAsync(ws->state, 0, sizeof(int), s));
     int64_t nk = 0;
     if (!use_graph) {
         int rc = enqueue_phased(P, ws, v, w, reps, scale, o, keep, s, &nk);
@@ -2906,7 +2922,7 @@ static int launch_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, d
     }
     for (size_t i = 0; i < P->graphs.size(); i++) {
         auto &g = P->graphs[i];
-        if (g.v == v && g.w == w && g.ws == ws && g.window == o.window && g.fill == (ws->captured || !keep) && g.reps == reps && g.scale == scale &&
+        if (g.v == v && g.w == w && g.ws == ws && g.window == o.window && g.keep == keep && g.reps == reps && g.scale == scale &&
             g.prec == o.precision && g.vec == o.vec && g.tile_rows == o.tile_rows &&
             g.tile_nnz == o.tile_nnz && g.engine == o.engine && g.stages == o.stages &&
             g.pipeline == o.pipeline && g.ctas_per_sm == o.ctas_per_sm && g.halo == o.halo) {
@@ -2932,7 +2948,7 @@ static int launch_phased(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, d
         cudaGraphExecDestroy(P->graphs.front().exec);
         P->graphs.erase(P->graphs.begin());
     }
-    P->graphs.push_back({v, w, ws, o.window, ws->captured || !keep, reps, o.precision, o.vec, o.tile_rows, o.tile_nnz, o.engine,
+    P->graphs.push_back({v, w, ws, o.window, keep, reps, o.precision, o.vec, o.tile_rows, o.tile_nnz, o.engine,
                          o.stages, o.pipeline, o.ctas_per_sm, o.halo, scale, exec, nk});
     NAP_CUDA(cudaGraphLaunch(exec, s));
     count_launch(nk);
@@ -3020,18 +3036,15 @@ static int launch_windows(int count, napspmv_plan_t *const *plans, napspmv_ws_t 
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     NAP_CUDA(cudaStreamIsCapturing(s, &cs));
     const bool capturing = cs != cudaStreamCaptureStatusNone;
-    bool fill = capturing;
-    for (int i = 0; i < count; i++) fill = fill || ws[i]->captured;
     for (int i = 0; i < count; i++) {
         ws[i]->recv_f32 = f32;
         if (!keep) continue;
-        if (int rc = note_receives(ws[i], false, !fill, capturing, s)) return rc;
+        // (the precision that the fused engine, the batches' other path, leaves)
+        note_receives(ws[i], false, true, capturing);
     }
     int64_t nk = 0;
-    const int rc = f32 ? enqueue_windows<float, 64>(count, plans, ws, v, w, reps, scale, o, keep,
-                                                    fill, s, &nk)
-                       : enqueue_windows<double, 64>(count, plans, ws, v, w, reps, scale, o, keep,
-                                                     fill, s, &nk);
+    const int rc = f32 ? enqueue_windows<float, 64>(count, plans, ws, v, w, reps, scale, o, keep, s, &nk)
+                       : enqueue_windows<double, 64>(count, plans, ws, v, w, reps, scale, o, keep, s, &nk);
     if (!rc) count_launch(nk);
     return rc;
 }
@@ -3273,7 +3286,7 @@ extern "C" int napspmv_spmv_step(napspmv_plan_t *P, napspmv_ws_t *ws, const doub
     if ((rc = build_items(P, o.tile_rows, o.tile_nnz))) return rc;
     const bool f32 = o.precision == NAPSPMV_PREC_F32;
     // launched as the phased engine launches its SpMV pass
-    const bool pdl = o.engine == NAPSPMV_ENGINE_PHASED;
+    bool pdl = o.engine == NAPSPMV_ENGINE_PHASED;
     if (W->buf_f32 != (f32 ? 1 : 0)) {
         set_error(NAPSPMV_ERR_STATE, "the receive buffers hold the other precision's copies: "
                                      "apply once in this precision (phased or overlapped engine "
@@ -3287,6 +3300,10 @@ extern "C" int napspmv_spmv_step(napspmv_plan_t *P, napspmv_ws_t *ws, const doub
         k_to_f32<<<g, NT, 0, st>>>(src, dst, nullptr, P->n, W->err);
         count_launch(1);
     };
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    NAP_CUDA(cudaStreamIsCapturing(st, &cs));
+    // a replay of this step comes after applies that the host does not know of now
+    if (cs != cudaStreamCaptureStatusNone) W->captured = true;
     if (o.window && W->recv_vector && !W->captured && W->recv_f32 == f32) {
         // on the windows: on-node receives from the kept vector, off-node from g_recv.
         // It receives again what an apply that filled the buffers had received: a step
@@ -3306,14 +3323,14 @@ extern "C" int napspmv_spmv_step(napspmv_plan_t *P, napspmv_ws_t *ws, const doub
         if ((rc = window_launch<1>(1, pl, jobs, convert ? 1 : f32 ? 2 : 0, true, o, st))) return rc;
         count_launch(1);
     } else {
-        if (W->recv_vector || W->captured) {
-            // the receive buffers from the kept vector (after a capture, if the
-            // device word says that the last apply kept one)
-            const int *state = W->captured ? W->state : nullptr;
-            if (f32) receives_launch<float>(P, W, W->xtmp, state, st);
-            else receives_launch<double>(P, W, W->xtmp, state, st);
+        if (P->win.blocks && (W->recv_vector || W->captured)) {
+            // the receive buffers from the kept vector, if the device word says that
+            // the last apply kept one; they are what a later step reads
+            if (f32) receives_launch<float>(P, W, W->xtmp, st);
+            else receives_launch<double>(P, W, W->xtmp, st);
             count_launch(1);
-            if (!W->captured) W->recv_vector = false;
+            W->recv_vector = false;
+            pdl = true;
         }
         SpmvLaunch L;
         if ((rc = spmv_launch(P, o, kFull, L))) return rc;

@@ -175,11 +175,12 @@ struct napspmv_ws_s {
     int buf_f32 = 0;
     // the staged windows keep the receives in shared memory: what a later
     // napspmv_spmv_step takes them from is the last apply's vector, in xtmp, and
-    // g_recv (recv_f32: of FP32 copies).  captured: the caller captured an apply,
-    // whose replays the host does not see; *state (device) is then 1 only while
-    // the last apply that ran kept its vector, and later applies fill the buffers.
+    // g_recv (recv_f32: of FP32 copies).  *state (device) is 1 while the last apply
+    // that ran kept its vector, 0 while the receive buffers hold its receives;
+    // recv_vector is the same as the host sees it, which it does until the caller
+    // captures an apply or a step of this workspace (captured).
     bool recv_vector = false, recv_f32 = false, captured = false;
-    int *state = nullptr;
+    int *state = nullptr;  // two words, see k_receives
     double *hv = nullptr, *hw = nullptr;  // staging of napspmv_apply_host
     unsigned long long *ctr = nullptr;  // the fused engine's grid barrier: arrivals, generation
     int *err = nullptr;                 // sticky device status
@@ -238,7 +239,7 @@ struct napspmv_plan_s {
     // instantiated CUDA graphs of chained phased applies, newest last
     struct GraphEntry {
         const void *v, *w, *ws;
-        bool window, fill;
+        bool window, keep;
         int32_t reps, prec, vec, tile_rows, tile_nnz, engine, stages, pipeline, ctas_per_sm, halo;
         double scale;
         cudaGraphExec_t exec;

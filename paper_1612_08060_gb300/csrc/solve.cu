@@ -752,7 +752,7 @@ bool slots_on_windows(int32_t count, const napspmv_cg_slot *slots, int32_t preci
         const napspmv_cg_slot &c = slots[i];
         const napspmv_ws_t *W = c.ws ? c.ws : c.plan->ws;
         if (!runs_on_windows(c.plan, precision) || c.plan->device != dev || W->plan != c.plan ||
-            W->captured || c.p == c.q || (precision == NAPSPMV_PREC_F32 && !c.plan->d_val32))
+            c.p == c.q || (precision == NAPSPMV_PREC_F32 && !c.plan->d_val32))
             return false;
         for (int q = 0; q < i; q++)
             if (W == (slots[q].ws ? slots[q].ws : slots[q].plan->ws)) return false;

@@ -1,5 +1,6 @@
 """Which path a call takes around the staged windows, and that it answers the same on every
-path: batches of plans with different default options, workspaces in error."""
+path: batches of plans with different default options, workspaces in error, steps and
+applies that a caller captured."""
 import numpy as np
 import pytest
 import torch
@@ -7,6 +8,7 @@ import torch
 from gpu_util import gpu_plan
 from paper_1612_08060_gb300 import inputs as I
 from paper_1612_08060_gb300 import napspmv as nap
+from test_windows_gpu import near_and_far
 
 pytestmark = pytest.mark.gpu
 
@@ -69,3 +71,86 @@ def test_workspace_in_error_leaves_the_rest_of_a_windowed_batch_alone(message_le
     assert torch.all(wa == 7.0) and nap.napspmv_status(A) == nap.ERR_TIMEOUT
     nap.napspmv_apply_batch([A, B], [va, vb2], [wa, wb], [1, 1])
     assert nap.napspmv_status(A) == nap.OK and not torch.any(wa == 7.0)
+
+
+TILES = dict(engine=nap.ENGINE_PHASED, pipeline=nap.PIPELINE_CTA, vec=1)
+FUSED = dict(engine=nap.ENGINE_FUSED)
+
+
+def short_or_long(mat):
+    """A plan of short rows, or of long rows whose far messages the windows reorder."""
+    if mat == "short":
+        return gpu_plan(I.poisson3d(18), 7, 3)
+    return gpu_plan(near_and_far(300 * 80 + 1, 700, 1, 300), 80, 1)
+
+
+class Steps:
+    """Applies on one path or another, and the step that follows, of one plan."""
+
+    def __init__(self, mat, prec):
+        self.plan, self.prec = short_or_long(mat), prec
+        self.v, self.w, self.z = vec(self.plan.n, 1), vec(self.plan.n, 2), vec(self.plan.n, 3)
+        self.ws = nap.Workspace(self.plan)  # for what is expected
+
+    def apply(self, x, path, ws=None):
+        nap.napspmv_apply_ex(self.plan, x, self.w, 1, 1.0, nap.make_opts(precision=self.prec, **path), ws=ws)
+
+    def step(self, path, ws=None):
+        self.z.fill_(float("nan"))
+        nap.napspmv_spmv_step(self.plan, self.v, self.z, 1.0, nap.make_opts(precision=self.prec, **path), ws=ws)
+        return self.z
+
+    def want(self, x):
+        self.apply(x, TILES, self.ws)
+        return bits(self.step(TILES, self.ws))
+
+
+def paths(prec):  # (the fused engine leaves FP64 receives, which an FP32 step refuses)
+    return [{}, TILES] if prec else [{}, TILES, FUSED]
+
+
+@pytest.mark.parametrize("prec", [nap.PREC_F64, nap.PREC_F32])
+@pytest.mark.parametrize("mat", ["short", "long"])
+def test_captured_step_takes_the_receives_of_the_apply_before_the_replay(mat, prec):
+    S = Steps(mat, prec)
+    x = [vec(S.plan.n, 30 + k) for k in range(2)]
+    want = [S.want(y) for y in x]
+    for step in ({}, TILES):
+        for before in paths(prec):
+            S.ws2 = nap.Workspace(S.plan)  # nothing on it was captured yet
+            S.apply(x[0], before, S.ws2)
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                S.step(step, S.ws2)
+            graph.replay()
+            assert np.array_equal(bits(S.z), want[0]), (step, before)
+            for after in paths(prec):
+                S.apply(x[1], after, S.ws2)
+                for _ in range(2):
+                    graph.replay()
+                    assert np.array_equal(bits(S.z), want[1]), (step, before, after)
+                assert np.array_equal(bits(S.step({}, S.ws2)), want[1]), (step, before, after)
+            del graph
+
+
+@pytest.mark.parametrize("prec", [nap.PREC_F64, nap.PREC_F32])
+@pytest.mark.parametrize("mat", ["short", "long"])
+def test_step_after_a_capture_that_did_not_run(mat, prec):
+    """An apply that was captured and not replayed changes no receives, whatever ran before."""
+    S = Steps(mat, prec)
+    x = [vec(S.plan.n, 40 + k) for k in range(3)]
+    want = [S.want(y) for y in x]
+    for one in paths(prec):
+        for two in paths(prec):
+            ws = nap.Workspace(S.plan)
+            S.apply(x[0], one, ws)
+            S.apply(x[1], two, ws)
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                S.apply(x[2], {}, ws)
+            assert np.array_equal(bits(S.step({}, ws)), want[1]), (one, two)
+            graph.replay()
+            assert np.array_equal(bits(S.step({}, ws)), want[2]), (one, two)
+            S.apply(x[0], two, ws)
+            assert np.array_equal(bits(S.step(TILES, ws)), want[0]), (one, two)
+            del graph
