@@ -117,9 +117,13 @@ extern "C" {
  * apply runs on staged windows where it can: every process's rows are cut into
  * blocks, a CTA brings the values its block multiplies into shared memory, each
  * once, and sums its sliced rows from there (the bits of vec = 1).  That takes at
- * least 64 rows per process on average, no row of more than 256 entries and no
- * composed gathers; otherwise, and once napspmv_set_default_opts has set a plan's
- * defaults, the engine and pipeline of napspmv_get_default_opts run. */
+ * least 64 rows per process on average, no row of more than 256 entries, no
+ * composed gathers, processes of at most 819,200 values (own rows and receives),
+ * and blocks that fit the shared memory.  Otherwise the engine and pipeline of
+ * napspmv_get_default_opts run, as they do once napspmv_set_default_opts was given
+ * any of these fields; options read by napspmv_get_default_opts and written back
+ * with all of them as they were leave the path open.  ENGINE_PHASED with
+ * PIPELINE_SELL as defaults run on staged windows again. */
 #define NAPSPMV_ENGINE_DEFAULT 0 /* the plan's default engine               */
 #define NAPSPMV_ENGINE_FUSED 1   /* one persistent, cooperative launch for all
                                     phases and all chained applies, in levels

@@ -9,7 +9,7 @@ coordinate descent: starting from the plan's defaults, each parameter in turn
 is set to each candidate while the others stay fixed, the fastest is kept, and
 the sweep repeats until nothing improves.  Each candidate is timed with CUDA
 events over chained applies (inputs already on the device).  The winner is
-installed with napspmv_set_default_opts and cached per (N, nnz, nnz-per-row
+installed with napspmv_set_default_opts and cached per (paths, N, nnz, nnz-per-row
 histogram, n_p, ppn, precision) key, in memory and optionally in a JSON file.
 """
 from __future__ import annotations
@@ -35,11 +35,17 @@ CANDIDATES = {
 _cache: dict = {}
 
 
+# Leads every key: options measured against other paths than today's are not taken from a
+# file (before the staged windows the best of a short-row plan was the overlapped engine,
+# which as a default would keep the plan off the windows).
+PATHS = "windows1"
+
+
 def matrix_key(row_ptr, n_p, ppn, precision):
     lens = np.diff(np.asarray(row_ptr))
     hist = np.histogram(np.minimum(lens, 64), bins=[0, 2, 4, 8, 12, 16, 24, 32, 48, 65])[0]
     hist = tuple(int(round(10 * h / max(1, len(lens)))) for h in hist)
-    return f"n{len(lens)}_nnz{int(lens.sum())}_h{hist}_np{n_p}_ppn{ppn}_p{precision}"
+    return f"{PATHS}_n{len(lens)}_nnz{int(lens.sum())}_h{hist}_np{n_p}_ppn{ppn}_p{precision}"
 
 
 def time_opts(plan, v, w, opts, reps=20, trials=3, stream=None):

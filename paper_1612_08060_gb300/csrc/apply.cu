@@ -1945,6 +1945,13 @@ bool leaves_path_open(const napspmv_opts &o)
            !o.tile_rows && !o.tile_nnz && !o.stages && !o.halo;
 }
 
+bool same_path(const napspmv_opts &a, const napspmv_opts &b)
+{
+    return a.engine == b.engine && a.pipeline == b.pipeline && a.vec == b.vec &&
+           a.tile_rows == b.tile_rows && a.tile_nnz == b.tile_nnz && a.stages == b.stages &&
+           a.halo == b.halo;
+}
+
 Opts resolve_opts(const napspmv_plan_t *P, const napspmv_opts *o)
 {
     Opts r;

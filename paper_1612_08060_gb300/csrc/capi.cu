@@ -219,8 +219,10 @@ int napspmv_set_default_opts(napspmv_plan_t *P, const napspmv_opts *opts)
     int rc = build_items(P, o.tile_rows, o.tile_nnz);
     if (cur != P->device) cudaSetDevice(cur);
     if (rc) return rc;
+    // a path that is named is one to take, staged windows or not; one that reads as
+    // napspmv_get_default_opts gave it is not named
+    if (!leaves_path_open(*opts) && !same_path(*opts, P->defaults)) P->auto_window = false;
     P->defaults = o;
-    if (!leaves_path_open(*opts)) P->auto_window = false;
     return NAPSPMV_OK;
 }
 

@@ -232,7 +232,7 @@ struct napspmv_plan_s {
     nap::WinPart win;  // staged windows over sell[0]
     int64_t wave_gather[2] = {}, wave_send[2] = {};  // CTAs the GPU holds at once (FP64, FP32)
     // an apply that leaves engine, pipeline and tile options unset runs on the
-    // staged windows (until napspmv_set_default_opts names an engine or pipeline)
+    // staged windows (until napspmv_set_default_opts names some of them)
     bool auto_window = true;
 
     nap::ItemSet items;
@@ -269,6 +269,8 @@ struct Opts : napspmv_opts {
 Opts resolve_opts(const napspmv_plan_t *P, const napspmv_opts *o);
 // the fields that name an engine, a pipeline or a tile shape are all unset
 bool leaves_path_open(const napspmv_opts &o);
+// they are all the same
+bool same_path(const napspmv_opts &a, const napspmv_opts &b);
 // ERR_ARG / ERR_STATE / ERR_UNSUPPORTED (with the message set) for resolved
 // options the plan cannot run, else NAPSPMV_OK
 int check_opts(const napspmv_plan_t *P, const napspmv_opts &o);

@@ -1,6 +1,6 @@
 """Which path a call takes around the staged windows, and that it answers the same on every
-path: batches of plans with different default options, workspaces in error, steps and
-applies that a caller captured."""
+path: batches of plans with different default options, default options read and written back,
+workspaces in error, steps and applies that a caller captured, the largest plan on windows."""
 import numpy as np
 import pytest
 import torch
@@ -154,3 +154,41 @@ def test_step_after_a_capture_that_did_not_run(mat, prec):
             S.apply(x[0], two, ws)
             assert np.array_equal(bits(S.step(TILES, ws)), want[0]), (one, two)
             del graph
+
+
+def launches(plan, v, w):
+    before = nap.napspmv_launch_count()
+    nap.napspmv_apply(plan, v, w)
+    return nap.napspmv_launch_count() - before
+
+
+@pytest.mark.parametrize("mat", ["short", "long"])
+def test_default_options_read_and_written_back_change_no_path(mat):
+    plan = short_or_long(mat)
+    v, w = vec(plan.n, 1), vec(plan.n, 2)
+    assert launches(plan, v, w) == 2  # messages, windows
+    d = nap.napspmv_get_default_opts(plan)
+    d.timeout_ms = 700
+    nap.napspmv_set_default_opts(plan, d)
+    assert launches(plan, v, w) == 2
+    # another tile shape is a path of its own, and stays one when written back
+    nap.napspmv_set_default_opts(plan, nap.make_opts(engine=nap.ENGINE_OVERLAP, pipeline=nap.PIPELINE_CTA))
+    assert launches(plan, v, w) > 2
+    nap.napspmv_set_default_opts(plan, nap.napspmv_get_default_opts(plan))
+    assert launches(plan, v, w) > 2
+    nap.napspmv_set_default_opts(plan, nap.make_opts(engine=nap.ENGINE_PHASED, pipeline=nap.PIPELINE_SELL))
+    assert launches(plan, v, w) == 2
+
+
+@pytest.mark.parametrize("rows,windows", [(819199, True), (819200, False)])
+def test_largest_process_on_windows(rows, windows):
+    """A process's rows and receives (one here) number 819,200 at most."""
+    n = 2 * rows
+    cols = np.arange(n)[:, None] + np.array([-1, 0, 1])
+    ok = (cols >= 0) & (cols < n)
+    row_ptr = np.concatenate([[0], np.cumsum(ok.sum(1))])
+    plan = gpu_plan(I.CSR(row_ptr, cols[ok].astype(np.int32), np.linspace(-1, 1, 3 * n)[:ok.sum()]), 2, 1)
+    v, w, z = vec(n, 1), vec(n, 2), vec(n, 3)
+    assert (launches(plan, v, w) == 2) == windows
+    nap.napspmv_apply_ex(plan, v, z, 1, 1.0, nap.make_opts(**TILES))
+    assert np.array_equal(bits(w), bits(z))
