@@ -2609,7 +2609,7 @@ static WinJob window_job(const napspmv_plan_t *P, const napspmv_ws_t *ws, const 
                          const void *l, double *y, float *y32, double scale)
 {
     const WinPart &W = P->win;
-    const SellPart &SP = P->sell[0];
+    const SellPart &SP = W.rows;
     WinJob J{};
     J.S = WinView{W.d_blk,  SP.d_info,  SP.d_perm, W.d_col, SP.d_val,
                   SP.d_val32, W.d_runs, (W.max_src + 7) & ~7, (W.max_slots + 7) & ~7, W.max_words};

@@ -129,9 +129,9 @@ struct SellPart {
 // block's window lists, once each, the values its rows multiply: own vector
 // entries, on-node receives (b_{l->l}) and off-node receives (b_{nl->l}), in
 // that order.  The CTA brings the window into shared memory (phase 4, and phase
-// 1's on-node part) and sums its sliced rows from there; the whole matrix's
-// sliced rows are sorted and cut per block, and stored entry s multiplies
-// window slot col[s].
+// 1's on-node part) and sums its sliced rows from there: the windows have sliced
+// rows of their own, sorted and cut per block, whose stored entry s multiplies window
+// slot col[s].
 // Where the window's values come from is kept as runs.  For every 32 slots: a
 // mask of the slots that start a run (the first always does) and the index of
 // its first run, as two words; after them the source of every run's first slot.
@@ -141,7 +141,7 @@ constexpr uint16_t kWinPad = 0xffff;      // padding slots, as kSellPad
 constexpr uint32_t kFromRecv = 0x80000000u;  // source in g_recv, else in x
 constexpr uint32_t kFromNode = 0x40000000u;  // an on-node receive, source in x
 struct WinBlock {
-    int32_t chunk0, chunks;  // its chunks of the whole matrix's sliced rows
+    int32_t chunk0, chunks;  // its chunks of the windows' sliced rows
     int32_t slot0, slots;    // its stored-entry slots
     int32_t srcs;            // window slots
     int32_t words, word0;    // its runs: words (a multiple of 4), and the first / 4
@@ -150,12 +150,12 @@ struct WinBlock {
 };
 struct WinPart {
     int32_t blocks = 0;   // 0: the plan has no windows
-    int32_t rows = 0;     // rows per block (a multiple of 32)
+    SellPart rows;        // the whole matrix's rows, sorted and cut per block (no d_col, d_long)
     int32_t threads = 0;  // per CTA
     bool long_rows = false;     // rows of more than 12 entries: k_window_long
     int32_t long_ctas[2] = {};  // its CTAs per SM (FP64, FP32)
     int32_t max_src = 0, max_slots = 0, max_words = 0;  // largest block: slots, entry slots, run words
-    uint16_t *d_col = nullptr;  // window slot of every sliced-row slot
+    uint16_t *d_col = nullptr;  // window slot of every slot of `rows`
     WinBlock *d_blk = nullptr;
     uint32_t *d_runs = nullptr;
     int32_t *d_send = nullptr;  // not null: the order of g_send the windows' receives want (order_receives)
@@ -229,7 +229,7 @@ struct napspmv_plan_s {
     // sliced-row copies of the whole matrix, its local part and its remote
     // part (index 0, 1, 2), for NAPSPMV_PIPELINE_SELL; built with the plan
     nap::SellPart sell[3];
-    nap::WinPart win;  // staged windows over sell[0]
+    nap::WinPart win;  // staged windows
     int64_t wave_gather[2] = {}, wave_send[2] = {};  // CTAs the GPU holds at once (FP64, FP32)
     // an apply that leaves engine, pipeline and tile options unset runs on the
     // staged windows (until napspmv_set_default_opts names some of them)

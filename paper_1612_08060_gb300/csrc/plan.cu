@@ -125,13 +125,6 @@ struct dvec {
         bytes = 0;
     }
     ~dvec() { drop(); }
-    T *release()
-    {
-        T *q = p;
-        p = nullptr;
-        bytes = 0;
-        return q;
-    }
     void swap(dvec &o)
     {
         std::swap(p, o.p);
@@ -885,6 +878,77 @@ void host_stats(napspmv_plan_t *P)
     S.bytes_msg = 20.0 * (double)(P->n_bll + P->n_lbuf + P->n_gs + P->n_bnl) + 20.0 * (double)P->n_gs;
 }
 
+// Rows sorted and cut into chunks, a part's or the staged windows'.
+//
+// One radix sort of (window, length) keys orders every window at once; a warp
+// per window then cuts it, 32 rows to a step.  Sorting and cutting on the host
+// (a stable sort per window, three parts, and the upload of the row lists) took
+// most of a plan build: 41 of 56 ms of a 10^6-row 7-point plan on GB300, against 2.3 of
+// 17 ms this way (810 of 1,180 ms of the 2^23-row banded random plan, against 6 of 370).
+struct RowCut {
+    int64_t n, nwin;
+    dvec<uint64_t> key;
+    dvec<int32_t> row;
+    // per window, first chunk and first slot; the last element of each is the total;
+    // then the first long row's position
+    dvec<int64_t> off;
+    int64_t total[3];  // chunks, slots, rows of at most kSellLong entries
+    const int64_t *och() const { return off.p; }
+    const int64_t *osl() const { return off.p + nwin + 1; }
+    int wblocks() const { return blocks_for(32 * (nwin + 1)); }
+
+    RowCut(Cub &cb, const int32_t *d_rp, int64_t rows, const Part &part, const SellCut &cut = SellCut())
+        : n(rows), nwin(cut.count(part, rows)), key(n), row(n), off(2 * (nwin + 1) + 1)
+    {
+        dvec<uint64_t> key2(n);
+        dvec<int32_t> row2(n);
+        k_sell_keys<<<blocks_for(n), 256>>>(d_rp, n, part, cut, nwin, key.p, row.p);
+        CK(cudaGetLastError());
+        cb.sort_pairs(key, key2, row, row2, n, kSellKeyBits + bits_for(nwin));
+        dvec<int64_t> cnt(2 * (nwin + 1));
+        int64_t *nch = cnt.p, *nsl = cnt.p + nwin + 1;
+        k_sell_cut<false><<<wblocks(), 256>>>(key.p, row.p, n, nwin, nch, nsl, nullptr, nullptr,
+                                              nullptr, nullptr, off.p + 2 * (nwin + 1));
+        CK(cudaGetLastError());
+        cb.exclusive_sum(nch, off.p, nwin + 1);
+        cb.exclusive_sum(nsl, off.p + nwin + 1, nwin + 1);
+        CK(cudaMemcpy(&total[0], och() + nwin, sizeof(int64_t), cudaMemcpyDeviceToHost));
+        CK(cudaMemcpy(&total[1], osl() + nwin, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost));
+    }
+    // 31-bit slots
+    bool fits() const { return total[1] <= (int64_t)INT32_MAX - 1024; }
+    // the chunks, and room for their slots
+    void chunks(SellPart &S, bool f32, bool columns) const
+    {
+        S.nch = total[0];
+        S.slots = total[1];
+        CK(device_alloc(&S.d_info, sizeof(int2) * std::max<int64_t>(S.nch, 1)));
+        CK(device_alloc(&S.d_perm, sizeof(int32_t) * 32 * std::max<int64_t>(S.nch, 1)));
+        k_sell_cut<true><<<wblocks(), 256>>>(key.p, row.p, n, nwin, nullptr, nullptr, och(), osl(),
+                                             S.d_info, S.d_perm, nullptr);
+        CK(cudaGetLastError());
+        // padded past the last slot: a block's bulk copy is widened to 16 bytes
+        auto al = [&](size_t sz, int fill) {
+            void *q = nullptr;
+            const size_t bytes = sz * (size_t)std::max<int64_t>(S.slots, 1) + 256;
+            CK(device_alloc(&q, bytes));
+            CK(cudaMemset(q, fill, bytes));
+            return q;
+        };
+        if (columns) S.d_col = (uint32_t *)al(4, 0xff);  // kSellPad between chunks too
+        S.d_val = (double *)al(8, 0);
+        if (f32) S.d_val32 = (float *)al(4, 0);
+    }
+};
+
+void free_sell(SellPart &S)
+{
+    void *p[] = {S.d_info, S.d_perm, S.d_col, S.d_val, S.d_val32, S.d_long};
+    for (void *q : p)
+        if (q) cudaFree(q);
+    S = SellPart();
+}
+
 // Sliced-row copy of one matrix part (which: 0 whole, 1 local, 2 remote) from
 // its CSR, built on the device.  Windows: the rows of each process (contiguous
 // partition) or of each 1024-row block (strided).  Within a window, rows of at
@@ -892,72 +956,28 @@ void host_stats(napspmv_plan_t *P)
 // cut into chunks of up to 32 whose counts are at least half the first one's;
 // longer rows are listed apart.  A part whose padded slots would not fit 31-bit
 // offsets is left without a sliced copy.
-//
-// One radix sort of (window, length) keys orders every window at once; a warp
-// per window then cuts it, 32 rows to a step.  Sorting and cutting on the host
-// (a stable sort per window, three parts, and the upload of the row lists) took
-// most of a plan build: 41 of 56 ms of a 10^6-row 7-point plan on GB300, against 2.3 of
-// 17 ms this way (810 of 1,180 ms of the 2^23-row banded random plan, against 6 of 370).
 void build_sell(napspmv_plan_t *P, Cub &cb, int which, const int32_t *d_rp, const uint32_t *d_col,
-                const double *d_val, const float *d_val32, const Part &part,
-                const SellCut &cut = SellCut(), dvec<int64_t> *win_off = nullptr)
+                const double *d_val, const float *d_val32, const Part &part)
 {
     SellPart &S = P->sell[which];
     const int64_t n = P->n;
-    const int64_t nwin = cut.count(part, n);
-    const int kb = kSellKeyBits + bits_for(nwin);
-    dvec<uint64_t> key(n), key2(n);
-    dvec<int32_t> row(n), row2(n);
-    k_sell_keys<<<blocks_for(n), 256>>>(d_rp, n, part, cut, nwin, key.p, row.p);
-    CK(cudaGetLastError());
-    cb.sort_pairs(key, key2, row, row2, n, kb);
-    // per window: chunks and slots, then their exclusive sums (the last element
-    // is the total) and the first long row's position
-    dvec<int64_t> cnt(2 * (nwin + 1)), off(2 * (nwin + 1) + 1);
-    int64_t *nch = cnt.p, *nsl = cnt.p + nwin + 1, *och = off.p, *osl = off.p + nwin + 1;
-    const int wblocks = blocks_for(32 * (nwin + 1));
-    k_sell_cut<false><<<wblocks, 256>>>(key.p, row.p, n, nwin, nch, nsl, nullptr, nullptr, nullptr,
-                                        nullptr, off.p + 2 * (nwin + 1));
-    CK(cudaGetLastError());
-    cb.exclusive_sum(nch, och, nwin + 1);
-    cb.exclusive_sum(nsl, osl, nwin + 1);
-    int64_t tot[3];
-    CK(cudaMemcpy(&tot[0], och + nwin, sizeof(int64_t), cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(&tot[1], osl + nwin, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost));
-    const int64_t slots = tot[1];
-    if (slots > (int64_t)INT32_MAX - 1024) {
+    RowCut R(cb, d_rp, n, part);
+    if (!R.fits()) {
         S.slots = -1;  // no sliced copy: NAPSPMV_PIPELINE_SELL is refused for this plan
         return;
     }
-    S.nch = tot[0];
-    S.slots = slots;
-    S.n_long = (int32_t)(n - tot[2]);
-    CK(device_alloc(&S.d_info, sizeof(int2) * std::max<int64_t>(S.nch, 1)));
-    CK(device_alloc(&S.d_perm, sizeof(int32_t) * 32 * std::max<int64_t>(S.nch, 1)));
+    R.chunks(S, d_val32 != nullptr, true);
+    S.n_long = (int32_t)(n - R.total[2]);
     CK(device_alloc(&S.d_long, sizeof(int32_t) * std::max<int64_t>(S.n_long, 1)));
     if (S.n_long)
-        CK(cudaMemcpy(S.d_long, row.p + tot[2], sizeof(int32_t) * S.n_long,
+        CK(cudaMemcpy(S.d_long, R.row.p + R.total[2], sizeof(int32_t) * S.n_long,
                       cudaMemcpyDeviceToDevice));
-    k_sell_cut<true><<<wblocks, 256>>>(key.p, row.p, n, nwin, nullptr, nullptr, och, osl, S.d_info,
-                                       S.d_perm, nullptr);
-    CK(cudaGetLastError());
-    // padded past the last slot: a block's bulk copy is widened to 16 bytes
-    auto al = [&](size_t sz, int fill = 0) {
-        void *q = nullptr;
-        CK(device_alloc(&q, sz * (size_t)std::max<int64_t>(slots, 1) + 256));
-        CK(cudaMemset(q, fill, sz * (size_t)std::max<int64_t>(slots, 1) + 256));
-        return q;
-    };
-    S.d_col = (uint32_t *)al(4, 0xff);  // kSellPad between chunks too
-    S.d_val = (double *)al(8);
-    if (d_val32) S.d_val32 = (float *)al(4);
     if (S.nch) {
         k_sell_fill<<<blocks_for(32 * S.nch), 256>>>(d_rp, d_col, d_val, d_val32, S.d_info,
                                                      S.d_perm, S.nch, S.d_col, S.d_val,
                                                      S.d_val32);
         CK(cudaGetLastError());
     }
-    if (win_off) win_off->swap(off);
 }
 
 // A block takes at most this much shared memory in FP64: four CTAs to an SM.
@@ -979,8 +999,8 @@ constexpr int64_t kWinLong512 = 140000000, kWinLong256 = 36000000;
 // One CTA per block of the staged windows.  The positions of a process's full
 // window (own rows, b_{l->l}, b_{nl->l}) that the block's rows use are marked in
 // a shared-memory bitmap; a position's slot is its rank among the marked ones.
-// COUNT: the size of the block's window.  FILL: its sources and the slot of
-// every stored entry of its sliced rows.
+// COUNT: the size of the block's window.  FILL: its sources, and the window slots and
+// values of its sliced rows (a warp per chunk).
 struct WinGeom {
     Part part;
     SellCut cut;
@@ -989,10 +1009,10 @@ struct WinGeom {
 };
 template <bool FILL>
 __global__ void k_win_block(const int32_t *rp, const uint32_t *col, WinGeom G, int64_t nblk,
-                            int32_t *nsrc, int32_t *nent, int32_t *stat, const int64_t *osl,
-                            const int64_t *osrc,
-                            const int32_t *bll_j, const int32_t *unp_src, const uint32_t *scol,
-                            uint32_t *src, uint16_t *col16)
+                            int32_t *nsrc, int32_t *nent, int32_t *stat, const int64_t *och,
+                            const int64_t *osrc, const int32_t *bll_j, const int32_t *unp_src,
+                            const double *val, const float *val32, SellPart S, uint32_t *src,
+                            uint16_t *col16)
 {
     extern __shared__ uint32_t bits[];  // [words], then (FILL) marked positions before each word
     __shared__ int warp_sum[8];         // 256 threads
@@ -1056,13 +1076,18 @@ __global__ void k_win_block(const int32_t *rp, const uint32_t *col, WinGeom G, i
                 }
             }
             __syncthreads();
-            for (int64_t q = osl[b] + tid; q < osl[b + 1]; q += blockDim.x) {
-                const uint32_t c = scol[q];
-                if (c == kSellPad) {
-                    col16[q] = kWinPad;
-                } else {
-                    const int32_t f = position(c);
+            for (int64_t c = och[b] + warp; c < och[b + 1]; c += blockDim.x >> 5) {
+                const int2 inf = S.d_info[c];
+                const int width = inf.y >> 6, nlane = inf.y & 63;
+                if (lane >= nlane) continue;
+                const int32_t i = S.d_perm[32 * c + lane], k0 = rp[i], len = rp[i + 1] - k0;
+                for (int k = 0; k < width; k++) {
+                    const int64_t q = (int64_t)inf.x + (int64_t)k * nlane + lane;
+                    if (k >= len) break;  // (the padding is there)
+                    const int32_t f = position(col[k0 + k]);
                     col16[q] = (uint16_t)(pre[f >> 5] + __popc(bits[f >> 5] & ((1u << (f & 31)) - 1)));
+                    S.d_val[q] = val[k0 + k];
+                    if (S.d_val32) S.d_val32[q] = val32[k0 + k];
                 }
             }
         }
@@ -1232,18 +1257,26 @@ int32_t *order_receives(napspmv_plan_t *P, Cub &cb, int64_t nblk, const int32_t 
     return send;
 }
 
-// Chooses the block size of the staged windows and builds them with the whole
-// matrix's sliced rows.  No windows (the sliced rows then keep their own): a
-// plan of composed gathers, a row of more than kSellLong entries, fewer than 64
-// rows per process, or blocks that do not fit the shared memory.
+void free_windows(WinPart &W)
+{
+    void *p[] = {W.d_col, W.d_blk, W.d_runs, W.d_send};
+    for (void *q : p)
+        if (q) cudaFree(q);
+    free_sell(W.rows);
+    W = WinPart();
+}
+
+// Chooses the block size of the staged windows and builds them, with sliced rows of
+// their own: those of the other engines are sorted over a whole process, where a
+// 20-entry row's chunks hold 2.3% padding against 15% over 128 rows.  (When the fused
+// engine took the windows' rows, a 150,000-row apply went from 50.5 to 59.5 us, a batch
+// of eight 100,000-row matrices from 130 to 143, the SpMV step of 10^6 rows from 74 to
+// 81.)  No windows: a plan of composed gathers, a row of more than kSellLong entries,
+// fewer than 64 rows per process, or blocks that do not fit the shared memory.
 void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *bll_ptr,
                    const int32_t *bnl_ptr, const int64_t *gs_off, int64_t n_msg)
 {
-    WinPart &W = P->win;
     const int64_t n = P->n;
-    auto plain = [&] {
-        build_sell(P, cb, 0, P->d_rowptr, P->d_colenc, P->d_val, P->d_val32, part);
-    };
     int64_t wide = 0;  // largest process window
     for (int64_t t = 0; t < part.np; t++)
         wide = std::max<int64_t>(wide, part.rows(t) + P->h_bll_rank[t + 1] - P->h_bll_rank[t] +
@@ -1252,7 +1285,10 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
     const int64_t max_rows = part.rows(0);
     if ((P->flags & NAPSPMV_COMPOSED_GATHERS) || n / part.np < 64 ||
         8 * words > 200 * 1024)
-        return plain();
+        return;
+    struct Made : WinPart {  // freed unless they become the plan's
+        ~Made() { free_windows(*this); }
+    } W;
     WinGeom G{part, SellCut(), (int32_t)words, bll_ptr, bnl_ptr};
     CK(cudaFuncSetAttribute((const void *)k_win_block<false>,
                             cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
@@ -1277,14 +1313,14 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
         CK(cudaMemset(nent.p, 0, sizeof(int32_t) * nblk));
         CK(cudaMemset(stat.p, 0, sizeof(st)));
         const int grid = (int)std::min<int64_t>(nblk, 1 << 20);
-        k_win_block<false><<<grid, 256, 4 * words>>>(P->d_rowptr, P->d_colenc, G, nblk, nsrc.p,
-                                                     nent.p, stat.p, nullptr, nullptr, nullptr,
-                                                     nullptr, nullptr, nullptr, nullptr);
+        k_win_block<false><<<grid, 256, 4 * words>>>(
+            P->d_rowptr, P->d_colenc, G, nblk, nsrc.p, nent.p, stat.p, nullptr, nullptr, nullptr,
+            nullptr, nullptr, nullptr, SellPart(), nullptr, nullptr);
         CK(cudaGetLastError());
         cb.max_i32(nsrc.p, stat.p + 1, nblk);
         cb.max_i32(nent.p, stat.p + 2, nblk);
         CK(cudaMemcpy(st, stat.p, sizeof(st), cudaMemcpyDeviceToHost));
-        if (st[0] > kSellLong) return plain();
+        if (st[0] > kSellLong) return;
         if (W.long_rows) {
             W.threads = 2 * std::max(64, G.cut.rows);
             fits = window_long_bytes(st[1], 8) <= kWinSmem &&
@@ -1295,13 +1331,14 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
         W.threads = sparse ? 2 * G.cut.rows : G.cut.rows;
         fits = window_bytes(st[1], st[2], st[1], 8) <= kWinBytes && !(sparse && rows > 128);
     }
-    if (!fits) return plain();
-    dvec<int64_t> off, wide_n(nblk + 1), osrc(nblk + 1), oword(nblk + 1);
+    if (!fits || st[1] >= kWinPad) return;
+    dvec<int64_t> wide_n(nblk + 1), osrc(nblk + 1), oword(nblk + 1);
     dvec<int32_t> nword(nblk);
-    build_sell(P, cb, 0, P->d_rowptr, P->d_colenc, P->d_val, P->d_val32, part, G.cut, &off);
-    if (P->sell[0].slots < 0) return;
+    const RowCut R(cb, P->d_rowptr, n, part, G.cut);
+    if (!R.fits()) return;
+    R.chunks(W.rows, P->d_val32 != nullptr, false);
     // the most slots a block has, padding included
-    k_win_slots<<<blocks_for(nblk), 256>>>(nblk, off.p + nblk + 1, nent.p);
+    k_win_slots<<<blocks_for(nblk), 256>>>(nblk, R.osl(), nent.p);
     CK(cudaGetLastError());
     cb.max_i32(nent.p, stat.p + 2, nblk);
     auto offsets = [&](const int32_t *cnt, dvec<int64_t> &o) {  // and their total
@@ -1313,45 +1350,47 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
         return total;
     };
     const int64_t total = offsets(nsrc.p, osrc);
-    const size_t slots = (size_t)std::max<int64_t>(P->sell[0].slots, 1);
-    dvec<uint32_t> src(std::max<int64_t>(total, 1));
+    if (W.long_rows && total > INT32_MAX) return;
+    // every window's sources: a temporary where they become runs
+    dvec<uint32_t> list(W.long_rows ? 0 : std::max<int64_t>(total, 1));
+    if (W.long_rows) CK(device_alloc(&W.d_runs, sizeof(uint32_t) * std::max<int64_t>(total, 1)));
+    uint32_t *src = W.long_rows ? W.d_runs : list.p;
+    const size_t slots = (size_t)std::max<int64_t>(W.rows.slots, 1);
     CK(device_alloc(&W.d_col, sizeof(uint16_t) * slots + 256));
+    CK(cudaMemset(W.d_col, 0xff, sizeof(uint16_t) * slots + 256));  // kWinPad
     const int grid = (int)std::min<int64_t>(nblk, 1 << 20);
     k_win_block<true><<<grid, 256, 8 * words>>>(
-        P->d_rowptr, P->d_colenc, G, nblk, nullptr, nullptr, nullptr, off.p + nblk + 1, osrc.p,
-        P->lists[L_BLL].d_idx, P->d_unp_src, P->sell[0].d_col, src.p, W.d_col);
+        P->d_rowptr, P->d_colenc, G, nblk, nullptr, nullptr, nullptr, R.och(), osrc.p,
+        P->lists[L_BLL].d_idx, P->d_unp_src, P->d_val, P->d_val32, W.rows, src, W.d_col);
     CK(cudaGetLastError());
-    if (st[1] >= kWinPad) return;
     CK(device_alloc(&W.d_blk, sizeof(WinBlock) * nblk));
     const int bgrid = (int)((nblk + 255) / 256);
     if (W.long_rows) {  // plain lists
-        if (total > INT32_MAX) return;
-        k_win_blocks<<<bgrid, 256>>>(nblk, off.p, off.p + nblk + 1, nsrc.p, nsrc.p, osrc.p, 1,
-                                     W.d_blk);
+        k_win_blocks<<<bgrid, 256>>>(nblk, R.och(), R.osl(), nsrc.p, nsrc.p, osrc.p, 1, W.d_blk);
         CK(cudaGetLastError());
-        W.d_send = order_receives(P, cb, nblk, nsrc.p, osrc.p, src.p, total, gs_off, n_msg);
-        W.d_runs = src.release();
+        W.d_send = order_receives(P, cb, nblk, nsrc.p, osrc.p, src, total, gs_off, n_msg);
+        CK(cudaMemcpy(st, stat.p, sizeof(st), cudaMemcpyDeviceToHost));
     } else {
         const int wgrid = blocks_for(32 * nblk);
-        k_win_runs<false><<<wgrid, 256>>>(nblk, src.p, osrc.p, nsrc.p, nword.p, nullptr, nullptr);
+        k_win_runs<false><<<wgrid, 256>>>(nblk, src, osrc.p, nsrc.p, nword.p, nullptr, nullptr);
         CK(cudaGetLastError());
         cb.max_i32(nword.p, stat.p + 3, nblk);
         const int64_t all = offsets(nword.p, oword);
         if (all / 4 > (int64_t)INT32_MAX) return;
         CK(device_alloc(&W.d_runs, sizeof(uint32_t) * std::max<int64_t>(all, 1)));
-        k_win_runs<true><<<wgrid, 256>>>(nblk, src.p, osrc.p, nsrc.p, nullptr, oword.p, W.d_runs);
+        k_win_runs<true><<<wgrid, 256>>>(nblk, src, osrc.p, nsrc.p, nullptr, oword.p, W.d_runs);
         CK(cudaGetLastError());
-        k_win_blocks<<<bgrid, 256>>>(nblk, off.p, off.p + nblk + 1, nsrc.p, nword.p, oword.p, 4,
-                                     W.d_blk);
+        k_win_blocks<<<bgrid, 256>>>(nblk, R.och(), R.osl(), nsrc.p, nword.p, oword.p, 4, W.d_blk);
         CK(cudaGetLastError());
         CK(cudaMemcpy(st, stat.p, sizeof(st), cudaMemcpyDeviceToHost));
         if (window_bytes(st[1], st[2], st[3], 8) > kWinSmem) return;
         W.max_words = st[3];
     }
-    W.rows = G.cut.rows;
     W.max_src = st[1];
     W.max_slots = st[2];
     W.blocks = (int32_t)nblk;
+    P->win = W;
+    static_cast<WinPart &>(W) = WinPart();
 }
 
 void build(napspmv_plan_t *P, const napspmv_csr *A)
@@ -1802,9 +1841,10 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
     CK(cudaDeviceSynchronize());
 
     // sliced-row copies of the whole matrix and of its two split parts
-    build_windows(P, cb, part, d_bll_ptr.p, d_bnl_ptr.p, d_gs_off.p, NM);
+    build_sell(P, cb, 0, P->d_rowptr, P->d_colenc, P->d_val, P->d_val32, part);
     build_sell(P, cb, 1, P->d_rowptrL, P->d_colL, P->d_valL, P->d_val32L, part);
     build_sell(P, cb, 2, P->d_rowptrR, P->d_colR, P->d_valR, P->d_val32R, part);
+    build_windows(P, cb, part, d_bll_ptr.p, d_bnl_ptr.p, d_gs_off.p, NM);
     CK(cudaDeviceSynchronize());
 
     host_stats(P);
@@ -1989,14 +2029,8 @@ void plan_free(napspmv_plan_t *P)
     if (P->ev_join) cudaEventDestroy(P->ev_join);
     for (void *p : ptrs)
         if (p) cudaFree(p);
-    for (auto &S : P->sell) {
-        void *sp[] = {S.d_info, S.d_perm, S.d_col, S.d_val, S.d_val32, S.d_long};
-        for (void *p : sp)
-            if (p) cudaFree(p);
-    }
-    void *wp[] = {P->win.d_col, P->win.d_blk, P->win.d_runs, P->win.d_send};
-    for (void *p : wp)
-        if (p) cudaFree(p);
+    for (auto &S : P->sell) free_sell(S);
+    free_windows(P->win);
     delete P;
     cudaSetDevice(cur);
 }
