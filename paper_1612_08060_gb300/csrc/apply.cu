@@ -1657,19 +1657,22 @@ __global__ void __launch_bounds__(NT) k_send(const __grid_constant__ SendJobs<MA
 
 // Both receive buffers from a kept vector, where *state is 1; the last CTA to finish
 // clears it (state[1]: their count), for the buffers are what a later step reads.
-template <class T>
+template <class T, class XS>
 __global__ void __launch_bounds__(NT)
-    k_receives(const double *x, const int32_t *bll_j, T *bll, int n_bll, const int32_t *bnl_j,
+    k_receives(const XS *x, const int32_t *bll_j, T *bll, int n_bll, const int32_t *bnl_j,
                T *bnl, int n_bnl, int *state, const int *err)
 {
     griddep_wait();
     if (*(volatile const int *)err || !*(volatile int *)state) return;
     const uint64_t pol = policy_evict_first();
     auto gather = [&](T *dst, const int32_t *idx, int b, int e) {
-        batched<8, T>(
-            b, e, threadIdx.x, [&](int k) { return (uint32_t)ld_stream_hint_s32(idx + k, pol); },
-            [&](int, uint32_t j) { return to_xt(T(0), __ldg(x + j)); },
-            [&](int k, uint32_t, T v) { dst[k] = v; });
+        if constexpr (sizeof(T) == sizeof(XS))
+            step_gather<false, 8, T>(dst, x, idx, b, e, threadIdx.x);
+        else
+            batched<8, T>(
+                b, e, threadIdx.x, [&](int k) { return (uint32_t)ld_stream_hint_s32(idx + k, pol); },
+                [&](int, uint32_t j) { return to_xt(T(0), __ldg(x + j)); },
+                [&](int k, uint32_t, T v) { dst[k] = v; });
     };
     const int64_t n = (int64_t)n_bll + n_bnl, per = NT * 8;
     for (int64_t b = blockIdx.x * per; b < n; b += gridDim.x * per) {
@@ -2082,6 +2085,7 @@ static void note_receives(napspmv_ws_t *ws, bool f32, bool vector, bool capturin
     ws->captured = ws->captured || capturing;
     ws->buf_f32 = f32 ? 1 : 0;
     ws->recv_vector = vector;
+    ws->stepped = false;
 }
 
 static FJob make_job(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, double *w, int reps,
@@ -2666,15 +2670,16 @@ static int window_launch(int count, const napspmv_plan_t *const *plans, WinJobs<
     return NAPSPMV_OK;
 }
 
-template <class T>
-static void receives_launch(const napspmv_plan_t *P, const napspmv_ws_t *ws, const double *x,
+template <class T, class XS>
+static void receives_launch(const napspmv_plan_t *P, const napspmv_ws_t *ws, const XS *x,
                             cudaStream_t s)
 {
-    // one resident wave: after a capture most launches find the buffers filled
+    // one resident wave: after a capture most launches find the buffers filled, and a
+    // fill sweeps x once (96 CTAs per SM, 10^6 rows of 20 entries: 73 us for 45)
     const int64_t n = P->n_bll + P->n_bnl;
     const int g = (int)std::max<int64_t>(1, std::min<int64_t>((n + NT * 8 - 1) / (NT * 8),
                                                               P->wave_gather[sizeof(T) == 4]));
-    launch_pdl(true, k_receives<T>, g, 0, s, x, (const int32_t *)P->lists[L_BLL].d_idx,
+    launch_pdl(true, k_receives<T, XS>, g, 0, s, x, (const int32_t *)P->lists[L_BLL].d_idx,
                reinterpret_cast<T *>(ws->bll), (int)P->n_bll,
                (const int32_t *)P->lists[L_BNL].d_idx, reinterpret_cast<T *>(ws->bnl),
                (int)P->n_bnl, ws->state, (const int *)ws->err);
@@ -3275,6 +3280,18 @@ extern "C" int napspmv_apply_noalloc(napspmv_plan_t *P, const double *v, double 
 
 // The three-block SpMV step alone (phase 5 / local_spmv over the three blocks),
 // on the receive buffers the workspace holds from its last apply.
+//
+// After a windowed apply it runs on the windows, which receive again what an apply that
+// filled the buffers had received.  For short rows that is faster than the sums from
+// filled buffers (128^3: 34 against 46 us), for long rows only in plans of few entries
+// (us per step on GB300 with FP64 values, windows / buffers, and with FP32 ones: 5 * 10^4
+// rows of 20 entries 9.4 / 14.6 and 18.3 / 18.8, 2.5 * 10^5 24.6 / 24.8 and 37 / 29, 10^6
+// 82 / 75 and 97 / 71, 4 * 10^6 378 / 303 and 338 / 246).  Above that the second step
+// after an apply (with FP32 values, whose apply gained less, the first) fills the
+// buffers, and it and those that follow sum from there.
+namespace nap {
+constexpr int64_t kStepFill64 = 6000000, kStepFill32 = 2000000;  // stored entries
+}
 extern "C" int napspmv_spmv_step(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, double *w,
                                  double scale, const napspmv_opts *opts, void *stream)
 {
@@ -3311,30 +3328,33 @@ extern "C" int napspmv_spmv_step(napspmv_plan_t *P, napspmv_ws_t *ws, const doub
     NAP_CUDA(cudaStreamIsCapturing(st, &cs));
     // a replay of this step comes after applies that the host does not know of now
     if (cs != cudaStreamCaptureStatusNone) W->captured = true;
-    if (o.window && W->recv_vector && !W->captured && W->recv_f32 == f32) {
-        // on the windows: on-node receives from the kept vector, off-node from g_recv.
-        // It receives again what an apply that filled the buffers had received: a step
-        // alone on 10^6 rows of 20 entries takes 88 us (73 from filled buffers), an
-        // apply and a step 188 (222).
+    // The kept vector and g_recv are those of the apply that the host saw last.
+    const bool kept = W->recv_vector && !W->captured;
+    // the FP32 copy that an apply of long rows made of its vector first is there too
+    const bool copy32 = kept && f32 && W->recv_f32 && P->win.long_rows;
+    const bool fill = P->win.long_rows && P->nnz >= (f32 ? kStepFill32 : kStepFill64) &&
+                      (f32 || W->stepped);
+    if (o.window && kept && W->recv_f32 == f32 && !fill) {
+        // on the windows: on-node receives from the kept vector, off-node from g_recv
         const void *x = v, *l = W->xtmp;
-        const bool convert = f32 && P->win.long_rows;  // as enqueue_windows
-        if (convert) {
-            to_f32(v, W->x32[0]);
-            to_f32(W->xtmp, W->x32[1]);
-            x = W->x32[0];
-            l = W->x32[1];
+        if (copy32) {  // as enqueue_windows
+            to_f32(v, W->x32[1]);
+            x = W->x32[1];
+            l = W->x32[0];
         }
         WinJobs<1> jobs{};
         jobs.job[0] = window_job(P, W, x, l, w, nullptr, scale);
         const napspmv_plan_t *pl[1] = {P};
-        if ((rc = window_launch<1>(1, pl, jobs, convert ? 1 : f32 ? 2 : 0, true, o, st))) return rc;
+        if ((rc = window_launch<1>(1, pl, jobs, copy32 ? 1 : f32 ? 2 : 0, true, o, st))) return rc;
         count_launch(1);
+        W->stepped = true;
     } else {
         if (P->win.blocks && (W->recv_vector || W->captured)) {
             // the receive buffers from the kept vector, if the device word says that
             // the last apply kept one; they are what a later step reads
-            if (f32) receives_launch<float>(P, W, W->xtmp, st);
-            else receives_launch<double>(P, W, W->xtmp, st);
+            if (copy32) receives_launch<float>(P, W, (const float *)W->x32[0], st);
+            else if (f32) receives_launch<float>(P, W, (const double *)W->xtmp, st);
+            else receives_launch<double>(P, W, (const double *)W->xtmp, st);
             count_launch(1);
             W->recv_vector = false;
             pdl = true;

@@ -179,7 +179,8 @@ struct napspmv_ws_s {
     // that ran kept its vector, 0 while the receive buffers hold its receives;
     // recv_vector is the same as the host sees it, which it does until the caller
     // captures an apply or a step of this workspace (captured).
-    bool recv_vector = false, recv_f32 = false, captured = false;
+    // stepped: a step has taken them on the windows.
+    bool recv_vector = false, recv_f32 = false, captured = false, stepped = false;
     int *state = nullptr;  // two words, see k_receives
     double *hv = nullptr, *hw = nullptr;  // staging of napspmv_apply_host
     unsigned long long *ctr = nullptr;  // the fused engine's grid barrier: arrivals, generation

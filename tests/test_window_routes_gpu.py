@@ -192,3 +192,32 @@ def test_largest_process_on_windows(rows, windows):
     assert (launches(plan, v, w) == 2) == windows
     nap.napspmv_apply_ex(plan, v, z, 1, 1.0, nap.make_opts(**TILES))
     assert np.array_equal(bits(w), bits(z))
+
+
+def test_repeated_steps_of_long_rows():
+    """From some millions of entries on, the second step after an apply (the first with FP32
+    values) fills the receive buffers, and later ones sum from there."""
+    plan = gpu_plan(near_and_far(350 * 1000 + 1, 900, 4, 3), 350, 16)
+    v, w, z = vec(plan.n, 1), vec(plan.n, 2), vec(plan.n, 3)
+    ws = nap.Workspace(plan)
+    for prec in (nap.PREC_F64, nap.PREC_F32):
+        def step(path, ws=None):
+            z.fill_(float("nan"))
+            before = nap.napspmv_launch_count()
+            nap.napspmv_spmv_step(plan, v, z, 1.0, nap.make_opts(precision=prec, **path), ws=ws)
+            return bits(z), nap.napspmv_launch_count() - before
+
+        for seed, reps in ((5, 1), (6, 1), (7, 3)):
+            x = vec(plan.n, seed)
+            nap.napspmv_apply_ex(plan, x, w, reps, 0.5, nap.make_opts(precision=prec, **TILES), ws=ws)
+            want = step(TILES, ws)[0]
+            nap.napspmv_apply_ex(plan, x, w, reps, 0.5, nap.make_opts(precision=prec))
+            counts = []
+            for _ in range(4):
+                got, n = step({})
+                assert np.array_equal(got, want), (prec, seed)
+                counts.append(n)
+            # (an FP32 step converts v first)
+            assert counts == ([1, 2, 1, 1] if prec == nap.PREC_F64 else [3, 2, 2, 2])
+            assert np.array_equal(step(TILES)[0], want)
+    assert nap.napspmv_status(plan) == 0
