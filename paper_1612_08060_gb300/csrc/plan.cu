@@ -178,6 +178,11 @@ struct Part {
     // first row of rank r (contiguous blocks only)
     __host__ __device__ int64_t start(int64_t r) const { return r * q + (r < rem ? r : rem); }
 };
+Part partition(const napspmv_plan_t *P)
+{
+    const int64_t q = P->n / P->np, rem = P->n % P->np;
+    return Part{q, rem, rem * (q + 1), P->np, (P->flags & NAPSPMV_PARTITION_STRIDED) != 0};
+}
 
 inline int blocks_for(int64_t n, int t = 256)
 {
@@ -1273,10 +1278,10 @@ void free_windows(WinPart &W)
 // of eight 100,000-row matrices from 130 to 143, the SpMV step of 10^6 rows from 74 to
 // 81.)  No windows: a plan of composed gathers, a row of more than kSellLong entries,
 // fewer than 64 rows per process, or blocks that do not fit the shared memory.
-void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *bll_ptr,
-                   const int32_t *bnl_ptr, const int64_t *gs_off, int64_t n_msg)
+void build_windows(napspmv_plan_t *P, Cub &cb)
 {
     const int64_t n = P->n;
+    const Part part = partition(P);
     int64_t wide = 0;  // largest process window
     for (int64_t t = 0; t < part.np; t++)
         wide = std::max<int64_t>(wide, part.rows(t) + P->h_bll_rank[t + 1] - P->h_bll_rank[t] +
@@ -1289,7 +1294,7 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
     struct Made : WinPart {  // freed unless they become the plan's
         ~Made() { free_windows(*this); }
     } W;
-    WinGeom G{part, SellCut(), (int32_t)words, bll_ptr, bnl_ptr};
+    WinGeom G{part, SellCut(), (int32_t)words, P->d_bll_rank, P->d_bnl_rank};
     CK(cudaFuncSetAttribute((const void *)k_win_block<false>,
                             cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     CK(cudaFuncSetAttribute((const void *)k_win_block<true>,
@@ -1368,7 +1373,11 @@ void build_windows(napspmv_plan_t *P, Cub &cb, const Part &part, const int32_t *
     if (W.long_rows) {  // plain lists
         k_win_blocks<<<bgrid, 256>>>(nblk, R.och(), R.osl(), nsrc.p, nsrc.p, osrc.p, 1, W.d_blk);
         CK(cudaGetLastError());
-        W.d_send = order_receives(P, cb, nblk, nsrc.p, osrc.p, src, total, gs_off, n_msg);
+        const HostList &In = P->lists[L_INTER];
+        dvec<int64_t> gs_off(In.m + 1);
+        if (P->n_gs)
+            CK(cudaMemcpy(gs_off.p, In.ptr.data(), sizeof(int64_t) * (In.m + 1), cudaMemcpyHostToDevice));
+        W.d_send = order_receives(P, cb, nblk, nsrc.p, osrc.p, src, total, gs_off.p, In.m);
         CK(cudaMemcpy(st, stat.p, sizeof(st), cudaMemcpyDeviceToHost));
     } else {
         const int wgrid = blocks_for(32 * nblk);
@@ -1399,8 +1408,7 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
     const int32_t np = P->np, ppn = P->ppn, nn = P->nn;
     Scratch scratch;  // outlives every temporary below
     Cub cb;
-    Part part{n / np, n % np, (n % np) * (n / np + 1), np,
-              (P->flags & NAPSPMV_PARTITION_STRIDED) != 0};
+    const Part part = partition(P);
     const int jb = bits_for(n - 1), rb = bits_for(np - 1), nb = bits_for(nn - 1);
     if (2 * rb + jb > 63)
         throw NapError{NAPSPMV_ERR_UNSUPPORTED, "N and n_p too large for 64-bit plan keys"};
@@ -1844,10 +1852,23 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
     build_sell(P, cb, 0, P->d_rowptr, P->d_colenc, P->d_val, P->d_val32, part);
     build_sell(P, cb, 1, P->d_rowptrL, P->d_colL, P->d_valL, P->d_val32L, part);
     build_sell(P, cb, 2, P->d_rowptrR, P->d_colR, P->d_valR, P->d_val32R, part);
-    build_windows(P, cb, part, d_bll_ptr.p, d_bnl_ptr.p, d_gs_off.p, NM);
     CK(cudaDeviceSynchronize());
 
     host_stats(P);
+}
+
+// The staged windows come last, when the build's temporaries are gone, and a plan that
+// the memory has room for only without them is one without them.
+void add_windows(napspmv_plan_t *P)
+{
+    try {
+        Scratch scratch;
+        Cub cb;
+        build_windows(P, cb);
+    } catch (const NapError &e) {
+        if (e.code != NAPSPMV_ERR_OOM) throw;
+        cudaGetLastError();
+    }
 }
 
 }  // namespace
@@ -1941,7 +1962,7 @@ int cut_tiles(napspmv_plan_t *P, int32_t tile_rows, int32_t tile_nnz)
         const int64_t n = P->n;
         const bool strided = (P->flags & NAPSPMV_PARTITION_STRIDED) != 0;
         TileCut C{};
-        C.part = Part{n / P->np, n % P->np, (n % P->np) * (n / P->np + 1), P->np, strided};
+        C.part = partition(P);
         C.n = n;
         int64_t all = 0;
         for (int q = 0; q < kTileLists; q++) {
@@ -2124,6 +2145,7 @@ int plan_create(const napspmv_csr *A, int32_t np, int32_t ppn, uint32_t flags,
         P->defaults.debug_stall = 0;
         rc = build_items(P, P->defaults.tile_rows, P->defaults.tile_nnz);
         if (rc) throw NapError{rc, "row-tile construction failed"};
+        add_windows(P);
         if ((rc = window_prepare(P))) throw NapError{rc, "staged windows"};
     } catch (const NapError &e) {
         plan_free(P);
