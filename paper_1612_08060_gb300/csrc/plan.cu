@@ -47,21 +47,34 @@ inline void ck(cudaError_t e, const char *what)
 // Temporaries of one plan build, on one stream: a block given back serves the next
 // request that fits it, and all are freed with the build.  About a hundred arrays
 // come and go, and each allocation and release of one synchronised the device:
-// about 3.4 of 12.4 ms of a 10^6-row 7-point plan (GB300).
+// about 3.4 of 12.4 ms of a 10^6-row 7-point plan (GB300).  A small build takes them
+// from one allocation (slab bytes), where some fifty of 3 us and as many releases were a
+// tenth of a 64 x 64 grid's plan.
+constexpr size_t kSlabMax = 8 << 20;
 struct Scratch {
     std::multimap<size_t, void *> idle;
+    char *slab = nullptr;
+    size_t slab_bytes = 0, used = 0;
     Scratch *outer = current;
     static thread_local Scratch *current;
-    Scratch() { current = this; }
+    explicit Scratch(size_t slab = 0) : slab_bytes(slab <= kSlabMax ? slab : 0) { current = this; }
     ~Scratch()
     {
         trim();
+        if (slab) cudaFree(slab);
         current = outer;
     }
+    bool in_slab(const void *p) const { return slab && p >= slab && p < slab + slab_bytes; }
     void trim()
     {
-        for (auto &b : idle) cudaFree(b.second);
-        idle.clear();
+        for (auto it = idle.begin(); it != idle.end();) {
+            if (in_slab(it->second)) {
+                ++it;
+            } else {
+                cudaFree(it->second);
+                it = idle.erase(it);
+            }
+        }
     }
     void *take(size_t &bytes)
     {
@@ -70,6 +83,16 @@ struct Scratch {
             void *p = it->second;
             bytes = it->first;
             idle.erase(it);
+            return p;
+        }
+        if (slab_bytes && !slab && cudaMalloc(&slab, slab_bytes) != cudaSuccess) {
+            cudaGetLastError();
+            slab = nullptr;
+            slab_bytes = 0;
+        }
+        if (used + bytes <= slab_bytes) {
+            void *p = slab + used;
+            used += bytes;
             return p;
         }
         void *p = nullptr;
@@ -104,6 +127,10 @@ struct dvec {
     size_t bytes = 0;  // of a block that came from the scratch
     dvec() = default;
     explicit dvec(int64_t count) { alloc(count); }
+    explicit dvec(const std::vector<T> &h) : dvec((int64_t)h.size())
+    {
+        if (n) CK(cudaMemcpy(p, h.data(), sizeof(T) * h.size(), cudaMemcpyHostToDevice));
+    }
     void alloc(int64_t count)
     {
         drop();
@@ -178,6 +205,8 @@ struct Part {
     // first row of rank r (contiguous blocks only)
     __host__ __device__ int64_t start(int64_t r) const { return r * q + (r < rem ? r : rem); }
 };
+// About what a build's temporaries take (see Scratch).
+size_t slab_for(int64_t n, int64_t nnz) { return (size_t)(64 * nnz + 64 * n); }
 Part partition(const napspmv_plan_t *P)
 {
     const int64_t q = P->n / P->np, rem = P->n % P->np;
@@ -574,12 +603,6 @@ struct Cub {
         if (dk.Current() != k.p) k.swap(k2);
         if (dv.Current() != v.p) v.swap(v2);
     }
-    void max_i32(const int32_t *in, int32_t *out, int64_t n)
-    {
-        size_t b = 0;
-        CK(cub::DeviceReduce::Max(nullptr, b, in, out, (int)n, st));
-        CK(cub::DeviceReduce::Max(temp(b), b, in, out, (int)n, st));
-    }
     template <class T>
     void exclusive_sum(const T *in, T *out, int64_t n)
     {
@@ -594,16 +617,67 @@ struct Cub {
         uniq.clear();
         len.clear();
         if (n == 0) return;
-        dvec<uint64_t> u(n);
-        dvec<int32_t> c(n);
+        // one array: the number of runs, the values, the lengths
+        dvec<uint64_t> all(1 + n + (n + 1) / 2);
+        int *m_out = reinterpret_cast<int *>(all.p);
+        uint64_t *u = all.p + 1;
+        int32_t *c = reinterpret_cast<int32_t *>(u + n);
         size_t b = 0;
-        CK(cub::DeviceRunLengthEncode::Encode(nullptr, b, in, u.p, c.p, num.p, (int)n, st));
-        CK(cub::DeviceRunLengthEncode::Encode(temp(b), b, in, u.p, c.p, num.p, (int)n, st));
-        int64_t m = read_num();
+        CK(cub::DeviceRunLengthEncode::Encode(nullptr, b, in, u, c, m_out, (int)n, st));
+        CK(cub::DeviceRunLengthEncode::Encode(temp(b), b, in, u, c, m_out, (int)n, st));
+        int m = 0;
+        if (n <= 8192) {  // a short list comes whole: three reads were 35 us, this is 17 (GB300)
+            std::vector<uint64_t> h(all.n);
+            CK(cudaMemcpy(h.data(), all.p, sizeof(uint64_t) * h.size(), cudaMemcpyDeviceToHost));
+            memcpy(&m, h.data(), sizeof(m));
+            uniq.assign(h.begin() + 1, h.begin() + 1 + m);
+            len.resize(m);
+            memcpy(len.data(), h.data() + 1 + n, sizeof(int32_t) * m);
+            return;
+        }
+        CK(cudaMemcpy(&m, m_out, sizeof(m), cudaMemcpyDeviceToHost));
         uniq.resize(m);
         len.resize(m);
-        CK(cudaMemcpy(uniq.data(), u.p, sizeof(uint64_t) * m, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(len.data(), c.p, sizeof(int32_t) * m, cudaMemcpyDeviceToHost));
+        CK(cudaMemcpy(uniq.data(), u, sizeof(uint64_t) * m, cudaMemcpyDeviceToHost));
+        CK(cudaMemcpy(len.data(), c, sizeof(int32_t) * m, cudaMemcpyDeviceToHost));
+    }
+};
+
+// Numbers on the device, brought to the host together: every read of its own stops the
+// stream, 9 to 16 us (GB300).
+struct Picked {
+    const void *p[32];
+    uint32_t wide;  // bit i: p[i] is of 64 bits
+};
+__global__ void k_pick(Picked P, int n, int64_t *out)
+{
+    const int i = threadIdx.x;
+    if (i < n)
+        out[i] = P.wide >> i & 1 ? *static_cast<const int64_t *>(P.p[i]) : *static_cast<const int32_t *>(P.p[i]);
+}
+struct Reads {
+    Picked P{};
+    int64_t *to[32];
+    int n = 0;
+    void ask(const int64_t *p, int64_t *h)
+    {
+        P.wide |= 1u << n;
+        P.p[n] = p;
+        to[n++] = h;
+    }
+    void ask(const int32_t *p, int64_t *h)
+    {
+        P.p[n] = p;
+        to[n++] = h;
+    }
+    void take()
+    {
+        dvec<int64_t> out(32);
+        int64_t h[32];
+        k_pick<<<1, 32>>>(P, n, out.p);
+        CK(cudaGetLastError());
+        CK(cudaMemcpy(h, out.p, sizeof(int64_t) * n, cudaMemcpyDeviceToHost));
+        for (int i = 0; i < n; i++) *to[i] = h[i];
     }
 };
 
@@ -654,12 +728,14 @@ __global__ void k_sell_cut(const uint64_t *key, const int32_t *row, int64_t n, i
     for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w <= nwin; w += warps) {
         int64_t lim[2];  // the window's rows in the sorted order
         for (int q = 0; q < 2; q++) {
+            // 32 probes a step: a load for every factor of 33
             int64_t lo = 0, hi = n;
             const uint64_t x = (uint64_t)(w + q) << kSellKeyBits;
             while (lo < hi) {
-                const int64_t mid = (lo + hi) >> 1;
-                if (key[mid] < x) lo = mid + 1;
-                else hi = mid;
+                const int64_t step = (hi - lo + 32) / 33, at = lo + (lane + 1) * step - 1;
+                const int below = __popc(__ballot_sync(0xffffffffu, at < hi && key[at] < x));
+                if (below < 32) hi = min(hi, lo + (below + 1) * step - 1);
+                lo += below * step;
             }
             lim[q] = lo;
         }
@@ -807,12 +883,24 @@ std::vector<int32_t> full_ptr(const HostList &L, int32_t np)
     return p;
 }
 
-int check_bad(const dvec<int> &bad, const char *what)
+// The flaws that kernels found so far, by their bits.
+void check(int64_t bad)
+{
+    static const char *const what[] = {"row_ptr must start at 0, never decrease and end at nnz",
+                                       "column index out of range [0, n)",
+                                       "an entry (i, j) is stored twice",
+                                       "internal: pack source missing from the aggregator buffer",
+                                       "internal: off-node column without a node-pair message",
+                                       "internal: column missing from its receive buffer",
+                                       "internal: off-node receive value without a node pair"};
+    for (int i = 0; i < 7; i++)
+        if (bad >> i & 1) throw NapError{NAPSPMV_ERR_ARG, what[i]};
+}
+void check(const dvec<int> &bad)
 {
     int h = 0;
     CK(cudaMemcpy(&h, bad.p, sizeof(int), cudaMemcpyDeviceToHost));
-    if (h) throw NapError{NAPSPMV_ERR_ARG, std::string(what)};
-    return 0;
+    check(h);
 }
 
 void host_stats(napspmv_plan_t *P)
@@ -897,12 +985,14 @@ struct RowCut {
     // per window, first chunk and first slot; the last element of each is the total;
     // then the first long row's position
     dvec<int64_t> off;
-    int64_t total[3];  // chunks, slots, rows of at most kSellLong entries
+    int64_t total[3] = {};  // chunks, slots, rows of at most kSellLong entries
     const int64_t *och() const { return off.p; }
     const int64_t *osl() const { return off.p + nwin + 1; }
     int wblocks() const { return blocks_for(32 * (nwin + 1)); }
 
-    RowCut(Cub &cb, const int32_t *d_rp, int64_t rows, const Part &part, const SellCut &cut = SellCut())
+    // (the totals are there once `reads` were taken)
+    RowCut(Cub &cb, Reads &reads, const int32_t *d_rp, int64_t rows, const Part &part,
+           const SellCut &cut = SellCut())
         : n(rows), nwin(cut.count(part, rows)), key(n), row(n), off(2 * (nwin + 1) + 1)
     {
         dvec<uint64_t> key2(n);
@@ -917,9 +1007,11 @@ struct RowCut {
         CK(cudaGetLastError());
         cb.exclusive_sum(nch, off.p, nwin + 1);
         cb.exclusive_sum(nsl, off.p + nwin + 1, nwin + 1);
-        CK(cudaMemcpy(&total[0], och() + nwin, sizeof(int64_t), cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(&total[1], osl() + nwin, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost));
+        reads.ask(och() + nwin, &total[0]);
+        reads.ask(osl() + nwin, &total[1]);
+        reads.ask(osl() + nwin + 1, &total[2]);
     }
+    RowCut(const RowCut &) = delete;
     // 31-bit slots
     bool fits() const { return total[1] <= (int64_t)INT32_MAX - 1024; }
     // the chunks, and room for their slots
@@ -932,17 +1024,15 @@ struct RowCut {
         k_sell_cut<true><<<wblocks(), 256>>>(key.p, row.p, n, nwin, nullptr, nullptr, och(), osl(),
                                              S.d_info, S.d_perm, nullptr);
         CK(cudaGetLastError());
-        // padded past the last slot: a block's bulk copy is widened to 16 bytes
-        auto al = [&](size_t sz, int fill) {
-            void *q = nullptr;
-            const size_t bytes = sz * (size_t)std::max<int64_t>(S.slots, 1) + 256;
-            CK(device_alloc(&q, bytes));
-            CK(cudaMemset(q, fill, bytes));
-            return q;
-        };
-        if (columns) S.d_col = (uint32_t *)al(4, 0xff);  // kSellPad between chunks too
-        S.d_val = (double *)al(8, 0);
-        if (f32) S.d_val32 = (float *)al(4, 0);
+        // padded past the last slot: a block's bulk copy is widened to 16 bytes; a value
+        // without a column is not used
+        const size_t n_slots = (size_t)std::max<int64_t>(S.slots, 1);
+        if (columns) {
+            CK(device_alloc(&S.d_col, 4 * n_slots + 256));
+            CK(cudaMemset(S.d_col, 0xff, 4 * n_slots + 256));  // kSellPad between chunks too
+        }
+        CK(device_alloc(&S.d_val, 8 * n_slots + 256));
+        if (f32) CK(device_alloc(&S.d_val32, 4 * n_slots + 256));
     }
 };
 
@@ -954,19 +1044,17 @@ void free_sell(SellPart &S)
     S = SellPart();
 }
 
-// Sliced-row copy of one matrix part (which: 0 whole, 1 local, 2 remote) from
-// its CSR, built on the device.  Windows: the rows of each process (contiguous
+// Sliced-row copy of one matrix part (0 whole, 1 local, 2 remote) from its cut CSR
+// rows, built on the device.  Windows: the rows of each process (contiguous
 // partition) or of each 1024-row block (strided).  Within a window, rows of at
 // most kSellLong entries are sorted by count, longest first (ties by row), and
 // cut into chunks of up to 32 whose counts are at least half the first one's;
 // longer rows are listed apart.  A part whose padded slots would not fit 31-bit
 // offsets is left without a sliced copy.
-void build_sell(napspmv_plan_t *P, Cub &cb, int which, const int32_t *d_rp, const uint32_t *d_col,
-                const double *d_val, const float *d_val32, const Part &part)
+void build_sell(SellPart &S, const RowCut &R, const int32_t *d_rp, const uint32_t *d_col,
+                const double *d_val, const float *d_val32)
 {
-    SellPart &S = P->sell[which];
-    const int64_t n = P->n;
-    RowCut R(cb, d_rp, n, part);
+    const int64_t n = R.n;
     if (!R.fits()) {
         S.slots = -1;  // no sliced copy: NAPSPMV_PIPELINE_SELL is refused for this plan
         return;
@@ -1014,13 +1102,13 @@ struct WinGeom {
 };
 template <bool FILL>
 __global__ void k_win_block(const int32_t *rp, const uint32_t *col, WinGeom G, int64_t nblk,
-                            int32_t *nsrc, int32_t *nent, int32_t *stat, const int64_t *och,
+                            int32_t *nsrc, int32_t *stat, const int64_t *och,
                             const int64_t *osrc, const int32_t *bll_j, const int32_t *unp_src,
                             const double *val, const float *val32, SellPart S, uint32_t *src,
                             uint16_t *col16)
 {
     extern __shared__ uint32_t bits[];  // [words], then (FILL) marked positions before each word
-    __shared__ int warp_sum[8];         // 256 threads
+    __shared__ int warp_sum[8], block_entries;  // 256 threads
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int64_t b = blockIdx.x; b < nblk; b += gridDim.x) {
         const int64_t t = b / G.cut.nsub, sub = b % G.cut.nsub;
@@ -1035,6 +1123,7 @@ __global__ void k_win_block(const int32_t *rp, const uint32_t *col, WinGeom G, i
             return blkno == 1 ? own + k - l0 : own + nl + k - r0;
         };
         for (int w = tid; w < words; w += blockDim.x) bits[w] = 0;
+        if (tid == 0) block_entries = 0;
         __syncthreads();
         const int32_t k1 = min(own, (int32_t)(sub + 1) * G.cut.rows);
         int longest = 0, entries = 0;
@@ -1064,9 +1153,14 @@ __global__ void k_win_block(const int32_t *rp, const uint32_t *col, WinGeom G, i
         int before = incl - mine;
         for (int w = 0; w < warp; w++) before += warp_sum[w];
         if (!FILL) {
-            if (tid == blockDim.x - 1) nsrc[b] = before + mine;
             if (lane == 0 && longest) atomicMax(&stat[0], longest);
-            if (lane == 0 && entries) atomicAdd(&nent[b], entries);
+            if (lane == 0 && entries) atomicAdd(&block_entries, entries);
+            __syncthreads();
+            if (tid == blockDim.x - 1) {
+                nsrc[b] = before + mine;
+                atomicMax(&stat[1], before + mine);
+                atomicMax(&stat[2], block_entries);
+            }
         } else {
             uint32_t *pre = bits + G.words;
             const int64_t s0 = osrc[b];
@@ -1104,8 +1198,8 @@ __global__ void k_win_block(const int32_t *rp, const uint32_t *col, WinGeom G, i
 // COUNT: words needed, a multiple of 4.  WRITE: the runs.
 template <bool WRITE>
 __global__ void k_win_runs(int64_t nblk, const uint32_t *src, const int64_t *osrc,
-                           const int32_t *nsrc, int32_t *words, const int64_t *oword,
-                           uint32_t *runs)
+                           const int32_t *nsrc, int32_t *words, int32_t *most,
+                           const int64_t *oword, uint32_t *runs)
 {
     const int lane = threadIdx.x & 31;
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1127,7 +1221,10 @@ __global__ void k_win_runs(int64_t nblk, const uint32_t *src, const int64_t *osr
             }
             r += __popc(m);
         }
-        if (!WRITE && lane == 0) words[b] = (2 * tiles + (int)r + 3) & ~3;
+        if (!WRITE && lane == 0) {
+            words[b] = (2 * tiles + (int)r + 3) & ~3;
+            atomicMax(most, words[b]);
+        }
     }
 }
 
@@ -1147,11 +1244,14 @@ __global__ void k_win_blocks(int64_t nblk, const int64_t *och, const int64_t *os
     B.word0 = (int32_t)(oword[b] / unit);
     blk[b] = B;
 }
-__global__ void k_win_slots(int64_t nblk, const int64_t *osl, int32_t *slots)
+__global__ void k_win_slots(int64_t nblk, const int64_t *osl, int32_t *most)
 {
+    int32_t m = 0;
     for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nblk;
          b += (int64_t)gridDim.x * blockDim.x)
-        slots[b] = (int32_t)(osl[b + 1] - osl[b]);
+        m = max(m, (int32_t)(osl[b + 1] - osl[b]));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(most, m);
 }
 __global__ void k_widen(const int32_t *in, int64_t n, int64_t *out)  // out[n] = 0
 {
@@ -1299,9 +1399,9 @@ void build_windows(napspmv_plan_t *P, Cub &cb)
                             cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     CK(cudaFuncSetAttribute((const void *)k_win_block<true>,
                             cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    dvec<int32_t> nsrc, nent, stat(4);  // per block; longest row, largest window, most entries, words
+    dvec<int32_t> nsrc, stat(5);  // per block; longest row, largest window, most entries, slots, words
     int64_t nblk = 0;
-    int32_t st[4] = {};
+    int32_t st[5] = {};
     bool fits = false;
     W.long_rows = P->nnz > 12 * n;
     int rows = !W.long_rows                           ? 256
@@ -1314,16 +1414,12 @@ void build_windows(napspmv_plan_t *P, Cub &cb)
         nblk = part.np * G.cut.nsub;
         if (nblk >= (1ll << 31) - 1) break;
         nsrc.alloc(nblk);
-        nent.alloc(nblk);
-        CK(cudaMemset(nent.p, 0, sizeof(int32_t) * nblk));
         CK(cudaMemset(stat.p, 0, sizeof(st)));
         const int grid = (int)std::min<int64_t>(nblk, 1 << 20);
         k_win_block<false><<<grid, 256, 4 * words>>>(
-            P->d_rowptr, P->d_colenc, G, nblk, nsrc.p, nent.p, stat.p, nullptr, nullptr, nullptr,
-            nullptr, nullptr, nullptr, SellPart(), nullptr, nullptr);
+            P->d_rowptr, P->d_colenc, G, nblk, nsrc.p, stat.p, nullptr, nullptr, nullptr, nullptr,
+            nullptr, nullptr, SellPart(), nullptr, nullptr);
         CK(cudaGetLastError());
-        cb.max_i32(nsrc.p, stat.p + 1, nblk);
-        cb.max_i32(nent.p, stat.p + 2, nblk);
         CK(cudaMemcpy(st, stat.p, sizeof(st), cudaMemcpyDeviceToHost));
         if (st[0] > kSellLong) return;
         if (W.long_rows) {
@@ -1339,22 +1435,23 @@ void build_windows(napspmv_plan_t *P, Cub &cb)
     if (!fits || st[1] >= kWinPad) return;
     dvec<int64_t> wide_n(nblk + 1), osrc(nblk + 1), oword(nblk + 1);
     dvec<int32_t> nword(nblk);
-    const RowCut R(cb, P->d_rowptr, n, part, G.cut);
-    if (!R.fits()) return;
-    R.chunks(W.rows, P->d_val32 != nullptr, false);
+    Reads reads;
+    const RowCut R(cb, reads, P->d_rowptr, n, part, G.cut);
     // the most slots a block has, padding included
-    k_win_slots<<<blocks_for(nblk), 256>>>(nblk, R.osl(), nent.p);
+    k_win_slots<<<blocks_for(nblk), 256>>>(nblk, R.osl(), stat.p + 3);
     CK(cudaGetLastError());
-    cb.max_i32(nent.p, stat.p + 2, nblk);
-    auto offsets = [&](const int32_t *cnt, dvec<int64_t> &o) {  // and their total
+    auto offsets = [&](const int32_t *cnt, dvec<int64_t> &o) {  // their total last
         k_widen<<<blocks_for(nblk + 1), 256>>>(cnt, nblk, wide_n.p);
         CK(cudaGetLastError());
         cb.exclusive_sum(wide_n.p, o.p, nblk + 1);
-        int64_t total = 0;
-        CK(cudaMemcpy(&total, o.p + nblk, sizeof(total), cudaMemcpyDeviceToHost));
-        return total;
+        return o.p + nblk;
     };
-    const int64_t total = offsets(nsrc.p, osrc);
+    int64_t total = 0, max_slots = 0;
+    reads.ask(offsets(nsrc.p, osrc), &total);
+    reads.ask(stat.p + 3, &max_slots);
+    reads.take();
+    if (!R.fits()) return;
+    R.chunks(W.rows, P->d_val32 != nullptr, false);
     if (W.long_rows && total > INT32_MAX) return;
     // every window's sources: a temporary where they become runs
     dvec<uint32_t> list(W.long_rows ? 0 : std::max<int64_t>(total, 1));
@@ -1365,7 +1462,7 @@ void build_windows(napspmv_plan_t *P, Cub &cb)
     CK(cudaMemset(W.d_col, 0xff, sizeof(uint16_t) * slots + 256));  // kWinPad
     const int grid = (int)std::min<int64_t>(nblk, 1 << 20);
     k_win_block<true><<<grid, 256, 8 * words>>>(
-        P->d_rowptr, P->d_colenc, G, nblk, nullptr, nullptr, nullptr, R.och(), osrc.p,
+        P->d_rowptr, P->d_colenc, G, nblk, nullptr, nullptr, R.och(), osrc.p,
         P->lists[L_BLL].d_idx, P->d_unp_src, P->d_val, P->d_val32, W.rows, src, W.d_col);
     CK(cudaGetLastError());
     CK(device_alloc(&W.d_blk, sizeof(WinBlock) * nblk));
@@ -1374,29 +1471,30 @@ void build_windows(napspmv_plan_t *P, Cub &cb)
         k_win_blocks<<<bgrid, 256>>>(nblk, R.och(), R.osl(), nsrc.p, nsrc.p, osrc.p, 1, W.d_blk);
         CK(cudaGetLastError());
         const HostList &In = P->lists[L_INTER];
-        dvec<int64_t> gs_off(In.m + 1);
-        if (P->n_gs)
-            CK(cudaMemcpy(gs_off.p, In.ptr.data(), sizeof(int64_t) * (In.m + 1), cudaMemcpyHostToDevice));
+        const dvec<int64_t> gs_off(In.ptr);
         W.d_send = order_receives(P, cb, nblk, nsrc.p, osrc.p, src, total, gs_off.p, In.m);
-        CK(cudaMemcpy(st, stat.p, sizeof(st), cudaMemcpyDeviceToHost));
     } else {
         const int wgrid = blocks_for(32 * nblk);
-        k_win_runs<false><<<wgrid, 256>>>(nblk, src, osrc.p, nsrc.p, nword.p, nullptr, nullptr);
+        k_win_runs<false><<<wgrid, 256>>>(nblk, src, osrc.p, nsrc.p, nword.p, stat.p + 4, nullptr,
+                                            nullptr);
         CK(cudaGetLastError());
-        cb.max_i32(nword.p, stat.p + 3, nblk);
-        const int64_t all = offsets(nword.p, oword);
-        if (all / 4 > (int64_t)INT32_MAX) return;
+        int64_t all = 0, max_words = 0;
+        Reads more;
+        more.ask(offsets(nword.p, oword), &all);
+        more.ask(stat.p + 4, &max_words);
+        more.take();
+        if (all / 4 > (int64_t)INT32_MAX || window_bytes(st[1], max_slots, max_words, 8) > kWinSmem)
+            return;
+        W.max_words = (int32_t)max_words;
         CK(device_alloc(&W.d_runs, sizeof(uint32_t) * std::max<int64_t>(all, 1)));
-        k_win_runs<true><<<wgrid, 256>>>(nblk, src, osrc.p, nsrc.p, nullptr, oword.p, W.d_runs);
+        k_win_runs<true><<<wgrid, 256>>>(nblk, src, osrc.p, nsrc.p, nullptr, nullptr, oword.p,
+                                           W.d_runs);
         CK(cudaGetLastError());
         k_win_blocks<<<bgrid, 256>>>(nblk, R.och(), R.osl(), nsrc.p, nword.p, oword.p, 4, W.d_blk);
         CK(cudaGetLastError());
-        CK(cudaMemcpy(st, stat.p, sizeof(st), cudaMemcpyDeviceToHost));
-        if (window_bytes(st[1], st[2], st[3], 8) > kWinSmem) return;
-        W.max_words = st[3];
     }
     W.max_src = st[1];
-    W.max_slots = st[2];
+    W.max_slots = (int32_t)max_slots;
     W.blocks = (int32_t)nblk;
     P->win = W;
     static_cast<WinPart &>(W) = WinPart();
@@ -1406,7 +1504,6 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
 {
     const int64_t n = A->n, nnz = A->nnz;
     const int32_t np = P->np, ppn = P->ppn, nn = P->nn;
-    Scratch scratch;  // outlives every temporary below
     Cub cb;
     const Part part = partition(P);
     const int jb = bits_for(n - 1), rb = bits_for(np - 1), nb = bits_for(nn - 1);
@@ -1426,11 +1523,11 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
     CK(cudaMemset(bad.p, 0, sizeof(int)));
     k_check_rowptr<<<blocks_for(n), 256>>>(rp.p, n, nnz, bad.p);
     CK(cudaGetLastError());
-    check_bad(bad, "row_ptr must start at 0, never decrease and end at nnz");
+    check(bad);
     dvec<int32_t> row_of(nnz);
     k_row_of<<<blocks_for(n), 256>>>(rp.p, n, col.p, row_of.p, bad.p);
     CK(cudaGetLastError());
-    check_bad(bad, "column index out of range [0, n)");
+    check(bad);
 
     dvec<uint64_t> keys(nnz), alt(nnz);
     if (nnz) {
@@ -1439,7 +1536,6 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
         cb.sort(keys.p, alt.p, nnz, 2 * jb);
         k_adjacent_equal<<<blocks_for(nnz), 256>>>(keys.p, nnz, bad.p);
         CK(cudaGetLastError());
-        check_bad(bad, "an entry (i, j) is stored twice");
     }
 
     // ---- classify; the standard plan (Eqs. P, D)
@@ -1451,11 +1547,17 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
                                              keys.p, blk.p);
         CK(cudaGetLastError());
     }
-    unsigned long long hb[3];
-    CK(cudaMemcpy(hb, blk.p, sizeof(hb), cudaMemcpyDeviceToHost));
-    P->stats.nnz_on_process = (int64_t)hb[0];
-    P->stats.nnz_on_node = (int64_t)hb[1];
-    P->stats.nnz_off_node = (int64_t)hb[2];
+    {
+        Reads reads;
+        int64_t flaw = 0;
+        reads.ask(bad.p, &flaw);
+        const int64_t *entries = reinterpret_cast<const int64_t *>(blk.p);
+        reads.ask(entries, &P->stats.nnz_on_process);
+        reads.ask(entries + 1, &P->stats.nnz_on_node);
+        reads.ask(entries + 2, &P->stats.nnz_off_node);
+        reads.take();
+        check(flaw);
+    }
     row_of.alloc(0);
 
     int64_t c = cb.select(keys.p, nnz, alt.p, NotSent{});
@@ -1532,12 +1634,9 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
             CK(cudaMemset(cr.p, 0, sizeof(int32_t) * M * ppn));
             std::vector<uint64_t> pk(M);
             for (int64_t k = 0; k < M; k++) pk[k] = ((uint64_t)ND.src[k] << nb) | (uint64_t)ND.dst[k];
-            dvec<int64_t> d_ptr;
-            d_ptr.p = upload(ND.ptr);
-            dvec<int32_t> d_src;
-            d_src.p = upload(ND.src);
-            dvec<uint64_t> d_pk;
-            d_pk.p = upload(pk);
+            const dvec<int64_t> d_ptr(ND.ptr);
+            const dvec<int32_t> d_src(ND.src);
+            const dvec<uint64_t> d_pk(pk);
             k_major_send<<<blocks_for(ND.total), 256>>>(ND.d_idx, ND.total, d_ptr.p, M, d_src.p,
                                                        part, ppn, cs.p);
             CK(cudaGetLastError());
@@ -1546,7 +1645,7 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
                                                            part, ppn, cr.p, bad.p);
                 CK(cudaGetLastError());
             }
-            check_bad(bad, "internal: off-node receive value without a node pair");
+            check(bad);
             std::vector<int32_t> hs(M * ppn), hr(M * ppn);
             CK(cudaMemcpy(hs.data(), cs.p, sizeof(int32_t) * M * ppn, cudaMemcpyDeviceToHost));
             CK(cudaMemcpy(hr.data(), cr.p, sizeof(int32_t) * M * ppn, cudaMemcpyDeviceToHost));
@@ -1693,15 +1792,8 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
     }
     std::vector<int32_t> node_ptr32(M + 1);
     for (int64_t k = 0; k <= M; k++) node_ptr32[k] = (int32_t)ND.ptr[k];
-    dvec<int64_t> d_gs_off;
-    d_gs_off.p = upload(gs_off);
-    dvec<int32_t> d_msg_pair, d_msg_src, d_node_ptr;
-    d_msg_pair.p = upload(msg_pair);
-    d_msg_src.p = upload(msg_src);
-    d_node_ptr.p = upload(node_ptr32);
-    dvec<int64_t> d_msg_gr, d_msg_lo;
-    d_msg_gr.p = upload(msg_gr);
-    d_msg_lo.p = upload(msg_lo);
+    const dvec<int64_t> d_gs_off(gs_off), d_msg_gr(msg_gr), d_msg_lo(msg_lo);
+    const dvec<int32_t> d_msg_pair(msg_pair), d_msg_src(msg_src), d_node_ptr(node_ptr32);
 
     const int64_t ngs = P->n_gs;
     dvec<int32_t> msg_of(ngs);
@@ -1747,17 +1839,13 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
     P->h_bnl_rank = bnl_ptr;
     P->d_bll_rank = upload(bll_ptr);
     P->d_bnl_rank = upload(bnl_ptr);
-    dvec<int32_t> d_lbuf_ptr, d_bll_ptr, d_bnl_ptr;
-    d_lbuf_ptr.p = upload(lbuf_ptr);
-    d_bll_ptr.p = upload(bll_ptr);
-    d_bnl_ptr.p = upload(bnl_ptr);
+    const dvec<int32_t> d_lbuf_ptr(lbuf_ptr);
     if (ngs) {
         CK(device_alloc(&P->d_pack_src, sizeof(uint32_t) * ngs));
         k_pack_src<<<blocks_for(ngs), 256>>>(ngs, P->lists[L_INTER].d_idx, msg_of.p, d_msg_src.p,
                                             d_lbuf_ptr.p, P->lists[L_LBUF].d_idx, part,
                                             P->d_pack_src, bad.p);
         CK(cudaGetLastError());
-        check_bad(bad, "internal: pack source missing from the aggregator buffer");
     }
     msg_of.alloc(0);
 
@@ -1765,14 +1853,9 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
     const int64_t nbnl = P->n_bnl;
     std::vector<uint64_t> pair_key(M);
     for (int64_t k = 0; k < M; k++) pair_key[k] = ((uint64_t)ND.src[k] << nb) | ND.dst[k];
-    dvec<uint64_t> d_pair_key;
-    d_pair_key.p = upload(pair_key);
-    dvec<int64_t> d_pair_piece, d_piece_lo, d_piece_gr;
-    dvec<int32_t> d_piece_dst;
-    d_pair_piece.p = upload(pair_piece);
-    d_piece_lo.p = upload(piece_lo);
-    d_piece_gr.p = upload(piece_gr);
-    d_piece_dst.p = upload(piece_dst);
+    const dvec<uint64_t> d_pair_key(pair_key);
+    const dvec<int64_t> d_pair_piece(pair_piece), d_piece_lo(piece_lo), d_piece_gr(piece_gr);
+    const dvec<int32_t> d_piece_dst(piece_dst);
     dvec<uint64_t> j1key(nbnl), j1alt(nbnl);
     if (nbnl) {
         CK(device_alloc(&P->d_unp_src, sizeof(int32_t) * nbnl));
@@ -1781,7 +1864,7 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
                                                d_piece_dst.p, d_piece_gr.p, d_node_ptr.p,
                                                ND.d_idx, rb, j1key.p, P->d_unp_src, bad.p);
         CK(cudaGetLastError());
-        check_bad(bad, "internal: off-node column without a node-pair message");
+        check(bad);
     }
     int64_t nj1 = cb.select(j1key.p, nbnl, j1alt.p, NotSent{});
     cb.sort(j1alt.p, j1key.p, nj1, 2 * rb + jb);
@@ -1799,12 +1882,11 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
     CK(device_alloc(&P->d_split, sizeof(int32_t) * 3 * n));
     if (P->flags & NAPSPMV_F32_VALUES)
         CK(device_alloc(&P->d_val32, sizeof(float) * std::max<int64_t>(nnz, 1) + 64));
-    k_three_block<<<blocks_for(n), 256>>>(rp.p, n, col.p, val.p, tag.p, part, d_bll_ptr.p,
-                                         P->lists[L_BLL].d_idx, d_bnl_ptr.p,
+    k_three_block<<<blocks_for(n), 256>>>(rp.p, n, col.p, val.p, tag.p, part, P->d_bll_rank,
+                                         P->lists[L_BLL].d_idx, P->d_bnl_rank,
                                          P->lists[L_BNL].d_idx, P->d_colenc, P->d_val,
                                          P->d_val32, P->d_split, P->d_rowptr, bad.p);
     CK(cudaGetLastError());
-    check_bad(bad, "internal: column missing from its receive buffer");
 
     // ---- local / remote split
     {
@@ -1846,23 +1928,31 @@ void build(napspmv_plan_t *P, const napspmv_csr *A)
         CK(cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming));
         CK(cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming));
     }
-    CK(cudaDeviceSynchronize());
 
     // sliced-row copies of the whole matrix and of its two split parts
-    build_sell(P, cb, 0, P->d_rowptr, P->d_colenc, P->d_val, P->d_val32, part);
-    build_sell(P, cb, 1, P->d_rowptrL, P->d_colL, P->d_valL, P->d_val32L, part);
-    build_sell(P, cb, 2, P->d_rowptrR, P->d_colR, P->d_valR, P->d_val32R, part);
+    {
+        Reads reads;
+        int64_t flaw = 0;
+        reads.ask(bad.p, &flaw);
+        const RowCut all(cb, reads, P->d_rowptr, n, part), local(cb, reads, P->d_rowptrL, n, part),
+            remote(cb, reads, P->d_rowptrR, n, part);
+        reads.take();
+        check(flaw);
+        build_sell(P->sell[0], all, P->d_rowptr, P->d_colenc, P->d_val, P->d_val32);
+        build_sell(P->sell[1], local, P->d_rowptrL, P->d_colL, P->d_valL, P->d_val32L);
+        build_sell(P->sell[2], remote, P->d_rowptrR, P->d_colR, P->d_valR, P->d_val32R);
+    }
     CK(cudaDeviceSynchronize());
 
     host_stats(P);
 }
 
-// The staged windows come last, when the build's temporaries are gone, and a plan that
-// the memory has room for only without them is one without them.
+// The staged windows come last, when the build's temporaries make room for them (see
+// device_alloc), and a plan that the memory has room for only without them is one
+// without them.
 void add_windows(napspmv_plan_t *P)
 {
     try {
-        Scratch scratch;
         Cub cb;
         build_windows(P, cb);
     } catch (const NapError &e) {
@@ -1880,7 +1970,7 @@ void add_windows(napspmv_plan_t *P)
 // row, took 5.1 of 17.6 ms of a 10^6-row 7-point plan, and their three row pointers
 // 0.8 ms to bring there; this way 0.65 ms (GB300).
 namespace {
-constexpr int kSegment = 16384;
+constexpr int kSegment = 16384, kStaged = 1024;
 struct TileCut {
     const int32_t *rp[kTileLists];
     int32_t rows[kTileLists], cap[kTileLists];
@@ -1893,7 +1983,8 @@ struct TileCut {
 template <bool WRITE>
 __global__ void k_cut_tiles(TileCut C, int32_t *count, const int64_t *off, int32_t *fit, Item *items)
 {
-    const int list = blockIdx.y, lane = threadIdx.x & 31;
+    __shared__ int32_t staged[8][kStaged];  // a warp's row pointers: its tiles follow one another
+    const int list = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int32_t *rp = C.rp[list];
     const int32_t rows = C.rows[list], cap = C.cap[list];
     int64_t base = 0;  // of this list among all segments
@@ -1914,13 +2005,23 @@ __global__ void k_cut_tiles(TileCut C, int32_t *count, const int64_t *off, int32
         }
         int64_t at = WRITE ? off[base + s] : 0;
         int32_t most = 0, tall = 0;
+        int64_t s0 = r;  // staged: row pointers s0 .. s0 + kStaged - 1
+        auto stage = [&](int64_t from) {
+            __syncwarp();
+            s0 = from;
+            for (int k = lane; k < kStaged; k += 32) staged[warp][k] = rp[min(s0 + k, e)];
+            __syncwarp();
+        };
+        auto ptr = [&](int64_t i) { return i - s0 < kStaged ? staged[warp][i - s0] : rp[i]; };
+        if (r < e) stage(r);
         while (r < e) {
-            const int32_t k0 = rp[r];
             const int32_t limit = (int32_t)min((int64_t)rows, e - r);
+            if (r - s0 + limit >= kStaged && r > s0) stage(r);
+            const int32_t k0 = ptr(r);
             int32_t m = 0;  // rows of the tile
             for (;;) {
                 const int32_t i = m + lane + 1;
-                const unsigned ok = __ballot_sync(0xffffffffu, i <= limit && rp[r + min(i, limit)] - k0 <= cap);
+                const unsigned ok = __ballot_sync(0xffffffffu, i <= limit && ptr(r + min(i, limit)) - k0 <= cap);
                 if (ok == 0xffffffffu) {
                     m += 32;
                     continue;
@@ -1929,7 +2030,7 @@ __global__ void k_cut_tiles(TileCut C, int32_t *count, const int64_t *off, int32
                 break;
             }
             m = max(m, 1);
-            const int32_t k1 = rp[r + m];
+            const int32_t k1 = ptr(r + m);
             if (WRITE && lane == 0) {
                 Item it{};
                 it.kind = kSpmv;
@@ -1993,13 +2094,14 @@ int cut_tiles(napspmv_plan_t *P, int32_t tile_rows, int32_t tile_nnz)
         k_widen<<<blocks_for(all + 1), 256>>>(count.p, all, wide.p);
         CK(cudaGetLastError());
         cb.exclusive_sum(wide.p, off.p, all + 1);
-        int64_t first[kTileLists + 1], base = 0;
-        int32_t hf[2 * kTileLists];
+        int64_t first[kTileLists + 1], hf[2 * kTileLists], base = 0;
+        Reads reads;
         for (int q = 0; q <= kTileLists; q++) {
-            CK(cudaMemcpyAsync(&first[q], off.p + base, sizeof(int64_t), cudaMemcpyDeviceToHost));
+            reads.ask(off.p + base, &first[q]);
             if (q < kTileLists) base += C.segs[q];
         }
-        CK(cudaMemcpy(hf, fit.p, sizeof(hf), cudaMemcpyDeviceToHost));
+        for (int q = 0; q < 2 * kTileLists; q++) reads.ask(fit.p + q, &hf[q]);
+        reads.take();
         Item *d = nullptr;
         CK(device_alloc(&d, sizeof(Item) * std::max<int64_t>(first[kTileLists], 1)));
         k_cut_tiles<true><<<grid, 256>>>(C, nullptr, off.p, nullptr, d);
@@ -2014,8 +2116,8 @@ int cut_tiles(napspmv_plan_t *P, int32_t tile_rows, int32_t tile_nnz)
             L.d = d + first[q];
             L.n = (int32_t)(first[q + 1] - first[q]);
             // the stage the list needs: its largest tile that is staged at all
-            L.fit_nnz = std::min(C.cap[q], (std::max(32, hf[2 * q]) + 15) & ~15);
-            L.fit_rows = std::max(1, hf[2 * q + 1]);
+            L.fit_nnz = std::min(C.cap[q], (std::max(32, (int32_t)hf[2 * q]) + 15) & ~15);
+            L.fit_rows = std::max(1, (int32_t)hf[2 * q + 1]);
         }
         S.tile_rows = tile_rows;
         S.tile_nnz = tile_nnz;
@@ -2097,9 +2199,14 @@ int plan_create(const napspmv_csr *A, int32_t np, int32_t ppn, uint32_t flags,
     try {
         CK(cudaGetDevice(&P->device));
         CK(cudaDeviceGetAttribute(&P->num_sms, cudaDevAttrMultiProcessorCount, P->device));
+        Scratch scratch(slab_for(A->n, A->nnz));  // outlives every temporary of the build
         build(P, A);
         P->ws = new napspmv_ws_t();
         int rc = ws_alloc(P, P->ws);
+        if (rc == NAPSPMV_ERR_OOM) {
+            scratch.trim();
+            rc = ws_alloc(P, P->ws);
+        }
         if (rc) throw NapError{rc, "workspace allocation failed"};
         P->ws->owned_by_plan = true;
         // defaults, measured on GB300 (FP64, per apply):
