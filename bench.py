@@ -172,9 +172,11 @@ def ncu_launches(csv_path):
 
 def ncu_summary(csv_path, nsteps=2, per_step=1):
     """DRAM record of one `--profile-spmv nsteps` run: the kernels after the
-    last plan-build kernel are one apply, then nsteps SpMV steps of per_step
-    launches each (FP32 values: the FP32 copy of x, then the SpMV; on the staged
-    windows, whose first launch ends the apply, as many as there are)."""
+    last plan-build kernel are one apply, and the last of them nsteps SpMV steps of
+    per_step launches each (FP32 values: the FP32 copy of x, then the SpMV; short
+    rows on the staged windows: the SpMV alone).  Between them, after an apply on
+    the windows, which its first windowed launch ends, a few steps that are not
+    counted: they may fill the receive buffers that the others sum from."""
     items = []
     for name, m in ncu_launches(csv_path):
         short = name.split("(")[0].replace("void ", "").replace("nap::", "")
@@ -182,9 +184,10 @@ def ncu_summary(csv_path, nsteps=2, per_step=1):
     first = max(j for j, (n, _) in enumerate(items) if not _APPLY_KERNELS.search(n))
     rest = items[first + 1:]
     if "k_window" in rest[-1][0]:
-        done = next(j for j, (n, _) in enumerate(rest) if "k_window" in n)
-        per_step = (len(rest) - done - 1) // nsteps
-    steps, apply_ = rest[len(rest) - nsteps * per_step:], rest[:len(rest) - nsteps * per_step]
+        per_step = 2 if "k_to_f32" in rest[-2][0] else 1
+    ends = [j + 1 for j, (n, _) in enumerate(rest) if "k_window" in n]
+    steps = rest[len(rest) - nsteps * per_step:]
+    apply_ = rest[:ends[0] if ends else len(rest) - nsteps * per_step]
     b = lambda m: m.get("dram__bytes_read.sum", 0) + m.get("dram__bytes_write.sum", 0)  # noqa: E731
     t = lambda m: m.get("gpu__time_duration.sum", 0) / 1e3  # noqa: E731
     return {
@@ -534,9 +537,9 @@ def measure(nap, torch, dev, args, cfg, precision, reps, steps, warmup, ws=1, wi
             "l2": "inputs larger than L2 (129 MB): each apply streams the matrix "
                   f"({(12 if not f32 else 8) * A.nnz / 1e6:.0f} MB of columns and values); "
                   "not flushed between steps"}
-    # messages and windows: two launches per apply (FP32 copies of x: one per step more)
-    cfgd["staged_windows"] = args.gathers == "literal" and launches in (
-        2 * reps * steps, (2 * reps + 1) * steps)
+    # (on staged windows, where the plan has them and no option names another path, the
+    # messages and the windows: two, and one a step for FP32 copies of x)
+    cfgd["launches_per_apply"] = round(launches / (reps * steps), 3)
     what = f"{precision}|{cfgd['engine']}|{cfgd['pipeline']}"
     rec = ncu_record(w.name, what)
     spmv_traffic = None if rec is None else rec.get("spmv_step_bytes")
@@ -554,13 +557,9 @@ def measure(nap, torch, dev, args, cfg, precision, reps, steps, warmup, ws=1, wi
                      "peak_kind": peak_kind, "traffic": spmv_traffic,
                      "kernel": "the three-block SpMV step (one launch = every row of one apply)",
                      "timing": f"CUDA events around {sp_n} back-to-back napspmv_spmv_step launches "
-                               "on the benchmark stream after the timed region" + (
-                                   "; inside it the overlapped engine runs the same rows as a "
-                                   "local and a remote launch" if engine == nap.ENGINE_OVERLAP
-                                   else "; inside it the apply runs the same launch"
-                                   if engine == nap.ENGINE_PHASED
-                                   else "; inside it the fused kernel's last level sums the "
-                                   "same rows"),
+                               "on the benchmark stream after the timed region and three more; "
+                               "on staged windows a step of long rows sums filled receive "
+                               "buffers and one of short rows receives again, as the apply does",
                      "algorithmic_bytes": B_spmv, "launch_ms": round(spmv_ms, 5)},
         "step_roofline": {"bound": "hbm", "achieved": round(achieved, 3), "peak": peak,
                           "frac": round(achieved / peak, 4),
@@ -658,8 +657,8 @@ def main():
                          "`--profile-spmv 2` runs, KEY = workload|precision|engine|pipeline; "
                          "no GPU needed")
     ap.add_argument("--profile-spmv", type=int, default=0,
-                    help="profiling mode: one apply, then this many SpMV-step launches; "
-                         "prints nothing")
+                    help="profiling mode: one apply, then this many SpMV steps (and two "
+                         "before them where no engine or pipeline is named); prints nothing")
     args = ap.parse_args()
     if args.ncu_record:
         write_ncu_records(args.ncu_record, os.path.join(ROOT, "profiles", "dram_traffic.json"))
@@ -693,7 +692,8 @@ def main():
         if args.precision == "f32":
             ro.engine = nap.ENGINE_PHASED
         nap.napspmv_apply_ex(plan, vd, wd, 1, 1.0, ro, stream=stream)
-        for _ in range(args.profile_spmv):
+        # (after an apply on the windows two steps first, as the timed ones have)
+        for _ in range(args.profile_spmv + 2 * (opts.engine == 0 and opts.pipeline == 0)):
             nap.napspmv_spmv_step(plan, vd, xd, 1.0, opts, stream=stream)
         stream.synchronize()
         assert nap.napspmv_status(plan, stream) == 0
@@ -710,6 +710,9 @@ def main():
         return
     w = ctx["w"]
     line = {"metric": METRIC, "value": round(main_fields["value"], 3), "unit": "GB/s",
+            "value_counts": "the bytes of the step-by-step exchange and the CSR (both arms): a "
+                            "rate of work, which the staged windows do with fewer bytes; the "
+                            "bytes that move are in apply_dram",
             "n_gpus": ws, "steps": args.steps, "warmup": args.warmup,
             "ms_per_step": round(main_fields["ms_per_step"], 4),
             "ms_per_step_median": round(main_fields["ms_per_step_median"], 4),

@@ -74,3 +74,20 @@ def test_committed_record_layout():
         assert len(key.split("|")) == 4
         assert r["apply_bytes"] > 0 and r["spmv_step_bytes"] > 0
         assert r["apply_bytes"] == sum(k["dram_read"] + k["dram_write"] for k in r["per_kernel"])
+
+
+def test_steps_after_a_windowed_apply(tmp_path):
+    """The first windowed launch ends the apply; steps between it and the last ones, which
+    settle the receive buffers, are not counted."""
+    head = [("nap::<unnamed>::k_sell_fill(const int *)", 10, 10, 100),
+            ("void nap::k_send<double, double, 1>(SendJobs)", 300, 200, 2000),
+            ("void nap::k_window_long<0, 0>(WinJob, int)", 3000, 60, 7000)]
+    spmv = ("void nap::k_spmv_s<0, 0, 8, 32>(SellView)", 3200, 80, 6000)
+    settle = [("void nap::k_window_long<0, 1>(WinJob, int)", 3100, 60, 7300),
+              ("void nap::k_receives<double, double>(const T2 *)", 900, 700, 500), spmv]
+    r = bench.ncu_summary(_log(tmp_path, head + settle + [spmv, spmv]), nsteps=2, per_step=1)
+    assert [k["kernel"] for k in r["per_kernel"]] == ["k_send<double, double, 1>", "k_window_long<0, 0>"]
+    assert r["spmv_step_kernels"] == ["k_spmv_s<0, 0, 8, 32>"] and r["spmv_step_bytes"] == 3280
+    short = ("void nap::k_window<0, double, 1, 1>(WinJobs)", 190, 10, 40)
+    r = bench.ncu_summary(_log(tmp_path, head[:2] + [short] * 5), nsteps=2, per_step=2)
+    assert len(r["per_kernel"]) == 2 and r["spmv_step_bytes"] == 200
