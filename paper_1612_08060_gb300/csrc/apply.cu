@@ -2007,23 +2007,35 @@ int ws_alloc(napspmv_plan_t *P, napspmv_ws_t *ws)
 {
     ws->plan = P;
     ws->device = P->device;
-    auto al = [](double **p, int64_t n) {
-        return cudaMalloc(p, sizeof(double) * (size_t)std::max<int64_t>(n, 1));
-    };
-    auto alf = [](float **p, int64_t n) {
-        return cudaMalloc(p, sizeof(float) * (size_t)std::max<int64_t>(n, 1));
+    // one allocation, as the plan's arrays lie in a few (see device_alloc)
+    size_t bytes = 0;
+    auto place = [&](int64_t n, size_t size) {
+        const size_t at = bytes;
+        bytes += (size * (size_t)std::max<int64_t>(n, 1) + 511) & ~(size_t)511;
+        return at;
     };
     // b_{l->l} and b_{nl->l} get 4 spare values: the remote pass copies each
     // process's segment widened to 16-byte boundaries
-    if (al(&ws->bll, P->n_bll + 4) || al(&ws->lbuf, P->n_lbuf) || al(&ws->gsend, P->n_gs) ||
-        al(&ws->grecv, P->n_gs) || al(&ws->bnl, P->n_bnl + 4) || al(&ws->xtmp, P->n) ||
-        alf(&ws->x32[0], P->n) || alf(&ws->x32[1], P->n) ||
-        cudaMalloc(&ws->ctr, sizeof(unsigned long long) * ctr_count(P)) ||
-        cudaMalloc(&ws->err, 3 * sizeof(int))) {
-        ws_free(ws);
+    const size_t words = place(ctr_count(P), sizeof(unsigned long long)), err = place(3, sizeof(int)),
+                 bll = place(P->n_bll + 4, 8), lbuf = place(P->n_lbuf, 8), gsend = place(P->n_gs, 8),
+                 grecv = place(P->n_gs, 8), bnl = place(P->n_bnl + 4, 8), xtmp = place(P->n, 8),
+                 x0 = place(P->n, 4), x1 = place(P->n, 4);
+    if (cudaMalloc(&ws->mem, bytes)) {
+        ws->mem = nullptr;
         return cuda_error(cudaErrorMemoryAllocation, "workspace");
     }
+    char *m = static_cast<char *>(ws->mem);
+    ws->ctr = reinterpret_cast<unsigned long long *>(m + words);
+    ws->err = reinterpret_cast<int *>(m + err);
     ws->state = ws->err + 1;
+    ws->bll = reinterpret_cast<double *>(m + bll);
+    ws->lbuf = reinterpret_cast<double *>(m + lbuf);
+    ws->gsend = reinterpret_cast<double *>(m + gsend);
+    ws->grecv = reinterpret_cast<double *>(m + grecv);
+    ws->bnl = reinterpret_cast<double *>(m + bnl);
+    ws->xtmp = reinterpret_cast<double *>(m + xtmp);
+    ws->x32[0] = reinterpret_cast<float *>(m + x0);
+    ws->x32[1] = reinterpret_cast<float *>(m + x1);
     if (cudaMemset(ws->err, 0, 3 * sizeof(int)) != cudaSuccess) {
         ws_free(ws);
         return cuda_error(cudaGetLastError(), "workspace");
@@ -2033,10 +2045,10 @@ int ws_alloc(napspmv_plan_t *P, napspmv_ws_t *ws)
 
 void ws_free(napspmv_ws_t *ws)
 {
-    void *p[] = {ws->bll, ws->lbuf, ws->gsend, ws->grecv, ws->bnl, ws->xtmp, ws->hv, ws->hw,
-                 ws->ctr, ws->err, ws->x32[0], ws->x32[1]};
+    void *p[] = {ws->mem, ws->hv, ws->hw};
     for (void *q : p)
         if (q) cudaFree(q);
+    ws->mem = nullptr;
     ws->bll = ws->lbuf = ws->gsend = ws->grecv = ws->bnl = ws->xtmp = ws->hv = ws->hw = nullptr;
     ws->x32[0] = ws->x32[1] = nullptr;
     ws->ctr = nullptr;

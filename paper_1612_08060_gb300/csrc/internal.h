@@ -166,6 +166,7 @@ struct WinPart {
 struct napspmv_ws_s {
     napspmv_plan_t *plan = nullptr;
     int device = 0;
+    void *mem = nullptr;  // what the buffers below (but hv, hw) lie in
     double *bll = nullptr, *lbuf = nullptr, *gsend = nullptr, *grecv = nullptr, *bnl = nullptr;
     double *xtmp = nullptr;            // chained-apply intermediate vector
     // FP32 mode of the phased engines: FP32 copies of the chain's vectors, and
@@ -194,6 +195,12 @@ struct napspmv_plan_s {
     int32_t np = 0, ppn = 0, nn = 0;
     uint32_t flags = 0;
     int num_sms = 0;
+
+    struct Block {  // device memory that arrays of the plan lie in
+        char *p;
+        size_t bytes, used;
+    };
+    std::vector<Block> blocks;
 
     nap::HostList lists[nap::L_COUNT];
     std::vector<int32_t> send_proc, recv_proc;  // per NODE pair
