@@ -267,8 +267,9 @@ int napspmv_apply_ex(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, doubl
 /* The three-block SpMV step alone (the three local_spmv calls of Algorithm
  * NAPSpMV, Sec. 4): w <- scale (A_on_process v + A_on_node b_{l->l} +
  * A_off_node b_{nl->l}) with the receive buffers the workspace (NULL = the
- * plan's own) holds from its last apply.  For measuring the step on its own;
- * after an apply of v it reproduces that apply's w.  Asynchronous. */
+ * plan's own) holds from its last apply (for a captured step: the last apply
+ * that ran before each replay).  For measuring the step on its own; after an
+ * apply of v it reproduces that apply's w.  Asynchronous. */
 int napspmv_spmv_step(napspmv_plan_t *P, napspmv_ws_t *ws, const double *v, double *w,
                       double scale, const napspmv_opts *opts, void *stream);
 
@@ -396,10 +397,11 @@ int napspmv_cg(napspmv_plan_t *P, const double *b, double *x, double rtol, int32
  * the call: its dot products use a partition fixed by its own N (one block
  * per 1,024 values, at most 4,096) and a fixed-order final sum, and its
  * products run with its own plan's default options (slots whose options
- * differ go into separate fused launches). */
+ * differ go into separate launches). */
 /* Slots (and served SpMV requests) whose matrix holds at least this many
- * stored entries are applied on their own with the phased engine: there one
- * product costs less than its share of a fused-engine launch. */
+ * stored entries get products of their own where a call's slots do not all run
+ * on the windows of short rows: there one product costs less than its share of
+ * a fused-engine launch. */
 #define NAPSPMV_SOLO_NNZ (1ll << 19)
 
 typedef struct {
@@ -419,10 +421,12 @@ int napspmv_cg_batch_init(int32_t count, const napspmv_cg_slot *slots, int32_t p
 /* `iters` CG iterations for every slot: q = A p, alpha = r.r / p.q,
  * x += alpha p, r -= alpha q, beta = r.r_new / r.r, p = r + beta p.
  * Asynchronous; the caller reads scal[0] to decide convergence.
- * The products q = A p (and r = b - A x of napspmv_cg_batch_init): slots whose
- * matrix holds at least NAPSPMV_SOLO_NNZ stored entries are applied one by one
- * on the phased engine, the others together in one fused-engine launch.  The
- * choice depends on the slot's own matrix, not on the rest of the batch. */
+ * The products q = A p (and r = b - A x of napspmv_cg_batch_init): where all
+ * slots' plans run on the windows of short rows, two or more iterations share
+ * their windowed launches, whatever their sizes.  Otherwise slots whose matrix
+ * holds at least NAPSPMV_SOLO_NNZ stored entries are applied one by one, the
+ * others as napspmv_apply_batch applies them.  A slot's bits are the same on
+ * every one of these paths, so they do not depend on the rest of the batch. */
 int napspmv_cg_batch_iterate(int32_t count, const napspmv_cg_slot *slots, int32_t precision,
                              int32_t iters, void *stream);
 

@@ -2012,7 +2012,7 @@ void add_windows(napspmv_plan_t *P)
 // tiles one after another, each as many rows as fit tile_rows rows and tile_nnz
 // entries (a longer single row alone).  Cutting the seven lists on the host, row by
 // row, took 5.1 of 17.6 ms of a 10^6-row 7-point plan, and their three row pointers
-// 0.8 ms to bring there; this way 0.65 ms (GB300).
+// 0.8 ms to bring there; this way 0.47 ms (GB300).
 namespace {
 constexpr int kSegment = 16384, kStaged = 1024;
 struct TileCut {
