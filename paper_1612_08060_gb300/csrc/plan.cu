@@ -118,7 +118,7 @@ thread_local Scratch *Scratch::current = nullptr;
 // small or medium plan lie together in a few blocks: fewer allocations, and fewer pages
 // for its kernels (a fused apply of 64 x 64 rows, spread among the build's temporaries,
 // took 26.3 us for 25.1; GB300).
-constexpr size_t kBlockMax = 128 << 20, kBlockMin = 2 << 20;
+constexpr size_t kBlockMax = 128 << 20;
 template <class T>
 cudaError_t device_alloc(T **p, size_t bytes)
 {
@@ -137,7 +137,7 @@ cudaError_t device_alloc(T **p, size_t bytes)
     if (room && bytes <= room) {
         auto &B = S->plan->blocks;
         if (B.empty() || B.back().used + bytes > B.back().bytes) {
-            const size_t want = B.empty() ? room : std::max(room / 8, std::max(bytes, kBlockMin));
+            const size_t want = B.empty() ? room : std::max(room / 8, bytes);
             void *q = nullptr;
             if (get(&q, want) == cudaSuccess) B.push_back({static_cast<char *>(q), want, 0});
             else cudaGetLastError();
@@ -246,8 +246,9 @@ struct Part {
 };
 size_t block_room(const napspmv_plan_t *P)
 {
-    const size_t b = (size_t)((P->flags & NAPSPMV_F32_VALUES ? 80 : 60) * P->nnz + 64 * P->n);
-    return b <= kBlockMax ? std::max(b, kBlockMin) : 0;
+    // some sixty arrays, each on a 512-byte boundary
+    const size_t b = (size_t)((P->flags & NAPSPMV_F32_VALUES ? 80 : 60) * P->nnz + 64 * P->n) + (48 << 10);
+    return b <= kBlockMax ? b : 0;
 }
 // About what a build's temporaries take (see Scratch).
 size_t slab_for(int64_t n, int64_t nnz) { return (size_t)(64 * nnz + 64 * n); }
