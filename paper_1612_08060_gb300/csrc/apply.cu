@@ -3299,8 +3299,7 @@ extern "C" int napspmv_apply_noalloc(napspmv_plan_t *P, const double *v, double 
 // (us per step on GB300 with FP64 values, windows / buffers, and with FP32 ones: 5 * 10^4
 // rows of 20 entries 9.4 / 14.6 and 18.3 / 18.8, 2.5 * 10^5 24.6 / 24.8 and 37 / 29, 10^6
 // 82 / 75 and 97 / 71, 4 * 10^6 378 / 303 and 338 / 246).  Above that the second step
-// after an apply (with FP32 values, whose apply gained less, the first) fills the
-// buffers, and it and those that follow sum from there.
+// after an apply fills the buffers, and it and those that follow sum from there.
 namespace nap {
 constexpr int64_t kStepFill64 = 6000000, kStepFill32 = 2000000;  // stored entries
 }
@@ -3344,8 +3343,7 @@ extern "C" int napspmv_spmv_step(napspmv_plan_t *P, napspmv_ws_t *ws, const doub
     const bool kept = W->recv_vector && !W->captured;
     // the FP32 copy that an apply of long rows made of its vector first is there too
     const bool copy32 = kept && f32 && W->recv_f32 && P->win.long_rows;
-    const bool fill = P->win.long_rows && P->nnz >= (f32 ? kStepFill32 : kStepFill64) &&
-                      (f32 || W->stepped);
+    const bool fill = P->win.long_rows && P->nnz >= (f32 ? kStepFill32 : kStepFill64) && W->stepped;
     if (o.window && kept && W->recv_f32 == f32 && !fill) {
         // on the windows: on-node receives from the kept vector, off-node from g_recv
         const void *x = v, *l = W->xtmp;
