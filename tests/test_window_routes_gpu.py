@@ -78,9 +78,10 @@ FUSED = dict(engine=nap.ENGINE_FUSED)
 
 
 def short_or_long(mat):
-    """A plan of short rows, or of long rows whose far messages the windows reorder."""
-    if mat == "short":
-        return gpu_plan(I.poisson3d(18), 7, 3)
+    """A plan of short rows (without inter-node messages; without any), or of long rows whose
+    far messages the windows reorder."""
+    if mat != "long":
+        return gpu_plan(I.poisson3d(18), *{"short": (7, 3), "one node": (7, 7), "one process": (1, 1)}[mat])
     return gpu_plan(near_and_far(300 * 80 + 1, 700, 1, 300), 80, 1)
 
 
@@ -110,7 +111,7 @@ def paths(prec):  # (the fused engine leaves FP64 receives, which an FP32 step r
 
 
 @pytest.mark.parametrize("prec", [nap.PREC_F64, nap.PREC_F32])
-@pytest.mark.parametrize("mat", ["short", "long"])
+@pytest.mark.parametrize("mat", ["short", "long", "one node", "one process"])
 def test_captured_step_takes_the_receives_of_the_apply_before_the_replay(mat, prec):
     S = Steps(mat, prec)
     x = [vec(S.plan.n, 30 + k) for k in range(2)]
@@ -134,7 +135,7 @@ def test_captured_step_takes_the_receives_of_the_apply_before_the_replay(mat, pr
 
 
 @pytest.mark.parametrize("prec", [nap.PREC_F64, nap.PREC_F32])
-@pytest.mark.parametrize("mat", ["short", "long"])
+@pytest.mark.parametrize("mat", ["short", "long", "one node", "one process"])
 def test_step_after_a_capture_that_did_not_run(mat, prec):
     """An apply that was captured and not replayed changes no receives, whatever ran before."""
     S = Steps(mat, prec)
