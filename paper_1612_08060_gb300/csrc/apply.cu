@@ -1572,7 +1572,7 @@ __global__ void __launch_bounds__(1024, 1)
 // 2^23-row banded matrix, 162 in index order and 205 with the far messages in the order
 // that the windows gain from.
 // The copy of x that a later napspmv_spmv_step takes the on-node receives from
-// (SendJob::keep) is made by further CTAs of the same launch.
+// (SendJob::keep) is made, and the device word written, by further CTAs of the launch.
 constexpr int kSendWarps = NT / 32;
 struct SendJob {
     const void *x;
@@ -1609,10 +1609,9 @@ __global__ void __launch_bounds__(NT) k_send(const __grid_constant__ SendJobs<MA
     const XS *x = static_cast<const XS *>(J.x);
     T *grecv = static_cast<T *>(J.grecv);
     const int block = (int)blockIdx.x - J.block0, n = J.n_gs;
-    const bool tells = J.state && block == J.blocks - 1 && threadIdx.x == 0;
     if (block >= J.send_blocks) {
         griddep_wait();
-        if (tells) *J.state = J.value;
+        if (J.state && block == J.send_blocks && threadIdx.x == 0) *J.state = J.value;
         if (J.keep)
             for (int64_t i = (int64_t)(block - J.send_blocks) * NT + threadIdx.x; i < J.n;
                  i += (int64_t)(J.blocks - J.send_blocks) * NT)
@@ -1647,10 +1646,6 @@ __global__ void __launch_bounds__(NT) k_send(const __grid_constant__ SendJobs<MA
 #pragma unroll
         for (int u = 0; u < U; u++)
             if (b + 32 * u + lane < n) grecv[to[u]] = v[u];
-    }
-    if (tells) {
-        griddep_wait();
-        *J.state = J.value;
     }
     griddep_done();
 }
@@ -2522,7 +2517,11 @@ static int64_t enqueue_send(const napspmv_plan_t *P, const T *x, T *grecv, int *
     SendJobs<1> S{};
     S.n = 1;
     S.job[0] = send_job(P, sizeof(T) == 4, false, x, grecv, err);
-    S.job[0].state = state;
+    if (state) {  // by a CTA of its own: written by a sending one, after its messages, the
+                  // word lengthened every launch, a 64 x 64 grid's chained apply 3.77 us for 3.65
+        S.job[0].state = state;
+        S.job[0].blocks++;
+    }
     launch_pdl(pdl, k_send<T, T, 1>, S.job[0].blocks, 0, s, S);
     return 1;
 }
